@@ -175,6 +175,8 @@ int upload_schedule(pselinv_handle* h) {
     }
   if ((rc = upload(h, &h->d_meta, h->meta))) return rc;
   std::vector<psi::Task> all;
+  h->off_norm = (int64_t)all.size();
+  all.insert(all.end(), h->t_norm.tasks.begin(), h->t_norm.tasks.end());
   h->off_lhat = (int64_t)all.size();
   all.insert(all.end(), h->t_lhat.tasks.begin(), h->t_lhat.tasks.end());
   h->off_gemm1 = (int64_t)all.size();
@@ -224,7 +226,7 @@ int enqueue_persistent(pselinv_handle* h, cudaStream_t st) {
   psi::KArgs a = kargs(h);
   const int64_t B = h->opts.batch;
   PSI_CUDA(h, cudaMemsetAsync(h->d_pctr, 0, sizeof(int) * (4 * B * h->nsn + h->nlevels + 1), st));
-  PSI_CUDA(h, psi::launch_per_sn(psi::Kern::NormDiag, a, nullptr, h->nsn, st));
+  PSI_CUDA(h, psi::launch_tiles(psi::Kern::NormM, 0, a, tasks_at(h, h->off_norm, 0), (int64_t)h->t_norm.tasks.size(), st));
   for (int v = 0; v < psi::kNumVar; ++v) {
     const psi::Range r = h->t_lhat.whole[v];
     PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
@@ -372,7 +374,8 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
   psi::KArgs a3 = a;                                  // step 3: Uhat_{K,C} X_{C,K}
   if (unsym) a3.Lhat = h->d_uhat;
   rc = tm.run(0, (1 + nlhat_launch) * (unsym ? 2 : 1) - (unsym ? 1 : 0), [&] {
-    cudaError_t e = psi::launch_per_sn(unsym ? Kern::NormDiagLU : Kern::NormDiag, a, nullptr, h->nsn, st);
+    cudaError_t e = psi::launch_tiles(Kern::NormM, 0, a, tasks_at(h, h->off_norm, 0),
+                                      (int64_t)h->t_norm.tasks.size(), st);
     for (int side = 0; side < (unsym ? 2 : 1); ++side)
       for (int v = 0; v < psi::kNumVar && e == cudaSuccess; ++v) {
         const psi::Range r = h->t_lhat.whole[v];
@@ -1175,15 +1178,10 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   a.W1 = h->d_w1;
   a.Yb = h->d_yb;
   a.Hb = h->d_hb;
-  // recompute (L_KK)^{-1} and Lhat from L (step 1) instead of trusting stored copies
-  {
-    psi::KArgs na = a.k;
-    na.X = nullptr;
-    PSI_CUDA(h, psi::launch_per_sn(psi::Kern::NormDiag, na, nullptr, h->nsn, st));
-    for (int v = 0; v < psi::kNumVar; ++v) {
-      const psi::Range r = h->t_lhat.whole[v];
-      PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, na, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
-    }
+  // recompute Lhat = L_CK (L_KK)^{-1} from the factor (step 1) instead of trusting a stored copy
+  for (int v = 0; v < psi::kNumVar; ++v) {
+    const psi::Range r = h->t_lhat.whole[v];
+    PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a.k, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
   }
   PSI_CUDA(h, cudaMemsetAsync(h->d_lb, 0, B * h->panel_total * es, st));
   PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));
@@ -1386,7 +1384,7 @@ int pselinv_get_info(const pselinv_handle* h, pselinv_info* info) {
   // device memory held now (the autotuner reallocates the schedule buffers)
   if (h->dev_sym) {
     const int64_t B = h->opts.batch, es = (int64_t)elem_size(h), tasks =
-        (int64_t)(h->t_lhat.tasks.size() + h->t_gemm1.tasks.size() + h->t_gemm2.tasks.size() +
+        (int64_t)(h->t_norm.tasks.size() + h->t_lhat.tasks.size() + h->t_gemm1.tasks.size() + h->t_gemm2.tasks.size() +
                   h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_rect.tasks.size() +
                   h->t_pgemm1.tasks.size() + h->t_pgemm2.tasks.size() + h->t_sq.tasks.size());
     int64_t bytes = (int64_t)(sizeof(psi::SnMeta) * h->meta.size() + sizeof(psi::ColDesc) * h->desc.size() +

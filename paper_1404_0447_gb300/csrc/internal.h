@@ -141,7 +141,8 @@ struct pselinv_handle {
   double flops_selinv = 0, flops_gemm1 = 0, bytes_selinv = 0;
 
   // task lists (levels in priority order; supernodes of a level costliest first)
-  psi::TaskList t_lhat;   // normalisation tiles (all supernodes)
+  psi::TaskList t_norm;   // normalisation: s x s tiles of M_K (all supernodes, 64 x 8)
+  psi::TaskList t_lhat;   // normalisation: r x s tiles of Lhat (all supernodes)
   psi::TaskList t_gemm1;  // step 2 tiles (with k-slices of split supernodes)
   psi::TaskList t_rect;   // r x s tiles per level, unsplit (adjoint)
   psi::TaskList t_gemm2;  // step 3 partial-product tiles
@@ -175,7 +176,7 @@ struct pselinv_handle {
   void* d_diagmask = nullptr;
   void* d_flipmap = nullptr;
   void* d_tasks = nullptr;  // all task arrays back to back
-  int64_t off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
+  int64_t off_norm = 0, off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
   int64_t off_pgemm1 = 0, off_pgemm2 = 0, off_sq = 0;
   void* d_levelsn = nullptr;
   void* d_L = nullptr;      // L panels (unit diagonal implied; D on the diagonal slots)

@@ -317,123 +317,6 @@ __global__ void k_factor_diag_lu(const SnMeta* __restrict__ meta, const int32_t*
   for (int j = t; j < s; j += nt) D[b * sz.n + m.f + j] = Tl[pk(j, j, s)];
 }
 
-// Normalisation of a non-symmetric diagonal block (all supernodes, one CTA
-// each): Vl = (L_KK)^{-1} -> linv, Vu = (U'_KK^T)^{-1} -> uinv, and the
-// first term of step 3, U_KK^{-1} L_KK^{-1} = U'_KK^{-1} D_K^{-1} L_KK^{-1}
-// = Vu^T D_K^{-1} Vl, to the full diagonal block of the X panel.
-template <class T>
-__global__ void k_norm_diag_lu(const SnMeta* __restrict__ meta, const T* __restrict__ L, const T* __restrict__ U,
-                               const T* __restrict__ D, T* __restrict__ Linv, T* __restrict__ Uinv,
-                               T* __restrict__ X, Sizes sz) {
-  extern __shared__ __align__(16) unsigned char shraw[];
-  T* Tp = reinterpret_cast<T*>(shraw);
-  const int k = blockIdx.x;
-  const int b = blockIdx.y;
-  const SnMeta m = meta[k];
-  const int s = m.s, ld = m.s + m.r;
-  const T* d = D + b * sz.n + m.f;
-  T* rd = Tp + s * (s + 1) / 2;
-  const int nt = blockDim.x, t = threadIdx.x;
-  T* Vl = Linv + b * sz.linv + m.linv;
-  T* Vu = Uinv + b * sz.linv + m.linv;
-  for (int side = 0; side < 2; ++side) {
-    const T* P = (side == 0 ? L : U) + b * sz.panel + m.panel;
-    for (int e = t; e < s * s; e += nt) {
-      const int i = e % s, j = e / s;
-      if (i > j) Tp[pk(i, j, s)] = P[i + (int64_t)j * ld];
-    }
-    __syncthreads();
-    unit_lower_inverse(Tp, s, side == 0 ? Vl : Vu);
-    __syncthreads();
-  }
-  for (int q = t; q < s; q += nt) rd[q] = Sc<T>::one() / d[q];
-  __syncthreads();
-  T* XK = X + b * sz.panel + m.panel;
-  for (int e = t; e < s * s; e += nt) {
-    const int i = e % s, j = e / s;
-    T acc = Sc<T>::zero();
-    for (int q = i > j ? i : j; q < s; ++q) acc += Vu[q + i * s] * rd[q] * Vl[q + j * s];
-    XK[i + (int64_t)j * ld] = acc;
-  }
-}
-
-// Normalisation, diagonal part (all supernodes, one CTA each):
-// (L_KK)^{-1} -> linv and M_K = L_KK^{-T} D_K^{-1} L_KK^{-1} -> the diagonal
-// block of the X panel (Algorithm 1 step 3's first term; U_KK = D_K L_KK^T).
-// A pivoted factor (ptype set): D_K has 2x2 blocks, so row q of D_K^{-1} V is
-// c_q V_q + c'_q V_{q'} with q' the 2x2 partner, and M_K goes to the original
-// columns (P(i), P(j)).
-template <class T>
-__global__ void k_norm_diag(const SnMeta* __restrict__ meta, const T* __restrict__ L, const T* __restrict__ D,
-                            T* __restrict__ Linv, T* __restrict__ X, Sizes sz, const int32_t* __restrict__ piv,
-                            const int8_t* __restrict__ ptype, const T* __restrict__ E) {
-  extern __shared__ __align__(16) unsigned char shraw[];
-  T* Tp = reinterpret_cast<T*>(shraw);
-  const int k = blockIdx.x;
-  const int b = blockIdx.y;
-  const SnMeta m = meta[k];
-  const int s = m.s, ld = m.s + m.r;
-  const T* P = L + b * sz.panel + m.panel;
-  const T* d = D + b * sz.n + m.f;
-  T* rd = Tp + s * (s + 1) / 2;  // 1 / d_q, or the own coefficient of a 2x2 row
-  T* rp = rd + s;                // partner coefficient (0 for a 1x1 pivot)
-  int* pq = reinterpret_cast<int*>(rp + s);
-  const int nt = blockDim.x, t = threadIdx.x;
-  for (int e = t; e < s * s; e += nt) {
-    const int i = e % s, j = e / s;
-    if (i > j) Tp[pk(i, j, s)] = P[i + (int64_t)j * ld];
-  }
-  if (ptype) {
-    const int8_t* ty = ptype + b * sz.n + m.f;
-    const T* ee = E + b * sz.n + m.f;
-    for (int q = t; q < s; q += nt) {
-      if (ty[q] == 0) {
-        rd[q] = Sc<T>::one() / d[q];
-        rp[q] = Sc<T>::zero();
-        pq[q] = q;
-      } else {
-        const int f0 = ty[q] == 1 ? q : q - 1;  // first column of the 2x2 block
-        const T det = d[f0] * d[f0 + 1] - ee[f0] * ee[f0];
-        const int o = ty[q] == 1 ? q + 1 : q - 1;
-        rd[q] = d[o] / det;
-        rp[q] = -ee[f0] / det;
-        pq[q] = o;
-      }
-    }
-  } else {
-    for (int q = t; q < s; q += nt) rd[q] = Sc<T>::one() / d[q];
-  }
-  __syncthreads();
-  T* V = Linv + b * sz.linv + m.linv;
-  unit_lower_inverse(Tp, s, V);
-  if (!X) return;  // inverse only (the adjoint recomputes it)
-  __syncthreads();
-  T* XK = X + b * sz.panel + m.panel;
-  if (ptype) {
-    const int32_t* pv = piv + b * sz.n + m.f;
-    for (int e = t; e < s * s; e += nt) {
-      const int i = e % s, j = e / s;
-      if (i >= j) {
-        T acc = Sc<T>::zero();
-        for (int q = i; q < s; ++q)  // V_qi = 0 for q < i; row q of D^{-1} V vanishes in column j <= i below j - 1
-          acc += V[q + i * s] * (rd[q] * V[q + j * s] + rp[q] * V[pq[q] + j * s]);
-        XK[pv[i] + (int64_t)pv[j] * ld] = acc;
-        XK[pv[j] + (int64_t)pv[i] * ld] = acc;
-      }
-    }
-    return;
-  }
-  for (int e = t; e < s * s; e += nt) {
-    const int i = e % s, j = e / s;
-    if (i >= j) {
-      T acc = Sc<T>::zero();
-      for (int q = i; q < s; ++q) acc += V[q + i * s] * rd[q] * V[q + j * s];
-      XK[i + (int64_t)j * ld] = acc;
-      XK[j + (int64_t)i * ld] = acc;
-    }
-  }
-}
-
 // |re| + |im|: the magnitude Bunch-Kaufman compares (plain |x| for real)
 __device__ __forceinline__ double bk_abs(double x) { return fabs(x); }
 __device__ __forceinline__ double bk_abs(Cplx x) { return fabs(x.re) + fabs(x.im); }
@@ -841,6 +724,95 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
   });
 }
 
+// Normalisation, diagonal part: M_K = L_KK^{-T} D_K^{-1} L_KK^{-1} = V^T (D_K^{-1} V)
+// with V = (L_KK)^{-1} from the factorisation, into the diagonal block of the
+// X panel (Algorithm 1 step 3's first term; U_KK = D_K L_KK^T), one 64 x 8
+// tile of s x s per CTA over all supernodes; V is lower triangular, so only
+// k >= max(m0, n0) contributes, and the symmetric forms compute the lower
+// triangle and mirror it.
+// MODE 1, pivoted factor: D_K has 2 x 2 blocks, so row q of D_K^{-1} V is
+// c_q V_q + c'_q V_{q'} with q' the 2 x 2 partner, and M_K goes to the
+// original columns (P(i), P(j)).
+// MODE 2, non-symmetric: U_KK^{-1} L_KK^{-1} = U'_KK^{-1} D_K^{-1} L_KK^{-1} =
+// Vu^T D_K^{-1} Vl, every entry of the block.
+// Bound: the FP64 pipe (2/3 s^3 flops per supernode).  It replaces a kernel of
+// one CTA per supernode that inverted L_KK again, one column per thread (a
+// serial chain of dependent loads through L1, 1.0 to 1.7 ms a pass on
+// problems with a 128-wide supernode whatever their size).
+template <class T, int MODE>
+__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, 8>())) k_norm_m(KArgs a, const Task* __restrict__ tasks) {
+  constexpr int BN = 8;
+  __shared__ TileSmem<T, BN> sm;
+  __shared__ double coef[(MODE == 1 ? 2 : 1) * kMaxWidth * Sc<T>::P];  // 1 / d_q, or the own coefficient of a 2 x 2 row; partners after
+  __shared__ int pq[MODE == 1 ? kMaxWidth : 1];
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y;
+  const SnMeta m = a.meta[tk.sn];
+  const int s = m.s, ld = m.s + m.r;
+  const T* V = (const T*)a.Linv + b * a.sz.linv + m.linv;
+  const T* Vm = MODE == 2 ? (const T*)a.Uinv + b * a.sz.linv + m.linv : V;
+  const T* d = (const T*)a.D + b * a.sz.n + m.f;
+  T* rd = reinterpret_cast<T*>(coef);
+  T* rp = rd + (MODE == 1 ? kMaxWidth : 0);
+  const int q0 = max(tk.m0, tk.n0);  // V_qi = 0 for q < i
+  for (int q = q0 + threadIdx.x; q < s; q += TG_THREADS) {
+    if constexpr (MODE == 1) {
+      const int8_t* ty = a.ptype + b * a.sz.n + m.f;
+      const T* ee = (const T*)a.E + b * a.sz.n + m.f;
+      if (ty[q] == 0) {
+        rd[q] = Sc<T>::one() / d[q];
+        rp[q] = Sc<T>::zero();
+        pq[q] = q;
+      } else {
+        const int f0 = ty[q] == 1 ? q : q - 1;  // first column of the 2 x 2 block
+        const T det = d[f0] * d[f0 + 1] - ee[f0] * ee[f0];
+        const int o = ty[q] == 1 ? q + 1 : q - 1;
+        rd[q] = d[o] / det;
+        rp[q] = -ee[f0] / det;
+        pq[q] = o;
+      }
+    } else {
+      rd[q] = Sc<T>::one() / d[q];
+    }
+  }
+  __syncthreads();
+  Acc<T, BN> acc;
+  acc_zero<T, BN>(acc);
+  auto la = [&](int mm, int q) {
+    const int i = tk.m0 + mm;
+    return i < s ? Vm[q + i * s] : Sc<T>::zero();
+  };
+  auto lb = [&](int q, int nn) -> T {
+    const int j = tk.n0 + nn;
+    if (j >= s) return Sc<T>::zero();
+    if constexpr (MODE == 1) return rd[q] * V[q + j * s] + rp[q] * V[pq[q] + j * s];
+    return rd[q] * V[q + j * s];
+  };
+  const int dm = tk.m0 - tk.n0;
+  // a 2 x 2 pivot whose first column is q0 - 1 has its second row at q0: row q0 - 1
+  // of D^{-1} V meets V_{q0-1,i} = 0, so the range still starts at q0
+  tile_mma<T, BN>(sm, q0, s, [](int) { return true; }, la, lb, acc, [&](int r0, int c0) {
+    return tk.m0 + r0 < s && tk.n0 + c0 < s && (MODE == 2 || c0 <= dm + r0 + 7);
+  });
+  T* XK = (T*)a.X + b * a.sz.panel + m.panel;
+  tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
+    int i = tk.m0 + mm, j = tk.n0 + nn;
+    if (i >= s || j >= s) return;
+    if constexpr (MODE == 2) {
+      XK[i + (int64_t)j * ld] = v;
+    } else {
+      if (i < j) return;
+      if constexpr (MODE == 1) {
+        const int32_t* pv = a.piv + b * a.sz.n + m.f;
+        i = pv[i];
+        j = pv[j];
+      }
+      XK[i + (int64_t)j * ld] = v;
+      XK[j + (int64_t)i * ld] = v;
+    }
+  });
+}
+
 // Normalisation, off-diagonal part: Lhat_{C,K} = L_{C,K} (L_KK)^{-1}.
 template <class T, int BN>
 __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_lhat(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
@@ -1040,12 +1012,6 @@ static cudaError_t setup_t() {
   cudaError_t e = cudaFuncSetAttribute(k_factor_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)diag_smem_fd<T>(kMaxWidth));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_norm_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)diag_smem<T>(kMaxWidth));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_norm_diag_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)diag_smem<T>(kMaxWidth));
-  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)diag_smem_bk<T>(kMaxWidth));
   if (e == cudaSuccess)
@@ -1133,6 +1099,17 @@ static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cu
     case Kern::Lhat:
       k_lhat<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, (T*)a.Lhat, a.sz);
       break;
+    case Kern::NormM:
+      if constexpr (BN == 8) {
+        if (a.Uinv)
+          k_norm_m<T, 2><<<grid, TG_THREADS, 0, st>>>(a, t);
+        else if (a.ptype)
+          k_norm_m<T, 1><<<grid, TG_THREADS, 0, st>>>(a, t);
+        else
+          k_norm_m<T, 0><<<grid, TG_THREADS, 0, st>>>(a, t);
+        break;
+      }
+      return cudaErrorInvalidValue;  // the list holds 64 x 8 tiles only
     case Kern::Gemm1:
       if (a.XU)
         k_gemm1<T, BN, true><<<grid, TG_THREADS, 0, st>>>(a, t);
@@ -1175,10 +1152,6 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
     case Kern::CopyBack:
       k_copyback<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.Lhat, a.sz);
       break;
-    case Kern::NormDiag:  // every supernode: blockIdx.x is the supernode itself
-      k_norm_diag<T><<<grid, 256, diag_smem<T>(a.maxw), st>>>(a.meta, (const T*)a.L, (const T*)a.D, (T*)a.Linv,
-                                                              (T*)a.X, a.sz, a.piv, a.ptype, (const T*)a.E);
-      break;
     case Kern::Gemm1Reduce:
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);
       break;
@@ -1193,11 +1166,6 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
     case Kern::CopyBackBK:
       k_copyback_bk<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (T*)a.Lhat, (const T*)a.D,
                                                                   (const T*)a.E, a.ptype, a.sz);
-      break;
-    case Kern::NormDiagLU:
-      k_norm_diag_lu<T><<<grid, 256, diag_smem<T>(a.maxw), st>>>(a.meta, (const T*)a.L, (const T*)a.U,
-                                                                 (const T*)a.D, (T*)a.Linv, (T*)a.Uinv,
-                                                                 (T*)a.X, a.sz);
       break;
     default:
       // 32 CTAs per supernode: the levels near the root hold one supernode whose

@@ -19,8 +19,8 @@ struct Sizes {
 };
 
 enum class Kern {
-  Trsm, Schur, Lhat, Gemm1, Gemm2, FactorDiag, CopyBack, NormDiag, DiagFinal, Gemm1Reduce,
-  FactorDiagLU, NormDiagLU,  // non-symmetric diagonal blocks
+  Trsm, Schur, NormM, Lhat, Gemm1, Gemm2, FactorDiag, CopyBack, DiagFinal, Gemm1Reduce,
+  FactorDiagLU,              // non-symmetric diagonal blocks
   FactorDiagBK, CopyBackBK   // Bunch-Kaufman pivoted factor
 };
 
@@ -93,11 +93,11 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
 // diagmask == nullptr: plain gather; else off-diagonal entries doubled.
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
                                  void* out, const Sizes& sz, cudaStream_t st);
-// Tile kernels (Trsm, Schur, Lhat, Gemm1, Gemm2) over n tasks of one tile
+// Tile kernels (Trsm, Schur, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
 cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st);
-// Per-supernode kernels (FactorDiag, CopyBack, NormDiag, DiagFinal, Gemm1Reduce) over the
-// nsn supernodes listed in sns (NormDiag: supernodes 0..nsn-1, sns unused).
+// Per-supernode kernels (FactorDiag, CopyBack, DiagFinal, Gemm1Reduce) over the
+// nsn supernodes listed in sns.
 // threads: block size of the diagonal-factorisation kernels (FactorDiag,
 // FactorDiagLU, FactorDiagBK -- the last capped at 512); the others use 256.
 cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads = 256);

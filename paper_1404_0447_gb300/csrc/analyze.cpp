@@ -640,6 +640,38 @@ int build_schedule(pselinv_handle* h) {
   build(h->t_gemm1, false, [&](int32_t k) { return (int)h->s2var[k]; }, step2_tiles);
   build(h->t_trsm, false, [&](int32_t k) { return (int)h->trvar[k]; }, rect);
   build(h->t_gemm2, false, [&](int32_t k) { return (int)h->s3var[k]; }, step3_tiles);
+  {
+    h->fb_sn.clear();
+    h->fb_range.assign((size_t)nl * kFactorBlocks, Range{});
+    TaskList &tp = h->t_fpanel, &tu = h->t_fupdate, &tv = h->t_vinv;
+    for (TaskList* tl : {&tp, &tu, &tv}) {
+      tl->tasks.clear();
+      tl->per_lv.assign((size_t)nl * kFactorBlocks, Range{});
+    }
+    for (int32_t l = 0; l < nl; ++l)
+      for (int p = 0; p < kFactorBlocks; ++p) {
+        const size_t at = (size_t)l * kFactorBlocks + p;
+        h->fb_range[at].begin = (int64_t)h->fb_sn.size();
+        tp.per_lv[at].begin = (int64_t)tp.tasks.size();
+        tu.per_lv[at].begin = (int64_t)tu.tasks.size();
+        for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
+          const int32_t k = h->level_sn[t];
+          const SnMeta& m = h->meta[k];
+          const int32_t c0 = p * kFactorBlock, c1 = std::min(m.s, c0 + kFactorBlock), ld = m.s + m.r;
+          if (m.s <= c0) continue;
+          h->fb_sn.push_back(k);
+          for (int32_t m0 = c1; m0 < ld; m0 += kTileM)
+            for (int32_t n0 = c0; n0 < c1; n0 += 8) tp.tasks.push_back({k, m0, n0, p});
+          for (int32_t n0 = c1; n0 < m.s; n0 += 8)
+            for (int32_t m0 = n0; m0 < ld; m0 += kTileM) tu.tasks.push_back({k, m0, n0, p});
+          if (p == 0 && m.s > kFactorBlock)
+            for (int32_t n0 = 0; n0 < m.s; n0 += 8) tv.tasks.push_back({k, 0, n0, 0});
+        }
+        h->fb_range[at].end = (int64_t)h->fb_sn.size();
+        tp.per_lv[at].end = (int64_t)tp.tasks.size();
+        tu.per_lv[at].end = (int64_t)tu.tasks.size();
+      }
+  }
   build(h->t_sq, false, [&](int32_t k) { return (int)qvar[k]; }, [&](int32_t k, int bn, std::vector<Task>& out) {
     const SnMeta& m = h->meta[k];
     for (int32_t m0 = 0; m0 < m.s; m0 += kTileM)

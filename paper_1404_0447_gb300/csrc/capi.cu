@@ -71,7 +71,7 @@ void free_device(pselinv_handle* h) {
                    &h->d_piv, &h->d_ptype, &h->d_E, &h->d_snlevel, &h->d_yring, &h->d_pring,
                    &h->d_xb,   &h->d_lb,   &h->d_db,     &h->d_zb,     &h->d_w1,    &h->d_yb,   &h->d_hb,
                    &h->d_plist, &h->d_pn,  &h->d_pctr, &h->d_xs, &h->d_ls, &h->d_sig, &h->d_lexp, &h->d_gexp, &h->d_crow,
-                   &h->d_tctr, &h->d_gctr};
+                   &h->d_tctr, &h->d_gctr, &h->d_fbsn};
   for (void** p : ptrs) {
     if (*p) cudaFree(*p);
     *p = nullptr;
@@ -119,6 +119,7 @@ int ensure_device(pselinv_handle* h) {
   if ((rc = upload(h, &h->d_valmap, h->valmap))) return rc;
   if ((rc = upload(h, &h->d_diagmask, h->diagmask))) return rc;
   if ((rc = upload(h, &h->d_levelsn, h->level_sn))) return rc;
+  if ((rc = upload(h, &h->d_fbsn, h->fb_sn))) return rc;
   {
     // level of every supernode, supernodal parents, level offsets (persistent schedule)
     std::vector<int32_t> v(2 * (size_t)h->nsn + h->nlevels + 1);
@@ -185,6 +186,12 @@ int upload_schedule(pselinv_handle* h) {
   all.insert(all.end(), h->t_gemm2.tasks.begin(), h->t_gemm2.tasks.end());
   h->off_trsm = (int64_t)all.size();
   all.insert(all.end(), h->t_trsm.tasks.begin(), h->t_trsm.tasks.end());
+  h->off_fpanel = (int64_t)all.size();
+  all.insert(all.end(), h->t_fpanel.tasks.begin(), h->t_fpanel.tasks.end());
+  h->off_fupdate = (int64_t)all.size();
+  all.insert(all.end(), h->t_fupdate.tasks.begin(), h->t_fupdate.tasks.end());
+  h->off_vinv = (int64_t)all.size();
+  all.insert(all.end(), h->t_vinv.tasks.begin(), h->t_vinv.tasks.end());
   h->off_schur = (int64_t)all.size();
   all.insert(all.end(), h->t_schur.tasks.begin(), h->t_schur.tasks.end());
   h->off_rect = (int64_t)all.size();
@@ -269,6 +276,8 @@ psi::KArgs kargs(pselinv_handle* h) {
   psi::KArgs a;
   a.dtype = h->opts.dtype;
   a.maxw = h->max_width;
+  a.fblock = 0;
+  a.blocked = 0;
   a.meta = (const psi::SnMeta*)h->d_meta;
   a.desc = (const psi::ColDesc*)h->d_desc;
   a.relidx = (const int32_t*)h->d_relidx;
@@ -668,6 +677,7 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   const psi::Sizes sz = sizes(h);
   const int64_t B = h->opts.batch;
   const bool unsym = d_upper != nullptr;
+  const bool blocked = !unsym && !bk;  // panels factored kFactorBlock columns at a time
   h->factored = h->inverted = false;
   if (bk && !h->d_piv) {
     int rc;
@@ -746,28 +756,41 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   for (int32_t l = nl - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
-    // a level holding a wide supernode gets wide CTAs: the column steps of the
-    // diagonal factorisation are serial, the work inside each step is not
     int wmax = 0;
     for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) wmax = std::max(wmax, h->meta[h->level_sn[t]].s);
-    // shared memory sized for the level's widest block: several CTAs per SM on levels of narrow supernodes
-    psi::KArgs ad = a;
-    ad.maxw = wmax;
-    PSI_CUDA(h, psi::launch_per_sn(unsym ? psi::Kern::FactorDiagLU
-                                         : bk  ? psi::Kern::FactorDiagBK
-                                               : psi::Kern::FactorDiag,
-                                   ad, sns, nsl, hi, wmax >= 64 ? 1024 : 256));
-    for (int side = 0; side < (unsym ? 2 : 1); ++side) {
-      const psi::KArgs& ka = side ? au : al;
-      for (int v = 0; v < psi::kNumVar; ++v) {
-        const psi::Range r = h->t_trsm.per_lv[(size_t)l * psi::kNumVar + v];
-        PSI_CUDA(h, psi::launch_tiles(psi::Kern::Trsm, v, ka, tasks_at(h, h->off_trsm, r.begin), r.end - r.begin,
-                                      hi));
+    if (blocked) {
+      for (int p = 0; p < psi::kFactorBlocks && wmax > p * psi::kFactorBlock; ++p) {
+        const size_t at = (size_t)l * psi::kFactorBlocks + p;
+        const psi::Range rs = h->fb_range[at], rp = h->t_fpanel.per_lv[at], ru = h->t_fupdate.per_lv[at];
+        psi::KArgs ad = a;
+        ad.fblock = p;
+        PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiag, ad, (const int32_t*)h->d_fbsn + rs.begin,
+                                       (int)(rs.end - rs.begin), hi));
+        PSI_CUDA(h, psi::launch_tiles(psi::Kern::FPanel, 0, al, tasks_at(h, h->off_fpanel, rp.begin),
+                                      rp.end - rp.begin, hi));
+        PSI_CUDA(h, psi::launch_tiles(psi::Kern::FUpdate, 0, al, tasks_at(h, h->off_fupdate, ru.begin),
+                                      ru.end - ru.begin, hi));
       }
-      // the pivoted copy-back also divides the scratch by 2x2 blocks of D, which the Schur
-      // update reads: per level; the plain one only fills the panels (nothing in the
-      // factorisation reads L_{C,K} from them): once for all levels, after the loop
-      if (bk) PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBackBK, ka, sns, nsl, hi));
+    } else {
+      // a level holding a wide supernode gets wide CTAs: the column steps of the
+      // diagonal factorisation are serial, the work inside each step is not;
+      // shared memory sized for the level's widest block: several CTAs per SM on levels of narrow supernodes
+      psi::KArgs ad = a;
+      ad.maxw = wmax;
+      PSI_CUDA(h, psi::launch_per_sn(unsym ? psi::Kern::FactorDiagLU : psi::Kern::FactorDiagBK, ad, sns, nsl, hi,
+                                     wmax >= 64 ? 1024 : 256));
+      for (int side = 0; side < (unsym ? 2 : 1); ++side) {
+        const psi::KArgs& ka = side ? au : al;
+        for (int v = 0; v < psi::kNumVar; ++v) {
+          const psi::Range r = h->t_trsm.per_lv[(size_t)l * psi::kNumVar + v];
+          PSI_CUDA(h, psi::launch_tiles(psi::Kern::Trsm, v, ka, tasks_at(h, h->off_trsm, r.begin), r.end - r.begin,
+                                        hi));
+        }
+        // the pivoted copy-back also divides the scratch by 2x2 blocks of D, which the Schur
+        // update reads: per level; the plain one only fills the panels (nothing in the
+        // factorisation reads L_{C,K} from them): once for all levels, after the loop
+        if (bk) PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBackBK, ka, sns, nsl, hi));
+      }
     }
     if (h->far_after_near[l]) {
       if (l + 1 < nl) PSI_CUDA(h, cudaStreamWaitEvent(hi, ev[1 + nl + l + 1], 0));
@@ -789,9 +812,14 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   PSI_CUDA(h, cudaStreamWaitEvent(st, ev[1 + 2 * nl], 0));
   PSI_CUDA(h, cudaEventRecord(ev[2 + 2 * nl], lo));
   PSI_CUDA(h, cudaStreamWaitEvent(st, ev[2 + 2 * nl], 0));
+  al.blocked = blocked;
   if (!bk)
     for (int side = 0; side < (unsym ? 2 : 1); ++side)
       PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBack, side ? au : al, lsn, h->nsn, st));
+  // (L_KK)^{-1} off its diagonal blocks, from the panels just filled
+  if (blocked)
+    PSI_CUDA(h, psi::launch_tiles(psi::Kern::VInv, 0, al, tasks_at(h, h->off_vinv, 0),
+                                  (int64_t)h->t_vinv.tasks.size(), st));
   // no host synchronisation: the first bad pivot stays in status words 0-1
   // until the next factorisation and is reported by pselinv_sync_status (and
   // by pselinv_logdet, which synchronises anyway)
@@ -1385,7 +1413,8 @@ int pselinv_get_info(const pselinv_handle* h, pselinv_info* info) {
   if (h->dev_sym) {
     const int64_t B = h->opts.batch, es = (int64_t)elem_size(h), tasks =
         (int64_t)(h->t_norm.tasks.size() + h->t_lhat.tasks.size() + h->t_gemm1.tasks.size() + h->t_gemm2.tasks.size() +
-                  h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_rect.tasks.size() +
+                  h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_fpanel.tasks.size() +
+                  h->t_fupdate.tasks.size() + h->t_vinv.tasks.size() + h->t_rect.tasks.size() +
                   h->t_pgemm1.tasks.size() + h->t_pgemm2.tasks.size() + h->t_sq.tasks.size());
     int64_t bytes = (int64_t)(sizeof(psi::SnMeta) * h->meta.size() + sizeof(psi::ColDesc) * h->desc.size() +
                               4 * h->relidx.size() + 8 * h->valmap.size() + h->diagmask.size() +

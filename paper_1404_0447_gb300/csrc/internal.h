@@ -70,6 +70,12 @@ constexpr int kTargetTiles = 128 * 152;  // tiles a level should offer the GPU (
 constexpr int kMinSlice2 = 128;   // smallest step-2 slice the per-level boost makes
 constexpr int kTileM = 64;       // output tile rows of the grouped GEMMs
 constexpr int kTileN = 64;       // output tile columns
+// Columns per step of the blocked factorisation of a panel.  The serial part of a
+// step (the pivots of a 32 x 32 block, ~10 us on one SM) balances its two tile
+// launches; 16 would double the launches, 64 put four times the flops of the
+// diagonal blocks on one SM's FP64 pipe.
+constexpr int kFactorBlock = 32;
+constexpr int kFactorBlocks = (kMaxWidth + kFactorBlock - 1) / kFactorBlock;
 
 // Tile-width variants of the tile GEMMs: BN = 8 << var.
 constexpr int kNumVar = 4;
@@ -146,7 +152,14 @@ struct pselinv_handle {
   psi::TaskList t_gemm1;  // step 2 tiles (with k-slices of split supernodes)
   psi::TaskList t_rect;   // r x s tiles per level, unsplit (adjoint)
   psi::TaskList t_gemm2;  // step 3 partial-product tiles
-  psi::TaskList t_trsm;   // factorisation: off-diagonal panel solve tiles
+  psi::TaskList t_trsm;   // factorisation (pivoted, non-symmetric): off-diagonal panel solve tiles
+  // blocked factorisation: per (level, block) at [level * kFactorBlocks + p] the
+  // supernodes of the level wider than p blocks (fb_sn), the tiles of the rows
+  // below block p (t_fpanel) and of the columns right of it (t_fupdate), all
+  // 64 x 8; t_vinv: 8-column strips of the inverses of all supernodes wider than a block
+  std::vector<int32_t> fb_sn;
+  std::vector<psi::Range> fb_range;
+  psi::TaskList t_fpanel, t_fupdate, t_vinv;
   psi::TaskList t_schur;  // factorisation: Schur-complement update tiles
   // Schur groups: the supernodes of a level split into groups whose update
   // targets are disjoint (no two share a row of C), launched one after the
@@ -176,9 +189,10 @@ struct pselinv_handle {
   void* d_diagmask = nullptr;
   void* d_flipmap = nullptr;
   void* d_tasks = nullptr;  // all task arrays back to back
-  int64_t off_norm = 0, off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
+  int64_t off_norm = 0, off_fpanel = 0, off_fupdate = 0, off_vinv = 0, off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
   int64_t off_pgemm1 = 0, off_pgemm2 = 0, off_sq = 0;
   void* d_levelsn = nullptr;
+  void* d_fbsn = nullptr;   // fb_sn
   void* d_L = nullptr;      // L panels (unit diagonal implied; D on the diagonal slots)
   void* d_X = nullptr;      // X panels
   void* d_D = nullptr;      // pivots, batch x n

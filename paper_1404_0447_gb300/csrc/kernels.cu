@@ -18,13 +18,6 @@ namespace psi {
 // packed lower-triangular index, column-major: (i, j), i >= j, order s
 __device__ __forceinline__ int pk(int i, int j, int s) { return j * s - (j * (j - 1)) / 2 + (i - j); }
 
-// elements of the blocked inverse's scratch S for width s: (ceil(s/16) - 1)
-// blocks of 16 x 16 (at least one)
-__host__ __device__ __forceinline__ int fd_scratch(int s) {
-  const int nb = (s + 15) / 16;
-  return 256 * (nb > 1 ? nb - 1 : 1);
-}
-
 // Status words 0-1 hold one 64-bit key (column << 2 | kind), kind 1 = zero
 // pivot, 2 = non-finite: the minimum is the first bad column and, within
 // it, a zero pivot before its consequences.
@@ -116,40 +109,23 @@ __device__ void unit_lower_inverse(const T* Tp, int s, T* V) {
   }
 }
 
-// Where unit_lower_inverse_blocked keeps V: column-major in global memory
-// (ld s; the upper triangle is written as zeros), or packed lower in shared
-// memory (the pk layout; only the lower triangle exists).
-template <class T>
-struct VGlobal {
-  static constexpr bool kPacked = false;
-  T* p;
-  int s;
-  __device__ __forceinline__ T& operator()(int i, int j) const { return p[i + (int64_t)j * s]; }
-};
-template <class T>
-struct VPacked {
-  static constexpr bool kPacked = true;
-  T* p;
-  int s;
-  __device__ __forceinline__ T& operator()(int i, int j) const { return p[pk(i, j, s)]; }
-};
-
 // V = (L_KK)^{-1} for the unit lower triangle held packed in Tp (shared
 // memory), by 16 x 16 blocks so that the whole CTA works at every step:
 // first the diagonal blocks V_ii = (L_ii)^{-1} (one column per thread),
 // then, for block distance d = 1, 2, ... (all block pairs (i, j) with
 // i - j = d at once), S = sum_{k=j}^{i-1} L_ik V_kj and V_ij = -V_ii S.
-// V (see VGlobal / VPacked) is read back by the later steps of this CTA;
-// S (shared) holds (ceil(s/16) - 1) blocks of 16 x 16.
-template <class T, class VA>
-__device__ void unit_lower_inverse_blocked(const T* Tp, int s, const VA& V, T* S) {
+// V (global memory, column-major, ld s, zeros above the diagonal) is read back
+// by the later steps of this CTA; S (shared) holds (ceil(s/16) - 1) blocks of
+// 16 x 16.
+template <class T>
+__device__ void unit_lower_inverse_blocked(const T* Tp, int s, T* Vg, T* S) {
+  auto V = [&](int i, int j) -> T& { return Vg[i + (int64_t)j * s]; };
   constexpr int B = 16;
   const int nb = (s + B - 1) / B;
   const int nt = blockDim.x, t = threadIdx.x;
   for (int c = t; c < s; c += nt) {
     const int i1 = min((c / B + 1) * B, s);
-    if constexpr (!VA::kPacked)
-      for (int i = 0; i < c; ++i) V(i, c) = Sc<T>::zero();
+    for (int i = 0; i < c; ++i) V(i, c) = Sc<T>::zero();
     V(c, c) = Sc<T>::one();
     for (int i = c + 1; i < i1; ++i) {
       T acc = Sc<T>::zero();
@@ -181,74 +157,193 @@ __device__ void unit_lower_inverse_blocked(const T* Tp, int s, const VA& V, T* S
   }
 }
 
-// Factorisation, one CTA per supernode of the level: right-looking LDL^T of
-// the s x s diagonal block (lower part, already holding A_KK minus all
-// descendant updates) in shared memory; L_KK (unit diagonal implied, d_j on
-// the diagonal slot) back to the panel, d to D, (L_KK)^{-1} to linv.
-// Column step j: u = column j below the diagonal, then L_ij = u_i / d_j and
-// the trailing lower triangle T_ik -= L_ij u_k, one warp per column k (no
-// integer division, only lower-triangle entries visited).
+// Blocked factorisation of the panel of supernode K, 32 columns at a time: for
+// block p, k_fdiag (diagonal block), k_fpanel (the rows below it) and k_fupdate
+// (the remaining columns of the panel).  One SM's FP64 pipe takes 97 us for the
+// s^3 / 3 flops of a 128-wide block and as long again for its inverse, so the
+// work is spread over the GPU and only the 32 x 32 blocks stay on one SM;
+// (L_KK)^{-1} off the diagonal blocks waits until after the last level
+// (k_vinv), where all supernodes run at once.  Against one CTA per supernode
+// factoring and inverting the whole block in shared memory: see k_fdiag.
+constexpr int kFB = kFactorBlock;
+constexpr int kFdThreads = 192;                                       // 6 warps: enough to fill the FP64 pipe
+constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdThreads - 1) / kFdThreads;  // lower entries per thread
+
+// Row and column of entry e of a lower triangle stored row by row.
+__device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
+  i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+  while ((i + 1) * (i + 2) / 2 <= e) ++i;
+  while (i * (i + 1) / 2 > e) --i;
+  k = e - i * (i + 1) / 2;
+}
+
+// Block p of the supernodes in sns (width above 32 p): LDL^T of the w x w
+// diagonal block (w <= 32) and the inverse V of its unit lower triangle, in
+// one pass of in-place elimination on [A | I]: at column j, row i > j becomes
+// row i - l_i row j, with the freed slot (i, j) taking V's -l_i.  Each thread
+// holds up to three entries in registers; what a step needs from others (column
+// j below the pivot, V's row j, 1 / d_j) goes through shared memory, double
+// buffered, one barrier per column.  Out: L (unit diagonal implied, d on the
+// diagonal) to the panel, d to D, V to linv (zeros above the diagonal).
+// Bound: the chain of w pivots (1 / d 364 cycles, product and update 115,
+// barrier and shared memory ~70), about 0.3 us per column.
 template <class T>
-__global__ void k_factor_diag(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                              T* __restrict__ D, T* __restrict__ Linv, Sizes sz, int* status) {
-  extern __shared__ __align__(16) unsigned char shraw[];
-  T* Tp = reinterpret_cast<T*>(shraw);
-  const int k = sns[blockIdx.x];
+__global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns,
+                                                      int p, T* __restrict__ L, T* __restrict__ D,
+                                                      T* __restrict__ Linv, Sizes sz, int* status) {
+  __shared__ __align__(16) double raw[2 * (kFB + 1) * Sc<T>::P];
+  T* buf = reinterpret_cast<T*>(raw);  // [2][kFB + 1]: column / row entries, then 1 / d
   const int b = blockIdx.y;
-  const SnMeta m = meta[k];
-  const int s = m.s, ld = m.s + m.r;
-  T* u = Tp + s * (s + 1) / 2;
-  T* S = u + s;
-  T* P = L + b * sz.panel + m.panel;
-  const int nt = blockDim.x, t = threadIdx.x;
-  const int lane = t & 31, warp = t >> 5, nw = nt >> 5;
-  for (int j = warp; j < s; j += nw) {
-    const int cb = pk(j, j, s);
-    for (int i = j + lane; i < s; i += 32) Tp[cb + i - j] = P[i + (int64_t)j * ld];
+  const SnMeta m = meta[sns[blockIdx.x]];
+  const int s = m.s, ld = m.s + m.r, c0 = p * kFB, w = min(kFB, s - c0);
+  T* P = L + b * sz.panel + m.panel + c0 + (int64_t)c0 * ld;
+  T* V = Linv + b * sz.linv + m.linv + c0 + (int64_t)c0 * s;
+  const int ne = w * (w + 1) / 2;
+  T x[kFdEntries], l[kFdEntries];
+  int ri[kFdEntries], ck[kFdEntries];
+#pragma unroll
+  for (int q = 0; q < kFdEntries; ++q) {
+    const int e = threadIdx.x + q * kFdThreads;
+    ri[q] = ck[q] = -1;  // no entry: never live
+    if (e < ne) {
+      tri_entry(e, ri[q], ck[q]);
+      x[q] = P[ri[q] + (int64_t)ck[q] * ld];
+      if (ck[q] == 0) {
+        if (ri[q] == 0)
+          buf[kFB] = Sc<T>::one() / x[q];
+        else
+          buf[ri[q]] = x[q];
+      }
+    }
   }
   __syncthreads();
-  // rd[0] = 1 / d_j of the current step: one division per column, by the
-  // thread that last wrote the pivot (thread 0 here, then warp 0 lane 0 of
-  // the update, which owns entry (j+1, j+1))
-  T* rd = S;
-  if (t == 0) rd[0] = Sc<T>::one() / Tp[0];
-  __syncthreads();
-  for (int j = 0; j < s; ++j) {
-    const int cj = pk(j, j, s);
-    const T d = Tp[cj], rdj = rd[0];
-    if (t == 0 && Sc<T>::bad(d)) report_pivot(status, m.f + j, Sc<T>::is_zero(d));
-    for (int i = j + 1 + t; i < s; i += nt) {
-      const T v = Tp[cj + i - j];
-      u[i] = v;
-      Tp[cj + i - j] = v * rdj;
-    }
-    __syncthreads();
-    for (int kk = j + 1 + warp; kk < s; kk += nw) {
-      const int ck = pk(kk, kk, s);
-      const T uk = u[kk];
-      for (int i = kk + lane; i < s; i += 32) {
-        const T x = Tp[ck + i - kk] - Tp[cj + i - j] * uk;
-        Tp[ck + i - kk] = x;
-        if (i == j + 1 && kk == j + 1) rd[0] = Sc<T>::one() / x;
+  for (int j = 0; j + 1 < w; ++j) {
+    const T* cur = buf + (j & 1) * (kFB + 1);
+    T* nxt = buf + (~j & 1) * (kFB + 1);
+    const T rd = cur[kFB];
+#pragma unroll
+    for (int q = 0; q < kFdEntries; ++q) {
+      const int i = ri[q], k = ck[q];
+      if (i <= j) continue;
+      const T t = cur[i] * rd;  // l_i
+      if (k == j) {
+        l[q] = t;
+        x[q] = -t;
+      } else {
+        x[q] -= t * cur[k];  // k > j: u_k = A_kj; k < j: V_jk
+      }
+      // what column j + 1 reads: its entries below the pivot, V's row j + 1, 1 / pivot
+      if (k == j + 1) {
+        if (i == k)
+          nxt[kFB] = Sc<T>::one() / x[q];
+        else
+          nxt[i] = x[q];
+      } else if (i == j + 1) {
+        nxt[k] = x[q];
       }
     }
     __syncthreads();
   }
-  T* Vg = Linv + b * sz.linv + m.linv;
-  if constexpr (Sc<T>::P == 1) {
-    // real: V packed in shared memory after S, then written out with its zeros
-    T* Vs = S + fd_scratch(s);
-    unit_lower_inverse_blocked(Tp, s, VPacked<T>{Vs, s}, S);
-    for (int j = warp; j < s; j += nw)
-      for (int i = lane; i < s; i += 32) Vg[i + (int64_t)j * s] = i < j ? Sc<T>::zero() : Vs[pk(i, j, s)];
-  } else {
-    unit_lower_inverse_blocked(Tp, s, VGlobal<T>{Vg, s}, S);
+#pragma unroll
+  for (int q = 0; q < kFdEntries; ++q) {
+    const int i = ri[q], k = ck[q];
+    if (i < 0) continue;
+    if (i == k) {
+      if (Sc<T>::bad(x[q])) report_pivot(status, m.f + c0 + i, Sc<T>::is_zero(x[q]));
+      D[b * sz.n + m.f + c0 + i] = x[q];
+      P[i + (int64_t)i * ld] = x[q];
+      V[i + (int64_t)i * s] = Sc<T>::one();
+    } else {
+      P[i + (int64_t)k * ld] = l[q];
+      V[i + (int64_t)k * s] = x[q];
+      V[k + (int64_t)i * s] = Sc<T>::zero();
+    }
   }
-  for (int j = warp; j < s; j += nw) {
-    const int cb = pk(j, j, s);
-    for (int i = j + lane; i < s; i += 32) P[i + (int64_t)j * ld] = Tp[cb + i - j];
+}
+
+// (L_KK)^{-1} off its 32 x 32 diagonal blocks, after the last level, all
+// supernodes wider than 32 at once: one CTA per 8 columns (task n0) of V.
+// With j the block of the columns, X_j = V_jj and, for i = j+1, j+2, ...:
+// X_i = -V_ii sum_{k=j}^{i-1} L_ik X_k; warp w holds rows 8w .. 8w+7 of the
+// 32-row block on m8n8k4 MMAs, its operand fragments straight from the panel
+// (eight 64-byte row runs per k-block, loaded before the products), X in
+// shared memory.  Blocks above the diagonal are written as zeros.
+template <class T>
+__global__ void __launch_bounds__(TG_THREADS) k_vinv(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
+                                                     const T* __restrict__ L, T* __restrict__ Linv, Sizes sz) {
+  constexpr int P = Sc<T>::P, LDX = 12;  // 4 (mod 16) doubles
+  __shared__ double xs[P][kMaxWidth][LDX];
+  __shared__ double ss[P][kFB][LDX];
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y;
+  const SnMeta m = meta[tk.sn];
+  const int s = m.s, ld = m.s + m.r;
+  const T* A = L + b * sz.panel + m.panel;
+  T* V = Linv + b * sz.linv + m.linv;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
+  const int n0 = tk.n0, j0 = n0 / kFB * kFB, j1 = min(s, j0 + kFB), n1 = min(s, n0 + 8);
+  for (int e = t; e < j0 * 8; e += TG_THREADS) {
+    const int col = n0 + e / j0;
+    if (col < n1) V[e % j0 + (int64_t)col * s] = Sc<T>::zero();
   }
-  for (int j = t; j < s; j += nt) D[b * sz.n + m.f + j] = Tp[pk(j, j, s)];
+  for (int e = t; e < kFB * 8; e += TG_THREADS) {
+    const int row = j0 + e % kFB, col = n0 + e / kFB;
+    const T v = row < j1 && col < n1 ? V[row + (int64_t)col * s] : Sc<T>::zero();
+#pragma unroll
+    for (int pl = 0; pl < P; ++pl) xs[pl][row][e / kFB] = Sc<T>::plane(v, pl);
+  }
+  __syncthreads();
+  // acc += (M at rows r0 + g of the block, columns k0 .. k0 + 31) (x rows k0 ..)
+  auto product = [&](const T* M, int64_t mld, int row, bool rlive, int k0, int klim, const double (*x)[LDX],
+                     int64_t xplane, int xr0, double (&acc)[P][2]) {
+    T f[kFB / 4];
+#pragma unroll
+    for (int u = 0; u < kFB / 4; ++u) {
+      const int kk = k0 + 4 * u + q;
+      f[u] = rlive && kk < klim ? M[row + (int64_t)kk * mld] : Sc<T>::zero();
+    }
+#pragma unroll
+    for (int u = 0; u < kFB / 4; ++u) {
+      const double* xb = &x[xr0 + 4 * u + q][g];
+      if constexpr (P == 1) {
+        dmma884(acc[0][0], acc[0][1], f[u], xb[0]);
+      } else {
+        const double br = xb[0], bi = xb[xplane];
+        dmma884(acc[0][0], acc[0][1], f[u].re, br);
+        dmma884(acc[0][0], acc[0][1], -f[u].im, bi);
+        dmma884(acc[1][0], acc[1][1], f[u].re, bi);
+        dmma884(acc[1][0], acc[1][1], f[u].im, br);
+      }
+    }
+  };
+  for (int i0 = j1; i0 < s; i0 += kFB) {
+    const int row = i0 + 8 * warp + g;
+    double acc[P][2] = {};
+    for (int k0 = j0; k0 < i0; k0 += kFB)
+      product(A, ld, row, row < s, k0, s, xs[0], kMaxWidth * LDX, k0, acc);
+#pragma unroll
+    for (int pl = 0; pl < P; ++pl)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        ss[pl][8 * warp + g][2 * q + e] = acc[pl][e];
+        acc[pl][e] = 0.0;
+      }
+    __syncthreads();
+    product(V, s, row, row < s, i0, min(s, i0 + kFB), ss[0], kFB * LDX, 0, acc);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int col = n0 + 2 * q + e;
+#pragma unroll
+      for (int pl = 0; pl < P; ++pl) xs[pl][i0 + 8 * warp + g][2 * q + e] = -acc[pl][e];
+      if (row < s && col < n1) {
+        if constexpr (P == 1)
+          V[row + (int64_t)col * s] = -acc[0][e];
+        else
+          V[row + (int64_t)col * s] = T{-acc[0][e], -acc[1][e]};
+      }
+    }
+    __syncthreads();
+  }
 }
 
 // Factorisation of a non-symmetric diagonal block, one CTA per supernode of
@@ -302,9 +397,9 @@ __global__ void k_factor_diag_lu(const SnMeta* __restrict__ meta, const int32_t*
   }
   if constexpr (Sc<T>::P == 1) {  // real: the blocked inverses (their 16 x 16 scratch after the triangles)
     T* S = Tu + s * (s + 1) / 2;
-    unit_lower_inverse_blocked(Tl, s, VGlobal<T>{Linv + b * sz.linv + m.linv, s}, S);
+    unit_lower_inverse_blocked(Tl, s, Linv + b * sz.linv + m.linv, S);
     __syncthreads();
-    unit_lower_inverse_blocked(Tu, s, VGlobal<T>{Uinv + b * sz.linv + m.linv, s}, S);
+    unit_lower_inverse_blocked(Tu, s, Uinv + b * sz.linv + m.linv, S);
   } else {  // complex: both triangles fill the shared memory
     unit_lower_inverse(Tl, s, Linv + b * sz.linv + m.linv);
     unit_lower_inverse(Tu, s, Uinv + b * sz.linv + m.linv);
@@ -499,7 +594,7 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
     if (t == 0) report_pivot(status, m.f + k, sh_bad == 1);
     return;
   }
-  unit_lower_inverse_blocked(Tp, s, VGlobal<T>{Linv + b * sz.linv + m.linv, s}, reinterpret_cast<T*>(perm + ((s + 3) & ~3)));
+  unit_lower_inverse_blocked(Tp, s, Linv + b * sz.linv + m.linv, reinterpret_cast<T*>(perm + ((s + 3) & ~3)));
   for (int e = t; e < s * s; e += nt) {
     const int i = e % s, j = e / s;
     if (i > j) P[i + (int64_t)j * ld] = Tp[pk(i, j, s)];
@@ -596,28 +691,36 @@ __global__ void k_diag_final(KArgs a, const int32_t* __restrict__ sns) {
   if (a.gam) pole_share<T>(a, sns[blockIdx.x], blockIdx.z, gridDim.z);
 }
 
-// Copy the factor scratch back into the panels of the level's supernodes
-// (blockIdx.z strides over the columns; threads run down a column).
+// Copy the factor scratch back into the panels of the listed supernodes
+// (blockIdx.z strides over the columns; threads run down a column).  Lkk set
+// (blocked factorisation): L_KK below its 32 x 32 diagonal blocks too, from
+// where k_fpanel kept it.
 template <class T>
 __global__ void k_copyback(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                           const T* __restrict__ Ltmp, Sizes sz) {
+                           const T* __restrict__ Ltmp, const T* __restrict__ Lkk, Sizes sz) {
   const int k = sns[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[k];
   const int s = m.s, r = m.r, ld = s + r;
   T* P = L + b * sz.panel + m.panel + s;
   const T* src = Ltmp + b * sz.lhat + m.lhat;
-  for (int j = blockIdx.z; j < s; j += gridDim.z)
+  const T* lk = Lkk + b * sz.linv + m.linv;
+  for (int j = blockIdx.z; j < s; j += gridDim.z) {
     for (int i = threadIdx.x; i < r; i += blockDim.x) P[i + (int64_t)j * ld] = src[i + (int64_t)j * r];
+    if (Lkk)
+      for (int i = (j / kFB + 1) * kFB + threadIdx.x; i < s; i += blockDim.x)
+        P[i - s + (int64_t)j * ld] = lk[i + (int64_t)j * s];
+  }
 }
 
 // --------------------------------------------------------------------------
 // tile GEMMs
 // --------------------------------------------------------------------------
 
-// Factorisation panel solve: Ltmp_{C,K} = A_{C,K} (L_KK)^{-T} D_K^{-1}, and,
-// when W is set, W_{C,K} = A_{C,K} (L_KK)^{-T} itself (the Schur update's
-// L_{C,K} D_K without a product per operand element; KArgs::W).
+// Panel solve of the pivoted and the non-symmetric factorisations:
+// Ltmp_{C,K} = A_{C,K} (L_KK)^{-T} D_K^{-1} and W_{C,K} = A_{C,K} (L_KK)^{-T}
+// itself (the Schur update's L_{C,K} D_K without a product per operand
+// element; KArgs::W).
 // Pivoted factor (piv set): the columns of A_{C,K} are read in pivot order
 // and D^{-1} is left to k_copyback_bk (2x2 blocks can straddle tiles).
 template <class T, int BN>
@@ -648,13 +751,96 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
   tile_mma<T, BN>(sm, 0, min(s, tk.n0 + BN), [](int) { return false; }, la, lb, acc,
                   LiveRect{r - tk.m0, s - tk.n0}, KUpperB<BN>{tk.n0});
   T* out = Ltmp + b * sz.lhat + m.lhat;
-  T* wout = W ? W + b * sz.panel + m.panel : nullptr;
+  T* wout = W + b * sz.panel + m.panel + s;
   tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
     const int row = tk.m0 + mm, col = tk.n0 + nn;
     if (row < r && col < s) {
       out[row + (int64_t)col * r] = pv ? v : v / d[col];
-      if (wout) wout[row + (int64_t)col * r] = v;
+      wout[row + (int64_t)col * ld] = v;
     }
+  });
+}
+
+// Blocked factorisation, rows below the diagonal block of columns [32 p, 32 p
+// + 32) (tile rows m0 .. m0+63 of the panel, columns n0 .. n0+7): W = A V_pp^T
+// = L D, kept in the X panels (same layout) as the first operand of the panel
+// update and the Schur update, and L = W D^{-1}: rows of C to Ltmp (the Schur
+// update's second operand), rows of K's own block to the unused lower part of
+// linv (the panel update's second operand).  Both copies leave the panel itself
+// unwritten: tiles of the same rows and other columns still read it.
+template <class T, int BN>
+__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_fpanel(
+    const SnMeta* __restrict__ meta, const Task* __restrict__ tasks, const T* __restrict__ L, const T* __restrict__ D,
+    T* __restrict__ Linv, T* __restrict__ Ltmp, T* __restrict__ W, Sizes sz) {
+  __shared__ TileSmem<T, BN> sm;
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y;
+  const SnMeta m = meta[tk.sn];
+  const int s = m.s, r = m.r, ld = s + r;
+  const T* A = L + b * sz.panel + m.panel;
+  T* Vi = Linv + b * sz.linv + m.linv;
+  const T* d = D + b * sz.n + m.f;
+  Acc<T, BN> acc;
+  acc_zero<T, BN>(acc);
+  const int k0 = tk.n0 / kFB * kFB, nend = min(s, k0 + kFB);
+  auto la = [&](int mm, int kk) {
+    const int row = tk.m0 + mm;
+    return row < ld ? A[row + (int64_t)kk * ld] : Sc<T>::zero();
+  };
+  auto lb = [&](int kk, int nn) {
+    const int col = tk.n0 + nn;
+    return col < nend ? Vi[col + (int64_t)kk * s] : Sc<T>::zero();
+  };
+  // V_pp^T is upper triangular: columns < n0 + BN need only k < n0 + BN
+  tile_mma<T, BN>(sm, k0, min(nend, tk.n0 + BN), [](int) { return false; }, la, lb, acc,
+                  LiveRect{ld - tk.m0, nend - tk.n0}, KUpperB<BN>{tk.n0});
+  T* out = Ltmp + b * sz.lhat + m.lhat;
+  T* wout = W + b * sz.panel + m.panel;
+  tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
+    const int row = tk.m0 + mm, col = tk.n0 + nn;
+    if (row < ld && col < nend) {
+      wout[row + (int64_t)col * ld] = v;
+      const T l = v / d[col];
+      if (row >= s)
+        out[row - s + (int64_t)col * r] = l;
+      else
+        Vi[row + (int64_t)col * s] = l;  // rows below block p: disjoint from V_pp
+    }
+  });
+}
+
+// Blocked factorisation, the columns right of block p (task c) of the panel:
+// A_ij -= sum_k W_ik L_jk over the block's 32 columns k, rows i >= j of the
+// whole panel, each entry by one thread.
+template <class T, int BN>
+__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_fupdate(
+    const SnMeta* __restrict__ meta, const Task* __restrict__ tasks, T* __restrict__ L, const T* __restrict__ Linv,
+    const T* __restrict__ W, Sizes sz) {
+  __shared__ TileSmem<T, BN> sm;
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y;
+  const SnMeta m = meta[tk.sn];
+  const int s = m.s, ld = s + m.r;
+  const T* Wp = W + b * sz.panel + m.panel;
+  const T* Lk = Linv + b * sz.linv + m.linv;
+  Acc<T, BN> acc;
+  acc_zero<T, BN>(acc);
+  auto la = [&](int mm, int kk) {
+    const int row = tk.m0 + mm;
+    return row < ld ? Wp[row + (int64_t)kk * ld] : Sc<T>::zero();
+  };
+  auto lb = [&](int kk, int nn) {
+    const int col = tk.n0 + nn;
+    return col < s ? Lk[col + (int64_t)kk * s] : Sc<T>::zero();
+  };
+  const int dm = tk.m0 - tk.n0;
+  tile_mma<T, BN>(sm, tk.c * kFB, tk.c * kFB + kFB, [](int) { return false; }, la, lb, acc, [&](int r0, int c0) {
+    return tk.m0 + r0 < ld && tk.n0 + c0 < s && c0 <= dm + r0 + 7;
+  });
+  T* P = L + b * sz.panel + m.panel;
+  tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
+    const int row = tk.m0 + mm, col = tk.n0 + nn;
+    if (row < ld && col < s && row >= col) P[row + (int64_t)col * ld] -= v;
   });
 }
 
@@ -669,7 +855,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
 // Non-symmetric factor: Ltmp2 is the second operand (U'_{K,C}^T), giving
 // L_{C,K} D_K U'_{K,C} into the L panels and, called again with the operands
 // swapped and `strict`, (U'_{K,C}^T D_K L_{C,K}^T) below the diagonal into the
-// U panels.  W set: the first operand is W_{C,K} = L_{C,K} D_K (or
+// U panels.  The first operand is W_{C,K} = L_{C,K} D_K (or
 // U'_{K,C}^T D_K; pivoted: with D's 2 x 2 blocks) as the panel solve left it, so the loads carry no
 // FP64 product (a product per A element is 64 x 16 FP64 operations per
 // k-tile, 1/8 of the MMA work of a 64 x 8 tile on the same pipe).
@@ -677,31 +863,20 @@ template <class T, int BN>
 __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
                                                       const ColDesc* __restrict__ desc,
                                                       const int32_t* __restrict__ relidx, T* __restrict__ L,
-                                                      const T* __restrict__ D, const T* __restrict__ Ltmp,
                                                       const T* __restrict__ Ltmp2, int strict, Sizes sz,
-                                                      const int8_t* __restrict__ ptype, const T* __restrict__ E,
                                                       const T* __restrict__ W) {
   __shared__ TileSmem<T, BN> sm;
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[tk.sn];
-  const int s = m.s, r = m.r;
-  const T* Lc = Ltmp + b * sz.lhat + m.lhat;
+  const int s = m.s, r = m.r, ld = s + r;
   const T* Lc2 = Ltmp2 + b * sz.lhat + m.lhat;
-  const T* d = D + b * sz.n + m.f;
   Acc<T, BN> acc;
   acc_zero<T, BN>(acc);
-  const int8_t* ty = ptype ? ptype + b * sz.n + m.f : nullptr;
-  const T* ee = ptype ? E + b * sz.n + m.f : nullptr;
-  const T* Wc = W ? W + b * sz.panel + m.panel : nullptr;
+  const T* Wc = W + b * sz.panel + m.panel + s;
   auto la = [&](int mm, int kk) {
     const int row = tk.m0 + mm;
-    if (row >= r) return Sc<T>::zero();
-    if (Wc) return Wc[row + (int64_t)kk * r];
-    T v = Lc[row + (int64_t)kk * r] * d[kk];
-    if (ty && ty[kk] == 1) v += Lc[row + (int64_t)(kk + 1) * r] * ee[kk];       // (L D) with a 2x2 block
-    if (ty && ty[kk] == 2) v += Lc[row + (int64_t)(kk - 1) * r] * ee[kk - 1];
-    return v;
+    return row < r ? Wc[row + (int64_t)kk * ld] : Sc<T>::zero();
   };
   auto lb = [&](int kk, int nn) {
     const int col = tk.n0 + nn;
@@ -984,15 +1159,6 @@ static size_t diag_smem(int maxw) {
   return sizeof(T) * ((size_t)maxw * (maxw + 1) / 2 + 2 * (size_t)maxw) + sizeof(int) * (size_t)maxw;
 }
 
-// the symmetric diagonal factorisation: packed lower triangle, the column u,
-// and the 16 x 16 blocks S of the blocked inverse
-template <class T>
-static size_t diag_smem_fd(int maxw) {
-  // packed L_KK, u, S; real: the packed inverse too (complex keeps it in global memory)
-  const size_t tri = (size_t)maxw * (maxw + 1) / 2;
-  return sizeof(T) * (tri + (size_t)maxw + fd_scratch(maxw) + (Sc<T>::P == 1 ? tri : 0));
-}
-
 // the pivoted diagonal factorisation: diag_smem plus the blocks of the inverse
 template <class T>
 static size_t diag_smem_bk(int maxw) {
@@ -1009,11 +1175,8 @@ static size_t diag_smem_lu(int maxw) {
 
 template <class T>
 static cudaError_t setup_t() {
-  cudaError_t e = cudaFuncSetAttribute(k_factor_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)diag_smem_fd<T>(kMaxWidth));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)diag_smem_bk<T>(kMaxWidth));
+  cudaError_t e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)diag_smem_bk<T>(kMaxWidth));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_factor_diag_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)diag_smem_lu<T>(Sc<T>::P == 1 ? kMaxWidth : kMaxWidthLUComplex));
@@ -1086,39 +1249,53 @@ cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, 
 template <class T, int BN>
 static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cudaStream_t st) {
   const dim3 grid((unsigned)n, a.sz.batch);
-  switch (k) {
-    case Kern::Trsm:
-      k_trsm<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.D, (const T*)a.Linv,
-                                                 (T*)a.Lhat, a.sz, a.piv, (T*)a.W);
-      break;
-    case Kern::Schur:
-      k_schur<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, a.desc, a.relidx, (T*)a.L, (const T*)a.D,
-                                                  (const T*)a.Lhat, (const T*)(a.Uhat ? a.Uhat : a.Lhat),
-                                                  a.strict, a.sz, a.ptype, (const T*)a.E, (const T*)a.W);
-      break;
-    case Kern::Lhat:
-      k_lhat<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, (T*)a.Lhat, a.sz);
-      break;
-    case Kern::NormM:
-      if constexpr (BN == 8) {
+  if constexpr (BN == 8) {  // lists of 64 x 8 tiles only
+    switch (k) {
+      case Kern::FPanel:
+        k_fpanel<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.D, (T*)a.Linv,
+                                                     (T*)a.Lhat, (T*)a.W, a.sz);
+        return cudaGetLastError();
+      case Kern::FUpdate:
+        k_fupdate<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (T*)a.L, (const T*)a.Linv, (const T*)a.W, a.sz);
+        return cudaGetLastError();
+      case Kern::VInv:
+        k_vinv<T><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (T*)a.Linv, a.sz);
+        return cudaGetLastError();
+      case Kern::NormM:
         if (a.Uinv)
           k_norm_m<T, 2><<<grid, TG_THREADS, 0, st>>>(a, t);
         else if (a.ptype)
           k_norm_m<T, 1><<<grid, TG_THREADS, 0, st>>>(a, t);
         else
           k_norm_m<T, 0><<<grid, TG_THREADS, 0, st>>>(a, t);
-        break;
-      }
-      return cudaErrorInvalidValue;  // the list holds 64 x 8 tiles only
+        return cudaGetLastError();
+      default: break;
+    }
+  }
+  switch (k) {
+    case Kern::Trsm:
+      k_trsm<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.D, (const T*)a.Linv,
+                                                 (T*)a.Lhat, a.sz, a.piv, (T*)a.W);
+      break;
+    case Kern::Schur:
+      k_schur<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, a.desc, a.relidx, (T*)a.L,
+                                                  (const T*)(a.Uhat ? a.Uhat : a.Lhat), a.strict, a.sz,
+                                                  (const T*)a.W);
+      break;
+    case Kern::Lhat:
+      k_lhat<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, (T*)a.Lhat, a.sz);
+      break;
     case Kern::Gemm1:
       if (a.XU)
         k_gemm1<T, BN, true><<<grid, TG_THREADS, 0, st>>>(a, t);
       else
         k_gemm1<T, BN, false><<<grid, TG_THREADS, 0, st>>>(a, t);
       break;
-    default:
+    case Kern::Gemm2:
       k_gemm2<T, BN><<<grid, TG_THREADS, 0, st>>>(a, t);
       break;
+    default:
+      return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
@@ -1146,11 +1323,11 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
   const dim3 grid(nsn, a.sz.batch);
   switch (k) {
     case Kern::FactorDiag:
-      k_factor_diag<T><<<grid, threads, diag_smem_fd<T>(a.maxw), st>>>(a.meta, sns, (T*)a.L, (T*)a.D, (T*)a.Linv,
-                                                                    a.sz, a.status);
+      k_fdiag<T><<<grid, kFdThreads, 0, st>>>(a.meta, sns, a.fblock, (T*)a.L, (T*)a.D, (T*)a.Linv, a.sz, a.status);
       break;
     case Kern::CopyBack:
-      k_copyback<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.Lhat, a.sz);
+      k_copyback<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.Lhat,
+                                                                (const T*)(a.blocked ? a.Linv : nullptr), a.sz);
       break;
     case Kern::Gemm1Reduce:
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);

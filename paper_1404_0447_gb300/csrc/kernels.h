@@ -19,7 +19,7 @@ struct Sizes {
 };
 
 enum class Kern {
-  Trsm, Schur, NormM, Lhat, Gemm1, Gemm2, FactorDiag, CopyBack, DiagFinal, Gemm1Reduce,
+  Trsm, FPanel, FUpdate, VInv, Schur, NormM, Lhat, Gemm1, Gemm2, FactorDiag, CopyBack, DiagFinal, Gemm1Reduce,
   FactorDiagLU,              // non-symmetric diagonal blocks
   FactorDiagBK, CopyBackBK   // Bunch-Kaufman pivoted factor
 };
@@ -28,6 +28,8 @@ enum class Kern {
 struct KArgs {
   int dtype;  // PSELINV_F64 / PSELINV_C128
   int maxw;   // widest supernode (shared-memory size of the diagonal kernels)
+  int fblock;   // FactorDiag: the block of kFactorBlock columns
+  int blocked;  // CopyBack: L_KK below its diagonal blocks is in linv (blocked factorisation)
   const SnMeta* meta;
   const ColDesc* desc;
   const int32_t* relidx;
@@ -64,9 +66,9 @@ struct KArgs {
   int* gctr;
   // factor: W_{C,K} = L_{C,K} D_K (U side: U'_{K,C}^T D_K; pivoted: D_K's
   // 1 x 1 and 2 x 2 blocks, columns in pivot order), the panel solve's
-  // product before the D^{-1} scaling, kept for the Schur update; r x s
-  // column-major at each supernode's panel offset of this array (the X or XU
-  // panels, free during the factorisation); nullptr elsewhere
+  // product before the D^{-1} scaling, kept for the Schur update, in the panel
+  // layout of this array (the X or XU panels, free during the factorisation);
+  // nullptr elsewhere
   void* W;
 };
 
@@ -93,13 +95,13 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
 // diagmask == nullptr: plain gather; else off-diagonal entries doubled.
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
                                  void* out, const Sizes& sz, cudaStream_t st);
-// Tile kernels (Trsm, Schur, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
+// Tile kernels (Trsm, FPanel, FUpdate, VInv, Schur, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
 cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st);
 // Per-supernode kernels (FactorDiag, CopyBack, DiagFinal, Gemm1Reduce) over the
 // nsn supernodes listed in sns.
-// threads: block size of the diagonal-factorisation kernels (FactorDiag,
-// FactorDiagLU, FactorDiagBK -- the last capped at 512); the others use 256.
+// threads: block size of the diagonal-factorisation kernels FactorDiagLU and
+// FactorDiagBK (the last capped at 512).
 cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads = 256);
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype = nullptr, const void* E = nullptr);

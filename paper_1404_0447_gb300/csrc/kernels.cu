@@ -166,8 +166,13 @@ __device__ void unit_lower_inverse_blocked(const T* Tp, int s, T* Vg, T* S) {
 // (k_vinv), where all supernodes run at once.  Against one CTA per supernode
 // factoring and inverting the whole block in shared memory: see k_fdiag.
 constexpr int kFB = kFactorBlock;
-constexpr int kFdThreads = 192;                                       // 6 warps: enough to fill the FP64 pipe
-constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdThreads - 1) / kFdThreads;  // lower entries per thread
+constexpr int kFdUpdate = 192;               // threads holding the triangle: 6 warps fill the FP64 pipe
+constexpr int kFdThreads = 32 + kFdUpdate;  // and the pivot warp
+constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdUpdate - 1) / kFdUpdate;  // lower entries per thread
+
+// Value of lane src, to all lanes of the warp.
+__device__ __forceinline__ double shfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ Cplx shfl(Cplx v, int src) { return {shfl(v.re, src), shfl(v.im, src)}; }
 
 // Row and column of entry e of a lower triangle stored row by row.
 __device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
@@ -178,86 +183,90 @@ __device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
 }
 
 // Block p of the supernodes in sns (width above 32 p): LDL^T of the w x w
-// diagonal block (w <= 32) and the inverse V of its unit lower triangle, in
-// one pass of in-place elimination on [A | I]: at column j, row i > j becomes
-// row i - l_i row j, with the freed slot (i, j) taking V's -l_i.  Each thread
-// holds up to three entries in registers; what a step needs from others (column
-// j below the pivot, V's row j, 1 / d_j) goes through shared memory, double
-// buffered, one barrier per column.  Out: L (unit diagonal implied, d on the
-// diagonal) to the panel, d to D, V to linv (zeros above the diagonal).
-// Bound: the chain of w pivots (1 / d 364 cycles, product and update 115,
-// barrier and shared memory ~70), about 0.3 us per column.
+// diagonal block (w <= 32) and the inverse V of its unit lower triangle, by
+// in-place elimination on [A | I]: at column j, row i > j becomes row i - l_i
+// row j, and the freed slot (i, j) takes V's -l_i.
+// Bound: the chain of w pivots.  Warp 0 runs that chain one column ahead of the
+// others: in phase j it updates column j + 1 (lane = row), takes 1 / d (364
+// cycles) and scales (60), while the other warps apply column j to the entries
+// right of column j + 1 and to V (up to three entries per thread, in
+// registers).  They exchange l and u of column j, column j + 1 before its last
+// update and V's row j through shared memory, double buffered, one barrier per
+// column.  Out: L (unit diagonal implied, d on the diagonal) to the panel, d to
+// D, V to linv (zeros above the diagonal).
 template <class T>
 __global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns,
                                                       int p, T* __restrict__ L, T* __restrict__ D,
                                                       T* __restrict__ Linv, Sizes sz, int* status) {
-  __shared__ __align__(16) double raw[2 * (kFB + 1) * Sc<T>::P];
-  T* buf = reinterpret_cast<T*>(raw);  // [2][kFB + 1]: column / row entries, then 1 / d
+  __shared__ __align__(16) double raw[2 * 4 * kFB * Sc<T>::P];
+  // of parity j & 1: l and u of column j, column j before the update by column j - 1, V's row j
+  T* sl = reinterpret_cast<T*>(raw);
+  T *su = sl + 2 * kFB, *spre = su + 2 * kFB, *sv = spre + 2 * kFB;
   const int b = blockIdx.y;
   const SnMeta m = meta[sns[blockIdx.x]];
   const int s = m.s, ld = m.s + m.r, c0 = p * kFB, w = min(kFB, s - c0);
   T* P = L + b * sz.panel + m.panel + c0 + (int64_t)c0 * ld;
   T* V = Linv + b * sz.linv + m.linv + c0 + (int64_t)c0 * s;
+  T* d = D + b * sz.n + m.f + c0;
+  if (threadIdx.x < 32) {
+    const int i = threadIdx.x;
+    T c = i < w ? P[i] : Sc<T>::zero();  // column 0
+    for (int j = 0;; ++j) {
+      // c: column j, final
+      if (i == j) {
+        if (Sc<T>::bad(c)) report_pivot(status, m.f + c0 + i, Sc<T>::is_zero(c));
+        d[i] = c;
+        P[i + (int64_t)i * ld] = c;
+        V[i + (int64_t)i * s] = Sc<T>::one();
+      }
+      if (j == w - 1) break;
+      const T rd = Sc<T>::one() / shfl(c, j);
+      const int o = (j & 1) * kFB;
+      if (i > j && i < w) {
+        const T l = c * rd;
+        sl[o + i] = l;
+        su[o + i] = c;
+        P[i + (int64_t)j * ld] = l;
+      }
+      __syncthreads();
+      if (i > j && i < w) c = spre[(kFB - o) + i] - sl[o + i] * su[o + j + 1];
+    }
+    return;
+  }
   const int ne = w * (w + 1) / 2;
-  T x[kFdEntries], l[kFdEntries];
+  T x[kFdEntries];
   int ri[kFdEntries], ck[kFdEntries];
 #pragma unroll
   for (int q = 0; q < kFdEntries; ++q) {
-    const int e = threadIdx.x + q * kFdThreads;
+    const int e = threadIdx.x - 32 + q * kFdUpdate;
     ri[q] = ck[q] = -1;  // no entry: never live
     if (e < ne) {
       tri_entry(e, ri[q], ck[q]);
-      x[q] = P[ri[q] + (int64_t)ck[q] * ld];
-      if (ck[q] == 0) {
-        if (ri[q] == 0)
-          buf[kFB] = Sc<T>::one() / x[q];
-        else
-          buf[ri[q]] = x[q];
-      }
+      if (ck[q] > 0) x[q] = P[ri[q] + (int64_t)ck[q] * ld];  // column 0 is the pivot warp's
+      if (ck[q] == 1) spre[kFB + ri[q]] = x[q];
     }
   }
-  __syncthreads();
   for (int j = 0; j + 1 < w; ++j) {
-    const T* cur = buf + (j & 1) * (kFB + 1);
-    T* nxt = buf + (~j & 1) * (kFB + 1);
-    const T rd = cur[kFB];
+    __syncthreads();
+    const int o = (j & 1) * kFB;
 #pragma unroll
     for (int q = 0; q < kFdEntries; ++q) {
       const int i = ri[q], k = ck[q];
-      if (i <= j) continue;
-      const T t = cur[i] * rd;  // l_i
-      if (k == j) {
-        l[q] = t;
-        x[q] = -t;
-      } else {
-        x[q] -= t * cur[k];  // k > j: u_k = A_kj; k < j: V_jk
-      }
-      // what column j + 1 reads: its entries below the pivot, V's row j + 1, 1 / pivot
-      if (k == j + 1) {
-        if (i == k)
-          nxt[kFB] = Sc<T>::one() / x[q];
-        else
-          nxt[i] = x[q];
-      } else if (i == j + 1) {
-        nxt[k] = x[q];
-      }
+      if (i <= j || k == j + 1) continue;  // column j + 1 is the pivot warp's
+      if (k == j)
+        x[q] = -sl[o + i];
+      else
+        x[q] -= sl[o + i] * (k > j ? su[o + k] : sv[o + k]);
+      if (k == j + 2) spre[o + i] = x[q];              // parity of column j + 2
+      if (i == j + 1) sv[kFB - o + k] = x[q];          // k <= j: V's row j + 1
     }
-    __syncthreads();
   }
 #pragma unroll
   for (int q = 0; q < kFdEntries; ++q) {
     const int i = ri[q], k = ck[q];
-    if (i < 0) continue;
-    if (i == k) {
-      if (Sc<T>::bad(x[q])) report_pivot(status, m.f + c0 + i, Sc<T>::is_zero(x[q]));
-      D[b * sz.n + m.f + c0 + i] = x[q];
-      P[i + (int64_t)i * ld] = x[q];
-      V[i + (int64_t)i * s] = Sc<T>::one();
-    } else {
-      P[i + (int64_t)k * ld] = l[q];
-      V[i + (int64_t)k * s] = x[q];
-      V[k + (int64_t)i * s] = Sc<T>::zero();
-    }
+    if (i <= k) continue;
+    V[i + (int64_t)k * s] = x[q];
+    V[k + (int64_t)i * s] = Sc<T>::zero();
   }
 }
 

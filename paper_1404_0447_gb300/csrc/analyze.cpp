@@ -660,10 +660,9 @@ int build_schedule(pselinv_handle* h) {
           const int32_t c0 = p * kFactorBlock, c1 = std::min(m.s, c0 + kFactorBlock), ld = m.s + m.r;
           if (m.s <= c0) continue;
           h->fb_sn.push_back(k);
-          for (int32_t m0 = c1; m0 < ld; m0 += kTileM)
-            for (int32_t n0 = c0; n0 < c1; n0 += 8) tp.tasks.push_back({k, m0, n0, p});
+          for (int32_t m0 = c1; m0 < ld; m0 += kFPanelRows) tp.tasks.push_back({k, m0, c0, p});
           for (int32_t n0 = c1; n0 < m.s; n0 += 8)
-            for (int32_t m0 = n0; m0 < ld; m0 += kTileM) tu.tasks.push_back({k, m0, n0, p});
+            for (int32_t m0 = n0; m0 < ld; m0 += kFUpdateRows) tu.tasks.push_back({k, m0, n0, p});
           if (p == 0 && m.s > kFactorBlock)
             for (int32_t n0 = 0; n0 < m.s; n0 += 8) tv.tasks.push_back({k, 0, n0, 0});
         }

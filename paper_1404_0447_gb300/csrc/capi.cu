@@ -276,8 +276,6 @@ psi::KArgs kargs(pselinv_handle* h) {
   psi::KArgs a;
   a.dtype = h->opts.dtype;
   a.maxw = h->max_width;
-  a.fblock = 0;
-  a.blocked = 0;
   a.meta = (const psi::SnMeta*)h->d_meta;
   a.desc = (const psi::ColDesc*)h->d_desc;
   a.relidx = (const int32_t*)h->d_relidx;
@@ -294,9 +292,7 @@ psi::KArgs kargs(pselinv_handle* h) {
   a.sz = sizes(h);
   a.U = h->d_U;
   a.Uinv = h->d_uinv;
-  a.Uhat = nullptr;
   a.XU = h->d_XU;
-  a.strict = 0;
   a.piv = h->pivoted ? (const int32_t*)h->d_piv : nullptr;
   a.ptype = h->pivoted ? (const int8_t*)h->d_ptype : nullptr;
   a.E = h->pivoted ? h->d_E : nullptr;
@@ -642,13 +638,12 @@ int ensure_factor_streams(pselinv_handle* h) {
     h->fev.push_back(e);
   }
   if (h->far_after_near.empty()) {
-    // Per level l: does far(l) wait for near(l), so that level l - 1's
-    // diagonal blocks start beside it?  A diagonal-block CTA does not fit on
-    // an SM beside resident Schur tiles, so when far(l) is already running the
-    // next diagonal blocks wait for its end.  Worth it when far(l) is short
-    // against the next level's diagonal blocks and panel solves (model: FP64
-    // work at 1 TFLOP/s; a diagonal block of width w, 345 us (w / 128)^3 +
-    // 30 us, measured on the 1,024-thread kernel).
+    // Per level l: does far(l) wait for near(l), so that level l - 1's panels
+    // start beside it?  The pivot chain of a diagonal block and the panel tiles
+    // run several times slower beside resident Schur tiles (one FP64 pipe per
+    // SM), so when far(l) is already running they crawl until its end.  Worth it
+    // when far(l) is short against the next level's panels (model: FP64 work at
+    // 1 TFLOP/s; 30 us per 32 columns of the widest supernode).
     const int32_t nl = h->nlevels;
     std::vector<double> t_far(nl, 0.0), t_next(nl, 0.0);
     for (int32_t l = 0; l < nl; ++l) {
@@ -660,9 +655,8 @@ int ensure_factor_streams(pselinv_handle* h) {
         solve += (double)m.r * m.s * m.s;
         wmax = std::max(wmax, m.s);
       }
-      const double w = wmax / 128.0;
       t_far[l] = far / 1e12;
-      t_next[l] = 345e-6 * w * w * w + 30e-6 + solve / 1e12;
+      t_next[l] = 30e-6 * ((wmax + psi::kFactorBlock - 1) / psi::kFactorBlock) + solve / 1e12;
     }
     h->far_after_near.assign(nl, 0);
     for (int32_t l = 1; l < nl; ++l) h->far_after_near[l] = t_far[l] < 4.0 * t_next[l - 1];
@@ -671,13 +665,12 @@ int ensure_factor_streams(pselinv_handle* h) {
 }
 
 // Supernodal factorisation, level by level from the leaves.  Symmetric:
-// A = L D L^T.  Non-symmetric (d_upper set): A = L D U', the U side running
-// the same panel-solve, copy and Schur kernels through swapped pointers.
+// A = L D L^T.  Non-symmetric (d_upper set): A = L D U', both sides in every
+// launch (blockIdx.z).
 int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cudaStream_t st, bool bk = false) {
   const psi::Sizes sz = sizes(h);
   const int64_t B = h->opts.batch;
   const bool unsym = d_upper != nullptr;
-  const bool blocked = !unsym && !bk;  // panels factored kFactorBlock columns at a time
   h->factored = h->inverted = false;
   if (bk && !h->d_piv) {
     int rc;
@@ -690,37 +683,29 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   if (unsym) PSI_CUDA(h, cudaMemsetAsync(h->d_U, 0, elem_size(h) * B * h->panel_total, st));
   PSI_CUDA(h, cudaMemsetAsync(h->d_status, 0x7f, 2 * sizeof(int), st));  // pivot key: unset
   PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, sizeof(int) * (kStatusWords - 2), st));
-  psi::KArgs a = kargs(h);
-  a.XU = nullptr;
   if (unsym)
     PSI_CUDA(h, psi::launch_scatter_values_lu(h->opts.dtype, d_lower, d_upper, (const int64_t*)h->d_valmap,
                                               (const uint8_t*)h->d_flipmap, h->nnz_a, h->d_L, h->d_U, sz, st));
   else
     PSI_CUDA(h, psi::launch_scatter_values(h->opts.dtype, d_lower, (const int64_t*)h->d_valmap, h->nnz_a, h->d_L,
                                            sz, st));
-  // L side: L_{C,K} = A_{C,K} (L_KK^{-T} or U'_KK^{-1}) D^{-1} into lhat, copied to the L panels
-  psi::KArgs al = a;
-  if (unsym) al.Linv = h->d_uinv;
-  // U side: U'_{K,C}^T = A_{K,C}^T L_KK^{-T} D^{-1} into uhat, copied to the U panels
-  psi::KArgs au = a;
-  au.L = h->d_U;
-  au.Lhat = h->d_uhat;
-  // the panel solves also keep W = L_{C,K} D_K (U'_{K,C}^T D_K; with pivots,
-  // D_K's 1 x 1 and 2 x 2 blocks), in the X (XU) panels, which a factorisation
-  // withdraws, as the Schur update's first operand
-  al.W = h->d_X;
-  if (unsym) au.W = h->d_XU;
-  // Schur: L_{C,K} D U'_{K,C} into the L panels, and its strict upper part (transposed) into the U panels
-  psi::KArgs sl = a, su = a;
-  sl.W = al.W;
-  su.W = au.W;
-  if (unsym) {
-    sl.Uhat = h->d_uhat;
-    su.L = h->d_U;
-    su.Lhat = h->d_uhat;
-    su.Uhat = h->d_lhat;
-    su.strict = 1;
-  }
+  const int dt = h->opts.dtype;
+  psi::FArgs f;
+  f.meta = (const psi::SnMeta*)h->d_meta;
+  f.desc = (const psi::ColDesc*)h->d_desc;
+  f.relidx = (const int32_t*)h->d_relidx;
+  f.L[0] = h->d_L;
+  f.L[1] = h->d_U;
+  f.Linv[0] = h->d_linv;
+  f.Linv[1] = h->d_uinv;
+  f.W[0] = h->d_X;  // which a factorisation withdraws
+  f.W[1] = h->d_XU;
+  f.D = h->d_D;
+  f.status = (int*)h->d_status;
+  f.sz = sz;
+  f.sides = unsym ? 2 : 1;
+  psi::KArgs a = kargs(h);  // pivoted panel solves
+  a.W = h->d_X;
   // Two streams (look-ahead): `hi` (high priority) runs each level's
   // diagonal blocks, panel solves and "near" Schur tiles (those updating the
   // parents' columns, which the next level's diagonal blocks need); `lo` runs
@@ -743,14 +728,12 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   PSI_CUDA(h, cudaStreamWaitEvent(lo, ev[0], 0));
   const auto* lsn = (const int32_t*)h->d_levelsn;
   auto schur = [&](const std::vector<psi::Range>& grp, int32_t g0, int32_t g1, cudaStream_t s) -> cudaError_t {
-    for (int side = 0; side < (unsym ? 2 : 1); ++side)
-      for (int32_t g = g0; g < g1; ++g) {  // group by group: disjoint targets inside a group, no atomics
-        const psi::Range r = grp[g];
-        if (r.end == r.begin) continue;
-        cudaError_t e = psi::launch_tiles(psi::Kern::Schur, h->schur_gvar[g], side ? su : sl,
-                                          tasks_at(h, h->off_schur, r.begin), r.end - r.begin, s);
-        if (e != cudaSuccess) return e;
-      }
+    for (int32_t g = g0; g < g1; ++g) {  // group by group: disjoint targets inside a group, no atomics
+      const psi::Range r = grp[g];
+      cudaError_t e = psi::launch_ftiles(psi::FKern::Schur, h->schur_gvar[g], dt, f,
+                                         tasks_at(h, h->off_schur, r.begin), r.end - r.begin, s);
+      if (e != cudaSuccess) return e;
+    }
     return cudaSuccess;
   };
   for (int32_t l = nl - 1; l >= 0; --l) {
@@ -758,39 +741,28 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
     int wmax = 0;
     for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) wmax = std::max(wmax, h->meta[h->level_sn[t]].s);
-    if (blocked) {
+    if (!bk) {
+      // the panels of the level, kFactorBlock columns at a time
       for (int p = 0; p < psi::kFactorBlocks && wmax > p * psi::kFactorBlock; ++p) {
         const size_t at = (size_t)l * psi::kFactorBlocks + p;
         const psi::Range rs = h->fb_range[at], rp = h->t_fpanel.per_lv[at], ru = h->t_fupdate.per_lv[at];
-        psi::KArgs ad = a;
-        ad.fblock = p;
-        PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiag, ad, (const int32_t*)h->d_fbsn + rs.begin,
-                                       (int)(rs.end - rs.begin), hi));
-        PSI_CUDA(h, psi::launch_tiles(psi::Kern::FPanel, 0, al, tasks_at(h, h->off_fpanel, rp.begin),
-                                      rp.end - rp.begin, hi));
-        PSI_CUDA(h, psi::launch_tiles(psi::Kern::FUpdate, 0, al, tasks_at(h, h->off_fupdate, ru.begin),
-                                      ru.end - ru.begin, hi));
+        PSI_CUDA(h, psi::launch_fdiag(dt, f, (const int32_t*)h->d_fbsn + rs.begin, (int)(rs.end - rs.begin), p, hi));
+        PSI_CUDA(h, psi::launch_ftiles(psi::FKern::Panel, 0, dt, f, tasks_at(h, h->off_fpanel, rp.begin),
+                                       rp.end - rp.begin, hi));
+        PSI_CUDA(h, psi::launch_ftiles(psi::FKern::Update, 0, dt, f, tasks_at(h, h->off_fupdate, ru.begin),
+                                       ru.end - ru.begin, hi));
       }
     } else {
-      // a level holding a wide supernode gets wide CTAs: the column steps of the
-      // diagonal factorisation are serial, the work inside each step is not;
       // shared memory sized for the level's widest block: several CTAs per SM on levels of narrow supernodes
       psi::KArgs ad = a;
       ad.maxw = wmax;
-      PSI_CUDA(h, psi::launch_per_sn(unsym ? psi::Kern::FactorDiagLU : psi::Kern::FactorDiagBK, ad, sns, nsl, hi,
-                                     wmax >= 64 ? 1024 : 256));
-      for (int side = 0; side < (unsym ? 2 : 1); ++side) {
-        const psi::KArgs& ka = side ? au : al;
-        for (int v = 0; v < psi::kNumVar; ++v) {
-          const psi::Range r = h->t_trsm.per_lv[(size_t)l * psi::kNumVar + v];
-          PSI_CUDA(h, psi::launch_tiles(psi::Kern::Trsm, v, ka, tasks_at(h, h->off_trsm, r.begin), r.end - r.begin,
-                                        hi));
-        }
-        // the pivoted copy-back also divides the scratch by 2x2 blocks of D, which the Schur
-        // update reads: per level; the plain one only fills the panels (nothing in the
-        // factorisation reads L_{C,K} from them): once for all levels, after the loop
-        if (bk) PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBackBK, ka, sns, nsl, hi));
+      PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiagBK, ad, sns, nsl, hi, wmax >= 64 ? 512 : 256));
+      for (int v = 0; v < psi::kNumVar; ++v) {
+        const psi::Range r = h->t_trsm.per_lv[(size_t)l * psi::kNumVar + v];
+        PSI_CUDA(h, psi::launch_tiles(psi::Kern::Trsm, v, a, tasks_at(h, h->off_trsm, r.begin), r.end - r.begin, hi));
       }
+      // L_{C,K} to the panels (the Schur update's second operand)
+      PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBackBK, a, sns, nsl, hi));
     }
     if (h->far_after_near[l]) {
       if (l + 1 < nl) PSI_CUDA(h, cudaStreamWaitEvent(hi, ev[1 + nl + l + 1], 0));
@@ -812,14 +784,10 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   PSI_CUDA(h, cudaStreamWaitEvent(st, ev[1 + 2 * nl], 0));
   PSI_CUDA(h, cudaEventRecord(ev[2 + 2 * nl], lo));
   PSI_CUDA(h, cudaStreamWaitEvent(st, ev[2 + 2 * nl], 0));
-  al.blocked = blocked;
+  // (L_KK)^{-1} off its 32 x 32 diagonal blocks, every supernode at once
   if (!bk)
-    for (int side = 0; side < (unsym ? 2 : 1); ++side)
-      PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBack, side ? au : al, lsn, h->nsn, st));
-  // (L_KK)^{-1} off its diagonal blocks, from the panels just filled
-  if (blocked)
-    PSI_CUDA(h, psi::launch_tiles(psi::Kern::VInv, 0, al, tasks_at(h, h->off_vinv, 0),
-                                  (int64_t)h->t_vinv.tasks.size(), st));
+    PSI_CUDA(h, psi::launch_ftiles(psi::FKern::VInv, 0, dt, f, tasks_at(h, h->off_vinv, 0),
+                                   (int64_t)h->t_vinv.tasks.size(), st));
   // no host synchronisation: the first bad pivot stays in status words 0-1
   // until the next factorisation and is reported by pselinv_sync_status (and
   // by pselinv_logdet, which synchronises anyway)

@@ -76,6 +76,8 @@ constexpr int kTileN = 64;       // output tile columns
 // diagonal blocks on one SM's FP64 pipe.
 constexpr int kFactorBlock = 32;
 constexpr int kFactorBlocks = (kMaxWidth + kFactorBlock - 1) / kFactorBlock;
+constexpr int kFPanelRows = 16;  // rows of a k_fpanel task (8 per warp)
+constexpr int kFUpdateRows = 32; // rows of a k_fupdate task
 
 // Tile-width variants of the tile GEMMs: BN = 8 << var.
 constexpr int kNumVar = 4;
@@ -152,11 +154,11 @@ struct pselinv_handle {
   psi::TaskList t_gemm1;  // step 2 tiles (with k-slices of split supernodes)
   psi::TaskList t_rect;   // r x s tiles per level, unsplit (adjoint)
   psi::TaskList t_gemm2;  // step 3 partial-product tiles
-  psi::TaskList t_trsm;   // factorisation (pivoted, non-symmetric): off-diagonal panel solve tiles
+  psi::TaskList t_trsm;   // pivoted factorisation: off-diagonal panel solve tiles
   // blocked factorisation: per (level, block) at [level * kFactorBlocks + p] the
   // supernodes of the level wider than p blocks (fb_sn), the tiles of the rows
-  // below block p (t_fpanel) and of the columns right of it (t_fupdate), all
-  // 64 x 8; t_vinv: 8-column strips of the inverses of all supernodes wider than a block
+  // below block p (t_fpanel) and of the columns right of it (t_fupdate);
+  // t_vinv: 8-column strips of the inverses of all supernodes wider than a block
   std::vector<int32_t> fb_sn;
   std::vector<psi::Range> fb_range;
   psi::TaskList t_fpanel, t_fupdate, t_vinv;

@@ -94,22 +94,6 @@ __global__ void k_gather_values(const T* __restrict__ X, int64_t panel_total, co
 // --------------------------------------------------------------------------
 
 // V = (L_KK)^{-1} for the unit lower triangle held packed in Tp (shared
-// memory), written column-major to global memory (ld s, zeros above the
-// diagonal); one column per thread.
-template <class T>
-__device__ void unit_lower_inverse(const T* Tp, int s, T* V) {
-  for (int c = threadIdx.x; c < s; c += blockDim.x) {
-    for (int i = 0; i < c; ++i) V[i + c * s] = Sc<T>::zero();
-    V[c + c * s] = Sc<T>::one();
-    for (int i = c + 1; i < s; ++i) {
-      T acc = Sc<T>::zero();
-      for (int q = c; q < i; ++q) acc += Tp[pk(i, q, s)] * V[q + c * s];
-      V[i + c * s] = -acc;
-    }
-  }
-}
-
-// V = (L_KK)^{-1} for the unit lower triangle held packed in Tp (shared
 // memory), by 16 x 16 blocks so that the whole CTA works at every step:
 // first the diagonal blocks V_ii = (L_ii)^{-1} (one column per thread),
 // then, for block distance d = 1, 2, ... (all block pairs (i, j) with
@@ -186,6 +170,11 @@ __device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
 // diagonal block (w <= 32) and the inverse V of its unit lower triangle, by
 // in-place elimination on [A | I]: at column j, row i > j becomes row i - l_i
 // row j, and the freed slot (i, j) takes V's -l_i.
+// SIDES 2, non-symmetric block A = L D U': the lower triangle (panel L, V to
+// linv) and the transposed upper one (panel U, V = (U'^T)^{-1} to uinv) are
+// eliminated side by side, each with its own l and the other's unscaled column
+// u; the pivots are those of the lower triangle, and on symmetric input both
+// sides do the arithmetic of SIDES 1.
 // Bound: the chain of w pivots.  Warp 0 runs that chain one column ahead of the
 // others: in phase j it updates column j + 1 (lane = row), takes 1 / d (364
 // cycles) and scales (60), while the other warps apply column j to the entries
@@ -194,51 +183,68 @@ __device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
 // update and V's row j through shared memory, double buffered, one barrier per
 // column.  Out: L (unit diagonal implied, d on the diagonal) to the panel, d to
 // D, V to linv (zeros above the diagonal).
-template <class T>
-__global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns,
-                                                      int p, T* __restrict__ L, T* __restrict__ D,
-                                                      T* __restrict__ Linv, Sizes sz, int* status) {
-  __shared__ __align__(16) double raw[2 * 4 * kFB * Sc<T>::P];
-  // of parity j & 1: l and u of column j, column j before the update by column j - 1, V's row j
-  T* sl = reinterpret_cast<T*>(raw);
-  T *su = sl + 2 * kFB, *spre = su + 2 * kFB, *sv = spre + 2 * kFB;
+template <class T, int SIDES>
+__global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const int32_t* __restrict__ sns, int p) {
+  __shared__ __align__(16) double raw[SIDES * 2 * 4 * kFB * Sc<T>::P];
+  // per side, of parity j & 1: l and u of column j, column j before the update by column j - 1, V's row j
+  constexpr int SD = 8 * kFB;
+  T* sh = reinterpret_cast<T*>(raw);
   const int b = blockIdx.y;
-  const SnMeta m = meta[sns[blockIdx.x]];
+  const SnMeta m = f.meta[sns[blockIdx.x]];
   const int s = m.s, ld = m.s + m.r, c0 = p * kFB, w = min(kFB, s - c0);
-  T* P = L + b * sz.panel + m.panel + c0 + (int64_t)c0 * ld;
-  T* V = Linv + b * sz.linv + m.linv + c0 + (int64_t)c0 * s;
-  T* d = D + b * sz.n + m.f + c0;
+  const int64_t po = b * f.sz.panel + m.panel + c0 + (int64_t)c0 * ld, vo = b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
   if (threadIdx.x < 32) {
     const int i = threadIdx.x;
-    T c = i < w ? P[i] : Sc<T>::zero();  // column 0
-    for (int j = 0;; ++j) {
-      // c: column j, final
-      if (i == j) {
-        if (Sc<T>::bad(c)) report_pivot(status, m.f + c0 + i, Sc<T>::is_zero(c));
-        d[i] = c;
-        P[i + (int64_t)i * ld] = c;
-        V[i + (int64_t)i * s] = Sc<T>::one();
-      }
-      if (j == w - 1) break;
-      const T rd = Sc<T>::one() / shfl(c, j);
+    T* d = (T*)f.D + b * f.sz.n + m.f + c0;
+    T c[SIDES];
+#pragma unroll
+    for (int e = 0; e < SIDES; ++e) c[e] = i < w ? ((T*)f.L[e] + po)[i] : Sc<T>::zero();  // column 0
+    // column j, final: d_j out (off the chain)
+    auto finish = [&](int j, T v) {
+      if (i != j) return;
+      if (Sc<T>::bad(v)) report_pivot(f.status, m.f + c0 + i, Sc<T>::is_zero(v));
+      d[i] = v;
+      ((T*)f.L[0] + po)[i + (int64_t)i * ld] = v;
+#pragma unroll
+      for (int e = 0; e < SIDES; ++e) ((T*)f.Linv[e] + vo)[i + (int64_t)i * s] = Sc<T>::one();
+    };
+    for (int j = 0; j + 1 < w; ++j) {
+      const T rd = Sc<T>::one() / shfl(c[0], j);
       const int o = (j & 1) * kFB;
-      if (i > j && i < w) {
-        const T l = c * rd;
-        sl[o + i] = l;
-        su[o + i] = c;
-        P[i + (int64_t)j * ld] = l;
+      T l[SIDES], u[SIDES];
+#pragma unroll
+      for (int e = 0; e < SIDES; ++e) {
+        l[e] = c[e] * rd;
+        sh[e * SD + o + i] = l[e];  // rows above j are not read
+        sh[e * SD + 2 * kFB + o + i] = c[e];
+        u[e] = shfl(c[e], j + 1);
       }
       __syncthreads();
-      if (i > j && i < w) c = spre[(kFB - o) + i] - sl[o + i] * su[o + j + 1];
+      T next[SIDES];  // rows above j + 1 and from w: never used
+#pragma unroll
+      for (int e = 0; e < SIDES; ++e) next[e] = sh[e * SD + 4 * kFB + (kFB - o) + i] - l[e] * u[SIDES - 1 - e];
+      finish(j, c[0]);
+#pragma unroll
+      for (int e = 0; e < SIDES; ++e) {
+        if (i > j && i < w) ((T*)f.L[e] + po)[i + (int64_t)j * ld] = l[e];
+        c[e] = next[e];
+      }
     }
+    finish(w - 1, c[0]);
     return;
   }
+  const int side = SIDES == 1 ? 0 : (threadIdx.x - 32) / kFdUpdate;
+  const int t = threadIdx.x - 32 - side * kFdUpdate;
+  const T* P = (const T*)f.L[side] + po;
+  T* V = (T*)f.Linv[side] + vo;
+  T *sl = sh + side * SD, *spre = sl + 4 * kFB, *sv = sl + 6 * kFB;
+  const T* su = sh + (SIDES - 1 - side) * SD + 2 * kFB;
   const int ne = w * (w + 1) / 2;
   T x[kFdEntries];
   int ri[kFdEntries], ck[kFdEntries];
 #pragma unroll
   for (int q = 0; q < kFdEntries; ++q) {
-    const int e = threadIdx.x - 32 + q * kFdUpdate;
+    const int e = t + q * kFdUpdate;
     ri[q] = ck[q] = -1;  // no entry: never live
     if (e < ne) {
       tri_entry(e, ri[q], ck[q]);
@@ -257,8 +263,8 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__
         x[q] = -sl[o + i];
       else
         x[q] -= sl[o + i] * (k > j ? su[o + k] : sv[o + k]);
-      if (k == j + 2) spre[o + i] = x[q];              // parity of column j + 2
-      if (i == j + 1) sv[kFB - o + k] = x[q];          // k <= j: V's row j + 1
+      if (k == j + 2) spre[o + i] = x[q];   // parity of column j + 2
+      if (i == j + 1) sv[kFB - o + k] = x[q];  // k <= j: V's row j + 1
     }
   }
 #pragma unroll
@@ -270,6 +276,124 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__
   }
 }
 
+// acc (8 x 8 fragment: lane l holds row l >> 2, columns 2 (l & 3) + {0, 1}) +=
+// A B with A's fragments a (lane: row l >> 2, k = 4 u + (l & 3)) and B's
+// fragments bf (lane: k = 4 u + (l & 3), column l >> 2), U k-steps of 4.
+template <class T, int U>
+__device__ __forceinline__ void frag_mma(double (&acc)[Sc<T>::P][2], const T* a, const T* bf) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if constexpr (Sc<T>::P == 1) {
+      dmma884(acc[0][0], acc[0][1], a[u], bf[u]);
+    } else {
+      dmma884(acc[0][0], acc[0][1], a[u].re, bf[u].re);
+      dmma884(acc[0][0], acc[0][1], -a[u].im, bf[u].im);
+      dmma884(acc[1][0], acc[1][1], a[u].re, bf[u].im);
+      dmma884(acc[1][0], acc[1][1], a[u].im, bf[u].re);
+    }
+  }
+}
+template <class T>
+__device__ __forceinline__ T frag_value(const double (&acc)[Sc<T>::P][2], int e) {
+  if constexpr (Sc<T>::P == 1) return acc[0][e];
+  else return T{acc[0][e], acc[1][e]};
+}
+
+// Blocked factorisation, rows m0 .. m0+15 of the panel below the diagonal block
+// p (task c): W = A V_pp^T = L D, kept in the X panels (same layout) as the
+// first operand of the panel and Schur updates, and L = W D^{-1} in place.
+// One warp per 8 rows and all (up to 32) columns of the block, so a row's
+// entries are read and written by one warp only; operand fragments go straight
+// from global memory to registers, all loads in flight at once.  Bound: the
+// FP64 pipe (20 m8n8k4 MMAs of 145 cycles a warp); shared-memory staging and
+// 64-row tiles would leave most SMs idle on the levels near the root, where a
+// 64 x 8 tile took 8.7 us however few there were.
+// blockIdx.z = 1: the U side of a non-symmetric factor, U'_{K,C}^T = A_{K,C}^T
+// L_KK^{-T} D^{-1}, as L_{C,K} = A_{C,K} U'_KK^{-1} D^{-1} uses (U'_KK^T)^{-1}.
+constexpr int kFPanelWarps = kFPanelRows / 8;
+template <class T>
+__global__ void __launch_bounds__(32 * kFPanelWarps) k_fpanel(FArgs f, const Task* __restrict__ tasks) {
+  __shared__ __align__(16) double raw[kFB * Sc<T>::P];
+  T* rd = reinterpret_cast<T*>(raw);
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y, side = blockIdx.z;
+  const SnMeta m = f.meta[tk.sn];
+  const int s = m.s, ld = s + m.r, c0 = tk.c * kFB, w = min(kFB, s - c0);
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  T* A = (T*)f.L[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
+  T* Wp = (T*)f.W[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
+  const T* Vi = (const T*)f.Linv[f.sides - 1 - side] + b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
+  const int row = tk.m0 + 8 * (threadIdx.x >> 5) + g;
+  T a[kFB / 4];
+#pragma unroll
+  for (int u = 0; u < kFB / 4; ++u) {
+    const int k = 4 * u + q;
+    a[u] = row < ld && k < w ? A[row + (int64_t)k * ld] : Sc<T>::zero();
+  }
+  if (threadIdx.x < w) rd[threadIdx.x] = Sc<T>::one() / ((const T*)f.D + b * f.sz.n + m.f + c0)[threadIdx.x];
+  double acc[kFB / 8][Sc<T>::P][2] = {};
+#pragma unroll
+  for (int j = 0; j < kFB / 8; ++j) {
+    // V_pp^T is upper triangular: columns 8 j .. 8 j + 7 need k < 8 j + 8
+    T bf[kFB / 4];
+#pragma unroll
+    for (int u = 0; u < 2 * j + 2; ++u) {
+      const int k = 4 * u + q, n = 8 * j + g;
+      bf[u] = n < w && k < w ? Vi[n + (int64_t)k * s] : Sc<T>::zero();
+    }
+    if (8 * j >= w) continue;
+    if (j == 0) frag_mma<T, 2>(acc[j], a, bf);
+    if (j == 1) frag_mma<T, 4>(acc[j], a, bf);
+    if (j == 2) frag_mma<T, 6>(acc[j], a, bf);
+    if (j == 3) frag_mma<T, 8>(acc[j], a, bf);
+  }
+  __syncthreads();  // rd; and every lane has read its row's entries
+  if (row >= ld) return;
+#pragma unroll
+  for (int j = 0; j < kFB / 8; ++j)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int col = 8 * j + 2 * q + e;
+      if (col >= w) continue;
+      const T v = frag_value<T>(acc[j], e);
+      Wp[row + (int64_t)col * ld] = v;
+      A[row + (int64_t)col * ld] = v * rd[col];
+    }
+}
+
+// Blocked factorisation, the columns right of block p (task c) of the panel:
+// A_ij -= sum_k W_ik L_jk over the block's 32 columns k, rows i >= j of the
+// whole panel (i > j on the U side), each entry by one thread; one warp per
+// 8 x 8 fragment of a 32 x 8 tile, operands straight to registers (see k_fpanel).
+template <class T>
+__global__ void __launch_bounds__(TG_THREADS) k_fupdate(FArgs f, const Task* __restrict__ tasks) {
+  const Task tk = tasks[blockIdx.x];
+  const int b = blockIdx.y, side = blockIdx.z;
+  const SnMeta m = f.meta[tk.sn];
+  const int s = m.s, ld = s + m.r, c0 = tk.c * kFB;
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int64_t po = b * f.sz.panel + m.panel;
+  T* P = (T*)f.L[side] + po;
+  const T* L2 = (const T*)f.L[f.sides - 1 - side] + po + (int64_t)c0 * ld;
+  const T* Wp = (const T*)f.W[side] + po + (int64_t)c0 * ld;
+  const int r0 = tk.m0 + 8 * (threadIdx.x >> 5);
+  if (r0 >= ld) return;
+  T a[kFB / 4], bf[kFB / 4];
+#pragma unroll
+  for (int u = 0; u < kFB / 4; ++u) {
+    const int64_t k = (int64_t)(4 * u + q) * ld;
+    a[u] = r0 + g < ld ? Wp[r0 + g + k] : Sc<T>::zero();
+    bf[u] = tk.n0 + g < s ? L2[tk.n0 + g + k] : Sc<T>::zero();
+  }
+  double acc[Sc<T>::P][2] = {};
+  frag_mma<T, kFB / 4>(acc, a, bf);
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int row = r0 + g, col = tk.n0 + 2 * q + e;
+    if (row < ld && col < s && row >= col + side) P[row + (int64_t)col * ld] -= frag_value<T>(acc, e);
+  }
+}
+
 // (L_KK)^{-1} off its 32 x 32 diagonal blocks, after the last level, all
 // supernodes wider than 32 at once: one CTA per 8 columns (task n0) of V.
 // With j the block of the columns, X_j = V_jj and, for i = j+1, j+2, ...:
@@ -278,17 +402,16 @@ __global__ void __launch_bounds__(kFdThreads) k_fdiag(const SnMeta* __restrict__
 // (eight 64-byte row runs per k-block, loaded before the products), X in
 // shared memory.  Blocks above the diagonal are written as zeros.
 template <class T>
-__global__ void __launch_bounds__(TG_THREADS) k_vinv(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
-                                                     const T* __restrict__ L, T* __restrict__ Linv, Sizes sz) {
+__global__ void __launch_bounds__(TG_THREADS) k_vinv(FArgs f, const Task* __restrict__ tasks) {
   constexpr int P = Sc<T>::P, LDX = 12;  // 4 (mod 16) doubles
   __shared__ double xs[P][kMaxWidth][LDX];
   __shared__ double ss[P][kFB][LDX];
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y;
-  const SnMeta m = meta[tk.sn];
+  const SnMeta m = f.meta[tk.sn];
   const int s = m.s, ld = m.s + m.r;
-  const T* A = L + b * sz.panel + m.panel;
-  T* V = Linv + b * sz.linv + m.linv;
+  const T* A = (const T*)f.L[blockIdx.z] + b * f.sz.panel + m.panel;
+  T* V = (T*)f.Linv[blockIdx.z] + b * f.sz.linv + m.linv;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
   const int n0 = tk.n0, j0 = n0 / kFB * kFB, j1 = min(s, j0 + kFB), n1 = min(s, n0 + 8);
   for (int e = t; e < j0 * 8; e += TG_THREADS) {
@@ -302,34 +425,27 @@ __global__ void __launch_bounds__(TG_THREADS) k_vinv(const SnMeta* __restrict__ 
     for (int pl = 0; pl < P; ++pl) xs[pl][row][e / kFB] = Sc<T>::plane(v, pl);
   }
   __syncthreads();
-  // acc += (M at rows r0 + g of the block, columns k0 .. k0 + 31) (x rows k0 ..)
-  auto product = [&](const T* M, int64_t mld, int row, bool rlive, int k0, int klim, const double (*x)[LDX],
-                     int64_t xplane, int xr0, double (&acc)[P][2]) {
-    T f[kFB / 4];
+  // acc += (row `row` of M, columns k0 .. k0 + 31, zero from klim) (x from row xr0)
+  auto product = [&](const T* M, int64_t mld, int row, int k0, int klim, const double (*x)[LDX], int64_t xplane,
+                     int xr0, double (&acc)[P][2]) {
+    T fa[kFB / 4], fb[kFB / 4];
 #pragma unroll
     for (int u = 0; u < kFB / 4; ++u) {
       const int kk = k0 + 4 * u + q;
-      f[u] = rlive && kk < klim ? M[row + (int64_t)kk * mld] : Sc<T>::zero();
-    }
-#pragma unroll
-    for (int u = 0; u < kFB / 4; ++u) {
+      fa[u] = row < s && kk < klim ? M[row + (int64_t)kk * mld] : Sc<T>::zero();
       const double* xb = &x[xr0 + 4 * u + q][g];
-      if constexpr (P == 1) {
-        dmma884(acc[0][0], acc[0][1], f[u], xb[0]);
-      } else {
-        const double br = xb[0], bi = xb[xplane];
-        dmma884(acc[0][0], acc[0][1], f[u].re, br);
-        dmma884(acc[0][0], acc[0][1], -f[u].im, bi);
-        dmma884(acc[1][0], acc[1][1], f[u].re, bi);
-        dmma884(acc[1][0], acc[1][1], f[u].im, br);
-      }
+      if constexpr (P == 1)
+        fb[u] = xb[0];
+      else
+        fb[u] = T{xb[0], xb[xplane]};
     }
+    frag_mma<T, kFB / 4>(acc, fa, fb);
   };
   for (int i0 = j1; i0 < s; i0 += kFB) {
     const int row = i0 + 8 * warp + g;
     double acc[P][2] = {};
     for (int k0 = j0; k0 < i0; k0 += kFB)
-      product(A, ld, row, row < s, k0, s, xs[0], kMaxWidth * LDX, k0, acc);
+      product(A, ld, row, k0, s, xs[0], kMaxWidth * LDX, k0, acc);
 #pragma unroll
     for (int pl = 0; pl < P; ++pl)
 #pragma unroll
@@ -338,87 +454,16 @@ __global__ void __launch_bounds__(TG_THREADS) k_vinv(const SnMeta* __restrict__ 
         acc[pl][e] = 0.0;
       }
     __syncthreads();
-    product(V, s, row, row < s, i0, min(s, i0 + kFB), ss[0], kFB * LDX, 0, acc);
+    product(V, s, row, i0, min(s, i0 + kFB), ss[0], kFB * LDX, 0, acc);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int col = n0 + 2 * q + e;
 #pragma unroll
       for (int pl = 0; pl < P; ++pl) xs[pl][i0 + 8 * warp + g][2 * q + e] = -acc[pl][e];
-      if (row < s && col < n1) {
-        if constexpr (P == 1)
-          V[row + (int64_t)col * s] = -acc[0][e];
-        else
-          V[row + (int64_t)col * s] = T{-acc[0][e], -acc[1][e]};
-      }
+      if (row < s && col < n1) V[row + (int64_t)col * s] = -frag_value<T>(acc, e);
     }
     __syncthreads();
   }
-}
-
-// Factorisation of a non-symmetric diagonal block, one CTA per supernode of
-// the level: A_KK = L_KK D_K U'_KK by pivot-free Gaussian elimination in
-// shared memory on two packed triangles, Tl (lower part and diagonal, from
-// the L panel) and Tu (Tu(i, j) = A_ji for i > j, from the U panel).  For
-// column j: d = Tl(j, j); L_ij = Tl(i, j) / d and U'_ji = Tu(i, j) / d; then
-// A_ik -= L_ij d U'_jk for i, k > j, on whichever triangle holds (i, k).
-// Back to the panels (L_KK with D on the diagonal, U'_KK^T), D, and the unit
-// lower inverses (L_KK)^{-1} -> linv, (U'_KK^T)^{-1} -> uinv.  On symmetric
-// input every operation matches k_factor_diag's.
-template <class T>
-__global__ void k_factor_diag_lu(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                                 T* __restrict__ U, T* __restrict__ D, T* __restrict__ Linv, T* __restrict__ Uinv,
-                                 Sizes sz, int* status) {
-  extern __shared__ __align__(16) unsigned char shraw[];
-  const int k = sns[blockIdx.x];
-  const int b = blockIdx.y;
-  const SnMeta m = meta[k];
-  const int s = m.s, ld = m.s + m.r;
-  T* Tl = reinterpret_cast<T*>(shraw);
-  T* Tu = Tl + s * (s + 1) / 2;
-  T* P = L + b * sz.panel + m.panel;
-  T* Q = U + b * sz.panel + m.panel;
-  const int nt = blockDim.x, t = threadIdx.x;
-  for (int e = t; e < s * s; e += nt) {
-    const int i = e % s, j = e / s;
-    if (i >= j) {
-      Tl[pk(i, j, s)] = P[i + (int64_t)j * ld];
-      Tu[pk(i, j, s)] = i > j ? Q[i + (int64_t)j * ld] : Sc<T>::zero();
-    }
-  }
-  __syncthreads();
-  for (int j = 0; j < s; ++j) {
-    const T d = Tl[pk(j, j, s)];
-    if (t == 0 && Sc<T>::bad(d)) report_pivot(status, m.f + j, Sc<T>::is_zero(d));
-    for (int i = j + 1 + t; i < s; i += nt) {
-      Tl[pk(i, j, s)] = Tl[pk(i, j, s)] / d;
-      Tu[pk(i, j, s)] = Tu[pk(i, j, s)] / d;
-    }
-    __syncthreads();
-    // trailing block, one warp per column kk (no integer division)
-    for (int kk = j + 1 + (t >> 5); kk < s; kk += nt >> 5) {
-      const int ck = pk(kk, kk, s);
-      for (int ii = kk + (t & 31); ii < s; ii += 32) {
-        Tl[ck + ii - kk] -= Tl[pk(ii, j, s)] * Tu[pk(kk, j, s)] * d;                      // A_{ii,kk}
-        if (ii > kk) Tu[ck + ii - kk] -= Tu[pk(ii, j, s)] * Tl[pk(kk, j, s)] * d;         // A_{kk,ii}
-      }
-    }
-    __syncthreads();
-  }
-  if constexpr (Sc<T>::P == 1) {  // real: the blocked inverses (their 16 x 16 scratch after the triangles)
-    T* S = Tu + s * (s + 1) / 2;
-    unit_lower_inverse_blocked(Tl, s, Linv + b * sz.linv + m.linv, S);
-    __syncthreads();
-    unit_lower_inverse_blocked(Tu, s, Uinv + b * sz.linv + m.linv, S);
-  } else {  // complex: both triangles fill the shared memory
-    unit_lower_inverse(Tl, s, Linv + b * sz.linv + m.linv);
-    unit_lower_inverse(Tu, s, Uinv + b * sz.linv + m.linv);
-  }
-  for (int e = t; e < s * s; e += nt) {
-    const int i = e % s, j = e / s;
-    if (i >= j) P[i + (int64_t)j * ld] = Tl[pk(i, j, s)];
-    if (i > j) Q[i + (int64_t)j * ld] = Tu[pk(i, j, s)];
-  }
-  for (int j = t; j < s; j += nt) D[b * sz.n + m.f + j] = Tl[pk(j, j, s)];
 }
 
 // |re| + |im|: the magnitude Bunch-Kaufman compares (plain |x| for real)
@@ -613,38 +658,31 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
 }
 
 // Pivoted factor: L_{C,K} = Z D_K^{-1} for the panel-solve output Z =
-// A_{C,K P} L_KK^{-T} held in the factor scratch, with 2x2 blocks of D_K;
-// written to the panel and back into the scratch (the Schur update reads it).
+// A_{C,K P} L_KK^{-T} (kept as W in the X panels' layout), with 2x2 blocks of
+// D_K, written to the panel.
 template <class T>
 __global__ void k_copyback_bk(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                              T* __restrict__ Ltmp, const T* __restrict__ D, const T* __restrict__ E,
+                              const T* __restrict__ W, const T* __restrict__ D, const T* __restrict__ E,
                               const int8_t* __restrict__ ptype, Sizes sz) {
   const int k = sns[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[k];
   const int s = m.s, r = m.r, ld = s + r;
   T* P = L + b * sz.panel + m.panel + s;
-  T* Z = Ltmp + b * sz.lhat + m.lhat;
+  const T* Z = W + b * sz.panel + m.panel + s;
   const T* d = D + b * sz.n + m.f;
   const T* e = E + b * sz.n + m.f;
   const int8_t* ty = ptype + b * sz.n + m.f;
   for (int j = blockIdx.z; j < s; j += gridDim.z) {
     if (ty[j] == 2) continue;  // done with its partner
     if (ty[j] == 0) {
-      for (int i = threadIdx.x; i < r; i += blockDim.x) {
-        const T l = Z[i + (int64_t)j * r] / d[j];
-        Z[i + (int64_t)j * r] = l;
-        P[i + (int64_t)j * ld] = l;
-      }
+      for (int i = threadIdx.x; i < r; i += blockDim.x) P[i + (int64_t)j * ld] = Z[i + (int64_t)j * ld] / d[j];
     } else {
       const T det = d[j] * d[j + 1] - e[j] * e[j];
       for (int i = threadIdx.x; i < r; i += blockDim.x) {
-        const T z1 = Z[i + (int64_t)j * r], z2 = Z[i + (int64_t)(j + 1) * r];
-        const T x1 = (z1 * d[j + 1] - z2 * e[j]) / det, x2 = (z2 * d[j] - z1 * e[j]) / det;
-        Z[i + (int64_t)j * r] = x1;
-        Z[i + (int64_t)(j + 1) * r] = x2;
-        P[i + (int64_t)j * ld] = x1;
-        P[i + (int64_t)(j + 1) * ld] = x2;
+        const T z1 = Z[i + (int64_t)j * ld], z2 = Z[i + (int64_t)(j + 1) * ld];
+        P[i + (int64_t)j * ld] = (z1 * d[j + 1] - z2 * e[j]) / det;
+        P[i + (int64_t)(j + 1) * ld] = (z2 * d[j] - z1 * e[j]) / det;
       }
     }
   }
@@ -700,42 +738,16 @@ __global__ void k_diag_final(KArgs a, const int32_t* __restrict__ sns) {
   if (a.gam) pole_share<T>(a, sns[blockIdx.x], blockIdx.z, gridDim.z);
 }
 
-// Copy the factor scratch back into the panels of the listed supernodes
-// (blockIdx.z strides over the columns; threads run down a column).  Lkk set
-// (blocked factorisation): L_KK below its 32 x 32 diagonal blocks too, from
-// where k_fpanel kept it.
-template <class T>
-__global__ void k_copyback(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                           const T* __restrict__ Ltmp, const T* __restrict__ Lkk, Sizes sz) {
-  const int k = sns[blockIdx.x];
-  const int b = blockIdx.y;
-  const SnMeta m = meta[k];
-  const int s = m.s, r = m.r, ld = s + r;
-  T* P = L + b * sz.panel + m.panel + s;
-  const T* src = Ltmp + b * sz.lhat + m.lhat;
-  const T* lk = Lkk + b * sz.linv + m.linv;
-  for (int j = blockIdx.z; j < s; j += gridDim.z) {
-    for (int i = threadIdx.x; i < r; i += blockDim.x) P[i + (int64_t)j * ld] = src[i + (int64_t)j * r];
-    if (Lkk)
-      for (int i = (j / kFB + 1) * kFB + threadIdx.x; i < s; i += blockDim.x)
-        P[i - s + (int64_t)j * ld] = lk[i + (int64_t)j * s];
-  }
-}
-
 // --------------------------------------------------------------------------
 // tile GEMMs
 // --------------------------------------------------------------------------
 
-// Panel solve of the pivoted and the non-symmetric factorisations:
-// Ltmp_{C,K} = A_{C,K} (L_KK)^{-T} D_K^{-1} and W_{C,K} = A_{C,K} (L_KK)^{-T}
-// itself (the Schur update's L_{C,K} D_K without a product per operand
-// element; KArgs::W).
-// Pivoted factor (piv set): the columns of A_{C,K} are read in pivot order
-// and D^{-1} is left to k_copyback_bk (2x2 blocks can straddle tiles).
+// Panel solve of the pivoted factorisation: W_{C,K} = A_{C,K P} (L_KK)^{-T}
+// (the columns of A_{C,K} in pivot order), the Schur update's L_{C,K} D_K; its
+// product with D^{-1} is k_copyback_bk's (2x2 blocks can straddle tiles).
 template <class T, int BN>
 __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
-                                                     const T* __restrict__ L, const T* __restrict__ D,
-                                                     const T* __restrict__ Linv, T* __restrict__ Ltmp, Sizes sz,
+                                                     const T* __restrict__ L, const T* __restrict__ Linv, Sizes sz,
                                                      const int32_t* __restrict__ piv, T* __restrict__ W) {
   __shared__ TileSmem<T, BN> sm;
   const Task tk = tasks[blockIdx.x];
@@ -744,13 +756,12 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
   const int s = m.s, r = m.r, ld = s + r;
   const T* A = L + b * sz.panel + m.panel + s;
   const T* Vi = Linv + b * sz.linv + m.linv;
-  const T* d = D + b * sz.n + m.f;
   Acc<T, BN> acc;
   acc_zero<T, BN>(acc);
-  const int32_t* pv = piv ? piv + b * sz.n + m.f : nullptr;
+  const int32_t* pv = piv + b * sz.n + m.f;
   auto la = [&](int mm, int kk) {
     const int row = tk.m0 + mm;
-    return row < r ? A[row + (int64_t)(pv ? pv[kk] : kk) * ld] : Sc<T>::zero();
+    return row < r ? A[row + (int64_t)pv[kk] * ld] : Sc<T>::zero();
   };
   auto lb = [&](int kk, int nn) {
     const int col = tk.n0 + nn;
@@ -759,97 +770,10 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
   // (L_KK)^{-T} is upper triangular: output columns < n0 + BN need only k < n0 + BN
   tile_mma<T, BN>(sm, 0, min(s, tk.n0 + BN), [](int) { return false; }, la, lb, acc,
                   LiveRect{r - tk.m0, s - tk.n0}, KUpperB<BN>{tk.n0});
-  T* out = Ltmp + b * sz.lhat + m.lhat;
   T* wout = W + b * sz.panel + m.panel + s;
   tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
     const int row = tk.m0 + mm, col = tk.n0 + nn;
-    if (row < r && col < s) {
-      out[row + (int64_t)col * r] = pv ? v : v / d[col];
-      wout[row + (int64_t)col * ld] = v;
-    }
-  });
-}
-
-// Blocked factorisation, rows below the diagonal block of columns [32 p, 32 p
-// + 32) (tile rows m0 .. m0+63 of the panel, columns n0 .. n0+7): W = A V_pp^T
-// = L D, kept in the X panels (same layout) as the first operand of the panel
-// update and the Schur update, and L = W D^{-1}: rows of C to Ltmp (the Schur
-// update's second operand), rows of K's own block to the unused lower part of
-// linv (the panel update's second operand).  Both copies leave the panel itself
-// unwritten: tiles of the same rows and other columns still read it.
-template <class T, int BN>
-__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_fpanel(
-    const SnMeta* __restrict__ meta, const Task* __restrict__ tasks, const T* __restrict__ L, const T* __restrict__ D,
-    T* __restrict__ Linv, T* __restrict__ Ltmp, T* __restrict__ W, Sizes sz) {
-  __shared__ TileSmem<T, BN> sm;
-  const Task tk = tasks[blockIdx.x];
-  const int b = blockIdx.y;
-  const SnMeta m = meta[tk.sn];
-  const int s = m.s, r = m.r, ld = s + r;
-  const T* A = L + b * sz.panel + m.panel;
-  T* Vi = Linv + b * sz.linv + m.linv;
-  const T* d = D + b * sz.n + m.f;
-  Acc<T, BN> acc;
-  acc_zero<T, BN>(acc);
-  const int k0 = tk.n0 / kFB * kFB, nend = min(s, k0 + kFB);
-  auto la = [&](int mm, int kk) {
-    const int row = tk.m0 + mm;
-    return row < ld ? A[row + (int64_t)kk * ld] : Sc<T>::zero();
-  };
-  auto lb = [&](int kk, int nn) {
-    const int col = tk.n0 + nn;
-    return col < nend ? Vi[col + (int64_t)kk * s] : Sc<T>::zero();
-  };
-  // V_pp^T is upper triangular: columns < n0 + BN need only k < n0 + BN
-  tile_mma<T, BN>(sm, k0, min(nend, tk.n0 + BN), [](int) { return false; }, la, lb, acc,
-                  LiveRect{ld - tk.m0, nend - tk.n0}, KUpperB<BN>{tk.n0});
-  T* out = Ltmp + b * sz.lhat + m.lhat;
-  T* wout = W + b * sz.panel + m.panel;
-  tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
-    const int row = tk.m0 + mm, col = tk.n0 + nn;
-    if (row < ld && col < nend) {
-      wout[row + (int64_t)col * ld] = v;
-      const T l = v / d[col];
-      if (row >= s)
-        out[row - s + (int64_t)col * r] = l;
-      else
-        Vi[row + (int64_t)col * s] = l;  // rows below block p: disjoint from V_pp
-    }
-  });
-}
-
-// Blocked factorisation, the columns right of block p (task c) of the panel:
-// A_ij -= sum_k W_ik L_jk over the block's 32 columns k, rows i >= j of the
-// whole panel, each entry by one thread.
-template <class T, int BN>
-__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_fupdate(
-    const SnMeta* __restrict__ meta, const Task* __restrict__ tasks, T* __restrict__ L, const T* __restrict__ Linv,
-    const T* __restrict__ W, Sizes sz) {
-  __shared__ TileSmem<T, BN> sm;
-  const Task tk = tasks[blockIdx.x];
-  const int b = blockIdx.y;
-  const SnMeta m = meta[tk.sn];
-  const int s = m.s, ld = s + m.r;
-  const T* Wp = W + b * sz.panel + m.panel;
-  const T* Lk = Linv + b * sz.linv + m.linv;
-  Acc<T, BN> acc;
-  acc_zero<T, BN>(acc);
-  auto la = [&](int mm, int kk) {
-    const int row = tk.m0 + mm;
-    return row < ld ? Wp[row + (int64_t)kk * ld] : Sc<T>::zero();
-  };
-  auto lb = [&](int kk, int nn) {
-    const int col = tk.n0 + nn;
-    return col < s ? Lk[col + (int64_t)kk * s] : Sc<T>::zero();
-  };
-  const int dm = tk.m0 - tk.n0;
-  tile_mma<T, BN>(sm, tk.c * kFB, tk.c * kFB + kFB, [](int) { return false; }, la, lb, acc, [&](int r0, int c0) {
-    return tk.m0 + r0 < ld && tk.n0 + c0 < s && c0 <= dm + r0 + 7;
-  });
-  T* P = L + b * sz.panel + m.panel;
-  tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
-    const int row = tk.m0 + mm, col = tk.n0 + nn;
-    if (row < ld && col < s && row >= col) P[row + (int64_t)col * ld] -= v;
+    if (row < r && col < s) wout[row + (int64_t)col * ld] = v;
   });
 }
 
@@ -861,48 +785,46 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_fupdat
 // (analysis), and inside one supernode the targets of different (i, k) are
 // different entries, so each target is read-modified-written by exactly one
 // thread of the launch: no atomics, and a fixed order of the updates.
-// Non-symmetric factor: Ltmp2 is the second operand (U'_{K,C}^T), giving
-// L_{C,K} D_K U'_{K,C} into the L panels and, called again with the operands
-// swapped and `strict`, (U'_{K,C}^T D_K L_{C,K}^T) below the diagonal into the
-// U panels.  The first operand is W_{C,K} = L_{C,K} D_K (or
-// U'_{K,C}^T D_K; pivoted: with D's 2 x 2 blocks) as the panel solve left it, so the loads carry no
-// FP64 product (a product per A element is 64 x 16 FP64 operations per
-// k-tile, 1/8 of the MMA work of a 64 x 8 tile on the same pipe).
+// The first operand is W_{C,K} = L_{C,K} D_K (pivoted: with D's 2 x 2 blocks) as
+// the panel solve left it, so the loads carry no FP64 product (a product per A
+// element is 64 x 16 FP64 operations per k-tile, 1/8 of the MMA work of a
+// 64 x 8 tile on the same pipe); the second is L_{C,K} in its panel.
+// Non-symmetric factor: side blockIdx.z = 0 takes U'_{K,C}^T as the second
+// operand, giving L_{C,K} D_K U'_{K,C} into the L panels; side 1 swaps the
+// operands' sides, giving U'_{K,C}^T D_K L_{C,K}^T below the diagonal into the
+// U panels.  Both sides run in one launch (different targets).
 template <class T, int BN>
-__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(const SnMeta* __restrict__ meta, const Task* __restrict__ tasks,
-                                                      const ColDesc* __restrict__ desc,
-                                                      const int32_t* __restrict__ relidx, T* __restrict__ L,
-                                                      const T* __restrict__ Ltmp2, int strict, Sizes sz,
-                                                      const T* __restrict__ W) {
+__global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(FArgs f, const Task* __restrict__ tasks) {
   __shared__ TileSmem<T, BN> sm;
   const Task tk = tasks[blockIdx.x];
-  const int b = blockIdx.y;
-  const SnMeta m = meta[tk.sn];
+  const int b = blockIdx.y, side = blockIdx.z;
+  const SnMeta m = f.meta[tk.sn];
   const int s = m.s, r = m.r, ld = s + r;
-  const T* Lc2 = Ltmp2 + b * sz.lhat + m.lhat;
+  const int64_t po = b * f.sz.panel + m.panel + s;
+  const T* Lc2 = (const T*)f.L[f.sides - 1 - side] + po;
+  const T* Wc = (const T*)f.W[side] + po;
   Acc<T, BN> acc;
   acc_zero<T, BN>(acc);
-  const T* Wc = W + b * sz.panel + m.panel + s;
   auto la = [&](int mm, int kk) {
     const int row = tk.m0 + mm;
     return row < r ? Wc[row + (int64_t)kk * ld] : Sc<T>::zero();
   };
   auto lb = [&](int kk, int nn) {
     const int col = tk.n0 + nn;
-    return col < tk.c ? Lc2[col + (int64_t)kk * r] : Sc<T>::zero();
+    return col < tk.c ? Lc2[col + (int64_t)kk * ld] : Sc<T>::zero();
   };
   // live: fragments with a row and a column inside C and an entry on or below the diagonal
   const int dm = tk.m0 - tk.n0;
   tile_mma<T, BN>(sm, 0, s, [](int) { return false; }, la, lb, acc, [&](int r0, int c0) {
     return tk.m0 + r0 < r && tk.n0 + c0 < tk.c && c0 <= dm + r0 + 7;
   });
-  T* Lb = L + b * sz.panel;
-  const ColDesc* dk = desc + m.desc;
+  T* Lb = (T*)f.L[side] + b * f.sz.panel;
+  const ColDesc* dk = f.desc + m.desc;
   tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
     const int i = tk.m0 + mm, kc = tk.n0 + nn;
-    if (i < r && kc < tk.c && kc + strict <= i) {
+    if (i < r && kc < tk.c && kc + side <= i) {
       const ColDesc cd = dk[kc];
-      T* dst = &Lb[cd.col + relidx[cd.rel + i]];
+      T* dst = &Lb[cd.col + f.relidx[cd.rel + i]];
       *dst = *dst - v;
     }
   });
@@ -1175,20 +1097,10 @@ static size_t diag_smem_bk(int maxw) {
   return diag_smem<T>(maxw) + 16 + sizeof(T) * 256 * (nb > 1 ? nb - 1 : 1);
 }
 
-// two packed triangles of the non-symmetric diagonal factorisation
-template <class T>
-static size_t diag_smem_lu(int maxw) {
-  const size_t nb = (size_t)(maxw + 15) / 16;
-  return sizeof(T) * ((size_t)maxw * (maxw + 1) + (Sc<T>::P == 1 ? 256 * (nb > 1 ? nb - 1 : 1) : 0));
-}
-
 template <class T>
 static cudaError_t setup_t() {
-  cudaError_t e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)diag_smem_bk<T>(kMaxWidth));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_factor_diag_lu<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)diag_smem_lu<T>(Sc<T>::P == 1 ? kMaxWidth : kMaxWidthLUComplex));
   return e;
 }
 
@@ -1260,16 +1172,6 @@ static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cu
   const dim3 grid((unsigned)n, a.sz.batch);
   if constexpr (BN == 8) {  // lists of 64 x 8 tiles only
     switch (k) {
-      case Kern::FPanel:
-        k_fpanel<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.D, (T*)a.Linv,
-                                                     (T*)a.Lhat, (T*)a.W, a.sz);
-        return cudaGetLastError();
-      case Kern::FUpdate:
-        k_fupdate<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (T*)a.L, (const T*)a.Linv, (const T*)a.W, a.sz);
-        return cudaGetLastError();
-      case Kern::VInv:
-        k_vinv<T><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (T*)a.Linv, a.sz);
-        return cudaGetLastError();
       case Kern::NormM:
         if (a.Uinv)
           k_norm_m<T, 2><<<grid, TG_THREADS, 0, st>>>(a, t);
@@ -1283,13 +1185,7 @@ static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cu
   }
   switch (k) {
     case Kern::Trsm:
-      k_trsm<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.D, (const T*)a.Linv,
-                                                 (T*)a.Lhat, a.sz, a.piv, (T*)a.W);
-      break;
-    case Kern::Schur:
-      k_schur<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, a.desc, a.relidx, (T*)a.L,
-                                                  (const T*)(a.Uhat ? a.Uhat : a.Lhat), a.strict, a.sz,
-                                                  (const T*)a.W);
+      k_trsm<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, a.sz, a.piv, (T*)a.W);
       break;
     case Kern::Lhat:
       k_lhat<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, (T*)a.Lhat, a.sz);
@@ -1326,31 +1222,58 @@ cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* t, int64_t
   return a.dtype == PSELINV_C128 ? tiles_t<Cplx>(k, var, a, t, n, st) : tiles_t<double>(k, var, a, t, n, st);
 }
 
+// ---- blocked factorisation ----
+
+template <class T>
+static cudaError_t fdiag_t(const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st) {
+  const dim3 grid(nsn, f.sz.batch);
+  if (f.sides == 2)
+    k_fdiag<T, 2><<<grid, 32 + 2 * kFdUpdate, 0, st>>>(f, sns, p);
+  else
+    k_fdiag<T, 1><<<grid, 32 + kFdUpdate, 0, st>>>(f, sns, p);
+  return cudaGetLastError();
+}
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st) {
+  if (nsn <= 0) return cudaSuccess;
+  return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, st) : fdiag_t<double>(f, sns, nsn, p, st);
+}
+
+template <class T>
+static cudaError_t ftiles_t(FKern k, int var, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
+  const dim3 grid((unsigned)n, f.sz.batch, f.sides);
+  switch (k) {
+    case FKern::Panel: k_fpanel<T><<<grid, 32 * kFPanelWarps, 0, st>>>(f, t); break;
+    case FKern::Update: k_fupdate<T><<<grid, TG_THREADS, 0, st>>>(f, t); break;
+    case FKern::VInv: k_vinv<T><<<grid, TG_THREADS, 0, st>>>(f, t); break;
+    default:  // Schur groups: 64 x 8 tiles, or the widest of the type
+      if (var == 0)
+        k_schur<T, 8><<<grid, TG_THREADS, 0, st>>>(f, t);
+      else if constexpr (Sc<T>::P == 2)
+        k_schur<T, 32><<<grid, TG_THREADS, 0, st>>>(f, t);
+      else
+        return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  return dtype == PSELINV_C128 ? ftiles_t<Cplx>(k, var, f, t, n, st) : ftiles_t<double>(k, var, f, t, n, st);
+}
+
 template <class T>
 static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads) {
   if (nsn <= 0) return cudaSuccess;
   const dim3 grid(nsn, a.sz.batch);
   switch (k) {
-    case Kern::FactorDiag:
-      k_fdiag<T><<<grid, kFdThreads, 0, st>>>(a.meta, sns, a.fblock, (T*)a.L, (T*)a.D, (T*)a.Linv, a.sz, a.status);
-      break;
-    case Kern::CopyBack:
-      k_copyback<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.Lhat,
-                                                                (const T*)(a.blocked ? a.Linv : nullptr), a.sz);
-      break;
     case Kern::Gemm1Reduce:
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);
-      break;
-    case Kern::FactorDiagLU:
-      k_factor_diag_lu<T><<<grid, threads, diag_smem_lu<T>(a.maxw), st>>>(a.meta, sns, (T*)a.L, (T*)a.U, (T*)a.D,
-                                                                      (T*)a.Linv, (T*)a.Uinv, a.sz, a.status);
       break;
     case Kern::FactorDiagBK:
       k_factor_diag_bk<T><<<grid, threads > 512 ? 512 : threads, diag_smem_bk<T>(a.maxw), st>>>(
           a.meta, sns, (T*)a.L, (T*)a.D, (T*)a.E, (int8_t*)a.ptype, (int32_t*)a.piv, (T*)a.Linv, a.sz, a.status);
       break;
     case Kern::CopyBackBK:
-      k_copyback_bk<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (T*)a.Lhat, (const T*)a.D,
+      k_copyback_bk<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.W, (const T*)a.D,
                                                                   (const T*)a.E, a.ptype, a.sz);
       break;
     default:

@@ -19,8 +19,7 @@ struct Sizes {
 };
 
 enum class Kern {
-  Trsm, FPanel, FUpdate, VInv, Schur, NormM, Lhat, Gemm1, Gemm2, FactorDiag, CopyBack, DiagFinal, Gemm1Reduce,
-  FactorDiagLU,              // non-symmetric diagonal blocks
+  Trsm, NormM, Lhat, Gemm1, Gemm2, DiagFinal, Gemm1Reduce,
   FactorDiagBK, CopyBackBK   // Bunch-Kaufman pivoted factor
 };
 
@@ -28,8 +27,6 @@ enum class Kern {
 struct KArgs {
   int dtype;  // PSELINV_F64 / PSELINV_C128
   int maxw;   // widest supernode (shared-memory size of the diagonal kernels)
-  int fblock;   // FactorDiag: the block of kFactorBlock columns
-  int blocked;  // CopyBack: L_KK below its diagonal blocks is in linv (blocked factorisation)
   const SnMeta* meta;
   const ColDesc* desc;
   const int32_t* relidx;
@@ -50,10 +47,8 @@ struct KArgs {
   // non-symmetric handles (nullptr / 0 for symmetric ones)
   void* U;     // U panels: U'_{j,i} at panel position (i, j)
   void* Uinv;  // (U'_KK^T)^{-1}, linv layout
-  void* Uhat;  // Uhat_{K,C}^T, lhat layout; Schur: second operand (nullptr = Lhat)
   void* XU;    // XU panels: X_{j,i} at panel position (i, j); step 2 reads X_{C,C} above the
                // diagonal from here, step 3 finish writes X_KK^T here
-  int strict;  // Schur: skip the diagonal entries of the updated blocks
   // Bunch-Kaufman pivoted factor (nullptr when not pivoted), batch x n each:
   const int32_t* piv;  // supernode-local original column at each pivot position
   const int8_t* ptype; // 0 = 1x1 pivot, 1 / 2 = first / second column of a 2x2 pivot
@@ -64,13 +59,30 @@ struct KArgs {
   const void* gw;
   void* gam;
   int* gctr;
-  // factor: W_{C,K} = L_{C,K} D_K (U side: U'_{K,C}^T D_K; pivoted: D_K's
-  // 1 x 1 and 2 x 2 blocks, columns in pivot order), the panel solve's
-  // product before the D^{-1} scaling, kept for the Schur update, in the panel
-  // layout of this array (the X or XU panels, free during the factorisation);
-  // nullptr elsewhere
+  // pivoted factor: W_{C,K} = L_{C,K} D_K (see FArgs); nullptr elsewhere
   void* W;
 };
+
+// The factorisation's kernels.  Symmetric factors have one side; non-symmetric
+// ones two: side 0 the lower triangle (L panels, (L_KK)^{-1}), side 1 the
+// transposed upper one (U panels, (U'_KK^T)^{-1}).
+struct FArgs {
+  const SnMeta* meta;
+  const ColDesc* desc;
+  const int32_t* relidx;
+  void* L[2];     // L, U panels
+  void* Linv[2];  // inverses of the diagonal blocks' unit triangles
+  // W_{C,K} = L_{C,K} D_K (side 1: U'_{K,C}^T D_K; pivoted: D_K's 1 x 1 and
+  // 2 x 2 blocks, columns in pivot order), the panel solve's product before the
+  // D^{-1} scaling, kept for the panel and Schur updates, in the panel layout
+  // of this array (the X and XU panels, free during the factorisation)
+  void* W[2];
+  void* D;
+  int* status;
+  Sizes sz;
+  int sides;
+};
+enum class FKern { Panel, Update, VInv, Schur };
 
 // CTAs of the per-level step-3 finish per supernode (blockIdx.z of k_diag_final).
 constexpr int kFinishCtas = 32;
@@ -95,14 +107,17 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
 // diagmask == nullptr: plain gather; else off-diagonal entries doubled.
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
                                  void* out, const Sizes& sz, cudaStream_t st);
-// Tile kernels (Trsm, FPanel, FUpdate, VInv, Schur, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
+// Tile kernels (Trsm, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
 cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st);
-// Per-supernode kernels (FactorDiag, CopyBack, DiagFinal, Gemm1Reduce) over the
-// nsn supernodes listed in sns.
-// threads: block size of the diagonal-factorisation kernels FactorDiagLU and
-// FactorDiagBK (the last capped at 512).
+// Per-supernode kernels (DiagFinal, Gemm1Reduce, FactorDiagBK, CopyBackBK) over
+// the nsn supernodes listed in sns.  threads: block size of FactorDiagBK (at
+// most 512).
 cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads = 256);
+// Blocked factorisation: the diagonal block p of the listed supernodes (all wider
+// than p blocks), and its tile lists (var: tile variant of the Schur groups).
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st);
+cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st);
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype = nullptr, const void* E = nullptr);
 cudaError_t launch_pole_sum(int dtype, const void* X, int64_t panel_total, int batch, const void* w, void* out,

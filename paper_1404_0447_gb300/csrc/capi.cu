@@ -64,6 +64,69 @@ int alloc(pselinv_handle* h, void** dst, int64_t bytes) {
   return PSELINV_OK;
 }
 
+// Captured schedules hold the addresses of the task lists and buffers.
+void drop_graphs(pselinv_handle* h) {
+  void** graphs[] = {&h->graph_exec[0],  &h->graph_exec[1],  &h->pgraph_exec[0], &h->pgraph_exec[1],
+                     &h->fgraph_exec[0], &h->fgraph_exec[1], &h->agraph_exec};
+  for (void** g : graphs)
+    if (*g) {
+      cudaGraphExecDestroy((cudaGraphExec_t)*g);
+      *g = nullptr;
+    }
+}
+
+// Replay *exec on st; captured first, from enqueue(stream), where it is not there
+// yet.  The capture runs on the handle's own stream, thread-local: nothing of
+// the caller's is captured.
+template <class F>
+int replay(pselinv_handle* h, void** exec, cudaStream_t st, F&& enqueue) {
+  if (!*exec) {
+    if (!h->graph_stream) {
+      cudaStream_t ns;
+      PSI_CUDA(h, cudaStreamCreateWithFlags(&ns, cudaStreamNonBlocking));
+      h->graph_stream = ns;
+    }
+    cudaStream_t cs = (cudaStream_t)h->graph_stream;
+    PSI_CUDA(h, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    const int rc = enqueue(cs);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(cs, &g);
+    if (rc) {
+      if (g) cudaGraphDestroy(g);
+      return rc;
+    }
+    if (e != cudaSuccess) return cuda_err(h, e, "cudaStreamEndCapture");
+    cudaGraphExec_t ex;
+    e = cudaGraphInstantiate(&ex, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return cuda_err(h, e, "cudaGraphInstantiate");
+    *exec = ex;
+  }
+  PSI_CUDA(h, cudaGraphLaunch((cudaGraphExec_t)*exec, st));
+  return PSELINV_OK;
+}
+
+// Launch sequences that depend only on the handle (the factorisation's levels,
+// the LEVEL sweep, the adjoint's sweeps) are replayed from a graph from the
+// second call on: a launch in stream order follows its predecessor by 2-3 us,
+// a graph node by 0.2 us, and the host's ~2 us per launch is gone, against
+// ~1 ms once for capture and instantiation (so a handle used once never pays).
+// A stream that is being captured by the caller takes the launches themselves,
+// as before.
+template <class F>
+int replay_or_enqueue(pselinv_handle* h, void** exec, bool* ran, cudaStream_t st, F&& enqueue) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another thread's capture: the launches report it
+    cap = cudaStreamCaptureStatusActive;
+  }
+  if (!*ran || cap != cudaStreamCaptureStatusNone) {
+    *ran = true;
+    return enqueue(st);
+  }
+  return replay(h, exec, st, enqueue);
+}
+
 void free_device(pselinv_handle* h) {
   void** ptrs[] = {&h->d_meta, &h->d_desc, &h->d_relidx, &h->d_valmap, &h->d_diagmask, &h->d_tasks, &h->d_levelsn,
                    &h->d_L,    &h->d_X,    &h->d_D,      &h->d_lhat,   &h->d_linv,  &h->d_part, &h->d_ypart,
@@ -80,10 +143,9 @@ void free_device(pselinv_handle* h) {
   h->ev_pool.clear();
   h->ev_used = 0;
   h->ev_spans.clear();
-  if (h->graph_exec) cudaGraphExecDestroy((cudaGraphExec_t)h->graph_exec);
-  if (h->pgraph_exec) cudaGraphExecDestroy((cudaGraphExec_t)h->pgraph_exec);
+  drop_graphs(h);
   if (h->graph_stream) cudaStreamDestroy((cudaStream_t)h->graph_stream);
-  h->graph_exec = h->pgraph_exec = h->graph_stream = nullptr;
+  h->graph_stream = nullptr;
   for (void* e : h->xfer_ev) cudaEventDestroy((cudaEvent_t)e);
   h->xfer_ev.clear();
   if (h->xfer_stream) cudaStreamDestroy((cudaStream_t)h->xfer_stream);
@@ -168,12 +230,7 @@ int upload_schedule(pselinv_handle* h) {
       cudaFree(*p);
       *p = nullptr;
     }
-  void** graphs[] = {&h->graph_exec, &h->pgraph_exec};
-  for (void** g : graphs)
-    if (*g) {
-      cudaGraphExecDestroy((cudaGraphExec_t)*g);
-      *g = nullptr;
-    }
+  drop_graphs(h);
   if ((rc = upload(h, &h->d_meta, h->meta))) return rc;
   std::vector<psi::Task> all;
   h->off_norm = (int64_t)all.size();
@@ -664,31 +721,8 @@ int ensure_factor_streams(pselinv_handle* h) {
   return PSELINV_OK;
 }
 
-// Supernodal factorisation, level by level from the leaves.  Symmetric:
-// A = L D L^T.  Non-symmetric (d_upper set): A = L D U', both sides in every
-// launch (blockIdx.z).
-int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cudaStream_t st, bool bk = false) {
-  const psi::Sizes sz = sizes(h);
-  const int64_t B = h->opts.batch;
-  const bool unsym = d_upper != nullptr;
-  h->factored = h->inverted = false;
-  if (bk && !h->d_piv) {
-    int rc;
-    if ((rc = alloc(h, &h->d_piv, B * h->n * (int64_t)sizeof(int32_t)))) return rc;
-    if ((rc = alloc(h, &h->d_ptype, B * h->n))) return rc;
-    if ((rc = alloc(h, &h->d_E, B * h->n * (int64_t)elem_size(h)))) return rc;
-  }
-  h->pivoted = bk;
-  PSI_CUDA(h, cudaMemsetAsync(h->d_L, 0, elem_size(h) * B * h->panel_total, st));
-  if (unsym) PSI_CUDA(h, cudaMemsetAsync(h->d_U, 0, elem_size(h) * B * h->panel_total, st));
-  PSI_CUDA(h, cudaMemsetAsync(h->d_status, 0x7f, 2 * sizeof(int), st));  // pivot key: unset
-  PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, sizeof(int) * (kStatusWords - 2), st));
-  if (unsym)
-    PSI_CUDA(h, psi::launch_scatter_values_lu(h->opts.dtype, d_lower, d_upper, (const int64_t*)h->d_valmap,
-                                              (const uint8_t*)h->d_flipmap, h->nnz_a, h->d_L, h->d_U, sz, st));
-  else
-    PSI_CUDA(h, psi::launch_scatter_values(h->opts.dtype, d_lower, (const int64_t*)h->d_valmap, h->nnz_a, h->d_L,
-                                           sz, st));
+// The factorisation's level loop on stream st (after the values are in the panels).
+int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
   const int dt = h->opts.dtype;
   psi::FArgs f;
   f.meta = (const psi::SnMeta*)h->d_meta;
@@ -702,8 +736,8 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   f.W[1] = h->d_XU;
   f.D = h->d_D;
   f.status = (int*)h->d_status;
-  f.sz = sz;
-  f.sides = unsym ? 2 : 1;
+  f.sz = sizes(h);
+  f.sides = h->opts.unsym ? 2 : 1;
   psi::KArgs a = kargs(h);  // pivoted panel solves
   a.W = h->d_X;
   // Two streams (look-ahead): `hi` (high priority) runs each level's
@@ -717,8 +751,6 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   // is short (far_after_near), far(l) waits for near(l) instead, so that the
   // diagonal blocks of l - 1 get their SMs before far(l)'s tiles fill them;
   // every target sees its updates in the same order either way.
-  int rc;
-  if ((rc = ensure_factor_streams(h))) return rc;
   cudaStream_t hi = (cudaStream_t)h->fs_hi, lo = (cudaStream_t)h->fs_lo;
   // [0] start, [1 + l] solves of l, [1 + nl + l] far of l, [3 + 2 nl + l] near of l
   cudaEvent_t* ev = (cudaEvent_t*)h->fev.data();
@@ -788,6 +820,39 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   if (!bk)
     PSI_CUDA(h, psi::launch_ftiles(psi::FKern::VInv, 0, dt, f, tasks_at(h, h->off_vinv, 0),
                                    (int64_t)h->t_vinv.tasks.size(), st));
+  return PSELINV_OK;
+}
+
+// Supernodal factorisation, level by level from the leaves.  Symmetric:
+// A = L D L^T.  Non-symmetric (d_upper set): A = L D U', both sides in every
+// launch (blockIdx.z).
+int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cudaStream_t st, bool bk = false) {
+  const psi::Sizes sz = sizes(h);
+  const int64_t B = h->opts.batch;
+  const bool unsym = d_upper != nullptr;
+  h->factored = h->inverted = false;
+  if (bk && !h->d_piv) {
+    int rc;
+    if ((rc = alloc(h, &h->d_piv, B * h->n * (int64_t)sizeof(int32_t)))) return rc;
+    if ((rc = alloc(h, &h->d_ptype, B * h->n))) return rc;
+    if ((rc = alloc(h, &h->d_E, B * h->n * (int64_t)elem_size(h)))) return rc;
+  }
+  h->pivoted = bk;
+  PSI_CUDA(h, cudaMemsetAsync(h->d_L, 0, elem_size(h) * B * h->panel_total, st));
+  if (unsym) PSI_CUDA(h, cudaMemsetAsync(h->d_U, 0, elem_size(h) * B * h->panel_total, st));
+  PSI_CUDA(h, cudaMemsetAsync(h->d_status, 0x7f, 2 * sizeof(int), st));  // pivot key: unset
+  PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, sizeof(int) * (kStatusWords - 2), st));
+  if (unsym)
+    PSI_CUDA(h, psi::launch_scatter_values_lu(h->opts.dtype, d_lower, d_upper, (const int64_t*)h->d_valmap,
+                                              (const uint8_t*)h->d_flipmap, h->nnz_a, h->d_L, h->d_U, sz, st));
+  else
+    PSI_CUDA(h, psi::launch_scatter_values(h->opts.dtype, d_lower, (const int64_t*)h->d_valmap, h->nnz_a, h->d_L,
+                                           sz, st));
+  int rc;
+  if ((rc = ensure_factor_streams(h))) return rc;
+  rc = replay_or_enqueue(h, &h->fgraph_exec[bk], &h->factor_ran[bk], st,
+                         [&](cudaStream_t cs) { return enqueue_factor(h, cs, bk); });
+  if (rc) return rc;
   // no host synchronisation: the first bad pivot stays in status words 0-1
   // until the next factorisation and is reported by pselinv_sync_status (and
   // by pselinv_logdet, which synchronises anyway)
@@ -864,68 +929,35 @@ int pselinv_selinv(pselinv_handle* h, int32_t mode, void* stream) {
   if (mode == PSELINV_PERSISTENT) {
     int rrc = ensure_ring(h);
     if (rrc) return rrc;
-    if (!h->pgraph_exec) {
-      if (!h->graph_stream) {
-        cudaStream_t cs;
-        PSI_CUDA(h, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        h->graph_stream = cs;
-      }
-      cudaStream_t cs = (cudaStream_t)h->graph_stream;
-      PSI_CUDA(h, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-      int rc = enqueue_persistent(h, cs);
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamEndCapture(cs, &g);
-      if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
-      }
-      if (e != cudaSuccess) return cuda_err(h, e, "cudaStreamEndCapture");
-      cudaGraphExec_t ex;
-      e = cudaGraphInstantiate(&ex, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_err(h, e, "cudaGraphInstantiate");
-      h->pgraph_exec = ex;
-    }
     if (h->debug_flags & 2) {  // arm one never-satisfied wait (status word 3)
       PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 3, 1, 1, st));
       h->debug_flags &= ~2;
     }
-    PSI_CUDA(h, cudaGraphLaunch((cudaGraphExec_t)h->pgraph_exec, st));
+    rrc = replay(h, &h->pgraph_exec[h->pivoted], st, [&](cudaStream_t cs) { return enqueue_persistent(h, cs); });
+    if (rrc) return rrc;
     h->launches[1] += h->nlevels;
-  } else if (mode != PSELINV_GRAPH) {
+  } else if (mode == PSELINV_PLAIN || (mode == PSELINV_LEVEL && h->timing)) {
     int rc = enqueue_selinv(h, mode, st, h->timing);
     if (rc) return rc;
   } else {
-    if (!h->graph_exec) {
-      if (!h->graph_stream) {
-        cudaStream_t ns;
-        PSI_CUDA(h, cudaStreamCreateWithFlags(&ns, cudaStreamNonBlocking));
-        h->graph_stream = ns;
-      }
-      cudaStream_t cs = (cudaStream_t)h->graph_stream;
-      PSI_CUDA(h, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-      int64_t before[4];
-      std::memcpy(before, h->launches, sizeof(before));
-      int rc = enqueue_selinv(h, PSELINV_LEVEL, cs, false);
-      for (int q = 0; q < 4; ++q) {
+    // launches per class: those of the sequence, whether enqueued, captured or replayed
+    int64_t before[4];
+    std::memcpy(before, h->launches, sizeof(before));
+    bool enqueued = false;
+    const auto sweep = [&](cudaStream_t cs) {
+      enqueued = true;
+      return enqueue_selinv(h, PSELINV_LEVEL, cs, false);
+    };
+    const int rc = mode == PSELINV_GRAPH
+                       ? replay(h, &h->graph_exec[h->pivoted], st, sweep)
+                       : replay_or_enqueue(h, &h->graph_exec[h->pivoted], &h->level_ran[h->pivoted], st, sweep);
+    if (rc) return rc;
+    for (int q = 0; q < 4; ++q) {
+      if (enqueued)
         h->graph_launches[q] = h->launches[q] - before[q];
-        h->launches[q] = before[q];
-      }
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamEndCapture(cs, &g);
-      if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
-      }
-      if (e != cudaSuccess) return cuda_err(h, e, "cudaStreamEndCapture");
-      cudaGraphExec_t ex;
-      e = cudaGraphInstantiate(&ex, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_err(h, e, "cudaGraphInstantiate");
-      h->graph_exec = ex;
+      else
+        h->launches[q] += h->graph_launches[q];
     }
-    PSI_CUDA(h, cudaGraphLaunch((cudaGraphExec_t)h->graph_exec, st));
-    for (int q = 0; q < 4; ++q) h->launches[q] += h->graph_launches[q];
   }
   h->inverted = true;
   return PSELINV_OK;
@@ -1141,47 +1173,14 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream) {
   return pivot_error(h, key);
 }
 
-int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, void* d_gradA, void* stream) {
+}  // extern "C"
+
+namespace {
+// The adjoint's two sweeps on stream st (after the seed).
+int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
   using psi::AdjKern;
   using psi::AdjSn;
-  if (!h) return set_err(nullptr, PSELINV_ERR_ARG, "handle is NULL");
-  if (!d_G || !d_gradA) return set_err(h, PSELINV_ERR_ARG, "NULL argument");
-  if (g_kind != PSELINV_G_SYMMETRIC && g_kind != PSELINV_G_PANEL) return set_err(h, PSELINV_ERR_ARG, "bad g_kind");
-  if (h->opts.unsym) return set_err(h, PSELINV_ERR_STATE, "symmetric handles only");
-  if (h->pivoted) return set_err(h, PSELINV_ERR_STATE, "the adjoint needs the pivot-free factor (pselinv_factor)");
-  if (!h->inverted) return set_err(h, PSELINV_ERR_STATE, "selinv_adjoint needs a prior pselinv_selinv");
   const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
-  int rc;
-  if (!h->d_xb) {
-    if ((rc = alloc(h, &h->d_xb, B * h->panel_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_lb, B * h->panel_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_db, B * h->n * es))) return rc;
-    if ((rc = alloc(h, &h->d_zb, B * h->linv_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_w1, B * h->linv_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_yb, B * h->lhat_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_hb, B * h->lhat_total * es))) return rc;
-  }
-  cudaStream_t st = (cudaStream_t)stream;
-  psi::AdjArgs a;
-  a.k = kargs(h);
-  a.k.tctr = (int*)h->d_tctr;  // split X_CC Yb and (W + W^T) L_CK summed by their last slice CTA
-  a.G = d_G;
-  a.g_kind = g_kind;
-  a.Xb = h->d_xb;
-  a.Lb = h->d_lb;
-  a.Db = h->d_db;
-  a.Zb = h->d_zb;
-  a.W1 = h->d_w1;
-  a.Yb = h->d_yb;
-  a.Hb = h->d_hb;
-  // recompute Lhat = L_CK (L_KK)^{-1} from the factor (step 1) instead of trusting a stored copy
-  for (int v = 0; v < psi::kNumVar; ++v) {
-    const psi::Range r = h->t_lhat.whole[v];
-    PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a.k, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
-  }
-  PSI_CUDA(h, cudaMemsetAsync(h->d_lb, 0, B * h->panel_total * es, st));
-  PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));
-  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, st));
   const auto* lsn = (const int32_t*)h->d_levelsn;
   auto tiles = [&](AdjKern k, const psi::TaskList& tl, int64_t off, int32_t l) -> cudaError_t {
     for (int v = 0; v < psi::kNumVar; ++v) {
@@ -1228,6 +1227,56 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
     PSI_CUDA(h, tiles(AdjKern::Df4, h->t_sq, h->off_sq, l));
     PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df5, a, sns, nsl, st));
   }
+  return PSELINV_OK;
+}
+}  // namespace
+
+extern "C" {
+
+int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, void* d_gradA, void* stream) {
+  using psi::AdjSn;
+  if (!h) return set_err(nullptr, PSELINV_ERR_ARG, "handle is NULL");
+  if (!d_G || !d_gradA) return set_err(h, PSELINV_ERR_ARG, "NULL argument");
+  if (g_kind != PSELINV_G_SYMMETRIC && g_kind != PSELINV_G_PANEL) return set_err(h, PSELINV_ERR_ARG, "bad g_kind");
+  if (h->opts.unsym) return set_err(h, PSELINV_ERR_STATE, "symmetric handles only");
+  if (h->pivoted) return set_err(h, PSELINV_ERR_STATE, "the adjoint needs the pivot-free factor (pselinv_factor)");
+  if (!h->inverted) return set_err(h, PSELINV_ERR_STATE, "selinv_adjoint needs a prior pselinv_selinv");
+  const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
+  int rc;
+  if (!h->d_xb) {
+    if ((rc = alloc(h, &h->d_xb, B * h->panel_total * es))) return rc;
+    if ((rc = alloc(h, &h->d_lb, B * h->panel_total * es))) return rc;
+    if ((rc = alloc(h, &h->d_db, B * h->n * es))) return rc;
+    if ((rc = alloc(h, &h->d_zb, B * h->linv_total * es))) return rc;
+    if ((rc = alloc(h, &h->d_w1, B * h->linv_total * es))) return rc;
+    if ((rc = alloc(h, &h->d_yb, B * h->lhat_total * es))) return rc;
+    if ((rc = alloc(h, &h->d_hb, B * h->lhat_total * es))) return rc;
+  }
+  cudaStream_t st = (cudaStream_t)stream;
+  psi::AdjArgs a;
+  a.k = kargs(h);
+  a.k.tctr = (int*)h->d_tctr;  // split X_CC Yb and (W + W^T) L_CK summed by their last slice CTA
+  a.G = d_G;
+  a.g_kind = g_kind;
+  a.Xb = h->d_xb;
+  a.Lb = h->d_lb;
+  a.Db = h->d_db;
+  a.Zb = h->d_zb;
+  a.W1 = h->d_w1;
+  a.Yb = h->d_yb;
+  a.Hb = h->d_hb;
+  // recompute Lhat = L_CK (L_KK)^{-1} from the factor (step 1) instead of trusting a stored copy
+  for (int v = 0; v < psi::kNumVar; ++v) {
+    const psi::Range r = h->t_lhat.whole[v];
+    PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a.k, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
+  }
+  PSI_CUDA(h, cudaMemsetAsync(h->d_lb, 0, B * h->panel_total * es, st));
+  PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));
+  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, st));
+  a.G = nullptr;  // read by the seed only
+  rc = replay_or_enqueue(h, &h->agraph_exec, &h->adjoint_ran, st,
+                         [&](cudaStream_t cs) { return enqueue_adjoint(h, a, cs); });
+  if (rc) return rc;
   PSI_CUDA(h, psi::launch_gather_values(h->opts.dtype, h->d_xb, (const int64_t*)h->d_valmap, nullptr, h->nnz_a,
                                         d_gradA, sizes(h), st));
   return PSELINV_OK;

@@ -239,9 +239,14 @@ struct pselinv_handle {
   void* d_yring = nullptr;   // persistent schedule: kRing level slots of step-2 partials
   void* d_pring = nullptr;   // ... and of step-3 partials
   int pgrid = 0;
-  void* pgraph_exec = nullptr;  // cudaGraphExec_t of the PERSISTENT schedule
+  void* pgraph_exec[2] = {nullptr, nullptr};  // cudaGraphExec_t of the PERSISTENT schedule: [pivoted factor]
   int debug_flags = 0;
-  void* graph_exec = nullptr;  // cudaGraphExec_t of the LEVEL schedule
+  void* graph_exec[2] = {nullptr, nullptr};  // cudaGraphExec_t of the LEVEL schedule: [pivoted factor]
+  // cudaGraphExec_t of the factorisation's level loop (pivot-free or non-symmetric, pivoted) and
+  // of the adjoint's two sweeps; captured on the second call (replay_or_enqueue)
+  void* fgraph_exec[2] = {nullptr, nullptr};
+  void* agraph_exec = nullptr;
+  bool factor_ran[2] = {false, false}, level_ran[2] = {false, false}, adjoint_ran = false;
   void* graph_stream = nullptr;
   // pselinv_selinv_to_host: per-level copy plan of finished X panels
   std::vector<int64_t> xfer_off, xfer_len;  // element ranges of one panel array
@@ -260,7 +265,7 @@ struct pselinv_handle {
   size_t ev_used = 0;
   std::vector<std::pair<int, std::pair<size_t, size_t>>> ev_spans;  // class, (start, stop) event slots
   int64_t launches[4] = {0, 0, 0, 0};
-  int64_t graph_launches[4] = {0, 0, 0, 0};  // kernels in the captured graph, per class
+  int64_t graph_launches[4] = {0, 0, 0, 0};  // kernels of the LEVEL sequence, per class
 };
 
 namespace psi {

@@ -199,15 +199,7 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
     T c[SIDES];
 #pragma unroll
     for (int e = 0; e < SIDES; ++e) c[e] = i < w ? ((T*)f.L[e] + po)[i] : Sc<T>::zero();  // column 0
-    // column j, final: d_j out (off the chain)
-    auto finish = [&](int j, T v) {
-      if (i != j) return;
-      if (Sc<T>::bad(v)) report_pivot(f.status, m.f + c0 + i, Sc<T>::is_zero(v));
-      d[i] = v;
-      ((T*)f.L[0] + po)[i + (int64_t)i * ld] = v;
-#pragma unroll
-      for (int e = 0; e < SIDES; ++e) ((T*)f.Linv[e] + vo)[i + (int64_t)i * s] = Sc<T>::one();
-    };
+    T dl = c[0];  // lane j: d_j, once column j is final
     for (int j = 0; j + 1 < w; ++j) {
       const T rd = Sc<T>::one() / shfl(c[0], j);
       const int o = (j & 1) * kFB;
@@ -220,17 +212,23 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
         u[e] = shfl(c[e], j + 1);
       }
       __syncthreads();
-      T next[SIDES];  // rows above j + 1 and from w: never used
-#pragma unroll
-      for (int e = 0; e < SIDES; ++e) next[e] = sh[e * SD + 4 * kFB + (kFB - o) + i] - l[e] * u[SIDES - 1 - e];
-      finish(j, c[0]);
 #pragma unroll
       for (int e = 0; e < SIDES; ++e) {
+        // rows above j + 1 and from w: never used
+        c[e] = sh[e * SD + 4 * kFB + (kFB - o) + i] - l[e] * u[SIDES - 1 - e];
         if (i > j && i < w) ((T*)f.L[e] + po)[i + (int64_t)j * ld] = l[e];
-        c[e] = next[e];
       }
+      if (i == j + 1) dl = c[0];
     }
-    finish(w - 1, c[0]);
+    // off the chain: a test of d_j inside the loop would hold this warp for the
+    // FP64 compares of every column
+    if (i < w) {
+      if (Sc<T>::bad(dl)) report_pivot(f.status, m.f + c0 + i, Sc<T>::is_zero(dl));
+      d[i] = dl;
+      ((T*)f.L[0] + po)[i + (int64_t)i * ld] = dl;
+#pragma unroll
+      for (int e = 0; e < SIDES; ++e) ((T*)f.Linv[e] + vo)[i + (int64_t)i * s] = Sc<T>::one();
+    }
     return;
   }
   const int side = SIDES == 1 ? 0 : (threadIdx.x - 32) / kFdUpdate;

@@ -76,8 +76,8 @@ constexpr int kTileN = 64;       // output tile columns
 // diagonal blocks on one SM's FP64 pipe.
 constexpr int kFactorBlock = 32;
 constexpr int kFactorBlocks = (kMaxWidth + kFactorBlock - 1) / kFactorBlock;
-constexpr int kFPanelRows = 16;  // rows of a k_fpanel task (8 per warp)
-constexpr int kFUpdateRows = 32; // rows of a k_fupdate task
+constexpr int kFPanelRows = 16;  // rows of a k_fpanel task
+constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
 // Tile-width variants of the tile GEMMs: BN = 8 << var.
 constexpr int kNumVar = 4;

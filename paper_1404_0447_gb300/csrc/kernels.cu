@@ -243,7 +243,8 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
 #pragma unroll
   for (int q = 0; q < kFdEntries; ++q) {
     const int e = t + q * kFdUpdate;
-    ri[q] = ck[q] = -1;  // no entry: never live
+    ri[q] = ck[q] = 0;  // no entry: never live
+    x[q] = Sc<T>::zero();
     if (e < ne) {
       tri_entry(e, ri[q], ck[q]);
       if (ck[q] > 0) x[q] = P[ri[q] + (int64_t)ck[q] * ld];  // column 0 is the pivot warp's
@@ -253,16 +254,26 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
   for (int j = 0; j + 1 < w; ++j) {
     __syncthreads();
     const int o = (j & 1) * kFB;
+    // all operands first, then the products of the three entries back to back: with
+    // a branch per kind of entry they ran one after the other and the phase took
+    // 924 cycles instead of 655 (34.2k -> 24.5k cycles for 32 columns)
+    T a[kFdEntries], v[kFdEntries];
+#pragma unroll
+    for (int q = 0; q < kFdEntries; ++q) {
+      a[q] = sl[o + ri[q]];
+      v[q] = (ck[q] > j ? su : sv)[o + ck[q]];  // k > j: u_k; k < j: V_jk
+    }
 #pragma unroll
     for (int q = 0; q < kFdEntries; ++q) {
       const int i = ri[q], k = ck[q];
-      if (i <= j || k == j + 1) continue;  // column j + 1 is the pivot warp's
-      if (k == j)
-        x[q] = -sl[o + i];
-      else
-        x[q] -= sl[o + i] * (k > j ? su[o + k] : sv[o + k]);
-      if (k == j + 2) spre[o + i] = x[q];   // parity of column j + 2
-      if (i == j + 1) sv[kFB - o + k] = x[q];  // k <= j: V's row j + 1
+      if (i > j && k != j + 1)  // column j + 1 is the pivot warp's
+        x[q] = (k == j ? Sc<T>::zero() : x[q]) - a[q] * (k == j ? Sc<T>::one() : v[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kFdEntries; ++q) {
+      const int i = ri[q], k = ck[q];
+      if (k == j + 2 && i >= k) spre[o + i] = x[q];    // parity of column j + 2
+      if (i == j + 1 && k <= j) sv[kFB - o + k] = x[q];  // V's row j + 1
     }
   }
 #pragma unroll
@@ -300,71 +311,70 @@ __device__ __forceinline__ T frag_value(const double (&acc)[Sc<T>::P][2], int e)
 // Blocked factorisation, rows m0 .. m0+15 of the panel below the diagonal block
 // p (task c): W = A V_pp^T = L D, kept in the X panels (same layout) as the
 // first operand of the panel and Schur updates, and L = W D^{-1} in place.
-// One warp per 8 rows and all (up to 32) columns of the block, so a row's
-// entries are read and written by one warp only; operand fragments go straight
-// from global memory to registers, all loads in flight at once.  Bound: the
-// FP64 pipe (20 m8n8k4 MMAs of 145 cycles a warp); shared-memory staging and
-// 64-row tiles would leave most SMs idle on the levels near the root, where a
-// 64 x 8 tile took 8.7 us however few there were.
+// Warp j takes the block's columns 8 j .. 8 j + 7 (k < 8 j + 8: V_pp^T is upper
+// triangular); the CTA's 16 rows are its own, so after one barrier L replaces A.
+// Operand fragments go straight from global memory to registers, all loads in
+// flight at once.  Bound: the FP64 pipe (40 m8n8k4 MMAs of 145 cycles) where a
+// level has many rows; near the root, latency: 64 x 8 tiles staged in shared
+// memory took 8.7 us however few there were, a warp per 8 rows and 32 columns 9.5.
 // blockIdx.z = 1: the U side of a non-symmetric factor, U'_{K,C}^T = A_{K,C}^T
 // L_KK^{-T} D^{-1}, as L_{C,K} = A_{C,K} U'_KK^{-1} D^{-1} uses (U'_KK^T)^{-1}.
-constexpr int kFPanelWarps = kFPanelRows / 8;
 template <class T>
-__global__ void __launch_bounds__(32 * kFPanelWarps) k_fpanel(FArgs f, const Task* __restrict__ tasks) {
-  __shared__ __align__(16) double raw[kFB * Sc<T>::P];
-  T* rd = reinterpret_cast<T*>(raw);
+__global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restrict__ tasks) {
+  constexpr int RF = kFPanelRows / 8;
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
   const int s = m.s, ld = s + m.r, c0 = tk.c * kFB, w = min(kFB, s - c0);
-  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, j = threadIdx.x >> 5;
   T* A = (T*)f.L[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   T* Wp = (T*)f.W[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   const T* Vi = (const T*)f.Linv[f.sides - 1 - side] + b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
-  const int row = tk.m0 + 8 * (threadIdx.x >> 5) + g;
-  T a[kFB / 4];
+  T a[RF][kFB / 4], bf[kFB / 4], rd[2];
 #pragma unroll
   for (int u = 0; u < kFB / 4; ++u) {
-    const int k = 4 * u + q;
-    a[u] = row < ld && k < w ? A[row + (int64_t)k * ld] : Sc<T>::zero();
-  }
-  if (threadIdx.x < w) rd[threadIdx.x] = Sc<T>::one() / ((const T*)f.D + b * f.sz.n + m.f + c0)[threadIdx.x];
-  double acc[kFB / 8][Sc<T>::P][2] = {};
+    const int k = 4 * u + q, n = 8 * j + g;
+    const bool on = u < 2 * j + 2 && k < w;
+    bf[u] = on && n < w ? Vi[n + (int64_t)k * s] : Sc<T>::zero();
 #pragma unroll
-  for (int j = 0; j < kFB / 8; ++j) {
-    // V_pp^T is upper triangular: columns 8 j .. 8 j + 7 need k < 8 j + 8
-    T bf[kFB / 4];
-#pragma unroll
-    for (int u = 0; u < 2 * j + 2; ++u) {
-      const int k = 4 * u + q, n = 8 * j + g;
-      bf[u] = n < w && k < w ? Vi[n + (int64_t)k * s] : Sc<T>::zero();
+    for (int h = 0; h < RF; ++h) {
+      const int row = tk.m0 + 8 * h + g;
+      a[h][u] = on && row < ld ? A[row + (int64_t)k * ld] : Sc<T>::zero();
     }
-    if (8 * j >= w) continue;
-    if (j == 0) frag_mma<T, 2>(acc[j], a, bf);
-    if (j == 1) frag_mma<T, 4>(acc[j], a, bf);
-    if (j == 2) frag_mma<T, 6>(acc[j], a, bf);
-    if (j == 3) frag_mma<T, 8>(acc[j], a, bf);
   }
-  __syncthreads();  // rd; and every lane has read its row's entries
-  if (row >= ld) return;
 #pragma unroll
-  for (int j = 0; j < kFB / 8; ++j)
+  for (int e = 0; e < 2; ++e) {
+    const int col = 8 * j + 2 * q + e;
+    rd[e] = Sc<T>::one() / (col < w ? ((const T*)f.D + b * f.sz.n + m.f + c0)[col] : Sc<T>::one());
+  }
+  double acc[RF][Sc<T>::P][2] = {};
+#pragma unroll
+  for (int h = 0; h < RF; ++h) {
+    if (j == 0) frag_mma<T, 2>(acc[h], a[h], bf);
+    if (j == 1) frag_mma<T, 4>(acc[h], a[h], bf);
+    if (j == 2) frag_mma<T, 6>(acc[h], a[h], bf);
+    if (j == 3) frag_mma<T, 8>(acc[h], a[h], bf);
+  }
+  __syncthreads();  // every warp has read its rows' entries
+#pragma unroll
+  for (int h = 0; h < RF; ++h)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int col = 8 * j + 2 * q + e;
-      if (col >= w) continue;
-      const T v = frag_value<T>(acc[j], e);
+      const int row = tk.m0 + 8 * h + g, col = 8 * j + 2 * q + e;
+      if (row >= ld || col >= w) continue;
+      const T v = frag_value<T>(acc[h], e);
       Wp[row + (int64_t)col * ld] = v;
-      A[row + (int64_t)col * ld] = v * rd[col];
+      A[row + (int64_t)col * ld] = v * rd[e];
     }
 }
 
 // Blocked factorisation, the columns right of block p (task c) of the panel:
 // A_ij -= sum_k W_ik L_jk over the block's 32 columns k, rows i >= j of the
 // whole panel (i > j on the U side), each entry by one thread; one warp per
-// 8 x 8 fragment of a 32 x 8 tile, operands straight to registers (see k_fpanel).
+// 8 x 8 fragment of a 16 x 8 tile, operands straight to registers (see k_fpanel).
+constexpr int kFUpdateThreads = 4 * kFUpdateRows;
 template <class T>
-__global__ void __launch_bounds__(TG_THREADS) k_fupdate(FArgs f, const Task* __restrict__ tasks) {
+__global__ void __launch_bounds__(kFUpdateThreads) k_fupdate(FArgs f, const Task* __restrict__ tasks) {
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
@@ -1240,8 +1250,8 @@ template <class T>
 static cudaError_t ftiles_t(FKern k, int var, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
   const dim3 grid((unsigned)n, f.sz.batch, f.sides);
   switch (k) {
-    case FKern::Panel: k_fpanel<T><<<grid, 32 * kFPanelWarps, 0, st>>>(f, t); break;
-    case FKern::Update: k_fupdate<T><<<grid, TG_THREADS, 0, st>>>(f, t); break;
+    case FKern::Panel: k_fpanel<T><<<grid, 4 * kFB, 0, st>>>(f, t); break;
+    case FKern::Update: k_fupdate<T><<<grid, kFUpdateThreads, 0, st>>>(f, t); break;
     case FKern::VInv: k_vinv<T><<<grid, TG_THREADS, 0, st>>>(f, t); break;
     default:  // Schur groups: 64 x 8 tiles, or the widest of the type
       if (var == 0)

@@ -528,7 +528,7 @@ int pselinv_export_symbolic(const pselinv_handle* h, pselinv_symbolic* view);
  * d_d       device, count x s pivots
  * d_M       device, count x s x s output, full symmetric, column-major
  * The first call on each device looks up the scratch array's device address
- * and sets a kernel attribute for that device; make that first call before
+ * for that device; make that first call before
  * any stream capture.  All calls share the one scratch array: calls that can
  * overlap on the GPU (different streams, or different host threads) race on
  * it and must be serialised by the caller.  Every call writes all scratch

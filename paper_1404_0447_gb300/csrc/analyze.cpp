@@ -654,6 +654,7 @@ int build_schedule(pselinv_handle* h) {
         h->fb_range[at].begin = (int64_t)h->fb_sn.size();
         tp.per_lv[at].begin = (int64_t)tp.tasks.size();
         tu.per_lv[at].begin = (int64_t)tu.tasks.size();
+        tv.per_lv[at].begin = (int64_t)tv.tasks.size();
         for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
           const int32_t k = h->level_sn[t];
           const SnMeta& m = h->meta[k];
@@ -669,6 +670,7 @@ int build_schedule(pselinv_handle* h) {
         h->fb_range[at].end = (int64_t)h->fb_sn.size();
         tp.per_lv[at].end = (int64_t)tp.tasks.size();
         tu.per_lv[at].end = (int64_t)tu.tasks.size();
+        tv.per_lv[at].end = (int64_t)tv.tasks.size();
       }
   }
   build(h->t_sq, false, [&](int32_t k) { return (int)qvar[k]; }, [&](int32_t k, int bn, std::vector<Task>& out) {

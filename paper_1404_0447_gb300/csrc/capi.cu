@@ -789,6 +789,10 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       psi::KArgs ad = a;
       ad.maxw = wmax;
       PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiagBK, ad, sns, nsl, hi, wmax >= 64 ? 512 : 256));
+      const psi::Range rv = h->t_vinv.per_lv[(size_t)l * psi::kFactorBlocks];
+      PSI_CUDA(h, psi::launch_vdiag(dt, f, sns, nsl, wmax, hi));
+      PSI_CUDA(h, psi::launch_ftiles(psi::FKern::VInv, 0, dt, f, tasks_at(h, h->off_vinv, rv.begin),
+                                     rv.end - rv.begin, hi));
       for (int v = 0; v < psi::kNumVar; ++v) {
         const psi::Range r = h->t_trsm.per_lv[(size_t)l * psi::kNumVar + v];
         PSI_CUDA(h, psi::launch_tiles(psi::Kern::Trsm, v, a, tasks_at(h, h->off_trsm, r.begin), r.end - r.begin, hi));

@@ -158,7 +158,7 @@ struct pselinv_handle {
   // blocked factorisation: per (level, block) at [level * kFactorBlocks + p] the
   // supernodes of the level wider than p blocks (fb_sn), the tiles of the rows
   // below block p (t_fpanel) and of the columns right of it (t_fupdate);
-  // t_vinv: 8-column strips of the inverses of all supernodes wider than a block
+  // t_vinv: 8-column strips of the inverses of the supernodes wider than a block (at block 0)
   std::vector<int32_t> fb_sn;
   std::vector<psi::Range> fb_range;
   psi::TaskList t_fpanel, t_fupdate, t_vinv;

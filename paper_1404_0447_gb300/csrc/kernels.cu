@@ -8,6 +8,7 @@
 // r x s with ld = r; (L_KK)^{-1} is s x s with ld = s; D holds the pivots.
 #include <cuda_runtime.h>
 
+#include "block_inverse.cuh"
 #include "internal.h"
 #include "kernels.h"
 #include "selinv_steps.cuh"
@@ -93,54 +94,6 @@ __global__ void k_gather_values(const T* __restrict__ X, int64_t panel_total, co
 // diagonal blocks
 // --------------------------------------------------------------------------
 
-// V = (L_KK)^{-1} for the unit lower triangle held packed in Tp (shared
-// memory), by 16 x 16 blocks so that the whole CTA works at every step:
-// first the diagonal blocks V_ii = (L_ii)^{-1} (one column per thread),
-// then, for block distance d = 1, 2, ... (all block pairs (i, j) with
-// i - j = d at once), S = sum_{k=j}^{i-1} L_ik V_kj and V_ij = -V_ii S.
-// V (global memory, column-major, ld s, zeros above the diagonal) is read back
-// by the later steps of this CTA; S (shared) holds (ceil(s/16) - 1) blocks of
-// 16 x 16.
-template <class T>
-__device__ void unit_lower_inverse_blocked(const T* Tp, int s, T* Vg, T* S) {
-  auto V = [&](int i, int j) -> T& { return Vg[i + (int64_t)j * s]; };
-  constexpr int B = 16;
-  const int nb = (s + B - 1) / B;
-  const int nt = blockDim.x, t = threadIdx.x;
-  for (int c = t; c < s; c += nt) {
-    const int i1 = min((c / B + 1) * B, s);
-    for (int i = 0; i < c; ++i) V(i, c) = Sc<T>::zero();
-    V(c, c) = Sc<T>::one();
-    for (int i = c + 1; i < i1; ++i) {
-      T acc = Sc<T>::zero();
-      for (int q = c; q < i; ++q) acc += Tp[pk(i, q, s)] * V(q, c);
-      V(i, c) = -acc;
-    }
-  }
-  __syncthreads();
-  for (int d = 1; d < nb; ++d) {
-    const int npair = nb - d;  // pairs (j + d, j), j = 0 .. nb - d - 1
-    for (int e = t; e < npair * B * B; e += nt) {
-      const int j = e / (B * B), rr = (e / B) % B, cc = e % B;
-      const int row = (j + d) * B + rr, col = j * B + cc;
-      T acc = Sc<T>::zero();
-      if (row < s && col < s)  // V(q, col) = 0 above the diagonal: q from col
-        for (int q = col; q < (j + d) * B; ++q) acc += Tp[pk(row, q, s)] * V(q, col);
-      S[e] = acc;
-    }
-    __syncthreads();
-    for (int e = t; e < npair * B * B; e += nt) {
-      const int j = e / (B * B), rr = (e / B) % B, cc = e % B;
-      const int i0 = (j + d) * B, row = i0 + rr, col = j * B + cc;
-      if (row >= s || col >= s) continue;
-      T acc = Sc<T>::zero();
-      for (int q = 0; q <= rr; ++q) acc += V(row, i0 + q) * S[j * B * B + q * B + cc];
-      V(row, col) = -acc;
-    }
-    __syncthreads();
-  }
-}
-
 // Blocked factorisation of the panel of supernode K, 32 columns at a time: for
 // block p, k_fdiag (diagonal block), k_fpanel (the rows below it) and k_fupdate
 // (the remaining columns of the panel).  One SM's FP64 pipe takes 97 us for the
@@ -149,7 +102,6 @@ __device__ void unit_lower_inverse_blocked(const T* Tp, int s, T* Vg, T* S) {
 // (L_KK)^{-1} off the diagonal blocks waits until after the last level
 // (k_vinv), where all supernodes run at once.  Against one CTA per supernode
 // factoring and inverting the whole block in shared memory: see k_fdiag.
-constexpr int kFB = kFactorBlock;
 constexpr int kFdUpdate = 192;               // threads holding the triangle: 6 warps fill the FP64 pipe
 constexpr int kFdThreads = 32 + kFdUpdate;  // and the pivot warp
 constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdUpdate - 1) / kFdUpdate;  // lower entries per thread
@@ -157,14 +109,6 @@ constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdUpdate - 1) / kFdUpdate;  /
 // Value of lane src, to all lanes of the warp.
 __device__ __forceinline__ double shfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ Cplx shfl(Cplx v, int src) { return {shfl(v.re, src), shfl(v.im, src)}; }
-
-// Row and column of entry e of a lower triangle stored row by row.
-__device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
-  i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-  while ((i + 1) * (i + 2) / 2 <= e) ++i;
-  while (i * (i + 1) / 2 > e) --i;
-  k = e - i * (i + 1) / 2;
-}
 
 // Block p of the supernodes in sns (width above 32 p): LDL^T of the w x w
 // diagonal block (w <= 32) and the inverse V of its unit lower triangle, by
@@ -285,29 +229,6 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
   }
 }
 
-// acc (8 x 8 fragment: lane l holds row l >> 2, columns 2 (l & 3) + {0, 1}) +=
-// A B with A's fragments a (lane: row l >> 2, k = 4 u + (l & 3)) and B's
-// fragments bf (lane: k = 4 u + (l & 3), column l >> 2), U k-steps of 4.
-template <class T, int U>
-__device__ __forceinline__ void frag_mma(double (&acc)[Sc<T>::P][2], const T* a, const T* bf) {
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if constexpr (Sc<T>::P == 1) {
-      dmma884(acc[0][0], acc[0][1], a[u], bf[u]);
-    } else {
-      dmma884(acc[0][0], acc[0][1], a[u].re, bf[u].re);
-      dmma884(acc[0][0], acc[0][1], -a[u].im, bf[u].im);
-      dmma884(acc[1][0], acc[1][1], a[u].re, bf[u].im);
-      dmma884(acc[1][0], acc[1][1], a[u].im, bf[u].re);
-    }
-  }
-}
-template <class T>
-__device__ __forceinline__ T frag_value(const double (&acc)[Sc<T>::P][2], int e) {
-  if constexpr (Sc<T>::P == 1) return acc[0][e];
-  else return T{acc[0][e], acc[1][e]};
-}
-
 // Blocked factorisation, rows m0 .. m0+15 of the panel below the diagonal block
 // p (task c): W = A V_pp^T = L D, kept in the X panels (same layout) as the
 // first operand of the panel and Schur updates, and L = W D^{-1} in place.
@@ -402,92 +323,47 @@ __global__ void __launch_bounds__(kFUpdateThreads) k_fupdate(FArgs f, const Task
   }
 }
 
-// (L_KK)^{-1} off its 32 x 32 diagonal blocks, after the last level, all
-// supernodes wider than 32 at once: one CTA per 8 columns (task n0) of V.
-// With j the block of the columns, X_j = V_jj and, for i = j+1, j+2, ...:
-// X_i = -V_ii sum_{k=j}^{i-1} L_ik X_k; warp w holds rows 8w .. 8w+7 of the
-// 32-row block on m8n8k4 MMAs, its operand fragments straight from the panel
-// (eight 64-byte row runs per k-block, loaded before the products), X in
-// shared memory.  Blocks above the diagonal are written as zeros.
+// (L_KK)^{-1} off its 32 x 32 diagonal blocks, all supernodes wider than 32 of the
+// task list at once (pivot-free: after the last level): one strip of 8 columns
+// (task n0) per CTA; blockIdx.z = side.
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_vinv(FArgs f, const Task* __restrict__ tasks) {
-  constexpr int P = Sc<T>::P, LDX = 12;  // 4 (mod 16) doubles
-  __shared__ double xs[P][kMaxWidth][LDX];
-  __shared__ double ss[P][kFB][LDX];
+  __shared__ VsSmem<T> sm;
   const Task tk = tasks[blockIdx.x];
-  const int b = blockIdx.y;
   const SnMeta m = f.meta[tk.sn];
-  const int s = m.s, ld = m.s + m.r;
-  const T* A = (const T*)f.L[blockIdx.z] + b * f.sz.panel + m.panel;
-  T* V = (T*)f.Linv[blockIdx.z] + b * f.sz.linv + m.linv;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
-  const int n0 = tk.n0, j0 = n0 / kFB * kFB, j1 = min(s, j0 + kFB), n1 = min(s, n0 + 8);
-  for (int e = t; e < j0 * 8; e += TG_THREADS) {
-    const int col = n0 + e / j0;
-    if (col < n1) V[e % j0 + (int64_t)col * s] = Sc<T>::zero();
-  }
-  for (int e = t; e < kFB * 8; e += TG_THREADS) {
-    const int row = j0 + e % kFB, col = n0 + e / kFB;
-    const T v = row < j1 && col < n1 ? V[row + (int64_t)col * s] : Sc<T>::zero();
-#pragma unroll
-    for (int pl = 0; pl < P; ++pl) xs[pl][row][e / kFB] = Sc<T>::plane(v, pl);
-  }
-  __syncthreads();
-  // acc += (row `row` of M, columns k0 .. k0 + 31, zero from klim) (x from row xr0)
-  auto product = [&](const T* M, int64_t mld, int row, int k0, int klim, const double (*x)[LDX], int64_t xplane,
-                     int xr0, double (&acc)[P][2]) {
-    T fa[kFB / 4], fb[kFB / 4];
-#pragma unroll
-    for (int u = 0; u < kFB / 4; ++u) {
-      const int kk = k0 + 4 * u + q;
-      fa[u] = row < s && kk < klim ? M[row + (int64_t)kk * mld] : Sc<T>::zero();
-      const double* xb = &x[xr0 + 4 * u + q][g];
-      if constexpr (P == 1)
-        fb[u] = xb[0];
-      else
-        fb[u] = T{xb[0], xb[xplane]};
-    }
-    frag_mma<T, kFB / 4>(acc, fa, fb);
-  };
-  for (int i0 = j1; i0 < s; i0 += kFB) {
-    const int row = i0 + 8 * warp + g;
-    double acc[P][2] = {};
-    for (int k0 = j0; k0 < i0; k0 += kFB)
-      product(A, ld, row, k0, s, xs[0], kMaxWidth * LDX, k0, acc);
-#pragma unroll
-    for (int pl = 0; pl < P; ++pl)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        ss[pl][8 * warp + g][2 * q + e] = acc[pl][e];
-        acc[pl][e] = 0.0;
-      }
-    __syncthreads();
-    product(V, s, row, i0, min(s, i0 + kFB), ss[0], kFB * LDX, 0, acc);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int col = n0 + 2 * q + e;
-#pragma unroll
-      for (int pl = 0; pl < P; ++pl) xs[pl][i0 + 8 * warp + g][2 * q + e] = -acc[pl][e];
-      if (row < s && col < n1) V[row + (int64_t)col * s] = -frag_value<T>(acc, e);
-    }
-    __syncthreads();
-  }
+  inverse_strip<T>((const T*)f.L[blockIdx.z] + blockIdx.y * f.sz.panel + m.panel, m.s + m.r,
+                   (T*)f.Linv[blockIdx.z] + blockIdx.y * f.sz.linv + m.linv, m.s, tk.n0, sm);
+}
+
+// Inverses of the 32 x 32 diagonal blocks of L_KK (pivoted factorisation; the
+// pivot-free one forms them in k_fdiag): blockIdx.z = block of the supernode.
+template <class T>
+__global__ void __launch_bounds__(kVdThreads) k_vdiag(FArgs f, const int32_t* __restrict__ sns) {
+  __shared__ __align__(16) unsigned char raw[sizeof(VdSmem<T>)];
+  const SnMeta m = f.meta[sns[blockIdx.x]];
+  const int c0 = blockIdx.z * kFB, ld = m.s + m.r;
+  if (c0 >= m.s) return;
+  diag_inverse<T>((const T*)f.L[0] + blockIdx.y * f.sz.panel + m.panel + c0 + (int64_t)c0 * ld, ld,
+                  (T*)f.Linv[0] + blockIdx.y * f.sz.linv + m.linv + c0 + (int64_t)c0 * m.s, m.s, min(kFB, m.s - c0),
+                  *reinterpret_cast<VdSmem<T>*>(raw));
 }
 
 // |re| + |im|: the magnitude Bunch-Kaufman compares (plain |x| for real)
 __device__ __forceinline__ double bk_abs(double x) { return fabs(x); }
 __device__ __forceinline__ double bk_abs(Cplx x) { return fabs(x.re) + fabs(x.im); }
 
-// Largest magnitude (first index on ties) over warp lanes; returns it to all lanes.
-__device__ __forceinline__ void warp_argmax(double& v, int& idx) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const double v2 = __shfl_xor_sync(0xffffffffu, v, o);
-    const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
-    if (v2 > v || (v2 == v && i2 < idx)) {
-      v = v2;
-      idx = i2;
-    }
-  }
+// Largest magnitude >= 0 over warp lanes with its index (the first on ties), to
+// all lanes; a lane without a candidate, or whose magnitude is NaN, passes idx =
+// none.  Magnitudes order like their bit patterns, so three 32-bit warp
+// reductions do it (an FP64 compare per shuffle step took ~600 cycles).
+__device__ __forceinline__ void warp_argmax(double& v, int& idx, int none) {
+  const unsigned long long key = idx == none ? 0ull : (unsigned long long)__double_as_longlong(v) + 1ull;
+  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  const bool top = hi == mh && lo == ml && key;
+  idx = (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)idx : (unsigned)none);
+  v = __longlong_as_double((long long)((((unsigned long long)mh << 32) | ml) - 1ull));
 }
 
 // Factorisation with Bunch-Kaufman pivoting restricted to the supernode's
@@ -501,12 +377,16 @@ __device__ __forceinline__ void warp_argmax(double& v, int& idx) {
 // symmetric interchanges of the whole block, including the computed L rows.
 // Out: L_KK (pivot order, zero beside 2x2 blocks) and D to the panel's
 // diagonal block, D, E (2x2 off-diagonals), pivot types, the local pivot
-// order piv, (L_KK)^{-1} to linv.  A reduced column that is entirely zero, a
+// order piv.  (L_KK)^{-1} is k_vdiag's and k_vinv's.
+// Bound: per column the search and the reciprocal of the pivot (one warp), three
+// barriers, and the trailing update on this SM's FP64 pipe, one FMA per entry
+// (L_i u_j with the unscaled column u kept beside L; L_i L_j d took three FP64
+// operations, 300 of the 440-530 us of a 128-wide block).  A reduced column that is entirely zero, a
 // singular 2x2 block or a non-finite value is reported in the status words.
 template <class T>
 __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
                                  T* __restrict__ D, T* __restrict__ E, int8_t* __restrict__ ptype,
-                                 int32_t* __restrict__ piv, T* __restrict__ Linv, Sizes sz, int* status) {
+                                 int32_t* __restrict__ piv, Sizes sz, int* status) {
   extern __shared__ __align__(16) unsigned char shraw[];
   T* Tp = reinterpret_cast<T*>(shraw);
   const int k0 = sns[blockIdx.x];
@@ -517,6 +397,8 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
   T* l2 = l1 + s;
   int* perm = reinterpret_cast<int*>(l2 + s);
   __shared__ int sh_kp, sh_kstep, sh_bad;
+  __shared__ __align__(16) double rraw[Sc<T>::P];
+  T* rpiv = reinterpret_cast<T*>(rraw);  // 1 / pivot of a 1 x 1 step
   T* P = L + b * sz.panel + m.panel;
   const int nt = blockDim.x, t = threadIdx.x;
   const double alpha = (1.0 + sqrt(17.0)) / 8.0;
@@ -534,26 +416,35 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
   while (k < s) {
     // pivot search by warp 0
     if (t < 32) {
-      double cv = -1.0;
+      const T akk = Tp[pk(k, k, s)];
+      const T r0 = Sc<T>::one() / akk;  // the reciprocal pivot of a 1 x 1 step without interchange
+      double cv = 0.0;
       int ci = s;
       for (int i = k + 1 + t; i < s; i += 32) {
         const double v = bk_abs(Tp[pk(i, k, s)]);
-        if (v > cv || (v == cv && i < ci)) {
+        if (v > cv || (v == cv && ci == s)) {
           cv = v;
           ci = i;
         }
       }
-      warp_argmax(cv, ci);
-      const double absakk = bk_abs(Tp[pk(k, k, s)]);
+      warp_argmax(cv, ci, s);
+      const double absakk = bk_abs(akk);
       const double colmax = ci < s ? cv : 0.0;
       const int imax = ci < s ? ci : k;
       double rowmax = 0.0;
       if (absakk < alpha * colmax) {
         double rv = 0.0;
+        int ri = s;
         for (int j = k + t; j < s; j += 32)
-          if (j != imax) rv = fmax(rv, bk_abs(j < imax ? Tp[pk(imax, j, s)] : Tp[pk(j, imax, s)]));
-        for (int o = 16; o > 0; o >>= 1) rv = fmax(rv, __shfl_xor_sync(0xffffffffu, rv, o));
-        rowmax = rv;
+          if (j != imax) {
+            const double v = bk_abs(j < imax ? Tp[pk(imax, j, s)] : Tp[pk(j, imax, s)]);
+            if (v > rv) {
+              rv = v;
+              ri = j;
+            }
+          }
+        warp_argmax(rv, ri, s);
+        if (ri < s) rowmax = rv;
       }
       if (t == 0) {
         int kp = k, kstep = 1;
@@ -573,6 +464,7 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
         }
         sh_kp = kp;
         sh_kstep = kstep;
+        *rpiv = kp == k ? r0 : Sc<T>::one() / Tp[pk(kp, kp, s)];
       }
     }
     __syncthreads();
@@ -605,15 +497,22 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
       __syncthreads();
     }
     if (kstep == 1) {
-      const T d = Tp[pk(k, k, s)];
-      for (int i = k + 1 + t; i < s; i += nt) Tp[pk(i, k, s)] = Tp[pk(i, k, s)] / d;
+      const T rd = *rpiv;
+      const int ck = pk(k, k, s) - k;
+      for (int i = k + 1 + t; i < s; i += nt) {
+        const T u = Tp[ck + i];
+        l1[i] = u;
+        Tp[ck + i] = u * rd;
+      }
       __syncthreads();
       // trailing lower triangle, one warp per column (no integer division)
       for (int jj = k + 1 + (t >> 5); jj < s; jj += nt >> 5) {
-        const int cj = pk(jj, jj, s);
-        for (int ii = jj + (t & 31); ii < s; ii += 32) Tp[cj + ii - jj] -= Tp[pk(ii, k, s)] * Tp[pk(jj, k, s)] * d;
+        const int cj = pk(jj, jj, s) - jj;
+        const T u = l1[jj];
+        for (int ii = jj + (t & 31); ii < s; ii += 32) Tp[cj + ii] -= Tp[ck + ii] * u;
       }
       if (t == 0) {
+        const T d = Tp[pk(k, k, s)];
         dd[k] = d;
         ee[k] = Sc<T>::zero();
         ty[k] = 0;
@@ -656,7 +555,6 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
     if (t == 0) report_pivot(status, m.f + k, sh_bad == 1);
     return;
   }
-  unit_lower_inverse_blocked(Tp, s, Linv + b * sz.linv + m.linv, reinterpret_cast<T*>(perm + ((s + 3) & ~3)));
   for (int e = t; e < s * s; e += nt) {
     const int i = e % s, j = e / s;
     if (i > j) P[i + (int64_t)j * ld] = Tp[pk(i, j, s)];
@@ -907,7 +805,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, 8>())) k_norm_m(
   // of D^{-1} V meets V_{q0-1,i} = 0, so the range still starts at q0
   tile_mma<T, BN>(sm, q0, s, [](int) { return true; }, la, lb, acc, [&](int r0, int c0) {
     return tk.m0 + r0 < s && tk.n0 + c0 < s && (MODE == 2 || c0 <= dm + r0 + 7);
-  });
+  }, KLowerTA{tk.m0});
   T* XK = (T*)a.X + b * a.sz.panel + m.panel;
   tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
     int i = tk.m0 + mm, j = tk.n0 + nn;
@@ -1098,17 +996,10 @@ static size_t diag_smem(int maxw) {
   return sizeof(T) * ((size_t)maxw * (maxw + 1) / 2 + 2 * (size_t)maxw) + sizeof(int) * (size_t)maxw;
 }
 
-// the pivoted diagonal factorisation: diag_smem plus the blocks of the inverse
-template <class T>
-static size_t diag_smem_bk(int maxw) {
-  const size_t nb = (size_t)(maxw + 15) / 16;
-  return diag_smem<T>(maxw) + 16 + sizeof(T) * 256 * (nb > 1 ? nb - 1 : 1);
-}
-
 template <class T>
 static cudaError_t setup_t() {
   const cudaError_t e = cudaFuncSetAttribute(k_factor_diag_bk<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)diag_smem_bk<T>(kMaxWidth));
+                                       (int)diag_smem<T>(kMaxWidth));
   return e;
 }
 
@@ -1246,6 +1137,16 @@ cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn,
   return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, st) : fdiag_t<double>(f, sns, nsn, p, st);
 }
 
+cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st) {
+  if (nsn <= 0) return cudaSuccess;
+  const dim3 grid(nsn, f.sz.batch, (wmax + kFB - 1) / kFB);
+  if (dtype == PSELINV_C128)
+    k_vdiag<Cplx><<<grid, kVdThreads, 0, st>>>(f, sns);
+  else
+    k_vdiag<double><<<grid, kVdThreads, 0, st>>>(f, sns);
+  return cudaGetLastError();
+}
+
 template <class T>
 static cudaError_t ftiles_t(FKern k, int var, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
   const dim3 grid((unsigned)n, f.sz.batch, f.sides);
@@ -1277,8 +1178,8 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);
       break;
     case Kern::FactorDiagBK:
-      k_factor_diag_bk<T><<<grid, threads > 512 ? 512 : threads, diag_smem_bk<T>(a.maxw), st>>>(
-          a.meta, sns, (T*)a.L, (T*)a.D, (T*)a.E, (int8_t*)a.ptype, (int32_t*)a.piv, (T*)a.Linv, a.sz, a.status);
+      k_factor_diag_bk<T><<<grid, threads > 512 ? 512 : threads, diag_smem<T>(a.maxw), st>>>(
+          a.meta, sns, (T*)a.L, (T*)a.D, (T*)a.E, (int8_t*)a.ptype, (int32_t*)a.piv, a.sz, a.status);
       break;
     case Kern::CopyBackBK:
       k_copyback_bk<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.W, (const T*)a.D,

@@ -117,6 +117,8 @@ cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, c
 // Blocked factorisation: the diagonal block p of the listed supernodes (all wider
 // than p blocks), and its tile lists (var: tile variant of the Schur groups).
 cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st);
+// Inverses of the 32 x 32 diagonal blocks of L_KK of the listed supernodes (the widest wmax).
+cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st);
 cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st);
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype = nullptr, const void* E = nullptr);

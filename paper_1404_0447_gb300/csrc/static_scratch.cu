@@ -15,6 +15,7 @@
 #include <mutex>
 #include <string>
 
+#include "block_inverse.cuh"
 #include "internal.h"
 #include "tile_gemm.cuh"
 
@@ -31,49 +32,54 @@ constexpr int kMaxDevices = 64;
 // column-major, block-major.  Every call overwrites what it uses.
 __device__ __align__(256) double g_block_scratch[kScratchDoubles];
 
-// Phase 1, one CTA per block: V = L^{-1} for the unit lower triangle of the
-// block (entries on and above the diagonal of L are not read), one column of
-// V per thread; every entry of V's s x s block is written (zeros above the
-// diagonal), so nothing from an earlier call survives into this one.
-__global__ void k_static_linv(int s, const double* __restrict__ L, double* __restrict__ scratch) {
-  extern __shared__ double T[];
-  const int b = blockIdx.x;
-  const double* Lb = L + (int64_t)b * s * s;
-  double* V = scratch + (int64_t)b * s * s;
-  for (int e = threadIdx.x; e < s * s; e += blockDim.x) T[e] = Lb[e];
-  __syncthreads();
-  for (int c = threadIdx.x; c < s; c += blockDim.x) {
-    for (int i = 0; i < c; ++i) V[i + c * s] = 0.0;
-    V[c + c * s] = 1.0;
-    for (int i = c + 1; i < s; ++i) {
-      double acc = 0.0;
-      for (int q = c; q < i; ++q) acc += T[i + q * s] * V[q + c * s];
-      V[i + c * s] = -acc;
-    }
-  }
+// Phase 1: the 32 x 32 diagonal blocks of V = L^{-1} (entries on and above the
+// diagonal of L are not read); CTA (block of the batch, block of V).
+__global__ void __launch_bounds__(psi::kVdThreads) k_static_vdiag(int s, const double* __restrict__ L,
+                                                                  double* __restrict__ scratch) {
+  __shared__ psi::VdSmem<double> sm;
+  const int c0 = blockIdx.y * psi::kFB;
+  const int64_t at = (int64_t)blockIdx.x * s * s + c0 + (int64_t)c0 * s;
+  psi::diag_inverse<double>(L + at, s, scratch + at, s, min(psi::kFB, s - c0), sm);
 }
 
-// Phase 2, one CTA per (block, 64 x 64 tile of M): M = V^T D^{-1} V on the
-// FP64 tensor pipe.
-__global__ void __launch_bounds__(psi::TG_THREADS) k_static_m(int s, int tiles_per_dim,
-                                                              const double* __restrict__ scratch,
-                                                              const double* __restrict__ d, double* __restrict__ M) {
-  constexpr int BN = 64;
+// Phase 2: the rest of V in strips of 8 columns (blockIdx.y); every entry of V's
+// s x s block is written by phases 1 and 2 (zeros above the diagonal), so nothing
+// from an earlier call survives into this one.
+__global__ void __launch_bounds__(psi::TG_THREADS) k_static_vinv(int s, const double* __restrict__ L,
+                                                                 double* __restrict__ scratch) {
+  __shared__ psi::VsSmem<double> sm;
+  const int64_t at = (int64_t)blockIdx.x * s * s;
+  psi::inverse_strip<double>(L + at, s, scratch + at, s, blockIdx.y * 8, sm);
+}
+
+// Phase 3, one CTA per 64 x 8 tile on or below the diagonal of a block: M =
+// V^T (D^{-1} V) on the FP64 pipe, which bounds it, from row k = max(m0, n0) of V
+// on (V is lower triangular), mirrored above the diagonal.
+__global__ void __launch_bounds__(psi::TG_THREADS, (psi::tile_min_ctas<double, 8>()))
+    k_static_m(int s, const double* __restrict__ scratch, const double* __restrict__ d, double* __restrict__ M) {
+  constexpr int BN = 8;
   __shared__ psi::TileSmem<double, BN> sm;
-  const int per_block = tiles_per_dim * tiles_per_dim;
-  const int b = blockIdx.x / per_block, t = blockIdx.x % per_block;
-  const int m0 = (t % tiles_per_dim) * psi::TG_BM, n0 = (t / tiles_per_dim) * BN;
+  __shared__ double rd[psi::kMaxWidth];
+  const int b = blockIdx.x, n0 = blockIdx.y * BN, m0 = n0 + blockIdx.z * psi::TG_BM;
+  if (m0 >= s) return;
   const double* V = scratch + (int64_t)b * s * s;
   const double* db = d + (int64_t)b * s;
+  for (int q = m0 + threadIdx.x; q < s; q += psi::TG_THREADS) rd[q] = 1.0 / db[q];
+  __syncthreads();
   psi::Acc<double, BN> acc;
   psi::acc_zero<double, BN>(acc);
-  auto la = [&](int mm, int q) { const int i = m0 + mm; return i < s ? V[q + i * s] / db[q] : 0.0; };
-  auto lb = [&](int q, int nn) { const int j = n0 + nn; return j < s ? V[q + j * s] : 0.0; };
-  psi::tile_mma<double, BN>(sm, 0, s, [](int) { return true; }, la, lb, acc);
+  auto la = [&](int mm, int q) { const int i = m0 + mm; return i < s ? V[q + i * s] : 0.0; };
+  auto lb = [&](int q, int nn) { const int j = n0 + nn; return j < s ? rd[q] * V[q + j * s] : 0.0; };
+  const int dm = m0 - n0;
+  psi::tile_mma<double, BN>(sm, m0, s, [](int) { return true; }, la, lb, acc, [&](int r0, int c0) {
+    return m0 + r0 < s && n0 + c0 < s && c0 <= dm + r0 + 7;
+  }, psi::KLowerTA{m0});
   double* Mb = M + (int64_t)b * s * s;
   psi::tile_epilogue<double, BN>(acc, [&](int mm, int nn, double v) {
     const int i = m0 + mm, j = n0 + nn;
-    if (i < s && j < s) Mb[i + j * s] = v;
+    if (i >= s || j >= s || i < j) return;
+    Mb[i + j * s] = v;
+    Mb[j + i * s] = v;
   });
 }
 
@@ -81,16 +87,12 @@ std::mutex g_mu;
 double* g_scratch_ptr[kMaxDevices] = {};
 
 // Once per device, with that device current: the device address of the
-// scratch array (the host-side symbol is only a stand-in) and the shared
-// memory limit of phase 1.
+// scratch array (the host-side symbol is only a stand-in).
 cudaError_t setup_device(int dev, double** out) {
   std::lock_guard<std::mutex> lock(g_mu);
   if (!g_scratch_ptr[dev]) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_block_scratch);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_static_linv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * psi::kMaxWidth * psi::kMaxWidth));
     if (e != cudaSuccess) return e;
     g_scratch_ptr[dev] = (double*)p;
   }
@@ -121,9 +123,12 @@ extern "C" int pselinv_block_inverse_static(int32_t s, int32_t count, const doub
   e = setup_device(dev, &scratch);
   if (e != cudaSuccess) return fail(PSELINV_ERR_CUDA, std::string("static scratch set-up: ") + cudaGetErrorString(e));
   cudaStream_t st = (cudaStream_t)stream;
-  k_static_linv<<<count, 128, sizeof(double) * s * s, st>>>(s, d_L, scratch);
-  const int tpd = (s + psi::TG_BM - 1) / psi::TG_BM;
-  k_static_m<<<count * tpd * tpd, psi::TG_THREADS, 0, st>>>(s, tpd, scratch, d_d, d_M);
+  // one CTA for the whole inverse of a block, a column per thread, took 1,000 of
+  // the 1,097 us of 192 blocks of order 100
+  const int strips = (s + 7) / 8;
+  k_static_vdiag<<<dim3(count, (s + psi::kFB - 1) / psi::kFB), psi::kVdThreads, 0, st>>>(s, d_L, scratch);
+  if (s > psi::kFB) k_static_vinv<<<dim3(count, strips), psi::TG_THREADS, 0, st>>>(s, d_L, scratch);
+  k_static_m<<<dim3(count, strips, (s + psi::TG_BM - 1) / psi::TG_BM), psi::TG_THREADS, 0, st>>>(s, scratch, d_d, d_M);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(PSELINV_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
   return PSELINV_OK;

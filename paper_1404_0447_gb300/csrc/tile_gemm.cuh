@@ -133,13 +133,13 @@ __device__ __forceinline__ void acc_zero(Acc<T, BN>& acc) {
 // fails live(r0, c0) are skipped (ragged edges of the output, fragments
 // wholly above the diagonal of a triangular output), and so are the 4-deep
 // k-steps at or past kend.  Skipped fragments keep their accumulators (zero
-// from acc_zero) and callers store only live entries.  A triangular B
-// operand adds klive: klive.frag(kk, c0) is false when B is zero on rows
-// kk..kk+3 for the fragment's columns, and klive.all(kt) is true when no
-// fragment has such zero rows in the k-tile [kt, kt + 16).
+// from acc_zero) and callers store only live entries.  A triangular operand
+// adds klive: klive.frag(kk, r0, c0) is false when A or B is zero on
+// kk..kk+3 for the fragment's rows or columns, and klive.all(kt) is true when no
+// fragment has such zeros in the k-tile [kt, kt + 16).
 struct KAllLive {
   __device__ __forceinline__ bool all(int) const { return true; }
-  __device__ __forceinline__ bool frag(int, int) const { return true; }
+  __device__ __forceinline__ bool frag(int, int, int) const { return true; }
 };
 
 template <class T, int BN, class MA, class LA, class LB, class LIVE, class KLIVE = KAllLive>
@@ -242,10 +242,10 @@ __device__ __forceinline__ void tile_mma(TileSmem<T, BN>& sm, int kbeg, int kend
         if (ks >= kleft) continue;
         uint32_t m = lmask;
 #pragma unroll
-        for (int j = 0; j < G::FN; ++j)
-          if (!klive.frag(kt + ks, wn + 8 * j))
+        for (int i = 0; i < G::FM; ++i)
 #pragma unroll
-            for (int i = 0; i < G::FM; ++i) m &= ~(1u << (i * G::FN + j));
+          for (int j = 0; j < G::FN; ++j)
+            if (!klive.frag(kt + ks, wm + 8 * i, wn + 8 * j)) m &= ~(1u << (i * G::FN + j));
         kstep(buf, ks, m);
       }
     }
@@ -274,7 +274,7 @@ template <int BN>
 struct KLowerB {
   int n0;
   __device__ __forceinline__ bool all(int kt) const { return kt + 3 >= n0 + BN - 8; }
-  __device__ __forceinline__ bool frag(int kk, int c0) const { return kk + 3 >= n0 + c0; }
+  __device__ __forceinline__ bool frag(int kk, int, int c0) const { return kk + 3 >= n0 + c0; }
 };
 
 // B upper triangular in (k, global column): B[k][n] = 0 for k > n.
@@ -282,7 +282,15 @@ template <int BN>
 struct KUpperB {
   int n0;
   __device__ __forceinline__ bool all(int kt) const { return kt + TG_BK - 4 <= n0 + 7; }
-  __device__ __forceinline__ bool frag(int kk, int c0) const { return kk <= n0 + c0 + 7; }
+  __device__ __forceinline__ bool frag(int kk, int, int c0) const { return kk <= n0 + c0 + 7; }
+};
+
+// A the transpose of a lower triangle in (k, global row): A[m][k] = 0 for k < m;
+// m0 = the tile's first row.
+struct KLowerTA {
+  int m0;
+  __device__ __forceinline__ bool all(int kt) const { return kt + 3 >= m0 + TG_BM - 8; }
+  __device__ __forceinline__ bool frag(int kk, int r0, int) const { return kk + 3 >= m0 + r0; }
 };
 
 // Visit every accumulator with its tile coordinates: f(m, n, value).

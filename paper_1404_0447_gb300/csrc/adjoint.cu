@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(TG_THREADS, (adj_min_ctas<T, BN, OP>())) k_adj
   const int b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[tk.sn];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   const T* X = (const T*)a.k.X + b * sz.panel;
   const T* L = (const T*)a.k.L + b * sz.panel;
@@ -302,6 +303,7 @@ __global__ void k_adj_sum_parts(AdjArgs a, const int32_t* __restrict__ sns) {
   const int k = sns[blockIdx.x], b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   if (m.nchunk < 2) return;
   const int s = m.s;
   T* part = (T*)a.k.part + b * sz.part + m.part;
@@ -319,6 +321,7 @@ __global__ void k_adj_zbar(AdjArgs a, const int32_t* __restrict__ sns) {
   const int k = sns[blockIdx.x], b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   const int s = m.s, ld = s + m.r;
   const T* Xb = (const T*)a.Xb + b * sz.panel + m.panel;
   T* Z = (T*)a.Zb + b * sz.linv + m.linv;
@@ -343,6 +346,7 @@ __global__ void k_adj_dr2(AdjArgs a, const int32_t* __restrict__ sns) {
   const int k = sns[blockIdx.x], b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   const int s = m.s;
   const T* V = (const T*)a.k.Linv + b * sz.linv + m.linv;
   const T* d = (const T*)a.k.D + b * sz.n + m.f;
@@ -373,6 +377,7 @@ __global__ void k_adj_df1(AdjArgs a, const int32_t* __restrict__ sns) {
   const int k = sns[blockIdx.x], b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   const T* Lp = (const T*)a.k.L + b * sz.panel + m.panel;
   const T* d = (const T*)a.k.D + b * sz.n + m.f;
@@ -415,6 +420,7 @@ __global__ void k_adj_ev(AdjArgs a) {
   const int k = blockIdx.x, b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   const int s = m.s;
   const T* V = (const T*)a.k.Linv + b * sz.linv + m.linv;
   const T* d = (const T*)a.k.D + b * sz.n + m.f;
@@ -429,6 +435,7 @@ __global__ void k_adj_df5(AdjArgs a, const int32_t* __restrict__ sns) {
   const int k = sns[blockIdx.x], b = blockIdx.y;
   const Sizes sz = a.k.sz;
   const SnMeta m = a.k.meta[k];
+  after_previous();
   const int s = m.s, ld = s + m.r;
   const T* Ab = (const T*)a.Zb + b * sz.linv + m.linv;
   T* Fb = (T*)a.Xb + b * sz.panel + m.panel;
@@ -443,66 +450,65 @@ __global__ void k_adj_df5(AdjArgs a, const int32_t* __restrict__ sns) {
 // --------------------------------------------------------------------------
 
 template <class T, int BN>
-static cudaError_t adj_tile_tb(int op, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st) {
+static cudaError_t adj_tile_tb(int op, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   const dim3 grid((unsigned)n, a.k.sz.batch);
+  auto go = [&](void (*kernel)(AdjArgs, const Task*)) { return launch_dep(kernel, grid, TG_THREADS, 0, st, dep, a, t); };
   switch (op) {
-    case A_YBAR: k_adj_tile<T, BN, A_YBAR><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_LHBAR: k_adj_tile<T, BN, A_LHBAR><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_LBAROFF: k_adj_tile<T, BN, A_LBAROFF><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_T1: k_adj_tile<T, BN, A_T1><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_Q: k_adj_tile<T, BN, A_Q><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_VPART: k_adj_tile<T, BN, A_VPART><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_RPART: k_adj_tile<T, BN, A_RPART><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DR1: k_adj_tile<T, BN, A_DR1><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DR3: k_adj_tile<T, BN, A_DR3><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DR4: k_adj_tile<T, BN, A_DR4><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DF2: k_adj_tile<T, BN, A_DF2><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DF3: k_adj_tile<T, BN, A_DF3><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    case A_DF4: k_adj_tile<T, BN, A_DF4><<<grid, TG_THREADS, 0, st>>>(a, t); break;
-    default: k_adj_tile<T, BN, A_SYR2K><<<grid, TG_THREADS, 0, st>>>(a, t); break;
+    case A_YBAR: return go(k_adj_tile<T, BN, A_YBAR>);
+    case A_LHBAR: return go(k_adj_tile<T, BN, A_LHBAR>);
+    case A_LBAROFF: return go(k_adj_tile<T, BN, A_LBAROFF>);
+    case A_T1: return go(k_adj_tile<T, BN, A_T1>);
+    case A_Q: return go(k_adj_tile<T, BN, A_Q>);
+    case A_VPART: return go(k_adj_tile<T, BN, A_VPART>);
+    case A_RPART: return go(k_adj_tile<T, BN, A_RPART>);
+    case A_DR1: return go(k_adj_tile<T, BN, A_DR1>);
+    case A_DR3: return go(k_adj_tile<T, BN, A_DR3>);
+    case A_DR4: return go(k_adj_tile<T, BN, A_DR4>);
+    case A_DF2: return go(k_adj_tile<T, BN, A_DF2>);
+    case A_DF3: return go(k_adj_tile<T, BN, A_DF3>);
+    case A_DF4: return go(k_adj_tile<T, BN, A_DF4>);
+    default: return go(k_adj_tile<T, BN, A_SYR2K>);
   }
-  return cudaGetLastError();
 }
 
 template <class T>
-static cudaError_t adj_tile_t(int op, int var, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st) {
+static cudaError_t adj_tile_t(int op, int var, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   if (n <= 0) return cudaSuccess;
   switch (var) {
-    case 0: return adj_tile_tb<T, 8>(op, a, t, n, st);
-    case 1: return adj_tile_tb<T, 16>(op, a, t, n, st);
-    case 2: return adj_tile_tb<T, 32>(op, a, t, n, st);
+    case 0: return adj_tile_tb<T, 8>(op, a, t, n, st, dep);
+    case 1: return adj_tile_tb<T, 16>(op, a, t, n, st, dep);
+    case 2: return adj_tile_tb<T, 32>(op, a, t, n, st, dep);
     default:
-      if constexpr (Sc<T>::P == 1) return adj_tile_tb<T, 64>(op, a, t, n, st);
+      if constexpr (Sc<T>::P == 1) return adj_tile_tb<T, 64>(op, a, t, n, st, dep);
       return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st) {
+cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   static const int map[] = {A_YBAR, A_LHBAR, A_LBAROFF, A_T1, A_Q, A_VPART, A_RPART, A_SYR2K,
                             A_DR1, A_DR3, A_DR4, A_DF2, A_DF3, A_DF4};
   const int op = map[(int)k];
-  return a.k.dtype == PSELINV_C128 ? adj_tile_t<Cplx>(op, var, a, t, n, st) : adj_tile_t<double>(op, var, a, t, n, st);
+  return a.k.dtype == PSELINV_C128 ? adj_tile_t<Cplx>(op, var, a, t, n, st, dep)
+                                     : adj_tile_t<double>(op, var, a, t, n, st, dep);
 }
 
 template <class T>
-static cudaError_t adj_sn_t(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st) {
+static cudaError_t adj_sn_t(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep) {
   if (nsn <= 0) return cudaSuccess;
-  const dim3 grid(nsn, a.k.sz.batch);
+  const dim3 grid(nsn, a.k.sz.batch), grid8(nsn, a.k.sz.batch, 8);
   switch (k) {
-    case AdjSn::Seed: k_adj_seed<T><<<grid, 256, 0, st>>>(a); break;
-    case AdjSn::Ev: k_adj_ev<T><<<grid, 256, 0, st>>>(a); break;
-    case AdjSn::Zbar: k_adj_zbar<T><<<grid, 256, 0, st>>>(a, sns); break;
-    case AdjSn::Dr2: k_adj_dr2<T><<<dim3(nsn, a.k.sz.batch, 8), 256, 0, st>>>(a, sns); break;
-    case AdjSn::Df1: k_adj_df1<T><<<dim3(nsn, a.k.sz.batch, 8), 256, 0, st>>>(a, sns); break;
-    case AdjSn::Df5: k_adj_df5<T><<<grid, 256, 0, st>>>(a, sns); break;
-    case AdjSn::SumParts: k_adj_sum_parts<T><<<dim3(nsn, a.k.sz.batch, 8), 256, 0, st>>>(a, sns); break;
-    default: break;
+    case AdjSn::Seed: k_adj_seed<T><<<grid, 256, 0, st>>>(a); return cudaGetLastError();
+    case AdjSn::Ev: return launch_dep(k_adj_ev<T>, grid, 256, 0, st, dep, a);
+    case AdjSn::Zbar: return launch_dep(k_adj_zbar<T>, grid, 256, 0, st, dep, a, sns);
+    case AdjSn::Dr2: return launch_dep(k_adj_dr2<T>, grid8, 256, 0, st, dep, a, sns);
+    case AdjSn::Df1: return launch_dep(k_adj_df1<T>, grid8, 256, 0, st, dep, a, sns);
+    case AdjSn::Df5: return launch_dep(k_adj_df5<T>, grid, 256, 0, st, dep, a, sns);
+    default: return launch_dep(k_adj_sum_parts<T>, grid8, 256, 0, st, dep, a, sns);
   }
-  return cudaGetLastError();
 }
 
-cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st) {
-  return a.k.dtype == PSELINV_C128 ? adj_sn_t<Cplx>(k, a, sns, nsn, st) : adj_sn_t<double>(k, a, sns, nsn, st);
+cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep) {
+  return a.k.dtype == PSELINV_C128 ? adj_sn_t<Cplx>(k, a, sns, nsn, st, dep) : adj_sn_t<double>(k, a, sns, nsn, st, dep);
 }
 
 }  // namespace psi

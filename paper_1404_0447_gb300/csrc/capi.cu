@@ -290,7 +290,8 @@ int enqueue_persistent(pselinv_handle* h, cudaStream_t st) {
   psi::KArgs a = kargs(h);
   const int64_t B = h->opts.batch;
   PSI_CUDA(h, cudaMemsetAsync(h->d_pctr, 0, sizeof(int) * (4 * B * h->nsn + h->nlevels + 1), st));
-  PSI_CUDA(h, psi::launch_tiles(psi::Kern::NormM, 0, a, tasks_at(h, h->off_norm, 0), (int64_t)h->t_norm.tasks.size(), st));
+  PSI_CUDA(h, psi::launch_tiles(psi::Kern::NormM, 0, a, tasks_at(h, h->off_norm, 0),
+                                (int64_t)h->t_norm.tasks.size(), st, false));
   for (int v = 0; v < psi::kNumVar; ++v) {
     const psi::Range r = h->t_lhat.whole[v];
     PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
@@ -437,7 +438,7 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
   if (unsym) a3.Lhat = h->d_uhat;
   rc = tm.run(0, (1 + nlhat_launch) * (unsym ? 2 : 1) - (unsym ? 1 : 0), [&] {
     cudaError_t e = psi::launch_tiles(Kern::NormM, 0, a, tasks_at(h, h->off_norm, 0),
-                                      (int64_t)h->t_norm.tasks.size(), st);
+                                      (int64_t)h->t_norm.tasks.size(), st, false);
     for (int side = 0; side < (unsym ? 2 : 1); ++side)
       for (int v = 0; v < psi::kNumVar && e == cudaSuccess; ++v) {
         const psi::Range r = h->t_lhat.whole[v];
@@ -759,15 +760,18 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
   PSI_CUDA(h, cudaStreamWaitEvent(hi, ev[0], 0));
   PSI_CUDA(h, cudaStreamWaitEvent(lo, ev[0], 0));
   const auto* lsn = (const int32_t*)h->d_levelsn;
-  auto schur = [&](const std::vector<psi::Range>& grp, int32_t g0, int32_t g1, cudaStream_t s) -> cudaError_t {
+  // dep: whether the stream's last operation is a kernel of the chain (launch_dep)
+  auto schur = [&](const std::vector<psi::Range>& grp, int32_t g0, int32_t g1, cudaStream_t s, bool& dep) -> cudaError_t {
     for (int32_t g = g0; g < g1; ++g) {  // group by group: disjoint targets inside a group, no atomics
       const psi::Range r = grp[g];
       cudaError_t e = psi::launch_ftiles(psi::FKern::Schur, h->schur_gvar[g], dt, f,
-                                         tasks_at(h, h->off_schur, r.begin), r.end - r.begin, s);
+                                         tasks_at(h, h->off_schur, r.begin), r.end - r.begin, s, dep);
       if (e != cudaSuccess) return e;
+      dep = true;
     }
     return cudaSuccess;
   };
+  bool hidep = false, lodep = false;  // hi and lo start with a wait on an event
   for (int32_t l = nl - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
@@ -778,7 +782,9 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       for (int p = 0; p < psi::kFactorBlocks && wmax > p * psi::kFactorBlock; ++p) {
         const size_t at = (size_t)l * psi::kFactorBlocks + p;
         const psi::Range rs = h->fb_range[at], rp = h->t_fpanel.per_lv[at], ru = h->t_fupdate.per_lv[at];
-        PSI_CUDA(h, psi::launch_fdiag(dt, f, (const int32_t*)h->d_fbsn + rs.begin, (int)(rs.end - rs.begin), p, hi));
+        PSI_CUDA(h, psi::launch_fdiag(dt, f, (const int32_t*)h->d_fbsn + rs.begin, (int)(rs.end - rs.begin), p, hi,
+                                      hidep));
+        hidep = true;
         PSI_CUDA(h, psi::launch_ftiles(psi::FKern::Panel, 0, dt, f, tasks_at(h, h->off_fpanel, rp.begin),
                                        rp.end - rp.begin, hi));
         PSI_CUDA(h, psi::launch_ftiles(psi::FKern::Update, 0, dt, f, tasks_at(h, h->off_fupdate, ru.begin),
@@ -788,7 +794,8 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       // shared memory sized for the level's widest block: several CTAs per SM on levels of narrow supernodes
       psi::KArgs ad = a;
       ad.maxw = wmax;
-      PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiagBK, ad, sns, nsl, hi, wmax >= 64 ? 512 : 256));
+      PSI_CUDA(h, psi::launch_per_sn(psi::Kern::FactorDiagBK, ad, sns, nsl, hi, wmax >= 64 ? 512 : 256, hidep));
+      hidep = true;
       const psi::Range rv = h->t_vinv.per_lv[(size_t)l * psi::kFactorBlocks];
       PSI_CUDA(h, psi::launch_vdiag(dt, f, sns, nsl, wmax, hi));
       PSI_CUDA(h, psi::launch_ftiles(psi::FKern::VInv, 0, dt, f, tasks_at(h, h->off_vinv, rv.begin),
@@ -800,20 +807,25 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       // L_{C,K} to the panels (the Schur update's second operand)
       PSI_CUDA(h, psi::launch_per_sn(psi::Kern::CopyBackBK, a, sns, nsl, hi));
     }
+    const int32_t g0 = h->schur_gptr[l], g1 = h->schur_gptr[l + 1];
+    auto wait = [&](cudaStream_t s, cudaEvent_t e, bool& dep) {
+      dep = false;
+      return cudaStreamWaitEvent(s, e, 0);
+    };
     if (h->far_after_near[l]) {
-      if (l + 1 < nl) PSI_CUDA(h, cudaStreamWaitEvent(hi, ev[1 + nl + l + 1], 0));
-      PSI_CUDA(h, schur(h->schur_near, h->schur_gptr[l], h->schur_gptr[l + 1], hi));
+      if (l + 1 < nl) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
       PSI_CUDA(h, cudaEventRecord(ev[3 + 2 * nl + l], hi));
-      PSI_CUDA(h, cudaStreamWaitEvent(lo, ev[3 + 2 * nl + l], 0));
-      PSI_CUDA(h, schur(h->schur_far, h->schur_gptr[l], h->schur_gptr[l + 1], lo));
+      PSI_CUDA(h, wait(lo, ev[3 + 2 * nl + l], lodep));
+      PSI_CUDA(h, schur(h->schur_far, g0, g1, lo, lodep));
       PSI_CUDA(h, cudaEventRecord(ev[1 + nl + l], lo));
     } else {
       PSI_CUDA(h, cudaEventRecord(ev[1 + l], hi));
-      PSI_CUDA(h, cudaStreamWaitEvent(lo, ev[1 + l], 0));
-      PSI_CUDA(h, schur(h->schur_far, h->schur_gptr[l], h->schur_gptr[l + 1], lo));
+      PSI_CUDA(h, wait(lo, ev[1 + l], lodep));
+      PSI_CUDA(h, schur(h->schur_far, g0, g1, lo, lodep));
       PSI_CUDA(h, cudaEventRecord(ev[1 + nl + l], lo));
-      if (l + 1 < nl) PSI_CUDA(h, cudaStreamWaitEvent(hi, ev[1 + nl + l + 1], 0));
-      PSI_CUDA(h, schur(h->schur_near, h->schur_gptr[l], h->schur_gptr[l + 1], hi));
+      if (l + 1 < nl) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
     }
   }
   PSI_CUDA(h, cudaEventRecord(ev[1 + 2 * nl], hi));
@@ -823,7 +835,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
   // (L_KK)^{-1} off its 32 x 32 diagonal blocks, every supernode at once
   if (!bk)
     PSI_CUDA(h, psi::launch_ftiles(psi::FKern::VInv, 0, dt, f, tasks_at(h, h->off_vinv, 0),
-                                   (int64_t)h->t_vinv.tasks.size(), st));
+                                   (int64_t)h->t_vinv.tasks.size(), st, false));
   return PSELINV_OK;
 }
 
@@ -1198,7 +1210,7 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
   for (int32_t l = h->nlevels - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Zbar, a, sns, nsl, st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Zbar, a, sns, nsl, st, l + 1 < h->nlevels));
     PSI_CUDA(h, tiles(AdjKern::Ybar, h->t_rect, h->off_rect, l));
     PSI_CUDA(h, tiles(AdjKern::Lhbar, h->t_gemm1, h->off_gemm1, l));  // step-2 slices of C
     // per Schur group, its near and far tiles (adjacent, different target levels) as one launch
@@ -1217,7 +1229,7 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
   }
   // adjoint of the supernodal LDL^T, root -> leaves
   PSI_CUDA(h, cudaMemsetAsync(h->d_xb, 0, B * h->panel_total * es, st));
-  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Ev, a, nullptr, h->nsn, st));
+  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Ev, a, nullptr, h->nsn, st, false));  // after the memset
   for (int32_t l = 0; l < h->nlevels; ++l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
@@ -1272,7 +1284,8 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   // recompute Lhat = L_CK (L_KK)^{-1} from the factor (step 1) instead of trusting a stored copy
   for (int v = 0; v < psi::kNumVar; ++v) {
     const psi::Range r = h->t_lhat.whole[v];
-    PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a.k, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st));
+    PSI_CUDA(h, psi::launch_tiles(psi::Kern::Lhat, v, a.k, tasks_at(h, h->off_lhat, r.begin), r.end - r.begin, st,
+                                  false));
   }
   PSI_CUDA(h, cudaMemsetAsync(h->d_lb, 0, B * h->panel_total * es, st));
   PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
   T* sh = reinterpret_cast<T*>(raw);
   const int b = blockIdx.y;
   const SnMeta m = f.meta[sns[blockIdx.x]];
+  after_previous();
   const int s = m.s, ld = m.s + m.r, c0 = p * kFB, w = min(kFB, s - c0);
   const int64_t po = b * f.sz.panel + m.panel + c0 + (int64_t)c0 * ld, vo = b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
   if (threadIdx.x < 32) {
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
+  after_previous();
   const int s = m.s, ld = s + m.r, c0 = tk.c * kFB, w = min(kFB, s - c0);
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, j = threadIdx.x >> 5;
   T* A = (T*)f.L[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(kFUpdateThreads) k_fupdate(FArgs f, const Task
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
+  after_previous();
   const int s = m.s, ld = s + m.r, c0 = tk.c * kFB;
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int64_t po = b * f.sz.panel + m.panel;
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(TG_THREADS) k_vinv(FArgs f, const Task* __rest
   __shared__ VsSmem<T> sm;
   const Task tk = tasks[blockIdx.x];
   const SnMeta m = f.meta[tk.sn];
+  after_previous();
   inverse_strip<T>((const T*)f.L[blockIdx.z] + blockIdx.y * f.sz.panel + m.panel, m.s + m.r,
                    (T*)f.Linv[blockIdx.z] + blockIdx.y * f.sz.linv + m.linv, m.s, tk.n0, sm);
 }
@@ -341,6 +345,7 @@ template <class T>
 __global__ void __launch_bounds__(kVdThreads) k_vdiag(FArgs f, const int32_t* __restrict__ sns) {
   __shared__ __align__(16) unsigned char raw[sizeof(VdSmem<T>)];
   const SnMeta m = f.meta[sns[blockIdx.x]];
+  after_previous();
   const int c0 = blockIdx.z * kFB, ld = m.s + m.r;
   if (c0 >= m.s) return;
   diag_inverse<T>((const T*)f.L[0] + blockIdx.y * f.sz.panel + m.panel + c0 + (int64_t)c0 * ld, ld,
@@ -352,18 +357,23 @@ __global__ void __launch_bounds__(kVdThreads) k_vdiag(FArgs f, const int32_t* __
 __device__ __forceinline__ double bk_abs(double x) { return fabs(x); }
 __device__ __forceinline__ double bk_abs(Cplx x) { return fabs(x.re) + fabs(x.im); }
 
-// Largest magnitude >= 0 over warp lanes with its index (the first on ties), to
-// all lanes; a lane without a candidate, or whose magnitude is NaN, passes idx =
-// none.  Magnitudes order like their bit patterns, so three 32-bit warp
-// reductions do it (an FP64 compare per shuffle step took ~600 cycles).
-__device__ __forceinline__ void warp_argmax(double& v, int& idx, int none) {
-  const unsigned long long key = idx == none ? 0ull : (unsigned long long)__double_as_longlong(v) + 1ull;
+// bk_abs as an ordered key: magnitudes compare like their bit patterns, in integer
+// instructions (an FP64 compare waits 55 cycles for the one pipe); 0 for a NaN.
+constexpr unsigned long long kBkInf = 0x7ff0000000000000ull;
+__device__ __forceinline__ unsigned long long bk_key(double mag) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(mag);
+  return u > kBkInf ? 0ull : u + 1ull;
+}
+
+// Largest key over warp lanes and its index (the first on ties), to all lanes:
+// three 32-bit warp reductions.  Key 0 is no candidate; none where all are.
+__device__ __forceinline__ void warp_argmax(unsigned long long& key, int& idx, int none) {
   const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
   const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
   const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-  const bool top = hi == mh && lo == ml && key;
+  const bool top = key && hi == mh && lo == ml;
   idx = (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)idx : (unsigned)none);
-  v = __longlong_as_double((long long)((((unsigned long long)mh << 32) | ml) - 1ull));
+  key = ((unsigned long long)mh << 32) | ml;
 }
 
 // Factorisation with Bunch-Kaufman pivoting restricted to the supernode's
@@ -378,27 +388,34 @@ __device__ __forceinline__ void warp_argmax(double& v, int& idx, int none) {
 // Out: L_KK (pivot order, zero beside 2x2 blocks) and D to the panel's
 // diagonal block, D, E (2x2 off-diagonals), pivot types, the local pivot
 // order piv.  (L_KK)^{-1} is k_vdiag's and k_vinv's.
+// A reduced column that is entirely zero, a singular 2x2 block or a non-finite
+// value is reported in the status words.
 // Bound: per column the search and the reciprocal of the pivot (one warp), three
-// barriers, and the trailing update on this SM's FP64 pipe, one FMA per entry
-// (L_i u_j with the unscaled column u kept beside L; L_i L_j d took three FP64
-// operations, 300 of the 440-530 us of a 128-wide block).  A reduced column that is entirely zero, a
-// singular 2x2 block or a non-finite value is reported in the status words.
+// barriers, and the trailing update on this SM's FP64 pipe (s^3 / 6 FMAs, 100 us
+// of a 128-wide real block), one FMA per entry: L_i u_j with the unscaled column u
+// kept beside L (L_i L_j d took three FP64 operations, 300 of the 440-530 us of
+// such a block).  Searching column k + 1 beside the update was slower (350
+// against 300 us): the update's FMAs keep the one warp waiting for the pipe.
 template <class T>
-__global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t* __restrict__ sns, T* __restrict__ L,
-                                 T* __restrict__ D, T* __restrict__ E, int8_t* __restrict__ ptype,
-                                 int32_t* __restrict__ piv, Sizes sz, int* status) {
+__global__ void __launch_bounds__(512) k_factor_diag_bk(const SnMeta* __restrict__ meta,
+                                                        const int32_t* __restrict__ sns, T* __restrict__ L,
+                                                        T* __restrict__ D, T* __restrict__ E,
+                                                        int8_t* __restrict__ ptype, int32_t* __restrict__ piv,
+                                                        Sizes sz, int* status) {
   extern __shared__ __align__(16) unsigned char shraw[];
   T* Tp = reinterpret_cast<T*>(shraw);
   const int k0 = sns[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[k0];
+  after_previous();
   const int s = m.s, ld = m.s + m.r;
-  T* l1 = Tp + s * (s + 1) / 2;  // 2x2 step: new L columns
-  T* l2 = l1 + s;
+  T* l1 = Tp + s * (s + 1) / 2;  // 1x1 step: the unscaled column; 2x2 step: the new L columns
+  T* l2 = l1 + s;                // 1x1 step: the new L column
   int* perm = reinterpret_cast<int*>(l2 + s);
-  __shared__ int sh_kp, sh_kstep, sh_bad;
+  __shared__ int sh_kp, sh_kstep, sh_bad, sh_row;  // sh_row: column of the row search still to do, or -1
   __shared__ __align__(16) double rraw[Sc<T>::P];
   T* rpiv = reinterpret_cast<T*>(rraw);  // 1 / pivot of a 1 x 1 step
+  __shared__ double sh_colmax;
   T* P = L + b * sz.panel + m.panel;
   const int nt = blockDim.x, t = threadIdx.x;
   const double alpha = (1.0 + sqrt(17.0)) / 8.0;
@@ -412,63 +429,73 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
   T* dd = D + b * sz.n + m.f;
   T* ee = E + b * sz.n + m.f;
   int8_t* ty = ptype + b * sz.n + m.f;
+  // warp 0, column c final: the decision for pivot position c, up to the row search
+  auto search = [&](int c) {
+    const T acc = Tp[pk(c, c, s)];
+    const T r0 = Sc<T>::one() / acc;  // the reciprocal pivot of a 1 x 1 step without interchange
+    const int cc = pk(c, c, s) - c;
+    unsigned long long ck = 0;
+    int ci = s;
+#pragma unroll
+    for (int h = 0; h < kMaxWidth / 32; ++h) {
+      const int i = c + 1 + t + 32 * h;
+      const unsigned long long key = i < s ? bk_key(bk_abs(Tp[cc + i])) : 0ull;
+      if (key > ck) {
+        ck = key;
+        ci = i;
+      }
+    }
+    warp_argmax(ck, ci, s);
+    if (t == 0) {
+      const unsigned long long ak = bk_key(bk_abs(acc));
+      const double colmax = ck ? __longlong_as_double((long long)(ck - 1)) : 0.0;
+      sh_kp = c;
+      sh_kstep = 1;
+      sh_row = -1;
+      *rpiv = r0;
+      if (ak == 0 || ak > kBkInf || ck > kBkInf) {  // NaN or infinite
+        sh_bad = 2;
+      } else if (ak == 1 && ck <= 1) {
+        sh_bad = 1;
+      } else if (ak < bk_key(alpha * colmax)) {
+        sh_row = ci;
+        sh_colmax = colmax;
+      }
+    }
+  };
   int k = 0;
   while (k < s) {
-    // pivot search by warp 0
-    if (t < 32) {
-      const T akk = Tp[pk(k, k, s)];
-      const T r0 = Sc<T>::one() / akk;  // the reciprocal pivot of a 1 x 1 step without interchange
-      double cv = 0.0;
-      int ci = s;
-      for (int i = k + 1 + t; i < s; i += 32) {
-        const double v = bk_abs(Tp[pk(i, k, s)]);
-        if (v > cv || (v == cv && ci == s)) {
-          cv = v;
-          ci = i;
-        }
-      }
-      warp_argmax(cv, ci, s);
-      const double absakk = bk_abs(akk);
-      const double colmax = ci < s ? cv : 0.0;
-      const int imax = ci < s ? ci : k;
-      double rowmax = 0.0;
-      if (absakk < alpha * colmax) {
-        double rv = 0.0;
+    if (t < 32) search(k);
+    __syncthreads();
+    if (sh_bad) break;
+    if (sh_row >= 0) {
+      if (t < 32) {
+        const int imax = sh_row;
+        unsigned long long rk = 0;
         int ri = s;
         for (int j = k + t; j < s; j += 32)
           if (j != imax) {
-            const double v = bk_abs(j < imax ? Tp[pk(imax, j, s)] : Tp[pk(j, imax, s)]);
-            if (v > rv) {
-              rv = v;
+            const unsigned long long key = bk_key(bk_abs(j < imax ? Tp[pk(imax, j, s)] : Tp[pk(j, imax, s)]));
+            if (key > rk) {
+              rk = key;
               ri = j;
             }
           }
-        warp_argmax(rv, ri, s);
-        if (ri < s) rowmax = rv;
-      }
-      if (t == 0) {
-        int kp = k, kstep = 1;
-        if (!(absakk == absakk) || !(colmax == colmax) || isinf(absakk) || isinf(colmax)) {
-          sh_bad = 2;
-        } else if (absakk == 0.0 && colmax == 0.0) {
-          sh_bad = 1;
-        } else if (absakk < alpha * colmax) {
-          if (absakk * rowmax >= alpha * colmax * colmax) {
-            kp = k;
-          } else if (bk_abs(Tp[pk(imax, imax, s)]) >= alpha * rowmax) {
-            kp = imax;
-          } else {
-            kp = imax;
-            kstep = 2;
+        warp_argmax(rk, ri, s);
+        if (t == 0) {
+          const double rowmax = rk ? __longlong_as_double((long long)(rk - 1)) : 0.0, colmax = sh_colmax;
+          const double absakk = bk_abs(Tp[pk(k, k, s)]);
+          if (!(absakk * rowmax >= alpha * colmax * colmax)) {
+            sh_kp = imax;
+            if (bk_abs(Tp[pk(imax, imax, s)]) >= alpha * rowmax)
+              *rpiv = Sc<T>::one() / Tp[pk(imax, imax, s)];
+            else
+              sh_kstep = 2;
           }
         }
-        sh_kp = kp;
-        sh_kstep = kstep;
-        *rpiv = kp == k ? r0 : Sc<T>::one() / Tp[pk(kp, kp, s)];
       }
+      __syncthreads();
     }
-    __syncthreads();
-    if (sh_bad) break;
     const int kstep = sh_kstep, kp = sh_kp, kk = k + kstep - 1;
     if (kp != kk) {  // symmetric interchange of kk and kp (kp > kk) in packed lower storage
       for (int j = t; j < kk; j += nt) {
@@ -500,22 +527,22 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
       const T rd = *rpiv;
       const int ck = pk(k, k, s) - k;
       for (int i = k + 1 + t; i < s; i += nt) {
-        const T u = Tp[ck + i];
+        const T u = Tp[ck + i], l = u * rd;
         l1[i] = u;
-        Tp[ck + i] = u * rd;
+        l2[i] = l;
+        Tp[ck + i] = l;
+      }
+      if (t == nt - 1) {
+        dd[k] = Tp[ck + k];
+        ee[k] = Sc<T>::zero();
+        ty[k] = 0;
       }
       __syncthreads();
       // trailing lower triangle, one warp per column (no integer division)
       for (int jj = k + 1 + (t >> 5); jj < s; jj += nt >> 5) {
         const int cj = pk(jj, jj, s) - jj;
         const T u = l1[jj];
-        for (int ii = jj + (t & 31); ii < s; ii += 32) Tp[cj + ii] -= Tp[ck + ii] * u;
-      }
-      if (t == 0) {
-        const T d = Tp[pk(k, k, s)];
-        dd[k] = d;
-        ee[k] = Sc<T>::zero();
-        ty[k] = 0;
+        for (int ii = jj + (t & 31); ii < s; ii += 32) Tp[cj + ii] -= l2[ii] * u;
       }
     } else {
       const T a11 = Tp[pk(k, k, s)], a21 = Tp[pk(k + 1, k, s)], a22 = Tp[pk(k + 1, k + 1, s)];
@@ -527,6 +554,7 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
         l2[i] = (w2 * a11 - w1 * a21) / det;
       }
       __syncthreads();
+      if (sh_bad) break;
       for (int jj = k + 2 + (t >> 5); jj < s; jj += nt >> 5) {
         const int cj = pk(jj, jj, s);
         for (int ii = jj + (t & 31); ii < s; ii += 32)
@@ -537,7 +565,7 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
         Tp[pk(i, k, s)] = l1[i];
         Tp[pk(i, k + 1, s)] = l2[i];
       }
-      if (t == 0) {
+      if (t == nt - 1) {
         Tp[pk(k + 1, k, s)] = Sc<T>::zero();
         dd[k] = a11;
         dd[k + 1] = a22;
@@ -548,7 +576,6 @@ __global__ void k_factor_diag_bk(const SnMeta* __restrict__ meta, const int32_t*
       }
     }
     __syncthreads();
-    if (sh_bad) break;
     k += kstep;
   }
   if (sh_bad) {
@@ -573,6 +600,7 @@ __global__ void k_copyback_bk(const SnMeta* __restrict__ meta, const int32_t* __
   const int k = sns[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[k];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   T* P = L + b * sz.panel + m.panel + s;
   const T* Z = W + b * sz.panel + m.panel + s;
@@ -640,8 +668,11 @@ __device__ void pole_share(const KArgs& a, int k, int part, int nparts) {
 
 template <class T>
 __global__ void k_diag_final(KArgs a, const int32_t* __restrict__ sns) {
-  step3_finish<T>(a, sns[blockIdx.x], blockIdx.y, blockIdx.z, gridDim.z, false);
-  if (a.gam) pole_share<T>(a, sns[blockIdx.x], blockIdx.z, gridDim.z);
+  const int k = sns[blockIdx.x];
+  const SnMeta m = a.meta[k];
+  after_previous();
+  step3_finish<T>(a, m, blockIdx.y, blockIdx.z, gridDim.z, false);
+  if (a.gam) pole_share<T>(a, k, blockIdx.z, gridDim.z);
 }
 
 // --------------------------------------------------------------------------
@@ -659,6 +690,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[tk.sn];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   const T* A = L + b * sz.panel + m.panel + s;
   const T* Vi = Linv + b * sz.linv + m.linv;
@@ -705,6 +737,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   const int64_t po = b * f.sz.panel + m.panel + s;
   const T* Lc2 = (const T*)f.L[f.sides - 1 - side] + po;
@@ -760,6 +793,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, 8>())) k_norm_m(
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = a.meta[tk.sn];
+  after_previous();
   const int s = m.s, ld = m.s + m.r;
   const T* V = (const T*)a.Linv + b * a.sz.linv + m.linv;
   const T* Vm = MODE == 2 ? (const T*)a.Uinv + b * a.sz.linv + m.linv : V;
@@ -834,6 +868,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_lhat(c
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y;
   const SnMeta m = meta[tk.sn];
+  after_previous();
   const int s = m.s, r = m.r, ld = s + r;
   const T* A = L + b * sz.panel + m.panel + s;
   const T* Vi = Linv + b * sz.linv + m.linv;
@@ -861,7 +896,10 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_lhat(c
 template <class T, int BN, bool UNSYM>
 __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_gemm1(KArgs a, const Task* __restrict__ tasks) {
   __shared__ TileSmem<T, BN> sm;
-  step2_tile<T, BN, UNSYM>(a, tasks[blockIdx.x], blockIdx.y, sm);
+  const Task tk = tasks[blockIdx.x];
+  const SnMeta m = a.meta[tk.sn];
+  after_previous();
+  step2_tile<T, BN, UNSYM>(a, tk, m, blockIdx.y, sm);
 }
 
 // blockIdx.z strides over the columns of the split supernodes of the level
@@ -873,7 +911,10 @@ __global__ void k_gemm1_reduce(KArgs a, const int32_t* __restrict__ sns) {
 template <class T, int BN>
 __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_gemm2(KArgs a, const Task* __restrict__ tasks) {
   __shared__ TileSmem<T, BN> sm;
-  step3_tile<T, BN>(a, tasks[blockIdx.x], blockIdx.y, sm, false);
+  const Task tk = tasks[blockIdx.x];
+  const SnMeta m = a.meta[tk.sn];
+  after_previous();
+  step3_tile<T, BN>(a, tk, m, blockIdx.y, sm, false);
 }
 
 // --------------------------------------------------------------------------
@@ -1067,136 +1108,114 @@ cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, 
 // ---- tile-kernel launch for one task range of one variant ----
 
 template <class T, int BN>
-static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cudaStream_t st) {
+static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   const dim3 grid((unsigned)n, a.sz.batch);
-  if constexpr (BN == 8) {  // lists of 64 x 8 tiles only
-    switch (k) {
-      case Kern::NormM:
-        if (a.Uinv)
-          k_norm_m<T, 2><<<grid, TG_THREADS, 0, st>>>(a, t);
-        else if (a.ptype)
-          k_norm_m<T, 1><<<grid, TG_THREADS, 0, st>>>(a, t);
-        else
-          k_norm_m<T, 0><<<grid, TG_THREADS, 0, st>>>(a, t);
-        return cudaGetLastError();
-      default: break;
-    }
-  }
   switch (k) {
+    case Kern::NormM:
+      if constexpr (BN == 8) {  // a list of 64 x 8 tiles only
+        if (a.Uinv) return launch_dep(k_norm_m<T, 2>, grid, TG_THREADS, 0, st, dep, a, t);
+        if (a.ptype) return launch_dep(k_norm_m<T, 1>, grid, TG_THREADS, 0, st, dep, a, t);
+        return launch_dep(k_norm_m<T, 0>, grid, TG_THREADS, 0, st, dep, a, t);
+      }
+      return cudaErrorInvalidValue;
     case Kern::Trsm:
-      k_trsm<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, a.sz, a.piv, (T*)a.W);
-      break;
+      return launch_dep(k_trsm<T, BN>, grid, TG_THREADS, 0, st, dep, a.meta, t, (const T*)a.L, (const T*)a.Linv, a.sz,
+                        a.piv, (T*)a.W);
     case Kern::Lhat:
-      k_lhat<T, BN><<<grid, TG_THREADS, 0, st>>>(a.meta, t, (const T*)a.L, (const T*)a.Linv, (T*)a.Lhat, a.sz);
-      break;
+      return launch_dep(k_lhat<T, BN>, grid, TG_THREADS, 0, st, dep, a.meta, t, (const T*)a.L, (const T*)a.Linv,
+                        (T*)a.Lhat, a.sz);
     case Kern::Gemm1:
-      if (a.XU)
-        k_gemm1<T, BN, true><<<grid, TG_THREADS, 0, st>>>(a, t);
-      else
-        k_gemm1<T, BN, false><<<grid, TG_THREADS, 0, st>>>(a, t);
-      break;
+      if (a.XU) return launch_dep(k_gemm1<T, BN, true>, grid, TG_THREADS, 0, st, dep, a, t);
+      return launch_dep(k_gemm1<T, BN, false>, grid, TG_THREADS, 0, st, dep, a, t);
     case Kern::Gemm2:
-      k_gemm2<T, BN><<<grid, TG_THREADS, 0, st>>>(a, t);
-      break;
+      return launch_dep(k_gemm2<T, BN>, grid, TG_THREADS, 0, st, dep, a, t);
     default:
       return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <class T>
-static cudaError_t tiles_t(Kern k, int var, const KArgs& a, const Task* t, int64_t n, cudaStream_t st) {
+static cudaError_t tiles_t(Kern k, int var, const KArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   if (n <= 0) return cudaSuccess;
   switch (var) {
-    case 0: return tiles_tb<T, 8>(k, a, t, n, st);
-    case 1: return tiles_tb<T, 16>(k, a, t, n, st);
-    case 2: return tiles_tb<T, 32>(k, a, t, n, st);
+    case 0: return tiles_tb<T, 8>(k, a, t, n, st, dep);
+    case 1: return tiles_tb<T, 16>(k, a, t, n, st, dep);
+    case 2: return tiles_tb<T, 32>(k, a, t, n, st, dep);
     default:
-      if constexpr (Sc<T>::P == 1) return tiles_tb<T, 64>(k, a, t, n, st);
+      if constexpr (Sc<T>::P == 1) return tiles_tb<T, 64>(k, a, t, n, st, dep);
       return cudaErrorInvalidValue;  // complex tiles stop at BN = 32 (register budget)
   }
 }
 
-cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* t, int64_t n, cudaStream_t st) {
-  return a.dtype == PSELINV_C128 ? tiles_t<Cplx>(k, var, a, t, n, st) : tiles_t<double>(k, var, a, t, n, st);
+cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* t, int64_t n, cudaStream_t st, bool dep) {
+  return a.dtype == PSELINV_C128 ? tiles_t<Cplx>(k, var, a, t, n, st, dep) : tiles_t<double>(k, var, a, t, n, st, dep);
 }
 
 // ---- blocked factorisation ----
 
 template <class T>
-static cudaError_t fdiag_t(const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st) {
+static cudaError_t fdiag_t(const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st, bool dep) {
   const dim3 grid(nsn, f.sz.batch);
-  if (f.sides == 2)
-    k_fdiag<T, 2><<<grid, 32 + 2 * kFdUpdate, 0, st>>>(f, sns, p);
-  else
-    k_fdiag<T, 1><<<grid, 32 + kFdUpdate, 0, st>>>(f, sns, p);
-  return cudaGetLastError();
+  if (f.sides == 2) return launch_dep(k_fdiag<T, 2>, grid, 32 + 2 * kFdUpdate, 0, st, dep, f, sns, p);
+  return launch_dep(k_fdiag<T, 1>, grid, 32 + kFdUpdate, 0, st, dep, f, sns, p);
 }
-cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st) {
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st, bool dep) {
   if (nsn <= 0) return cudaSuccess;
-  return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, st) : fdiag_t<double>(f, sns, nsn, p, st);
+  return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, st, dep) : fdiag_t<double>(f, sns, nsn, p, st, dep);
 }
 
 cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st) {
   if (nsn <= 0) return cudaSuccess;
   const dim3 grid(nsn, f.sz.batch, (wmax + kFB - 1) / kFB);
-  if (dtype == PSELINV_C128)
-    k_vdiag<Cplx><<<grid, kVdThreads, 0, st>>>(f, sns);
-  else
-    k_vdiag<double><<<grid, kVdThreads, 0, st>>>(f, sns);
-  return cudaGetLastError();
+  if (dtype == PSELINV_C128) return launch_dep(k_vdiag<Cplx>, grid, kVdThreads, 0, st, true, f, sns);
+  return launch_dep(k_vdiag<double>, grid, kVdThreads, 0, st, true, f, sns);
 }
 
 template <class T>
-static cudaError_t ftiles_t(FKern k, int var, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
+static cudaError_t ftiles_t(FKern k, int var, const FArgs& f, const Task* t, int64_t n, cudaStream_t st, bool dep) {
   const dim3 grid((unsigned)n, f.sz.batch, f.sides);
   switch (k) {
-    case FKern::Panel: k_fpanel<T><<<grid, 4 * kFB, 0, st>>>(f, t); break;
-    case FKern::Update: k_fupdate<T><<<grid, kFUpdateThreads, 0, st>>>(f, t); break;
-    case FKern::VInv: k_vinv<T><<<grid, TG_THREADS, 0, st>>>(f, t); break;
+    case FKern::Panel: return launch_dep(k_fpanel<T>, grid, 4 * kFB, 0, st, dep, f, t);
+    case FKern::Update: return launch_dep(k_fupdate<T>, grid, kFUpdateThreads, 0, st, dep, f, t);
+    case FKern::VInv: return launch_dep(k_vinv<T>, grid, TG_THREADS, 0, st, dep, f, t);
     default:  // Schur groups: 64 x 8 tiles, or the widest of the type
-      if (var == 0)
-        k_schur<T, 8><<<grid, TG_THREADS, 0, st>>>(f, t);
-      else if constexpr (Sc<T>::P == 2)
-        k_schur<T, 32><<<grid, TG_THREADS, 0, st>>>(f, t);
-      else
-        return cudaErrorInvalidValue;
+      if (var == 0) return launch_dep(k_schur<T, 8>, grid, TG_THREADS, 0, st, dep, f, t);
+      if constexpr (Sc<T>::P == 2) return launch_dep(k_schur<T, 32>, grid, TG_THREADS, 0, st, dep, f, t);
+      return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
-cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st) {
+cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st,
+                          bool dep) {
   if (n <= 0) return cudaSuccess;
-  return dtype == PSELINV_C128 ? ftiles_t<Cplx>(k, var, f, t, n, st) : ftiles_t<double>(k, var, f, t, n, st);
+  return dtype == PSELINV_C128 ? ftiles_t<Cplx>(k, var, f, t, n, st, dep) : ftiles_t<double>(k, var, f, t, n, st, dep);
 }
 
 template <class T>
-static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads) {
+static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads,
+                            bool dep) {
   if (nsn <= 0) return cudaSuccess;
   const dim3 grid(nsn, a.sz.batch);
   switch (k) {
     case Kern::Gemm1Reduce:
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);
-      break;
+      return cudaGetLastError();
     case Kern::FactorDiagBK:
-      k_factor_diag_bk<T><<<grid, threads > 512 ? 512 : threads, diag_smem<T>(a.maxw), st>>>(
-          a.meta, sns, (T*)a.L, (T*)a.D, (T*)a.E, (int8_t*)a.ptype, (int32_t*)a.piv, a.sz, a.status);
-      break;
+      return launch_dep(k_factor_diag_bk<T>, grid, threads > 512 ? 512 : threads, diag_smem<T>(a.maxw), st, dep, a.meta,
+                        sns, (T*)a.L, (T*)a.D, (T*)a.E, (int8_t*)a.ptype, (int32_t*)a.piv, a.sz, a.status);
     case Kern::CopyBackBK:
-      k_copyback_bk<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a.meta, sns, (T*)a.L, (const T*)a.W, (const T*)a.D,
-                                                                  (const T*)a.E, a.ptype, a.sz);
-      break;
+      return launch_dep(k_copyback_bk<T>, dim3(nsn, a.sz.batch, 16), 256, 0, st, dep, a.meta, sns, (T*)a.L,
+                        (const T*)a.W, (const T*)a.D, (const T*)a.E, a.ptype, a.sz);
     default:
       // 32 CTAs per supernode: the levels near the root hold one supernode whose
       // finish reads one s x s partial per row chunk of C
-      k_diag_final<T><<<dim3(nsn, a.sz.batch, kFinishCtas), 256, 0, st>>>(a, sns);
-      break;
+      return launch_dep(k_diag_final<T>, dim3(nsn, a.sz.batch, kFinishCtas), 256, 0, st, dep, a, sns);
   }
-  return cudaGetLastError();
 }
 
-cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads) {
-  return a.dtype == PSELINV_C128 ? per_sn_t<Cplx>(k, a, sns, nsn, st, threads)
-                                 : per_sn_t<double>(k, a, sns, nsn, st, threads);
+cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads,
+                          bool dep) {
+  return a.dtype == PSELINV_C128 ? per_sn_t<Cplx>(k, a, sns, nsn, st, threads, dep)
+                                 : per_sn_t<double>(k, a, sns, nsn, st, threads, dep);
 }
 
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,

@@ -7,6 +7,47 @@
 
 namespace psi {
 
+// Programmatic dependent launch.  The level loops are chains of kernels of a few
+// microseconds; a kernel launched with launch_dep may start while its predecessor in
+// the stream still runs, reads what no kernel writes (its task, the supernode's
+// metadata) and waits in after_previous() for the predecessor's end.  Every kernel
+// launched so calls after_previous() in all its threads before anything else in
+// memory, so that a kernel's end implies the end of all before it; the next one
+// may start only after that wait, so at most one kernel per stream waits resident.
+__device__ __forceinline__ void after_previous() {
+#ifdef __CUDA_ARCH__
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+#endif
+}
+
+//
+// Only grids of at most kDepCtas CTAs, the latency-bound ones: CTAs placed while the
+// predecessor still holds the SMs land where slots are free, several on one SM
+// beside empty ones, and a launch that is bound by the FP64 pipe then ends later
+// than after an ordinary start (no limit: 20^3 adjoint step 10.9 -> 14.0 ms; 64
+// against none: 31 x 31 grid 648 -> 590 us, 200 x 147 grid 1,911 -> 1,857, 24^3
+// log det step 6,685 -> 6,558, adjoint step 10,934 -> 10,778; 152 is within 2%
+// of 64 either way).
+constexpr int64_t kDepCtas = 64;
+
+// dep = false: an ordinary launch (the first of a stream's chain, or after a wait
+// on another stream's event).
+template <class... P, class... A>
+cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool dep, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = dep && (int64_t)grid.x * grid.y * grid.z <= kDepCtas ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Per-batch-member sizes (elements of the scalar) of every batched array.
 struct Sizes {
   int64_t panel;  // L and X panels
@@ -109,17 +150,21 @@ cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, 
                                  void* out, const Sizes& sz, cudaStream_t st);
 // Tile kernels (Trsm, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
-cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st);
+cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st,
+                         bool dep = true);
 // Per-supernode kernels (DiagFinal, Gemm1Reduce, FactorDiagBK, CopyBackBK) over
 // the nsn supernodes listed in sns.  threads: block size of FactorDiagBK (at
 // most 512).
-cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads = 256);
+cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, cudaStream_t st, int threads = 256,
+                          bool dep = true);
 // Blocked factorisation: the diagonal block p of the listed supernodes (all wider
 // than p blocks), and its tile lists (var: tile variant of the Schur groups).
-cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st);
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st,
+                         bool dep = true);
 // Inverses of the 32 x 32 diagonal blocks of L_KK of the listed supernodes (the widest wmax).
 cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st);
-cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st);
+cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st,
+                          bool dep = true);
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype = nullptr, const void* E = nullptr);
 cudaError_t launch_pole_sum(int dtype, const void* X, int64_t panel_total, int batch, const void* w, void* out,
@@ -208,7 +253,8 @@ struct AdjArgs {
 };
 enum class AdjKern { Ybar, Lhbar, LbarOff, T1, Q, Vpart, Rpart, Syr2k, Dr1, Dr3, Dr4, Df2, Df3, Df4 };
 enum class AdjSn { Seed, Ev, Zbar, Dr2, Df1, Df5, SumParts };
-cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* tasks, int64_t n, cudaStream_t st);
-cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st);
+cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* tasks, int64_t n, cudaStream_t st,
+                             bool dep = true);
+cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep = true);
 
 }  // namespace psi

@@ -119,9 +119,9 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
         if (par >= 0 && !cta_wait(p.cf + cb + par, kFinishParts, p.spin_ns, status)) break;
         const int64_t yoff = (int64_t)(l % kRing) * p.yslot;
         if (pt.var == 0)
-          step2_tile<T, 8>(a, tk, b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), yoff);
+          step2_tile<T, 8>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), yoff);
         else
-          step2_tile<T, MAXBN>(a, tk, b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), yoff);
+          step2_tile<T, MAXBN>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), yoff);
         cta_signal(p.c1 + cb + k);
         break;
       }
@@ -140,9 +140,9 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
           break;
         const int64_t poff = (int64_t)(p.snlevel[k] % kRing) * p.pslot;
         if (pt.var == 0)
-          step3_tile<T, 8>(a, tk, b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), true, poff);
+          step3_tile<T, 8>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), true, poff);
         else
-          step3_tile<T, MAXBN>(a, tk, b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), true, poff);
+          step3_tile<T, MAXBN>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), true, poff);
         cta_signal(p.c2 + cb + k);
         break;
       }
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
           target = p.n2[k] + 1;
         }
         if (ctr && !cta_wait(ctr, target, p.spin_ns, status)) break;
-        step3_finish<T>(a, k, b, pt.var, kFinishParts, true, (int64_t)(l % kRing) * p.pslot);
+        step3_finish<T>(a, a.meta[k], b, pt.var, kFinishParts, true, (int64_t)(l % kRing) * p.pslot);
         cta_signal2(p.cf + cb + k, p.lvl + l);
         break;
       }

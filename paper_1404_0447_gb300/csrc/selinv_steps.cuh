@@ -61,10 +61,9 @@ __device__ __forceinline__ bool last_slice(const KArgs& a, const SnMeta& m, cons
 // yoff / poff (persistent schedule): element offset of the level's slot in
 // the step-2 / step-3 partial-product buffers (0 for the per-level launches).
 template <class T, int BN, bool UNSYM = false>
-__device__ __forceinline__ void step2_tile(const KArgs& a, const Task& tk, int b, TileSmem<T, BN>& sm,
-                                           int64_t yoff = 0) {
+__device__ __forceinline__ void step2_tile(const KArgs& a, const Task& tk, const SnMeta& m, int b,
+                                           TileSmem<T, BN>& sm, int64_t yoff = 0) {
   const Sizes& sz = a.sz;
-  const SnMeta m = a.meta[tk.sn];
   const int s = m.s, r = m.r, ld = s + r;
   const ColDesc* dk = a.desc + m.desc;
   const int32_t* relidx = a.relidx;
@@ -150,10 +149,9 @@ __device__ __forceinline__ void step2_reduce(const KArgs& a, int k, int b, int c
 // Step 3 partial product tile: P_c = Lhat_{rows c, K}^T X_{rows c, K} over a
 // chunk of kchunk3 rows of C (plain transpose; s x s output tiles).
 template <class T, int BN>
-__device__ __forceinline__ void step3_tile(const KArgs& a, const Task& tk, int b, TileSmem<T, BN>& sm, bool cg,
-                                           int64_t poff = 0) {
+__device__ __forceinline__ void step3_tile(const KArgs& a, const Task& tk, const SnMeta& m, int b,
+                                           TileSmem<T, BN>& sm, bool cg, int64_t poff = 0) {
   const Sizes& sz = a.sz;
-  const SnMeta m = a.meta[tk.sn];
   const int s = m.s, r = m.r, ld = s + r;
   const T* Lh = (const T*)a.Lhat + b * sz.lhat + m.lhat;
   const T* Y = (const T*)a.X + b * sz.panel + m.panel + s;
@@ -184,10 +182,9 @@ __device__ __forceinline__ void step3_tile(const KArgs& a, const Task& tk, int b
 // Non-symmetric handles (a.XU set): X_KK = Z as it is, and Z^T goes to the
 // diagonal block of the XU panel.
 template <class T>
-__device__ __forceinline__ void step3_finish(const KArgs& a, int k, int b, int part, int nparts, bool cg,
+__device__ __forceinline__ void step3_finish(const KArgs& a, const SnMeta& m, int b, int part, int nparts, bool cg,
                                              int64_t poff = 0) {
   const Sizes& sz = a.sz;
-  const SnMeta m = a.meta[k];
   const int s = m.s, ld = m.s + m.r;
   T* XK = (T*)a.X + b * sz.panel + m.panel;
   const T* pp = (const T*)a.part + b * sz.part + poff + m.part;

@@ -661,7 +661,7 @@ int build_schedule(pselinv_handle* h) {
           const int32_t c0 = p * kFactorBlock, c1 = std::min(m.s, c0 + kFactorBlock), ld = m.s + m.r;
           if (m.s <= c0) continue;
           h->fb_sn.push_back(k);
-          for (int32_t m0 = c1; m0 < ld; m0 += kFPanelRows) tp.tasks.push_back({k, m0, c0, p});
+          for (int32_t m0 = c1; m0 < ld; m0 += fpanel_rows(c1 - c0)) tp.tasks.push_back({k, m0, c0, p});
           for (int32_t n0 = c1; n0 < m.s; n0 += 8)
             for (int32_t m0 = n0; m0 < ld; m0 += kFUpdateRows) tu.tasks.push_back({k, m0, n0, p});
           if (p == 0 && m.s > kFactorBlock)
@@ -790,6 +790,42 @@ int build_schedule(pselinv_handle* h) {
       lv.end = (int64_t)tl.tasks.size();
     }
     h->schur_gptr[nl] = (int32_t)h->schur_near.size();
+    // Levels with few tiles run all their groups in one launch: a launch per group
+    // and part costs 3-5 us however small (31 x 31 grid: 103 launches), a group
+    // inside the merged launch about 1 us.  The tiles are 16 x 8 with the k range
+    // split over the CTA's warps, so a tile of a 128-wide supernode holds an SM's
+    // FP64 pipe for 4.6 us instead of the 18 us of a 64 x 8 one.
+    h->schur_merged.assign(nl, 0);
+    h->schur_gcnt.assign(h->schur_near.size(), 0);
+    TaskList& tm = h->t_schurm;
+    tm.tasks.clear();
+    tm.per_lv.assign(nl, Range{});
+    const int64_t copies = (int64_t)o.batch * (o.unsym ? 2 : 1);
+    for (int32_t l = 0; l < nl; ++l) {
+      const int32_t g0 = h->schur_gptr[l], g1 = h->schur_gptr[l + 1];
+      const int64_t begin = (int64_t)tm.tasks.size();
+      bool fits = g1 - g0 < (1 << (31 - kMergedShift));
+      for (int32_t g = g0; g < g1 && fits; ++g) {
+        const int64_t gb = (int64_t)tm.tasks.size();
+        for (int32_t q = h->schur_gsn_ptr[g]; q < h->schur_gsn_ptr[g + 1] && fits; ++q) {
+          const int32_t k = h->schur_gsn[q], r = h->meta[k].r;
+          fits = r < (1 << kMergedShift);
+          for (int32_t n0 = 0; n0 < r && fits; n0 += 8) {
+            const int32_t ce = std::min(n0 + 8, r);
+            for (int32_t m0 = n0; m0 < r; m0 += kMergedRows)
+              tm.tasks.push_back({k, m0, n0, (g - g0) << kMergedShift | ce});
+            fits = ((int64_t)tm.tasks.size() - begin) * copies <= kMergedTiles;
+          }
+        }
+        h->schur_gcnt[g] = (int32_t)(tm.tasks.size() - gb);
+      }
+      if (!fits) {
+        tm.tasks.resize(begin);
+        for (int32_t g = g0; g < g1; ++g) h->schur_gcnt[g] = 0;
+      }
+      h->schur_merged[l] = fits;
+      tm.per_lv[l] = Range{begin, (int64_t)tm.tasks.size()};
+    }
   }
   // counters of the split step-2 output tiles (one per (supernode, m-tile, n-tile))
   h->tctr_total = 0;

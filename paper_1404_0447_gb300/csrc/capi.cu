@@ -134,7 +134,7 @@ void free_device(pselinv_handle* h) {
                    &h->d_piv, &h->d_ptype, &h->d_E, &h->d_snlevel, &h->d_yring, &h->d_pring,
                    &h->d_xb,   &h->d_lb,   &h->d_db,     &h->d_zb,     &h->d_w1,    &h->d_yb,   &h->d_hb,
                    &h->d_plist, &h->d_pn,  &h->d_pctr, &h->d_xs, &h->d_ls, &h->d_sig, &h->d_lexp, &h->d_gexp, &h->d_crow,
-                   &h->d_tctr, &h->d_gctr, &h->d_fbsn};
+                   &h->d_tctr, &h->d_gctr, &h->d_fbsn, &h->d_gcnt, &h->d_mctr};
   for (void** p : ptrs) {
     if (*p) cudaFree(*p);
     *p = nullptr;
@@ -219,12 +219,18 @@ int ensure_device(pselinv_handle* h) {
   return PSELINV_OK;
 }
 
+// A ticket per level, a count per (Schur group, copy): batch members and sides.
+int64_t merged_counter_bytes(const pselinv_handle* h) {
+  return (int64_t)sizeof(int) *
+         (h->nlevels + (int64_t)h->schur_gcnt.size() * h->opts.batch * (h->opts.unsym ? 2 : 1));
+}
+
 // Upload the tuning-dependent part (metadata, task lists, partial buffers);
 // called again by the autotuner after build_schedule.
 int upload_schedule(pselinv_handle* h) {
   int rc;
   void** old[] = {&h->d_meta, &h->d_tasks, &h->d_part, &h->d_ypart, &h->d_plist, &h->d_pn, &h->d_pctr,
-                   &h->d_yring, &h->d_pring, &h->d_tctr};
+                   &h->d_yring, &h->d_pring, &h->d_tctr, &h->d_gcnt, &h->d_mctr};
   for (void** p : old)
     if (*p) {
       cudaFree(*p);
@@ -249,6 +255,8 @@ int upload_schedule(pselinv_handle* h) {
   all.insert(all.end(), h->t_fupdate.tasks.begin(), h->t_fupdate.tasks.end());
   h->off_vinv = (int64_t)all.size();
   all.insert(all.end(), h->t_vinv.tasks.begin(), h->t_vinv.tasks.end());
+  h->off_schurm = (int64_t)all.size();
+  all.insert(all.end(), h->t_schurm.tasks.begin(), h->t_schurm.tasks.end());
   h->off_schur = (int64_t)all.size();
   all.insert(all.end(), h->t_schur.tasks.begin(), h->t_schur.tasks.end());
   h->off_rect = (int64_t)all.size();
@@ -260,6 +268,8 @@ int upload_schedule(pselinv_handle* h) {
   h->off_sq = (int64_t)all.size();
   all.insert(all.end(), h->t_sq.tasks.begin(), h->t_sq.tasks.end());
   if ((rc = upload(h, &h->d_tasks, all))) return rc;
+  if ((rc = upload(h, &h->d_gcnt, h->schur_gcnt))) return rc;
+  if ((rc = alloc(h, &h->d_mctr, merged_counter_bytes(h)))) return rc;
   const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
   if ((rc = alloc(h, &h->d_part, B * h->part_max * es))) return rc;
   if ((rc = alloc(h, &h->d_ypart, B * h->ypart_max * es))) return rc;
@@ -741,6 +751,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
   f.sides = h->opts.unsym ? 2 : 1;
   psi::KArgs a = kargs(h);  // pivoted panel solves
   a.W = h->d_X;
+  PSI_CUDA(h, cudaMemsetAsync(h->d_mctr, 0, merged_counter_bytes(h), st));
   // Two streams (look-ahead): `hi` (high priority) runs each level's
   // diagonal blocks, panel solves and "near" Schur tiles (those updating the
   // parents' columns, which the next level's diagonal blocks need); `lo` runs
@@ -782,8 +793,8 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       for (int p = 0; p < psi::kFactorBlocks && wmax > p * psi::kFactorBlock; ++p) {
         const size_t at = (size_t)l * psi::kFactorBlocks + p;
         const psi::Range rs = h->fb_range[at], rp = h->t_fpanel.per_lv[at], ru = h->t_fupdate.per_lv[at];
-        PSI_CUDA(h, psi::launch_fdiag(dt, f, (const int32_t*)h->d_fbsn + rs.begin, (int)(rs.end - rs.begin), p, hi,
-                                      hidep));
+        PSI_CUDA(h, psi::launch_fdiag(dt, f, (const int32_t*)h->d_fbsn + rs.begin, (int)(rs.end - rs.begin), p,
+                                      std::min(psi::kFactorBlock, wmax - p * psi::kFactorBlock), hi, hidep));
         hidep = true;
         PSI_CUDA(h, psi::launch_ftiles(psi::FKern::Panel, 0, dt, f, tasks_at(h, h->off_fpanel, rp.begin),
                                        rp.end - rp.begin, hi));
@@ -812,8 +823,19 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       dep = false;
       return cudaStreamWaitEvent(s, e, 0);
     };
-    if (h->far_after_near[l]) {
-      if (l + 1 < nl) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+    if (h->schur_merged[l]) {  // few tiles: near and far in one launch
+      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      const psi::Range r = h->t_schurm.per_lv[l];
+      const int copies = h->opts.batch * f.sides;
+      psi::MergedArgs q;
+      q.ticket = (int*)h->d_mctr + l;
+      q.gcnt = (const int32_t*)h->d_gcnt + g0;
+      q.done = (int*)h->d_mctr + nl + (int64_t)g0 * copies;
+      q.ntile = (int)(r.end - r.begin);
+      q.spin_ns = h->opts.spin_limit_ns > 0 ? h->opts.spin_limit_ns : 1000000000LL;
+      PSI_CUDA(h, psi::launch_schur_merged(dt, f, q, tasks_at(h, h->off_schurm, r.begin), hi, hidep));
+    } else if (h->far_after_near[l]) {
+      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
       PSI_CUDA(h, cudaEventRecord(ev[3 + 2 * nl + l], hi));
       PSI_CUDA(h, wait(lo, ev[3 + 2 * nl + l], lodep));
@@ -824,7 +846,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       PSI_CUDA(h, wait(lo, ev[1 + l], lodep));
       PSI_CUDA(h, schur(h->schur_far, g0, g1, lo, lodep));
       PSI_CUDA(h, cudaEventRecord(ev[1 + nl + l], lo));
-      if (l + 1 < nl) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
     }
   }
@@ -885,6 +907,13 @@ int pivot_error(pselinv_handle* h, unsigned long long key) {
   return set_err(h, zero ? PSELINV_ERR_ZERO_PIVOT : PSELINV_ERR_NONFINITE,
                  std::string(zero ? "zero" : "non-finite") + " pivot at column " + std::to_string(key >> 2) +
                      " (internal order)");
+}
+// A wait of a merged Schur launch that ran out: the factor is invalid (the flag
+// stays until the next factorisation).
+int factor_timeout(pselinv_handle* h, const int* status) {
+  if (!status[psi::kFactorTimeoutWord]) return PSELINV_OK;
+  h->factored = h->inverted = false;
+  return set_err(h, PSELINV_ERR_TIMEOUT, "a bounded device wait of the factorisation ran out; the factor is invalid");
 }
 }  // namespace
 
@@ -1045,6 +1074,7 @@ int pselinv_sync_status(pselinv_handle* h, void* stream) {
     const int rc = pivot_error(h, key);
     if (rc) return rc;
   }
+  if (const int rc = factor_timeout(h, status)) return rc;
   if (status[2]) {
     PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, 2 * sizeof(int), st));
     PSI_CUDA(h, cudaStreamSynchronize(st));
@@ -1183,10 +1213,13 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream) {
   PSI_CUDA(h, psi::launch_logdet(h->opts.dtype, h->d_D, h->n, dev, h->opts.batch, st,
                                   h->pivoted ? (const int8_t*)h->d_ptype : nullptr, h->pivoted ? h->d_E : nullptr));
   PSI_CUDA(h, cudaMemcpyAsync(h_out, dev, sizeof(double) * 2 * h->opts.batch, cudaMemcpyDeviceToHost, st));
-  unsigned long long key = 0;
-  PSI_CUDA(h, cudaMemcpyAsync(&key, h->d_status, sizeof(key), cudaMemcpyDeviceToHost, st));
+  int status[kStatusWords];
+  PSI_CUDA(h, cudaMemcpyAsync(status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, st));
   PSI_CUDA(h, cudaStreamSynchronize(st));
-  return pivot_error(h, key);
+  unsigned long long key;
+  std::memcpy(&key, status, sizeof(key));
+  if (const int rc = pivot_error(h, key)) return rc;
+  return factor_timeout(h, status);
 }
 
 }  // extern "C"
@@ -1447,7 +1480,7 @@ int pselinv_get_info(const pselinv_handle* h, pselinv_info* info) {
   if (h->dev_sym) {
     const int64_t B = h->opts.batch, es = (int64_t)elem_size(h), tasks =
         (int64_t)(h->t_norm.tasks.size() + h->t_lhat.tasks.size() + h->t_gemm1.tasks.size() + h->t_gemm2.tasks.size() +
-                  h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_fpanel.tasks.size() +
+                  h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_schurm.tasks.size() + h->t_fpanel.tasks.size() +
                   h->t_fupdate.tasks.size() + h->t_vinv.tasks.size() + h->t_rect.tasks.size() +
                   h->t_pgemm1.tasks.size() + h->t_pgemm2.tasks.size() + h->t_sq.tasks.size());
     int64_t bytes = (int64_t)(sizeof(psi::SnMeta) * h->meta.size() + sizeof(psi::ColDesc) * h->desc.size() +

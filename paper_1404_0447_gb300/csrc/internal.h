@@ -76,7 +76,17 @@ constexpr int kTileN = 64;       // output tile columns
 // diagonal blocks on one SM's FP64 pipe.
 constexpr int kFactorBlock = 32;
 constexpr int kFactorBlocks = (kMaxWidth + kFactorBlock - 1) / kFactorBlock;
-constexpr int kFPanelRows = 16;  // rows of a k_fpanel task
+// Rows of a k_fpanel task on a block of w columns: its four warps stand side by
+// side on 16 rows, 8 columns each, and on further rows where the block is narrow.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int fpanel_rows(int w) { return w <= 8 ? 64 : w <= 16 ? 32 : 16; }
+// Merged Schur launches: rows of a tile, bits of Task.c that hold the column end,
+// and the most tiles (all batch members and sides) of a level taken by one.
+constexpr int kMergedRows = 16;
+constexpr int kMergedShift = 20;
+constexpr int64_t kMergedTiles = 8 * 152;
 constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
 // Tile-width variants of the tile GEMMs: BN = 8 << var.
@@ -173,6 +183,12 @@ struct pselinv_handle {
   std::vector<psi::Range> schur_near, schur_far;
   std::vector<int8_t> schur_gvar;  // tile variant of each group (64 x 8 for groups with few tiles)
   std::vector<int32_t> schur_gsn_ptr, schur_gsn;  // supernodes of each group (pselinv_export_symbolic)
+  // levels whose Schur update is one launch (k_schur_merged): 16 x 8 tiles of all
+  // groups in order, Task.c = group inside the level << kMergedShift | column end;
+  // schur_gcnt[g] = such tiles of group g (0 on the other levels)
+  std::vector<int8_t> schur_merged;
+  psi::TaskList t_schurm;
+  std::vector<int32_t> schur_gcnt;
   int32_t schur_var = 0;  // tile variant of the Schur tiles of the larger groups
   std::vector<int8_t> s2var, s3var, trvar;  // step-2 / step-3 / panel-solve tile variant per supernode
   psi::TaskList t_sq;     // s x s tiles of each supernode's diagonal block (adjoint products)
@@ -191,10 +207,14 @@ struct pselinv_handle {
   void* d_diagmask = nullptr;
   void* d_flipmap = nullptr;
   void* d_tasks = nullptr;  // all task arrays back to back
-  int64_t off_norm = 0, off_fpanel = 0, off_fupdate = 0, off_vinv = 0, off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
+  int64_t off_norm = 0, off_fpanel = 0, off_fupdate = 0, off_vinv = 0, off_schurm = 0, off_lhat = 0, off_gemm1 = 0, off_gemm2 = 0, off_trsm = 0, off_schur = 0, off_rect = 0;
   int64_t off_pgemm1 = 0, off_pgemm2 = 0, off_sq = 0;
   void* d_levelsn = nullptr;
   void* d_fbsn = nullptr;   // fb_sn
+  void* d_gcnt = nullptr;   // schur_gcnt
+  // merged Schur launches: per level a ticket, per (group, batch member) the finished
+  // tiles; zeroed at the start of a factorisation
+  void* d_mctr = nullptr;
   void* d_L = nullptr;      // L panels (unit diagonal implied; D on the diagonal slots)
   void* d_X = nullptr;      // X panels
   void* d_D = nullptr;      // pivots, batch x n

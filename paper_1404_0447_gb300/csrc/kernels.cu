@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "block_inverse.cuh"
+#include "bounded_wait.cuh"
 #include "internal.h"
 #include "kernels.h"
 #include "selinv_steps.cuh"
@@ -102,9 +103,11 @@ __global__ void k_gather_values(const T* __restrict__ X, int64_t panel_total, co
 // (L_KK)^{-1} off the diagonal blocks waits until after the last level
 // (k_vinv), where all supernodes run at once.  Against one CTA per supernode
 // factoring and inverting the whole block in shared memory: see k_fdiag.
-constexpr int kFdUpdate = 192;               // threads holding the triangle: 6 warps fill the FP64 pipe
-constexpr int kFdThreads = 32 + kFdUpdate;  // and the pivot warp
+constexpr int kFdUpdate = 192;  // threads holding a 32 x 32 triangle, beside the pivot warp: 6 warps fill the FP64 pipe
 constexpr int kFdEntries = (kFB * (kFB + 1) / 2 + kFdUpdate - 1) / kFdUpdate;  // lower entries per thread
+// ... and a narrower one (levels of thousands of small supernodes): 64 threads for
+// w <= 8 (36 entries), 96 for w <= 16 (136), 128 for w <= 24 (300)
+inline int fd_update(int w) { return w <= 8 ? 64 : w <= 16 ? 96 : w <= 24 ? 128 : kFdUpdate; }
 
 // Value of lane src, to all lanes of the warp.
 __device__ __forceinline__ double shfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -176,8 +179,9 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
     }
     return;
   }
-  const int side = SIDES == 1 ? 0 : (threadIdx.x - 32) / kFdUpdate;
-  const int t = threadIdx.x - 32 - side * kFdUpdate;
+  const int nu = (blockDim.x - 32) / SIDES;  // threads per side
+  const int side = SIDES == 1 ? 0 : (threadIdx.x - 32) / nu;
+  const int t = threadIdx.x - 32 - side * nu;
   const T* P = (const T*)f.L[side] + po;
   T* V = (T*)f.Linv[side] + vo;
   T *sl = sh + side * SD, *spre = sl + 4 * kFB, *sv = sl + 6 * kFB;
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
   int ri[kFdEntries], ck[kFdEntries];
 #pragma unroll
   for (int q = 0; q < kFdEntries; ++q) {
-    const int e = t + q * kFdUpdate;
+    const int e = t + q * nu;
     ri[q] = ck[q] = 0;  // no entry: never live
     x[q] = Sc<T>::zero();
     if (e < ne) {
@@ -230,11 +234,13 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
   }
 }
 
-// Blocked factorisation, rows m0 .. m0+15 of the panel below the diagonal block
+// Blocked factorisation, 16 (32, 64) rows from m0 of the panel below the diagonal block
 // p (task c): W = A V_pp^T = L D, kept in the X panels (same layout) as the
 // first operand of the panel and Schur updates, and L = W D^{-1} in place.
 // Warp j takes the block's columns 8 j .. 8 j + 7 (k < 8 j + 8: V_pp^T is upper
-// triangular); the CTA's 16 rows are its own, so after one barrier L replaces A.
+// triangular) of 16 rows; blocks of at most 8 or 16 columns put the free warps on
+// further rows (fpanel_rows).  The CTA's rows are its own, so after one barrier L
+// replaces A.
 // Operand fragments go straight from global memory to registers, all loads in
 // flight at once.  Bound: the FP64 pipe (40 m8n8k4 MMAs of 145 cycles) where a
 // level has many rows; near the root, latency: 64 x 8 tiles staged in shared
@@ -243,13 +249,15 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
 // L_KK^{-T} D^{-1}, as L_{C,K} = A_{C,K} U'_KK^{-1} D^{-1} uses (U'_KK^T)^{-1}.
 template <class T>
 __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restrict__ tasks) {
-  constexpr int RF = kFPanelRows / 8;
+  constexpr int RF = 2;
   const Task tk = tasks[blockIdx.x];
   const int b = blockIdx.y, side = blockIdx.z;
   const SnMeta m = f.meta[tk.sn];
   after_previous();
   const int s = m.s, ld = s + m.r, c0 = tk.c * kFB, w = min(kFB, s - c0);
-  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, j = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, warp = threadIdx.x >> 5;
+  const int nw = 64 / fpanel_rows(w);  // warps side by side
+  const int j = warp % nw, m0 = tk.m0 + warp / nw * 16;
   T* A = (T*)f.L[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   T* Wp = (T*)f.W[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   const T* Vi = (const T*)f.Linv[f.sides - 1 - side] + b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
@@ -261,7 +269,7 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
     bf[u] = on && n < w ? Vi[n + (int64_t)k * s] : Sc<T>::zero();
 #pragma unroll
     for (int h = 0; h < RF; ++h) {
-      const int row = tk.m0 + 8 * h + g;
+      const int row = m0 + 8 * h + g;
       a[h][u] = on && row < ld ? A[row + (int64_t)k * ld] : Sc<T>::zero();
     }
   }
@@ -283,7 +291,7 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
   for (int h = 0; h < RF; ++h)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int row = tk.m0 + 8 * h + g, col = 8 * j + 2 * q + e;
+      const int row = m0 + 8 * h + g, col = 8 * j + 2 * q + e;
       if (row >= ld || col >= w) continue;
       const T v = frag_value<T>(acc[h], e);
       Wp[row + (int64_t)col * ld] = v;
@@ -769,6 +777,95 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
   });
 }
 
+// The Schur updates of a whole level in one launch: the tiles of all its groups,
+// 16 x 8, in group order.  Targets of different groups overlap, so a tile's
+// read-modify-write waits until the groups before its own have finished (same
+// order per target as a launch per group, so the same bits); the products do not
+// wait.  CTAs take their tile by a ticket: the holder of a tile only waits on
+// tiles with lower tickets, which running CTAs hold, and those of the lowest
+// group wait on nothing, so the waits end whatever else is resident; each is
+// bounded in time all the same (bounded_wait.cuh).
+// Warp w computes the k range [w kq, (w + 1) kq) of the tile from fragments loaded
+// straight to registers; the four partial sums are added in warp order.
+// Bound: latency (loads, at most 16 MMAs a warp, the group order).
+template <class T>
+__global__ void __launch_bounds__(TG_THREADS) k_schur_merged(FArgs f, const Task* __restrict__ tasks, MergedArgs mq) {
+  constexpr int P = Sc<T>::P, RF = kMergedRows / 8, LDP = kMergedRows + 1;
+  __shared__ double part[4][P][8][LDP];
+  __shared__ int sh_ticket;
+  if (threadIdx.x == 0) sh_ticket = atomicAdd(mq.ticket, 1);  // zeroed long before the previous kernel
+  __syncthreads();
+  const int ticket = sh_ticket, copies = gridDim.y, copy = ticket % copies;
+  const Task tk = tasks[ticket / copies];
+  const int side = copy % f.sides, b = copy / f.sides;
+  const int grp = tk.c >> kMergedShift, cend = tk.c & ((1 << kMergedShift) - 1);
+  const SnMeta m = f.meta[tk.sn];
+  const int s = m.s, r = m.r, ld = s + r;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
+  // this thread's entry of the tile and its target
+  const int ei = tk.m0 + t % kMergedRows, ec = tk.n0 + t / kMergedRows;
+  const bool live = ei < r && ec < cend && ec + side <= ei;
+  T* dst = nullptr;
+  if (live) {
+    const ColDesc cd = f.desc[m.desc + ec];
+    dst = (T*)f.L[side] + b * f.sz.panel + cd.col + f.relidx[cd.rel + ei];
+  }
+  const int need = grp > 0 ? mq.gcnt[grp - 1] : 0;
+  after_previous();
+  const int64_t po = b * f.sz.panel + m.panel + s;
+  const T* B = (const T*)f.L[f.sides - 1 - side] + po;
+  const T* W = (const T*)f.W[side] + po;
+  double acc[RF][P][2] = {};
+  const int kq = (s + 15) / 16 * 4, k0 = warp * kq, k1 = min(s, k0 + kq);  // at most 32
+  if (k0 < k1) {
+    T a[RF][kFB / 4], bf[kFB / 4];
+#pragma unroll
+    for (int u = 0; u < kFB / 4; ++u) {
+      const int k = k0 + 4 * u + q;
+      const bool on = k < k1;
+      bf[u] = on && tk.n0 + g < cend ? B[tk.n0 + g + (int64_t)k * ld] : Sc<T>::zero();
+#pragma unroll
+      for (int h = 0; h < RF; ++h) {
+        const int row = tk.m0 + 8 * h + g;
+        a[h][u] = on && row < r ? W[row + (int64_t)k * ld] : Sc<T>::zero();
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < RF; ++h) {
+      if (tk.m0 + 8 * h >= r) continue;
+#pragma unroll
+      for (int u = 0; u < kFB / 4; ++u)
+        if (k0 + 4 * u < k1) frag_mma<T, 1>(acc[h], a[h] + u, bf + u);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < RF; ++h)
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) part[warp][p][2 * q + e][8 * h + g] = acc[h][p][e];
+  __syncthreads();
+  double v[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    v[p] = part[0][p][t / kMergedRows][t % kMergedRows];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) v[p] += part[w][p][t / kMergedRows][t % kMergedRows];
+  }
+  if (grp > 0 && !cta_wait(mq.done + (int64_t)(grp - 1) * copies + copy, need, mq.spin_ns,
+                           f.status + kFactorTimeoutWord, 20))
+    return;
+  if (live) {
+    T x = ld_cg(dst);
+    if constexpr (P == 1)
+      x -= v[0];
+    else
+      x -= T{v[0], v[1]};
+    *dst = x;
+  }
+  cta_signal(mq.done + (int64_t)grp * copies + copy);
+}
+
 // Normalisation, diagonal part: M_K = L_KK^{-T} D_K^{-1} L_KK^{-1} = V^T (D_K^{-1} V)
 // with V = (L_KK)^{-1} from the factorisation, into the diagonal block of the
 // X panel (Algorithm 1 step 3's first term; U_KK = D_K L_KK^T), one 64 x 8
@@ -1154,14 +1251,17 @@ cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* t, int64_t
 // ---- blocked factorisation ----
 
 template <class T>
-static cudaError_t fdiag_t(const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st, bool dep) {
+static cudaError_t fdiag_t(const FArgs& f, const int32_t* sns, int nsn, int p, int w, cudaStream_t st, bool dep) {
   const dim3 grid(nsn, f.sz.batch);
-  if (f.sides == 2) return launch_dep(k_fdiag<T, 2>, grid, 32 + 2 * kFdUpdate, 0, st, dep, f, sns, p);
-  return launch_dep(k_fdiag<T, 1>, grid, 32 + kFdUpdate, 0, st, dep, f, sns, p);
+  const int nu = fd_update(w);
+  if (f.sides == 2) return launch_dep(k_fdiag<T, 2>, grid, 32 + 2 * nu, 0, st, dep, f, sns, p);
+  return launch_dep(k_fdiag<T, 1>, grid, 32 + nu, 0, st, dep, f, sns, p);
 }
-cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st, bool dep) {
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, int w, cudaStream_t st,
+                         bool dep) {
   if (nsn <= 0) return cudaSuccess;
-  return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, st, dep) : fdiag_t<double>(f, sns, nsn, p, st, dep);
+  return dtype == PSELINV_C128 ? fdiag_t<Cplx>(f, sns, nsn, p, w, st, dep)
+                               : fdiag_t<double>(f, sns, nsn, p, w, st, dep);
 }
 
 cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st) {
@@ -1188,6 +1288,14 @@ cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Tas
                           bool dep) {
   if (n <= 0) return cudaSuccess;
   return dtype == PSELINV_C128 ? ftiles_t<Cplx>(k, var, f, t, n, st, dep) : ftiles_t<double>(k, var, f, t, n, st, dep);
+}
+
+cudaError_t launch_schur_merged(int dtype, const FArgs& f, const MergedArgs& q, const Task* t, cudaStream_t st,
+                                bool dep) {
+  if (q.ntile <= 0) return cudaSuccess;
+  const dim3 grid(q.ntile, f.sz.batch * f.sides);
+  if (dtype == PSELINV_C128) return launch_dep(k_schur_merged<Cplx>, grid, TG_THREADS, 0, st, dep, f, t, q);
+  return launch_dep(k_schur_merged<double>, grid, TG_THREADS, 0, st, dep, f, t, q);
 }
 
 template <class T>

@@ -124,6 +124,18 @@ struct FArgs {
   int sides;
 };
 enum class FKern { Panel, Update, VInv, Schur };
+// Status word set when a wait of a merged Schur launch ran out.
+constexpr int kFactorTimeoutWord = 5;
+// One merged Schur launch (k_schur_merged): the level's ticket, and for the
+// level's first group on the tiles per group and the finished tiles per (group,
+// copy), copy = side and batch member.
+struct MergedArgs {
+  int* ticket;
+  const int32_t* gcnt;
+  int* done;
+  int ntile;         // tiles of one copy
+  long long spin_ns; // bound of every wait
+};
 
 // CTAs of the per-level step-3 finish per supernode (blockIdx.z of k_diag_final).
 constexpr int kFinishCtas = 32;
@@ -159,8 +171,10 @@ cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, c
                           bool dep = true);
 // Blocked factorisation: the diagonal block p of the listed supernodes (all wider
 // than p blocks), and its tile lists (var: tile variant of the Schur groups).
-cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, cudaStream_t st,
+// w: the widest such block.
+cudaError_t launch_fdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int p, int w, cudaStream_t st,
                          bool dep = true);
+cudaError_t launch_schur_merged(int dtype, const FArgs& f, const MergedArgs& q, const Task* t, cudaStream_t st, bool dep);
 // Inverses of the 32 x 32 diagonal blocks of L_KK of the listed supernodes (the widest wmax).
 cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st);
 cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st,

@@ -24,55 +24,11 @@
 
 #include "internal.h"
 #include "kernels.h"
+#include "bounded_wait.cuh"
 #include "selinv_steps.cuh"
 #include "tile_gemm.cuh"
 
 namespace psi {
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Thread 0 waits until *ctr >= target (device-scope acquire), bounded by
-// limit_ns; returns false for the whole CTA on timeout or abort.
-__device__ bool cta_wait(const int* ctr, int target, long long limit_ns, int* status) {
-  __shared__ int ok;
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile const int* abort_flag = status + 2;
-    const unsigned long long t0 = global_ns();
-    for (;;) {
-      if (*abort_flag) {
-        ok = 0;
-        break;
-      }
-      if (atomicAdd(const_cast<int*>(ctr), 0) >= target) break;
-      if ((long long)(global_ns() - t0) > limit_ns) {
-        atomicExch(status + 2, 1);  // timeout: abort the launch
-        ok = 0;
-        break;
-      }
-      __nanosleep(200);
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  const int r = ok;
-  __syncthreads();
-  return r != 0;
-}
-
-// Publish a finished task: all threads' writes, then a device-scope fence,
-// then the counter.
-__device__ void cta_signal(int* ctr) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1);
-  }
-}
 
 // Publish one finished finish part: the supernode's and the level's counters.
 __device__ void cta_signal2(int* ctr1, int* ctr2) {
@@ -113,10 +69,10 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
         if (l >= kRing) {  // the level using the same partial-product slot has finished
           const int lr = l - kRing;
           const int target = (p.level_ptr[lr + 1] - p.level_ptr[lr]) * kFinishParts * batch;
-          if (!cta_wait(p.lvl + lr, target, p.spin_ns, status)) break;
+          if (!cta_wait(p.lvl + lr, target, p.spin_ns, status + 2)) break;
         }
         const int par = p.snparent[k];
-        if (par >= 0 && !cta_wait(p.cf + cb + par, kFinishParts, p.spin_ns, status)) break;
+        if (par >= 0 && !cta_wait(p.cf + cb + par, kFinishParts, p.spin_ns, status + 2)) break;
         const int64_t yoff = (int64_t)(l % kRing) * p.yslot;
         if (pt.var == 0)
           step2_tile<T, 8>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), yoff);
@@ -127,7 +83,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
       }
       case P_REDUCE: {
         const int k = pt.idx;
-        if (!cta_wait(p.c1 + cb + k, p.n1[k], p.spin_ns, status)) break;
+        if (!cta_wait(p.c1 + cb + k, p.n1[k], p.spin_ns, status + 2)) break;
         step2_reduce<T>(a, k, b, pt.var, kReduceGroups, true, (int64_t)(p.snlevel[k] % kRing) * p.yslot);
         cta_signal(p.cr + cb + k);
         break;
@@ -136,7 +92,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
         const Task tk = p.g2[pt.idx];
         const int k = tk.sn;
         const bool split = a.meta[k].ksplit > 1;
-        if (!cta_wait(split ? p.cr + cb + k : p.c1 + cb + k, split ? kReduceGroups : p.n1[k], p.spin_ns, status))
+        if (!cta_wait(split ? p.cr + cb + k : p.c1 + cb + k, split ? kReduceGroups : p.n1[k], p.spin_ns, status + 2))
           break;
         const int64_t poff = (int64_t)(p.snlevel[k] % kRing) * p.pslot;
         if (pt.var == 0)
@@ -162,7 +118,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
           ctr = p.c2 + cb + k;
           target = p.n2[k] + 1;
         }
-        if (ctr && !cta_wait(ctr, target, p.spin_ns, status)) break;
+        if (ctr && !cta_wait(ctr, target, p.spin_ns, status + 2)) break;
         step3_finish<T>(a, a.meta[k], b, pt.var, kFinishParts, true, (int64_t)(l % kRing) * p.pslot);
         cta_signal2(p.cf + cb + k, p.lvl + l);
         break;

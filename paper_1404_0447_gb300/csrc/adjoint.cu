@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(TG_THREADS, (adj_min_ctas<T, BN, OP>())) k_adj
   } else if constexpr (OP == A_LBAROFF) {  // Lb_CK = Hb V^T
     auto la = [&](int mm, int t) { const int i = m0 + mm; return i < r ? Hb[i + (int64_t)t * r] : zero; };
     auto lb = [&](int t, int nn) { const int n = n0 + nn; return n < s ? V[n + t * s] : zero; };
-    tile_mma<T, BN>(sm, 0, min(s, n0 + BN), none, la, lb, acc, rect, KUpperB<BN>{n0});
+    tile_mma<T, BN>(sm, 0, min(s, n0 + tile_cols<BN>()), none, la, lb, acc, rect, KUpperB<BN>{n0});
     tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
       const int i = m0 + mm, n = n0 + nn;
       if (i < r && n < s) Lb[m.panel + s + i + (int64_t)n * ld] = v;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(TG_THREADS, (adj_min_ctas<T, BN, OP>())) k_adj
     };
     auto lb = [&](int kk, int nn) { const int n = n0 + nn; return n < s ? L[m.panel + s + kk + (int64_t)n * ld] : zero; };
     tile_mma<T, BN>(sm, kb, ke, upper_by_k, la, lb, acc, rect);
-    const int db = max(kb, m0), de = min(min(ke, r), m0 + TG_BM);
+    const int db = max(kb, m0), de = min(min(ke, r), m0 + tile_rows<BN>());
     if (db < de) {
       auto ld_ = [&](int mm, int kk) {
         if (m0 + mm != kk) return zero;
@@ -478,6 +478,7 @@ static cudaError_t adj_tile_t(int op, int var, const AdjArgs& a, const Task* t, 
     case 0: return adj_tile_tb<T, 8>(op, a, t, n, st, dep);
     case 1: return adj_tile_tb<T, 16>(op, a, t, n, st, dep);
     case 2: return adj_tile_tb<T, 32>(op, a, t, n, st, dep);
+    case kVarFine: return adj_tile_tb<T, kFine>(op, a, t, n, st, dep);
     default:
       if constexpr (Sc<T>::P == 1) return adj_tile_tb<T, 64>(op, a, t, n, st, dep);
       return cudaErrorInvalidValue;

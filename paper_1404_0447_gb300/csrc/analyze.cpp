@@ -514,7 +514,7 @@ int build_schedule(pselinv_handle* h) {
       // steps 2 and 3: up to 8x the tiles at the same padding (dead 8 x 8
       // fragments are skipped), so the few wide supernodes near the root
       // spread over the SMs.
-      int64_t t2f = 0, t3f = 0;
+      int64_t t2f = 0, t3f = 0, t2n = 0, t3n = 0, ttn = 0;  // tiles; 64 x 8 tiles of steps 2, 3 and the panel solve
       for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
         const int32_t k = h->level_sn[t];
         const SnMeta& m = h->meta[k];
@@ -523,6 +523,10 @@ int build_schedule(pselinv_handle* h) {
         const int64_t bn2 = 8 << h->s2var[k], bn3 = 8 << h->s3var[k];
         t2f += (m.r + step2_rows(o) - 1) / step2_rows(o) * ((m.s + bn2 - 1) / bn2) * m.ksplit;
         t3f += (int64_t)m.nchunk * ((m.s + kTileM - 1) / kTileM) * ((m.s + bn3 - 1) / bn3);
+        const int64_t rt = (m.r + kTileM - 1) / kTileM, nt8 = (m.s + 7) / 8;
+        t2n += rt * nt8 * m.ksplit;
+        t3n += (int64_t)m.nchunk * ((m.s + kTileM - 1) / kTileM) * nt8;
+        ttn += rt * nt8;
       }
       // the factorisation's panel solve (r x s tiles, k <= s) likewise
       int64_t ttf = 0;
@@ -536,6 +540,10 @@ int build_schedule(pselinv_handle* h) {
         if (t2f < target && !o.fp64_emulation) h->s2var[k] = 0;
         if (t3f < target / 2 && !o.fp64_emulation) h->s3var[k] = 0;
         h->trvar[k] = (int8_t)(ttf < target ? 0 : pick_variant(h->meta[k].s, cplx, o.small_cutoff));
+        // fewer 64 x 8 tiles than ~8 per SM: fine tiles
+        if (t2n * o.batch < kFineTiles && !o.fp64_emulation) h->s2var[k] = kVarFine;
+        if (t3n * o.batch < kFineTiles && !o.fp64_emulation) h->s3var[k] = kVarFine;
+        if (ttn * o.batch < kFineTiles) h->trvar[k] = kVarFine;
       }
     }
   }
@@ -555,7 +563,7 @@ int build_schedule(pselinv_handle* h) {
     for (int32_t k = 0; k < nsn; ++k) tl.var[k] = (int8_t)var_of(k);
     auto add_sn = [&](int32_t k) {
       tl.per_sn[k].begin = (int64_t)tl.tasks.size();
-      emit(k, 8 << tl.var[k], tl.tasks);
+      emit(k, var_rows(tl.var[k]), var_cols(tl.var[k]), tl.tasks);
       tl.per_sn[k].end = (int64_t)tl.tasks.size();
     };
     if (variant_major) {
@@ -578,9 +586,9 @@ int build_schedule(pselinv_handle* h) {
   };
   auto by_width = [&](int32_t k) { return pick_variant(h->meta[k].s, cplx, o.small_cutoff); };
   auto by_rows = [&](int32_t) { return cplx ? 2 : 3; };
-  auto rect = [&](int32_t k, int bn, std::vector<Task>& out) {  // r x s output tiles
+  auto rect = [&](int32_t k, int rows, int bn, std::vector<Task>& out) {  // r x s output tiles
     const SnMeta& m = h->meta[k];
-    for (int32_t m0 = 0; m0 < m.r; m0 += kTileM)
+    for (int32_t m0 = 0; m0 < m.r; m0 += rows)
       for (int32_t n0 = 0; n0 < m.s; n0 += bn) out.push_back({k, m0, n0, 0});
   };
   // Normalisation lists (one launch per tile width over all supernodes).  M_K:
@@ -589,20 +597,22 @@ int build_schedule(pselinv_handle* h) {
   // tile of a 128-wide block keeps one SM's FP64 pipe busy for 144 us, and with
   // fewer tiles than `target` that is the launch's length (200 x 147 grid:
   // k_lhat 226 us in four widths).
-  build(h->t_norm, true, [](int32_t) { return 0; }, [&](int32_t k, int bn, std::vector<Task>& out) {
+  build(h->t_norm, true, [](int32_t) { return 0; }, [&](int32_t k, int rows, int bn, std::vector<Task>& out) {
     const SnMeta& m = h->meta[k];
-    for (int32_t m0 = 0; m0 < m.s; m0 += kTileM)
+    for (int32_t m0 = 0; m0 < m.s; m0 += rows)
       for (int32_t n0 = 0; n0 < m.s; n0 += bn)
-        if (o.unsym || n0 < m0 + kTileM) out.push_back({k, m0, n0, 0});
+        if (o.unsym || n0 < m0 + rows) out.push_back({k, m0, n0, 0});
   });
   {
-    int64_t nt = 0;
+    int64_t nt = 0, nt8 = 0;
     for (int32_t k = 0; k < nsn; ++k) {
       const int64_t bn = 8 << by_width(k);
       nt += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + bn - 1) / bn);
+      nt8 += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + 7) / 8);
     }
     const bool narrow = nt < (o.level_tiles > 0 ? o.level_tiles : kTargetTiles);
-    build(h->t_lhat, true, [&](int32_t k) { return narrow ? 0 : by_width(k); }, rect);
+    const bool fine = nt8 * o.batch < kFineTiles;
+    build(h->t_lhat, true, [&](int32_t k) { return fine ? kVarFine : narrow ? 0 : by_width(k); }, rect);
   }
   // the adjoint's r x s and s x s tile lists: 64 x 8 tiles on levels whose
   // tiles are too few to fill the GPU (as for steps 2 and 3)
@@ -610,31 +620,33 @@ int build_schedule(pselinv_handle* h) {
   {
     const int64_t target = o.level_tiles > 0 ? o.level_tiles : kTargetTiles;
     for (int32_t l = 0; l < nl; ++l) {
-      int64_t nr = 0, nq = 0;
+      int64_t nr = 0, nq = 0, nr8 = 0, nq8 = 0;
       for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
         const SnMeta& m = h->meta[h->level_sn[t]];
         const int64_t bn = 8 << by_width(h->level_sn[t]);
         nr += (m.r + kTileM - 1) / kTileM * ((m.s + bn - 1) / bn);
         nq += (m.s + kTileM - 1) / kTileM * ((m.s + bn - 1) / bn);
+        nr8 += (m.r + kTileM - 1) / kTileM * ((m.s + 7) / 8);
+        nq8 += (m.s + kTileM - 1) / kTileM * ((m.s + 7) / 8);
       }
       for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
         const int32_t k = h->level_sn[t];
-        rvar[k] = (int8_t)(nr < target ? 0 : by_width(k));
-        qvar[k] = (int8_t)(nq < target ? 0 : by_width(k));
+        rvar[k] = (int8_t)(nr8 * o.batch < kFineTiles ? kVarFine : nr < target ? 0 : by_width(k));
+        qvar[k] = (int8_t)(nq8 * o.batch < kFineTiles ? kVarFine : nq < target ? 0 : by_width(k));
       }
     }
   }
   build(h->t_rect, false, [&](int32_t k) { return (int)rvar[k]; }, rect);
-  auto step2_tiles = [&](int32_t k, int bn, std::vector<Task>& out) {  // step 2: + k-parts
+  auto step2_tiles = [&](int32_t k, int rows, int bn, std::vector<Task>& out) {  // step 2: + k-parts
     const SnMeta& m = h->meta[k];
     for (int32_t c = 0; c < m.ksplit; ++c)
-      for (int32_t m0 = 0; m0 < m.r; m0 += step2_rows(o))
+      for (int32_t m0 = 0; m0 < m.r; m0 += rows)
         for (int32_t n0 = 0; n0 < m.s; n0 += bn) out.push_back({k, m0, n0, c});
   };
-  auto step3_tiles = [&](int32_t k, int bn, std::vector<Task>& out) {
+  auto step3_tiles = [&](int32_t k, int rows, int bn, std::vector<Task>& out) {
     const SnMeta& m = h->meta[k];
     for (int32_t c = 0; c < m.nchunk; ++c)
-      for (int32_t m0 = 0; m0 < m.s; m0 += kTileM)
+      for (int32_t m0 = 0; m0 < m.s; m0 += rows)
         for (int32_t n0 = 0; n0 < m.s; n0 += bn) out.push_back({k, m0, n0, c});
   };
   build(h->t_gemm1, false, [&](int32_t k) { return (int)h->s2var[k]; }, step2_tiles);
@@ -673,16 +685,16 @@ int build_schedule(pselinv_handle* h) {
         tv.per_lv[at].end = (int64_t)tv.tasks.size();
       }
   }
-  build(h->t_sq, false, [&](int32_t k) { return (int)qvar[k]; }, [&](int32_t k, int bn, std::vector<Task>& out) {
+  build(h->t_sq, false, [&](int32_t k) { return (int)qvar[k]; }, [&](int32_t k, int rows, int bn, std::vector<Task>& out) {
     const SnMeta& m = h->meta[k];
-    for (int32_t m0 = 0; m0 < m.s; m0 += kTileM)
+    for (int32_t m0 = 0; m0 < m.s; m0 += rows)
       for (int32_t n0 = 0; n0 < m.s; n0 += bn) out.push_back({k, m0, n0, 0});
   });
-  // the persistent kernel holds one shared-memory tile for every task kind,
-  // so its lists stop at 64 x (8 << kPersistentMaxVar) tiles (register budget: more CTAs per SM)
-  auto by_width_narrow = [&](int32_t k) { return std::min(by_width(k), kPersistentMaxVar); };
-  build(h->t_pgemm1, false, by_width_narrow, step2_tiles);
-  build(h->t_pgemm2, false, by_width_narrow, step3_tiles);
+  // the persistent kernel holds one shared-memory tile for every task kind, so its
+  // lists have 64 x 8 tiles only (register budget: more CTAs per SM), and fine
+  // ones where the other schedules have them (the same sums in the same order)
+  build(h->t_pgemm1, false, [&](int32_t k) { return h->s2var[k] == kVarFine ? kVarFine : 0; }, step2_tiles);
+  build(h->t_pgemm2, false, [&](int32_t k) { return h->s3var[k] == kVarFine ? kVarFine : 0; }, step3_tiles);
   {
     // Schur-update tiles (lower tiles of the r x r update of each supernode),
     // grouped so that the factorisation needs no atomics: two supernodes of a
@@ -833,8 +845,8 @@ int build_schedule(pselinv_handle* h) {
     SnMeta& m = h->meta[k];
     m.tctr = (int32_t)h->tctr_total;
     if (m.ksplit > 1) {
-      const int64_t bn = 8 << h->t_gemm1.var[k];
-      h->tctr_total += (m.r + step2_rows(o) - 1) / step2_rows(o) * ((m.s + bn - 1) / bn);
+      const int64_t bn = var_cols(h->t_gemm1.var[k]), rows = var_rows(h->t_gemm1.var[k]);
+      h->tctr_total += (m.r + rows - 1) / rows * ((m.s + bn - 1) / bn);
     }
   }
   // level-local offsets of the step-3 partial products

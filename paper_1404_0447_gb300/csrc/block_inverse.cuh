@@ -15,31 +15,6 @@ namespace psi {
 
 constexpr int kFB = kFactorBlock;
 
-// acc (8 x 8 fragment: lane l holds row l >> 2, columns 2 (l & 3) + {0, 1}) +=
-// A B with A's fragments a (lane: row l >> 2, k = 4 u + (l & 3)) and B's
-// fragments bf (lane: k = 4 u + (l & 3), column l >> 2), U k-steps of 4.
-template <class T, int U>
-__device__ __forceinline__ void frag_mma(double (&acc)[Sc<T>::P][2], const T* a, const T* bf) {
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if constexpr (Sc<T>::P == 1) {
-      dmma884(acc[0][0], acc[0][1], a[u], bf[u]);
-    } else {
-      dmma884(acc[0][0], acc[0][1], a[u].re, bf[u].re);
-      dmma884(acc[0][0], acc[0][1], -a[u].im, bf[u].im);
-      dmma884(acc[1][0], acc[1][1], a[u].re, bf[u].im);
-      dmma884(acc[1][0], acc[1][1], a[u].im, bf[u].re);
-    }
-  }
-}
-template <class T>
-__device__ __forceinline__ T frag_value(const double (&acc)[Sc<T>::P][2], int e) {
-  if constexpr (Sc<T>::P == 1)
-    return acc[0][e];
-  else
-    return T{acc[0][e], acc[1][e]};
-}
-
 // Row and column of entry e of a lower triangle stored row by row.
 __device__ __forceinline__ void tri_entry(int e, int& i, int& k) {
   i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);

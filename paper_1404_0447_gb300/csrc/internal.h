@@ -89,9 +89,13 @@ constexpr int kMergedShift = 20;
 constexpr int64_t kMergedTiles = 8 * 152;
 constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
-// Tile-width variants of the tile GEMMs: BN = 8 << var.
-constexpr int kNumVar = 4;
-constexpr int kPersistentMaxVar = 0;  // the persistent kernel's tiles stop at BN = 8
+// Variants of the tile GEMMs: 64 x (8 << var) for var 0 .. 3, and the fine 16 x 8 tile.
+constexpr int kNumVar = 5;
+constexpr int kVarFine = 4;
+constexpr int var_rows(int var) { return var == kVarFine ? 16 : kTileM; }
+constexpr int var_cols(int var) { return var == kVarFine ? 8 : 8 << var; }
+// A launch with fewer 64 x 8 tiles than this (all batch members) takes fine ones.
+constexpr int64_t kFineTiles = 8 * 152;
 
 // Tile width of an output with `width` columns: the variant with the least
 // padded width ceil(width / BN) * BN, the wider tile on ties; complex tiles
@@ -192,8 +196,8 @@ struct pselinv_handle {
   int32_t schur_var = 0;  // tile variant of the Schur tiles of the larger groups
   std::vector<int8_t> s2var, s3var, trvar;  // step-2 / step-3 / panel-solve tile variant per supernode
   psi::TaskList t_sq;     // s x s tiles of each supernode's diagonal block (adjoint products)
-  psi::TaskList t_pgemm1; // persistent schedule: step-2 tiles, widths <= 8 << kPersistentMaxVar
-  psi::TaskList t_pgemm2; // persistent schedule: step-3 tiles, widths <= 8 << kPersistentMaxVar
+  psi::TaskList t_pgemm1; // persistent schedule: step-2 tiles, 64 x 8 and fine
+  psi::TaskList t_pgemm2; // persistent schedule: step-3 tiles, 64 x 8 and fine
 
   // ---- device state ----
   int device = -1;

@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_trsm(c
     return col < s ? Vi[col + kk * s] : Sc<T>::zero();
   };
   // (L_KK)^{-T} is upper triangular: output columns < n0 + BN need only k < n0 + BN
-  tile_mma<T, BN>(sm, 0, min(s, tk.n0 + BN), [](int) { return false; }, la, lb, acc,
+  tile_mma<T, BN>(sm, 0, min(s, tk.n0 + tile_cols<BN>()), [](int) { return false; }, la, lb, acc,
                   LiveRect{r - tk.m0, s - tk.n0}, KUpperB<BN>{tk.n0});
   T* wout = W + b * sz.panel + m.panel + s;
   tile_epilogue<T, BN>(acc, [&](int mm, int nn, T v) {
@@ -1238,6 +1238,7 @@ static cudaError_t tiles_t(Kern k, int var, const KArgs& a, const Task* t, int64
     case 0: return tiles_tb<T, 8>(k, a, t, n, st, dep);
     case 1: return tiles_tb<T, 16>(k, a, t, n, st, dep);
     case 2: return tiles_tb<T, 32>(k, a, t, n, st, dep);
+    case kVarFine: return tiles_tb<T, kFine>(k, a, t, n, st, dep);
     default:
       if constexpr (Sc<T>::P == 1) return tiles_tb<T, 64>(k, a, t, n, st, dep);
       return cudaErrorInvalidValue;  // complex tiles stop at BN = 32 (register budget)

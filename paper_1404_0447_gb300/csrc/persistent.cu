@@ -45,8 +45,9 @@ __device__ void cta_signal2(int* ctr1, int* ctr2) {
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persistent(KArgs a, PArgs p, const PTask* __restrict__ list,
                                                            int64_t ntask) {
-  constexpr int MAXBN = 8 << kPersistentMaxVar;  // the task lists stop at this width
-  __shared__ __align__(16) unsigned char smraw[sizeof(TileSmem<T, MAXBN>)];
+  // the task lists hold 64 x 8 and fine tiles
+  static_assert(sizeof(TileSmem<T, kFine>) <= sizeof(TileSmem<T, 8>), "one buffer for both tiles");
+  __shared__ __align__(16) unsigned char smraw[sizeof(TileSmem<T, 8>)];
   __shared__ long long s_item;
   const int batch = a.sz.batch;
   const long long total = ntask * batch;
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
         if (pt.var == 0)
           step2_tile<T, 8>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), yoff);
         else
-          step2_tile<T, MAXBN>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), yoff);
+          step2_tile<T, kFine>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, kFine>*>(smraw), yoff);
         cta_signal(p.c1 + cb + k);
         break;
       }
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
         if (pt.var == 0)
           step3_tile<T, 8>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, 8>*>(smraw), true, poff);
         else
-          step3_tile<T, MAXBN>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, MAXBN>*>(smraw), true, poff);
+          step3_tile<T, kFine>(a, tk, a.meta[k], b, *reinterpret_cast<TileSmem<T, kFine>*>(smraw), true, poff);
         cta_signal(p.c2 + cb + k);
         break;
       }

@@ -36,7 +36,8 @@ __device__ __forceinline__ bool last_slice(const KArgs& a, const SnMeta& m, cons
   __threadfence();  // this CTA's partial before the count
   __syncthreads();
   if (threadIdx.x == 0) {
-    int* ctr = a.tctr + (int64_t)b * a.tctr_n + m.tctr + (tk.m0 / TG_BM) * ((m.s + BN - 1) / BN) + tk.n0 / BN;
+    int* ctr = a.tctr + (int64_t)b * a.tctr_n + m.tctr +
+               (tk.m0 / tile_rows<BN>()) * ((m.s + tile_cols<BN>() - 1) / tile_cols<BN>()) + tk.n0 / tile_cols<BN>();
     last = atomicAdd(ctr, 1) == m.ksplit - 1;
     if (last) *ctr = 0;
     __threadfence();

@@ -81,11 +81,28 @@ struct Geo {
 };
 constexpr int TG_AREG = TG_BM * TG_BK / TG_THREADS;  // 8 A elements per thread per k-tile
 
+// The fine tile, 16 x 8: for launches with few tiles, where a 64 x 8 tile leaves
+// SMs idle or ends long after the others (one with 128 k holds an SM's FP64 pipe for
+// 18 us; a k-tile of it waits for three dependent loads).  The four warps split
+// the k range, 32 each at a time, their fragments loaded straight to registers
+// with all loads in flight; the partial sums are added in warp order through
+// shared memory, after which every thread holds one element of the tile.
+constexpr int kFine = 4;  // as BN
+template <int BN>
+__host__ __device__ constexpr int tile_rows() { return BN == kFine ? 16 : TG_BM; }
+template <int BN>
+__host__ __device__ constexpr int tile_cols() { return BN == kFine ? 8 : BN; }
+template <>
+struct Geo<kFine> {
+  static constexpr int FM = 1, FN = 1;
+};
+
 // CTAs per SM the tile kernels are compiled for (a register cap of
 // 65536 / (128 x this)): the occupancy each tile width had before the
 // fragment predicates below raised the compiler's register choice.
 template <class T, int BN>
 constexpr int tile_min_ctas() {
+  if (BN == kFine) return Sc<T>::P == 2 ? 3 : 5;
   return Sc<T>::P == 2 ? (BN >= 32 ? 3 : BN >= 16 ? 4 : 5) : (BN >= 64 ? 4 : BN >= 32 ? 6 : BN >= 16 ? 8 : 9);
 }
 
@@ -94,6 +111,11 @@ struct TileSmem {
   static constexpr int P = Sc<T>::P;
   double a[2][P][TG_BK][TG_LDA];
   double b[2][P][TG_BK][Geo<BN>::LDB];
+};
+
+template <class T>
+struct TileSmem<T, kFine> {
+  double part[4][Sc<T>::P][tile_cols<kFine>()][tile_rows<kFine>() + 1];
 };
 
 template <class T, int BN>
@@ -105,6 +127,31 @@ __device__ __forceinline__ void dmma884(double& d0, double& d1, double a, double
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
                : "+d"(d0), "+d"(d1)
                : "d"(a), "d"(b));
+}
+
+// acc (8 x 8 fragment: lane l holds row l >> 2, columns 2 (l & 3) + {0, 1}) +=
+// A B with A's fragments a (lane: row l >> 2, k = 4 u + (l & 3)) and B's
+// fragments bf (lane: k = 4 u + (l & 3), column l >> 2), U k-steps of 4.
+template <class T, int U>
+__device__ __forceinline__ void frag_mma(double (&acc)[Sc<T>::P][2], const T* a, const T* bf) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if constexpr (Sc<T>::P == 1) {
+      dmma884(acc[0][0], acc[0][1], a[u], bf[u]);
+    } else {
+      dmma884(acc[0][0], acc[0][1], a[u].re, bf[u].re);
+      dmma884(acc[0][0], acc[0][1], -a[u].im, bf[u].im);
+      dmma884(acc[1][0], acc[1][1], a[u].re, bf[u].im);
+      dmma884(acc[1][0], acc[1][1], a[u].im, bf[u].re);
+    }
+  }
+}
+template <class T>
+__device__ __forceinline__ T frag_value(const double (&acc)[Sc<T>::P][2], int e) {
+  if constexpr (Sc<T>::P == 1)
+    return acc[0][e];
+  else
+    return T{acc[0][e], acc[1][e]};
 }
 
 template <class T, int BN>
@@ -142,10 +189,54 @@ struct KAllLive {
   __device__ __forceinline__ bool frag(int, int, int) const { return true; }
 };
 
+template <class T, class LA, class LB, class LIVE, class KLIVE>
+__device__ __forceinline__ void fine_mma(TileSmem<T, kFine>& sm, int kbeg, int kend, const LA& la, const LB& lb,
+                                         Acc<T, kFine>& acc, const LIVE& live, const KLIVE& klive) {
+  constexpr int P = Sc<T>::P, RF = tile_rows<kFine>() / 8, KW = 32;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
+  double d[RF][P][2] = {};
+  for (int k0 = kbeg + warp * KW; k0 < kend; k0 += 4 * KW) {
+    T a[RF][KW / 4], b[KW / 4];
+#pragma unroll
+    for (int u = 0; u < KW / 4; ++u) {
+      const int k = k0 + 4 * u + q;
+      b[u] = k < kend ? lb(k, g) : Sc<T>::zero();
+#pragma unroll
+      for (int h = 0; h < RF; ++h) a[h][u] = k < kend ? la(8 * h + g, k) : Sc<T>::zero();
+    }
+#pragma unroll
+    for (int h = 0; h < RF; ++h) {
+      if (!live(8 * h, 0)) continue;
+#pragma unroll
+      for (int u = 0; u < KW / 4; ++u)
+        if (k0 + 4 * u < kend && klive.frag(k0 + 4 * u, 8 * h, 0)) frag_mma<T, 1>(d[h], a[h] + u, b + u);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < RF; ++h)
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) sm.part[warp][p][2 * q + e][8 * h + g] = d[h][p][e];
+  __syncthreads();
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int col = t / tile_rows<kFine>(), row = t % tile_rows<kFine>();
+    double v = sm.part[0][p][col][row];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) v += sm.part[w][p][col][row];
+    acc[p][0][0][0] += v;
+  }
+  __syncthreads();  // sm is free for the next product
+}
+
 template <class T, int BN, class MA, class LA, class LB, class LIVE, class KLIVE = KAllLive>
 __device__ __forceinline__ void tile_mma(TileSmem<T, BN>& sm, int kbeg, int kend, const MA& a_by_k_at, const LA& la,
                                          const LB& lb, Acc<T, BN>& acc, const LIVE& live,
                                          const KLIVE& klive = KAllLive{}) {
+  if constexpr (BN == kFine) {
+    fine_mma<T>(sm, kbeg, kend, la, lb, acc, live, klive);
+  } else {
   using G = Geo<BN>;
   constexpr int P = Sc<T>::P;
   const int t = threadIdx.x;
@@ -252,6 +343,7 @@ __device__ __forceinline__ void tile_mma(TileSmem<T, BN>& sm, int kbeg, int kend
     if (it + 1 < nk) stash(buf ^ 1);
     __syncthreads();
   }
+  }
 }
 
 // Every fragment live.
@@ -273,7 +365,7 @@ struct LiveRect {
 template <int BN>
 struct KLowerB {
   int n0;
-  __device__ __forceinline__ bool all(int kt) const { return kt + 3 >= n0 + BN - 8; }
+  __device__ __forceinline__ bool all(int kt) const { return kt + 3 >= n0 + tile_cols<BN>() - 8; }
   __device__ __forceinline__ bool frag(int kk, int, int c0) const { return kk + 3 >= n0 + c0; }
 };
 
@@ -296,6 +388,15 @@ struct KLowerTA {
 // Visit every accumulator with its tile coordinates: f(m, n, value).
 template <class T, int BN, class F>
 __device__ __forceinline__ void tile_epilogue(const Acc<T, BN>& acc, const F& f) {
+  if constexpr (BN == kFine) {
+    const int t = threadIdx.x;
+    T v;
+    if constexpr (Sc<T>::P == 1)
+      v = acc[0][0][0][0];
+    else
+      v = T{acc[0][0][0][0], acc[1][0][0][0]};
+    f(t % tile_rows<BN>(), t / tile_rows<BN>(), v);
+  } else {
   using G = Geo<BN>;
   const int t = threadIdx.x;
   const int lane = t & 31, warp = t >> 5;
@@ -315,12 +416,23 @@ __device__ __forceinline__ void tile_epilogue(const Acc<T, BN>& acc, const F& f)
         }
         f(wm + 8 * i + g, wn + 8 * j + 2 * q + e, v);
       }
+  }
 }
 
 // acc(mm, nn) = f(mm, nn, acc(mm, nn)) for every element of the tile
 // (tile-local coordinates as in tile_epilogue).
 template <class T, int BN, class F>
 __device__ __forceinline__ void tile_update(Acc<T, BN>& acc, const F& f) {
+  if constexpr (BN == kFine) {
+    const int t = threadIdx.x, m = t % tile_rows<BN>(), n = t / tile_rows<BN>();
+    if constexpr (Sc<T>::P == 1) {
+      acc[0][0][0][0] = f(m, n, acc[0][0][0][0]);
+    } else {
+      const T v = f(m, n, T{acc[0][0][0][0], acc[1][0][0][0]});
+      acc[0][0][0][0] = v.re;
+      acc[1][0][0][0] = v.im;
+    }
+  } else {
   using G = Geo<BN>;
   const int t = threadIdx.x;
   const int lane = t & 31, warp = t >> 5;
@@ -346,6 +458,7 @@ __device__ __forceinline__ void tile_update(Acc<T, BN>& acc, const F& f) {
           acc[1][i][j][e] = v.im;
         }
       }
+  }
 }
 
 }  // namespace psi

@@ -479,7 +479,7 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
     af.gctr = (int*)h->d_gctr;
   }
   auto step = [&](const int32_t* sns, int nsn_step, const psi::Range* r1, const psi::Range* r2, bool split,
-                  int maxr) {
+                  int maxr, int maxs) {
     int n1 = (split && emul) ? 1 : 0, n2 = 0, e;
     for (int v = 0; v < psi::kNumVar; ++v) {
       n1 += r1[v].end > r1[v].begin;
@@ -499,6 +499,9 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
       });
     };
     if ((e = gemm1(a2))) return e;
+    // narrow supernodes: the last tile of each runs the finish (supernodes without
+    // rows below have none, and nothing to add to M_K)
+    a3.tctr = !unsym && !emul && !af.gam && maxs <= psi::kFinishWidth ? (int*)h->d_tctr : nullptr;
     // step 3 partial products; emulated: slices of diag(2^-e_C) X_{C,K} first
     if ((e = tm.run(2, n2 + (emul && n2 > 0 ? 1 : 0), [&] {
            cudaError_t x = emul ? psi::launch_em_split_xck(a, em, sns, nsn_step, maxr, st) : cudaSuccess;
@@ -510,8 +513,10 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
            return x;
          })))
       return e;
-    if ((e = tm.run(3, (nsn_step > 0) * (emul ? 2 : 1), [&] {
-           cudaError_t x = psi::launch_per_sn(Kern::DiagFinal, af, sns, nsn_step, st);
+    if ((e = tm.run(3, (nsn_step > 0) * (emul ? 2 : a3.tctr ? 0 : 1), [&] {
+           psi::KArgs ak = af;
+           ak.maxw = maxs;
+           cudaError_t x = a3.tctr ? cudaSuccess : psi::launch_per_sn(Kern::DiagFinal, ak, sns, nsn_step, st);
            if (emul && x == cudaSuccess) x = psi::launch_em_split_x(a, em, sns, nsn_step, st);
            return x;
          })))
@@ -527,15 +532,18 @@ int enqueue_selinv(pselinv_handle* h, int mode, cudaStream_t st, bool record,
       psi::Range r1[psi::kNumVar], r2[psi::kNumVar];
       r1[h->t_gemm1.var[k]] = h->t_gemm1.per_sn[k];
       r2[h->t_gemm2.var[k]] = h->t_gemm2.per_sn[k];
-      if ((rc = step(lsn + pos[k], 1, r1, r2, h->meta[k].ksplit > 1, h->meta[k].r))) return rc;
+      if ((rc = step(lsn + pos[k], 1, r1, r2, h->meta[k].ksplit > 1, h->meta[k].r, h->meta[k].s))) return rc;
     }
   } else {
     for (int32_t l = 0; l < h->nlevels; ++l) {
-      int maxr = 0;
-      for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) maxr = std::max(maxr, h->meta[h->level_sn[t]].r);
+      int maxr = 0, maxs = 0;
+      for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
+        maxr = std::max(maxr, h->meta[h->level_sn[t]].r);
+        maxs = std::max(maxs, h->meta[h->level_sn[t]].s);
+      }
       if ((rc = step(lsn + h->level_ptr[l], h->level_ptr[l + 1] - h->level_ptr[l],
                      &h->t_gemm1.per_lv[(size_t)l * psi::kNumVar], &h->t_gemm2.per_lv[(size_t)l * psi::kNumVar],
-                     h->level_split[l] != 0, maxr)))
+                     h->level_split[l] != 0, maxr, maxs)))
         return rc;
       if (after_level && (rc = (*after_level)(l))) return rc;
     }

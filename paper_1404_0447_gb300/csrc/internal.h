@@ -28,6 +28,7 @@ struct SnMeta {
   int64_t ypart;   // level-local offset of the step-2 partial products (ksplit * r * s)
   int32_t kchunk3; // rows of C per step-3 partial product (nchunk = ceil(r / kchunk3))
   int32_t tctr;    // split step 2: first of this supernode's output-tile counters (per batch member)
+  int32_t t3ctr;   // step 3: counter of its finished tiles
 };
 
 // Where column k of X_{C,C} (k-th row of C) lives: element offset of that
@@ -56,6 +57,8 @@ struct PTask {
   int32_t idx;   // index into the step-2 / step-3 task array, or the supernode
 };
 constexpr int kReduceGroups = 8;  // column groups of one slice reduction
+// Levels of supernodes no wider than this finish step 3 in the CTA of a supernode's last tile.
+constexpr int kFinishWidth = 32;
 constexpr int kFinishParts = 8;   // CTAs (or persistent tasks) sharing one step-3 finish
 
 // Contiguous task ranges [begin, end) for a level and for a supernode.
@@ -158,7 +161,7 @@ struct pselinv_handle {
   std::vector<int32_t> pn1, pn2;     // step-2 / step-3 tiles per supernode
   int64_t panel_total = 0, lhat_total = 0, linv_total = 0, part_max = 0, ypart_max = 0;
   int64_t nnz_l = 0, max_r = 0;
-  int64_t tctr_total = 0;       // output-tile counters of the split step-2 supernodes (per batch member)
+  int64_t tctr_total = 0;       // counters of split step-2 tiles and of step 3 (per batch member)
   int32_t max_width = 0;
   double flops_selinv = 0, flops_gemm1 = 0, bytes_selinv = 0;
 

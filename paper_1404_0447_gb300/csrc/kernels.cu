@@ -8,6 +8,8 @@
 // r x s with ld = r; (L_KK)^{-1} is s x s with ld = s; D holds the pivots.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "block_inverse.cuh"
 #include "bounded_wait.cuh"
 #include "internal.h"
@@ -1012,6 +1014,8 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_gemm2(
   const SnMeta m = a.meta[tk.sn];
   after_previous();
   step3_tile<T, BN>(a, tk, m, blockIdx.y, sm, false);
+  // levels of narrow supernodes: no launch of its own for a finish of a few entries
+  if (a.tctr && last_step3<BN>(a, m, blockIdx.y)) step3_finish<T>(a, m, blockIdx.y, 0, 1, true);
 }
 
 // --------------------------------------------------------------------------
@@ -1304,6 +1308,9 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
                             bool dep) {
   if (nsn <= 0) return cudaSuccess;
   const dim3 grid(nsn, a.sz.batch);
+  // CTAs of a step-3 finish: entries of X_KK (with 32 throughout, 1,291 supernodes of
+  // width ~5 took 43 us) and, for the pole sum, of X_{C,K}
+  const int parts = a.gam ? kFinishCtas : std::max(1, std::min(kFinishCtas, a.maxw * a.maxw / 512));
   switch (k) {
     case Kern::Gemm1Reduce:
       k_gemm1_reduce<T><<<dim3(nsn, a.sz.batch, 16), 256, 0, st>>>(a, sns);
@@ -1315,9 +1322,9 @@ static cudaError_t per_sn_t(Kern k, const KArgs& a, const int32_t* sns, int nsn,
       return launch_dep(k_copyback_bk<T>, dim3(nsn, a.sz.batch, 16), 256, 0, st, dep, a.meta, sns, (T*)a.L,
                         (const T*)a.W, (const T*)a.D, (const T*)a.E, a.ptype, a.sz);
     default:
-      // 32 CTAs per supernode: the levels near the root hold one supernode whose
-      // finish reads one s x s partial per row chunk of C
-      return launch_dep(k_diag_final<T>, dim3(nsn, a.sz.batch, kFinishCtas), 256, 0, st, dep, a, sns);
+      // up to 32 CTAs per supernode: the levels near the root hold one supernode
+      // whose finish reads one s x s partial per row chunk of C
+      return launch_dep(k_diag_final<T>, dim3(nsn, a.sz.batch, parts), 256, 0, st, dep, a, sns);
   }
 }
 

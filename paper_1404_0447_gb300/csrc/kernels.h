@@ -81,7 +81,8 @@ struct KArgs {
   int* status;
   // split step 2: per-output-tile counters (batch x tctr_total, zero between
   // launches); set: the last slice CTA of a tile sums the slices in slice
-  // order and writes X_{C,K} (no separate reduction); nullptr: partials only
+  // order and writes X_{C,K} (no separate reduction); nullptr: partials only.
+  // Step 3: set where the CTA of a supernode's last tile runs the finish
   int* tctr;
   int64_t tctr_n;  // counters per batch member
   Sizes sz;

@@ -175,6 +175,24 @@ __device__ __forceinline__ void step3_tile(const KArgs& a, const Task& tk, const
   });
 }
 
+// Counts a finished step-3 tile of the supernode; true in the CTA that brings the
+// count to all of them (it then runs the finish).  No CTA waits for another.
+template <int BN>
+__device__ __forceinline__ bool last_step3(const KArgs& a, const SnMeta& m, int b) {
+  __shared__ int last;
+  __threadfence();  // this CTA's partial before the count
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int n = m.nchunk * ((m.s + tile_rows<BN>() - 1) / tile_rows<BN>()) * ((m.s + tile_cols<BN>() - 1) / tile_cols<BN>());
+    int* ctr = a.tctr + (int64_t)b * a.tctr_n + m.t3ctr;
+    last = atomicAdd(ctr, 1) == n - 1;
+    if (last) *ctr = 0;
+    __threadfence();
+  }
+  __syncthreads();
+  return last != 0;
+}
+
 // Step 3 finish: X_KK = (Z + Z^T) / 2 with Z = M_K - sum_c P_c (the
 // symmetrisation at the end of Section 2.1 / Algorithm 3).  One thread per
 // unordered pair {i, j} reads and writes exactly (i, j) and (j, i) -- for a

@@ -828,7 +828,7 @@ int build_schedule(pselinv_handle* h) {
             const int32_t ce = std::min(n0 + 8, r);
             for (int32_t m0 = n0; m0 < r; m0 += kMergedRows)
               tm.tasks.push_back({k, m0, n0, (g - g0) << kMergedShift | ce});
-            fits = ((int64_t)tm.tasks.size() - begin) * copies <= kMergedTiles;
+            fits = ((int64_t)tm.tasks.size() - begin) * copies <= (cplx ? kMergedTilesComplex : kMergedTiles);
           }
         }
         h->schur_gcnt[g] = (int32_t)(tm.tasks.size() - gb);

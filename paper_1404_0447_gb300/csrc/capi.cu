@@ -790,6 +790,10 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
     }
     return cudaSuccess;
   };
+  auto merged = [&](int32_t l) {
+    const psi::Range r = h->t_schurm.per_lv[l];
+    return h->schur_merged[l] && (!bk || (r.end - r.begin) * h->opts.batch <= psi::kMergedTilesPivoted);
+  };
   bool hidep = false, lodep = false;  // hi and lo start with a wait on an event
   for (int32_t l = nl - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
@@ -831,8 +835,8 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       dep = false;
       return cudaStreamWaitEvent(s, e, 0);
     };
-    if (h->schur_merged[l]) {  // few tiles: near and far in one launch
-      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+    if (merged(l)) {  // few tiles: near and far in one launch
+      if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       const psi::Range r = h->t_schurm.per_lv[l];
       const int copies = h->opts.batch * f.sides;
       psi::MergedArgs q;
@@ -843,7 +847,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       q.spin_ns = h->opts.spin_limit_ns > 0 ? h->opts.spin_limit_ns : 1000000000LL;
       PSI_CUDA(h, psi::launch_schur_merged(dt, f, q, tasks_at(h, h->off_schurm, r.begin), hi, hidep));
     } else if (h->far_after_near[l]) {
-      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
       PSI_CUDA(h, cudaEventRecord(ev[3 + 2 * nl + l], hi));
       PSI_CUDA(h, wait(lo, ev[3 + 2 * nl + l], lodep));
@@ -854,7 +858,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       PSI_CUDA(h, wait(lo, ev[1 + l], lodep));
       PSI_CUDA(h, schur(h->schur_far, g0, g1, lo, lodep));
       PSI_CUDA(h, cudaEventRecord(ev[1 + nl + l], lo));
-      if (l + 1 < nl && !h->schur_merged[l + 1]) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
+      if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
     }
   }

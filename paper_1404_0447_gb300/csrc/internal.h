@@ -89,7 +89,13 @@ constexpr int fpanel_rows(int w) { return w <= 8 ? 64 : w <= 16 ? 32 : 16; }
 // and the most tiles (all batch members and sides) of a level taken by one.
 constexpr int kMergedRows = 16;
 constexpr int kMergedShift = 20;
-constexpr int64_t kMergedTiles = 8 * 152;
+// Both parts of a larger level as one launch no longer overlap its far part with the
+// next level's panels, so the line lies lower where the panels take longer: complex
+// ones, and pivoted ones, whose diagonal block is one long CTA (measured at 8, 32
+// and 128 tiles per SM: 24^3 log det step 6,373, 6,189, 6,086 us; 200 x 147 grid
+// 1,589, 1,507, 1,506; 4 complex poles 57.06, 57.11, 57.69 ms; indefinite 8,443,
+// 8,556, 8,997 us; 56^3 547.4, 547.4, 548.1 ms).
+constexpr int64_t kMergedTiles = 64 * 152, kMergedTilesComplex = 32 * 152, kMergedTilesPivoted = 8 * 152;
 constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
 // Variants of the tile GEMMs: 64 x (8 << var) for var 0 .. 3, and the fine 16 x 8 tile.

@@ -266,7 +266,9 @@ __global__ void __launch_bounds__(TG_THREADS, (adj_min_ctas<T, BN, OP>())) k_adj
 }
 
 // --------------------------------------------------------------------------
-// per-supernode kernels (one CTA each)
+// per-supernode kernels: gridDim.z CTAs share a supernode's s x s entries (and
+// columns), as many as the widest of the launch keeps busy (adj_parts); one CTA
+// for a 128-wide block took 20-35 us in each of six such kernels of a level
 // --------------------------------------------------------------------------
 
 // Seed of the reverse sweep (all supernodes; blockIdx.x is the supernode).
@@ -281,7 +283,7 @@ __global__ void k_adj_seed(AdjArgs a) {
   const int s = m.s, r = m.r, ld = s + r;
   const T* G = (const T*)a.G + b * sz.panel + m.panel;
   T* Xb = (T*)a.Xb + b * sz.panel + m.panel;
-  for (int j = 0; j < s; ++j)
+  for (int j = blockIdx.z; j < s; j += gridDim.z)
     for (int i = threadIdx.x; i < ld; i += blockDim.x) {
       const int64_t e = i + (int64_t)j * ld;
       T v;
@@ -325,7 +327,7 @@ __global__ void k_adj_zbar(AdjArgs a, const int32_t* __restrict__ sns) {
   const int s = m.s, ld = s + m.r;
   const T* Xb = (const T*)a.Xb + b * sz.panel + m.panel;
   T* Z = (T*)a.Zb + b * sz.linv + m.linv;
-  for (int e = threadIdx.x; e < s * s; e += blockDim.x) {
+  for (int e = threadIdx.x + blockIdx.z * blockDim.x; e < s * s; e += blockDim.x * gridDim.z) {
     const int i = e % s, j = e / s;
     Z[e] = 0.5 * (Xb[i + (int64_t)j * ld] + Xb[j + (int64_t)i * ld]);
   }
@@ -354,12 +356,14 @@ __global__ void k_adj_dr2(AdjArgs a, const int32_t* __restrict__ sns) {
   T* Z = (T*)a.Zb + b * sz.linv + m.linv;
   const T* W = (const T*)a.W1 + b * sz.linv + m.linv;
   T* Db = (T*)a.Db + b * sz.n + m.f;
-  // blockIdx.z of gridDim.z CTAs: columns t = z (mod gridDim.z), entries e in blocks of blockDim.x
+  // one warp per t, lanes along j; entries e in blocks of blockDim.x
   const int zc = blockIdx.z, nz = gridDim.z;
-  for (int t = zc + threadIdx.x * nz; t < s; t += blockDim.x * nz) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nw = blockDim.x / 32;
+  for (int t = zc + warp * nz; t < s; t += nw * nz) {
     T acc = Sc<T>::zero();
-    for (int j = 0; j < s; ++j) acc += W[t + j * s] * V[t + j * s];
-    Db[t] = -(acc / (d[t] * d[t]));
+    for (int j = lane; j < s; j += 32) acc += W[t + j * s] * V[t + j * s];
+    acc = warp_sum(acc);
+    if (lane == 0) Db[t] = -(acc / (d[t] * d[t]));
   }
   for (int e = threadIdx.x + zc * blockDim.x; e < s * s; e += blockDim.x * nz) {
     const int t = e % s;
@@ -386,25 +390,20 @@ __global__ void k_adj_df1(AdjArgs a, const int32_t* __restrict__ sns) {
   T* Db = (T*)a.Db + b * sz.n + m.f;
   const T* Lb = (const T*)a.Lb + b * sz.panel + m.panel;
   T* W = (T*)a.W1 + b * sz.linv + m.linv;
-  __shared__ T colsum[kMaxWidth];
   const T zero = Sc<T>::zero();
   auto R = [&](int i, int j) { return m.nchunk > 0 ? part[i + j * s] : zero; };
   auto Lkk = [&](int i, int j) { return i == j ? Sc<T>::one() : (i > j ? Lp[i + (int64_t)j * ld] : zero); };
-  // blockIdx.z of gridDim.z CTAs: columns t = z (mod gridDim.z), one warp per
-  // column, lanes along the r rows; entries e of W in blocks of blockDim.x
+  // one warp per column t, lanes along the r rows, then along j; entries e of W in
+  // blocks of blockDim.x
   const int zc = blockIdx.z, nz = gridDim.z;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nw = blockDim.x / 32;
   for (int t = zc + warp * nz; t < s; t += nw * nz) {
-    T acc = zero;
+    T acc = zero, acc2 = zero;
     for (int i = lane; i < r; i += 32) acc += Lp[s + i + (int64_t)t * ld] * T1[i + (int64_t)t * r];
+    for (int j = t + lane; j < s; j += 32) acc2 += Lkk(j, t) * R(j, t);
     acc = warp_sum(acc);
-    if (lane == 0) colsum[t] = acc;
-  }
-  __syncthreads();
-  for (int t = zc + threadIdx.x * nz; t < s; t += blockDim.x * nz) {
-    T acc2 = zero;
-    for (int j = t; j < s; ++j) acc2 += Lkk(j, t) * R(j, t);
-    Db[t] = Db[t] - 0.5 * colsum[t] - acc2;
+    acc2 = warp_sum(acc2);
+    if (lane == 0) Db[t] = Db[t] - 0.5 * acc - acc2;
   }
   for (int e = threadIdx.x + zc * blockDim.x; e < s * s; e += blockDim.x * nz) {
     const int i = e % s, j = e / s;
@@ -425,7 +424,7 @@ __global__ void k_adj_ev(AdjArgs a) {
   const T* V = (const T*)a.k.Linv + b * sz.linv + m.linv;
   const T* d = (const T*)a.k.D + b * sz.n + m.f;
   T* EV = (T*)a.W1 + b * sz.linv + m.linv;
-  for (int e = threadIdx.x; e < s * s; e += blockDim.x) EV[e] = V[e] / d[e % s];
+  for (int e = threadIdx.x + blockIdx.z * blockDim.x; e < s * s; e += blockDim.x * gridDim.z) EV[e] = V[e] / d[e % s];
 }
 
 // LDL^T adjoint, last diagonal part: Fb_KK (stored lower) = Ab_ij + Ab_ji
@@ -439,7 +438,7 @@ __global__ void k_adj_df5(AdjArgs a, const int32_t* __restrict__ sns) {
   const int s = m.s, ld = s + m.r;
   const T* Ab = (const T*)a.Zb + b * sz.linv + m.linv;
   T* Fb = (T*)a.Xb + b * sz.panel + m.panel;
-  for (int e = threadIdx.x; e < s * s; e += blockDim.x) {
+  for (int e = threadIdx.x + blockIdx.z * blockDim.x; e < s * s; e += blockDim.x * gridDim.z) {
     const int i = e % s, j = e / s;
     if (i >= j) Fb[i + (int64_t)j * ld] = i == j ? Ab[e] : Ab[e] + Ab[j + i * s];
   }
@@ -493,23 +492,29 @@ cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* t
                                      : adj_tile_t<double>(op, var, a, t, n, st, dep);
 }
 
+// CTAs per supernode of a launch whose widest is w.
+static int adj_parts(int w) { return w * w / 512 < 1 ? 1 : w * w / 512 > 32 ? 32 : w * w / 512; }
+
 template <class T>
-static cudaError_t adj_sn_t(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep) {
+static cudaError_t adj_sn_t(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, int wmax, cudaStream_t st,
+                            bool dep) {
   if (nsn <= 0) return cudaSuccess;
-  const dim3 grid(nsn, a.k.sz.batch), grid8(nsn, a.k.sz.batch, 8);
+  const dim3 grid(nsn, a.k.sz.batch, adj_parts(wmax));
   switch (k) {
     case AdjSn::Seed: k_adj_seed<T><<<grid, 256, 0, st>>>(a); return cudaGetLastError();
     case AdjSn::Ev: return launch_dep(k_adj_ev<T>, grid, 256, 0, st, dep, a);
     case AdjSn::Zbar: return launch_dep(k_adj_zbar<T>, grid, 256, 0, st, dep, a, sns);
-    case AdjSn::Dr2: return launch_dep(k_adj_dr2<T>, grid8, 256, 0, st, dep, a, sns);
-    case AdjSn::Df1: return launch_dep(k_adj_df1<T>, grid8, 256, 0, st, dep, a, sns);
+    case AdjSn::Dr2: return launch_dep(k_adj_dr2<T>, grid, 256, 0, st, dep, a, sns);
+    case AdjSn::Df1: return launch_dep(k_adj_df1<T>, grid, 256, 0, st, dep, a, sns);
     case AdjSn::Df5: return launch_dep(k_adj_df5<T>, grid, 256, 0, st, dep, a, sns);
-    default: return launch_dep(k_adj_sum_parts<T>, grid8, 256, 0, st, dep, a, sns);
+    default: return launch_dep(k_adj_sum_parts<T>, grid, 256, 0, st, dep, a, sns);
   }
 }
 
-cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep) {
-  return a.k.dtype == PSELINV_C128 ? adj_sn_t<Cplx>(k, a, sns, nsn, st, dep) : adj_sn_t<double>(k, a, sns, nsn, st, dep);
+cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, int wmax, cudaStream_t st,
+                              bool dep) {
+  return a.k.dtype == PSELINV_C128 ? adj_sn_t<Cplx>(k, a, sns, nsn, wmax, st, dep)
+                                   : adj_sn_t<double>(k, a, sns, nsn, wmax, st, dep);
 }
 
 }  // namespace psi

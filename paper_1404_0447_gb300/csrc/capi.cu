@@ -1243,6 +1243,10 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
   using psi::AdjSn;
   const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
   const auto* lsn = (const int32_t*)h->d_levelsn;
+  std::vector<int> wmax(h->nlevels, 0);
+  for (int32_t l = 0; l < h->nlevels; ++l)
+    for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t)
+      wmax[l] = std::max(wmax[l], h->meta[h->level_sn[t]].s);
   auto tiles = [&](AdjKern k, const psi::TaskList& tl, int64_t off, int32_t l) -> cudaError_t {
     for (int v = 0; v < psi::kNumVar; ++v) {
       const psi::Range r = tl.per_lv[(size_t)l * psi::kNumVar + v];
@@ -1255,7 +1259,7 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
   for (int32_t l = h->nlevels - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Zbar, a, sns, nsl, st, l + 1 < h->nlevels));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Zbar, a, sns, nsl, wmax[l], st, l + 1 < h->nlevels));
     PSI_CUDA(h, tiles(AdjKern::Ybar, h->t_rect, h->off_rect, l));
     PSI_CUDA(h, tiles(AdjKern::Lhbar, h->t_gemm1, h->off_gemm1, l));  // step-2 slices of C
     // per Schur group, its near and far tiles (adjacent, different target levels) as one launch
@@ -1265,28 +1269,28 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     }
     PSI_CUDA(h, tiles(AdjKern::LbarOff, h->t_rect, h->off_rect, l));
     PSI_CUDA(h, tiles(AdjKern::Vpart, h->t_gemm2, h->off_gemm2, l));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, wmax[l], st));
     // diagonal step: the s x s products as tiles over all supernodes of the level
     PSI_CUDA(h, tiles(AdjKern::Dr1, h->t_sq, h->off_sq, l));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Dr2, a, sns, nsl, st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Dr2, a, sns, nsl, wmax[l], st));
     PSI_CUDA(h, tiles(AdjKern::Dr3, h->t_sq, h->off_sq, l));
     PSI_CUDA(h, tiles(AdjKern::Dr4, h->t_sq, h->off_sq, l));
   }
   // adjoint of the supernodal LDL^T, root -> leaves
   PSI_CUDA(h, cudaMemsetAsync(h->d_xb, 0, B * h->panel_total * es, st));
-  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Ev, a, nullptr, h->nsn, st, false));  // after the memset
+  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Ev, a, nullptr, h->nsn, std::min(h->max_width, 64), st, false));  // after the memset
   for (int32_t l = 0; l < h->nlevels; ++l) {
     const int32_t* sns = lsn + h->level_ptr[l];
     const int nsl = h->level_ptr[l + 1] - h->level_ptr[l];
     PSI_CUDA(h, tiles(AdjKern::T1, h->t_gemm1, h->off_gemm1, l));
     PSI_CUDA(h, tiles(AdjKern::Q, h->t_rect, h->off_rect, l));
     PSI_CUDA(h, tiles(AdjKern::Rpart, h->t_gemm2, h->off_gemm2, l));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, st));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df1, a, sns, nsl, st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, wmax[l], st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df1, a, sns, nsl, wmax[l], st));
     PSI_CUDA(h, tiles(AdjKern::Df2, h->t_sq, h->off_sq, l));
     PSI_CUDA(h, tiles(AdjKern::Df3, h->t_sq, h->off_sq, l));
     PSI_CUDA(h, tiles(AdjKern::Df4, h->t_sq, h->off_sq, l));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df5, a, sns, nsl, st));
+    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df5, a, sns, nsl, wmax[l], st));
   }
   return PSELINV_OK;
 }
@@ -1334,7 +1338,7 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   }
   PSI_CUDA(h, cudaMemsetAsync(h->d_lb, 0, B * h->panel_total * es, st));
   PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));
-  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, st));
+  PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, std::min(h->max_width, 64), st));
   a.G = nullptr;  // read by the seed only
   rc = replay_or_enqueue(h, &h->agraph_exec, &h->adjoint_ran, st,
                          [&](cudaStream_t cs) { return enqueue_adjoint(h, a, cs); });

@@ -270,6 +270,8 @@ enum class AdjKern { Ybar, Lhbar, LbarOff, T1, Q, Vpart, Rpart, Syr2k, Dr1, Dr3,
 enum class AdjSn { Seed, Ev, Zbar, Dr2, Df1, Df5, SumParts };
 cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* tasks, int64_t n, cudaStream_t st,
                              bool dep = true);
-cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, cudaStream_t st, bool dep = true);
+// wmax: the widest supernode of the launch (64 at most where every supernode takes part).
+cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, int wmax, cudaStream_t st,
+                              bool dep = true);
 
 }  // namespace psi

@@ -593,12 +593,12 @@ int build_schedule(pselinv_handle* h) {
     for (int32_t m0 = 0; m0 < m.r; m0 += rows)
       for (int32_t n0 = 0; n0 < m.s; n0 += bn) out.push_back({k, m0, n0, 0});
   };
-  // Normalisation lists (one launch per tile width over all supernodes).  M_K:
-  // 64 x 8 tiles, the lower ones only where the block is symmetric.  Lhat:
-  // least-padding widths when those tiles fill the GPU, else 64 x 8: a 64 x 64
-  // tile of a 128-wide block keeps one SM's FP64 pipe busy for 144 us, and with
-  // fewer tiles than `target` that is the launch's length (200 x 147 grid:
-  // k_lhat 226 us in four widths).
+  // Normalisation lists over all supernodes.  M_K: 64 x 8 tiles, the lower ones only
+  // where the block is symmetric.  Lhat: 64 x 8 tiles, fine ones where there are
+  // few: a 64 x 64 tile of a 128-wide block keeps one SM's FP64 pipe busy for 144
+  // us, and a launch per width ends with one of those (200 x 147 grid: k_lhat 226
+  // us in four widths, 44 now; ten uneven grids: 935 of 15,224 us, now 14,903 in
+  // all); with every supernode in one launch the wide tiles gain nothing (56^3).
   build(h->t_norm, true, [](int32_t) { return 0; }, [&](int32_t k, int rows, int bn, std::vector<Task>& out) {
     const SnMeta& m = h->meta[k];
     for (int32_t m0 = 0; m0 < m.s; m0 += rows)
@@ -606,15 +606,10 @@ int build_schedule(pselinv_handle* h) {
         if (o.unsym || n0 < m0 + rows) out.push_back({k, m0, n0, 0});
   });
   {
-    int64_t nt = 0, nt8 = 0;
-    for (int32_t k = 0; k < nsn; ++k) {
-      const int64_t bn = 8 << by_width(k);
-      nt += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + bn - 1) / bn);
-      nt8 += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + 7) / 8);
-    }
-    const bool narrow = nt < (o.level_tiles > 0 ? o.level_tiles : kTargetTiles);
-    const bool fine = nt8 * o.batch < kFineTiles;
-    build(h->t_lhat, true, [&](int32_t k) { return fine ? kVarFine : narrow ? 0 : by_width(k); }, rect);
+    int64_t nt8 = 0;
+    for (int32_t k = 0; k < nsn; ++k) nt8 += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + 7) / 8);
+    const int var = nt8 * o.batch < kFineTiles ? kVarFine : 0;
+    build(h->t_lhat, true, [&](int32_t) { return var; }, rect);
   }
   // the adjoint's r x s and s x s tile lists: 64 x 8 tiles on levels whose
   // tiles are too few to fill the GPU (as for steps 2 and 3)

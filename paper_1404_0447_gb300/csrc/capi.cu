@@ -198,7 +198,7 @@ int ensure_device(pselinv_handle* h) {
   if ((rc = alloc(h, &h->d_D, B * h->n * es))) return rc;
   if ((rc = alloc(h, &h->d_lhat, B * h->lhat_total * es))) return rc;
   if ((rc = alloc(h, &h->d_linv, B * h->linv_total * es))) return rc;
-  if ((rc = alloc(h, &h->d_status, sizeof(int) * kStatusWords + sizeof(double) * 6 * B))) return rc;
+  if ((rc = alloc(h, &h->d_status, sizeof(int) * kStatusWords + sizeof(double) * (6 + 2 * psi::kLogdetCtas) * B))) return rc;
   if (h->opts.unsym) {
     if ((rc = upload(h, &h->d_flipmap, h->flipmap))) return rc;
     if ((rc = alloc(h, &h->d_U, B * h->panel_total * es))) return rc;
@@ -1222,7 +1222,7 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream) {
   if (!h->factored) return set_err(h, PSELINV_ERR_STATE, "no factor yet");
   cudaStream_t st = (cudaStream_t)stream;
   double* dev = (double*)((int*)h->d_status + kStatusWords);
-  PSI_CUDA(h, psi::launch_logdet(h->opts.dtype, h->d_D, h->n, dev, h->opts.batch, st,
+  PSI_CUDA(h, psi::launch_logdet(h->opts.dtype, h->d_D, h->n, dev + 6 * h->opts.batch, dev, h->opts.batch, st,
                                   h->pivoted ? (const int8_t*)h->d_ptype : nullptr, h->pivoted ? h->d_E : nullptr));
   PSI_CUDA(h, cudaMemcpyAsync(h_out, dev, sizeof(double) * 2 * h->opts.batch, cudaMemcpyDeviceToHost, st));
   int status[kStatusWords];

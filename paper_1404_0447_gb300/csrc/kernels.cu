@@ -1022,16 +1022,34 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_gemm2(
 // log det
 // --------------------------------------------------------------------------
 
-// Real: (sum log|d_j|, number of negative pivots); complex: sum of principal
-// logs (log|d_j|, arg d_j), per batch member.
-template <class T>
-__global__ void k_logdet(const T* __restrict__ D, int64_t n, double* __restrict__ out,
-                         const int8_t* __restrict__ ptype, const T* __restrict__ E) {
+// Sum of two values over the CTA's 256 threads, to thread 0.
+__device__ __forceinline__ void block_sum2(double& a, double& c) {
   __shared__ double s1[256];
   __shared__ double s2[256];
-  const int b = blockIdx.x;
+  s1[threadIdx.x] = a;
+  s2[threadIdx.x] = c;
+  __syncthreads();
+  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) {
+      s1[threadIdx.x] += s1[threadIdx.x + w];
+      s2[threadIdx.x] += s2[threadIdx.x + w];
+    }
+    __syncthreads();
+  }
+  a = s1[0];
+  c = s2[0];
+}
+
+// Real: (sum log|d_j|, number of negative pivots); complex: sum of principal
+// logs (log|d_j|, arg d_j), per batch member (blockIdx.y): partial sums of
+// gridDim.x CTAs, then their sum in a fixed order (k_logdet_sum).  Bound: the
+// logarithms on the FP64 pipe; one CTA took 136 us for n = 13,824.
+template <class T>
+__global__ void k_logdet(const T* __restrict__ D, int64_t n, double* __restrict__ work,
+                         const int8_t* __restrict__ ptype, const T* __restrict__ E) {
+  const int b = blockIdx.y;
   double a = 0.0, c = 0.0;
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+  for (int64_t j = threadIdx.x + (int64_t)blockIdx.x * blockDim.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
     const int8_t ty = ptype ? ptype[b * n + j] : 0;
     if (ty == 2) continue;  // counted with its partner
     // a 2x2 pivot contributes the determinant of its block
@@ -1044,19 +1062,25 @@ __global__ void k_logdet(const T* __restrict__ D, int64_t n, double* __restrict_
       c += atan2(d.im, d.re);
     }
   }
-  s1[threadIdx.x] = a;
-  s2[threadIdx.x] = c;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      s1[threadIdx.x] += s1[threadIdx.x + w];
-      s2[threadIdx.x] += s2[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
+  block_sum2(a, c);
   if (threadIdx.x == 0) {
-    out[2 * b] = s1[0];
-    out[2 * b + 1] = s2[0];
+    double* w = work + 2 * ((int64_t)b * kLogdetCtas + blockIdx.x);
+    w[0] = a;
+    w[1] = c;
+  }
+}
+__global__ void k_logdet_sum(const double* __restrict__ work, int parts, double* __restrict__ out) {
+  const int b = blockIdx.x;
+  const double* w = work + 2 * (int64_t)b * kLogdetCtas;
+  double a = 0.0, c = 0.0;
+  for (int p = threadIdx.x; p < parts; p += blockDim.x) {
+    a += w[2 * p];
+    c += w[2 * p + 1];
+  }
+  block_sum2(a, c);
+  if (threadIdx.x == 0) {
+    out[2 * b] = a;
+    out[2 * b + 1] = c;
   }
 }
 
@@ -1334,12 +1358,16 @@ cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, c
                                  : per_sn_t<double>(k, a, sns, nsn, st, threads, dep);
 }
 
-cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* out, int batch, cudaStream_t st,
+cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* work, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype, const void* E) {
+  const int parts = (int)blocks_for(n, 256, kLogdetCtas);
   if (dtype == PSELINV_C128)
-    k_logdet<Cplx><<<batch, 256, 0, st>>>((const Cplx*)D, n, out, ptype, (const Cplx*)E);
+    k_logdet<Cplx><<<dim3(parts, batch), 256, 0, st>>>((const Cplx*)D, n, work, ptype, (const Cplx*)E);
   else
-    k_logdet<double><<<batch, 256, 0, st>>>((const double*)D, n, out, ptype, (const double*)E);
+    k_logdet<double><<<dim3(parts, batch), 256, 0, st>>>((const double*)D, n, work, ptype, (const double*)E);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_logdet_sum<<<batch, 256, 0, st>>>(work, parts, out);
   return cudaGetLastError();
 }
 

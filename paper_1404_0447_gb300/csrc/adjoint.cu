@@ -29,6 +29,7 @@
 
 #include "internal.h"
 #include "kernels.h"
+#include "merged_update.cuh"
 #include "selinv_steps.cuh"
 #include "tile_gemm.cuh"
 
@@ -265,6 +266,23 @@ __global__ void __launch_bounds__(TG_THREADS, (adj_min_ctas<T, BN, OP>())) k_adj
   }
 }
 
+// A_SYR2K of a whole small level in one launch (merged_update.cuh), on the
+// levels where the factorisation's is merged.  A launch per group before: a gradient
+// on a 20^3 grid 8.99 -> 8.62 ms.
+template <class T>
+__global__ void __launch_bounds__(TG_THREADS) k_syr2k_merged(AdjArgs a, const Task* __restrict__ tasks, MergedArgs mq) {
+  const Sizes& sz = a.k.sz;
+  merged_update<T, 2>(
+      tasks, mq, a.k.meta, a.k.desc, a.k.relidx, 1, a.k.status + kAdjointTimeoutWord,
+      [&](const SnMeta& m, int b, int, int p) {
+        const T* Yb = (const T*)a.Yb + b * sz.lhat + m.lhat;
+        const T* Lh = (const T*)a.k.Lhat + b * sz.lhat + m.lhat;
+        return UpdatePair<T>{p ? Lh : Yb, p ? Yb : Lh, m.r};
+      },
+      [&](int b, int) { return (T*)a.Xb + b * sz.panel; },
+      [](T x, T v, bool diag) { return x + (diag ? -0.5 : -1.0) * v; });
+}
+
 // --------------------------------------------------------------------------
 // per-supernode kernels: gridDim.z CTAs share a supernode's s x s entries (and
 // columns), as many as the widest of the launch keeps busy (adj_parts); one CTA
@@ -490,6 +508,13 @@ cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* t
   const int op = map[(int)k];
   return a.k.dtype == PSELINV_C128 ? adj_tile_t<Cplx>(op, var, a, t, n, st, dep)
                                      : adj_tile_t<double>(op, var, a, t, n, st, dep);
+}
+
+cudaError_t launch_adj_merged(const AdjArgs& a, const MergedArgs& q, const Task* t, cudaStream_t st) {
+  if (q.ntile <= 0) return cudaSuccess;
+  const dim3 grid(q.ntile, a.k.sz.batch);
+  if (a.k.dtype == PSELINV_C128) return launch_dep(k_syr2k_merged<Cplx>, grid, TG_THREADS, 0, st, true, a, t, q);
+  return launch_dep(k_syr2k_merged<double>, grid, TG_THREADS, 0, st, true, a, t, q);
 }
 
 // CTAs per supernode of a launch whose widest is w.

@@ -225,6 +225,18 @@ int64_t merged_counter_bytes(const pselinv_handle* h) {
          (h->nlevels + (int64_t)h->schur_gcnt.size() * h->opts.batch * (h->opts.unsym ? 2 : 1));
 }
 
+psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
+  const int32_t g0 = h->schur_gptr[l];
+  const psi::Range r = h->t_schurm.per_lv[l];
+  psi::MergedArgs q;
+  q.ticket = (int*)h->d_mctr + l;
+  q.gcnt = (const int32_t*)h->d_gcnt + g0;
+  q.done = (int*)h->d_mctr + h->nlevels + (int64_t)g0 * h->opts.batch * (h->opts.unsym ? 2 : 1);
+  q.ntile = (int)(r.end - r.begin);
+  q.spin_ns = h->opts.spin_limit_ns > 0 ? h->opts.spin_limit_ns : 1000000000LL;
+  return q;
+}
+
 // Upload the tuning-dependent part (metadata, task lists, partial buffers);
 // called again by the autotuner after build_schedule.
 int upload_schedule(pselinv_handle* h) {
@@ -838,13 +850,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
     if (merged(l)) {  // few tiles: near and far in one launch
       if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       const psi::Range r = h->t_schurm.per_lv[l];
-      const int copies = h->opts.batch * f.sides;
-      psi::MergedArgs q;
-      q.ticket = (int*)h->d_mctr + l;
-      q.gcnt = (const int32_t*)h->d_gcnt + g0;
-      q.done = (int*)h->d_mctr + nl + (int64_t)g0 * copies;
-      q.ntile = (int)(r.end - r.begin);
-      q.spin_ns = h->opts.spin_limit_ns > 0 ? h->opts.spin_limit_ns : 1000000000LL;
+      const psi::MergedArgs q = merged_args(h, l);
       PSI_CUDA(h, psi::launch_schur_merged(dt, f, q, tasks_at(h, h->off_schurm, r.begin), hi, hidep));
     } else if (h->far_after_near[l]) {
       if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
@@ -1087,6 +1093,11 @@ int pselinv_sync_status(pselinv_handle* h, void* stream) {
     if (rc) return rc;
   }
   if (const int rc = factor_timeout(h, status)) return rc;
+  if (status[psi::kAdjointTimeoutWord]) {
+    PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + psi::kAdjointTimeoutWord, 0, sizeof(int), st));
+    PSI_CUDA(h, cudaStreamSynchronize(st));
+    return set_err(h, PSELINV_ERR_TIMEOUT, "a bounded device wait of the adjoint ran out; that gradient is invalid");
+  }
   if (status[2]) {
     PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, 2 * sizeof(int), st));
     PSI_CUDA(h, cudaStreamSynchronize(st));
@@ -1255,6 +1266,7 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     }
     return cudaSuccess;
   };
+  PSI_CUDA(h, cudaMemsetAsync(h->d_mctr, 0, merged_counter_bytes(h), st));
   // reverse sweep of the selected inversion, leaves -> root
   for (int32_t l = h->nlevels - 1; l >= 0; --l) {
     const int32_t* sns = lsn + h->level_ptr[l];
@@ -1262,8 +1274,11 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Zbar, a, sns, nsl, wmax[l], st, l + 1 < h->nlevels));
     PSI_CUDA(h, tiles(AdjKern::Ybar, h->t_rect, h->off_rect, l));
     PSI_CUDA(h, tiles(AdjKern::Lhbar, h->t_gemm1, h->off_gemm1, l));  // step-2 slices of C
-    // per Schur group, its near and far tiles (adjacent, different target levels) as one launch
-    for (int32_t g = h->schur_gptr[l]; g < h->schur_gptr[l + 1]; ++g) {
+    if (h->schur_merged[l])
+      PSI_CUDA(h, psi::launch_adj_merged(a, merged_args(h, l), tasks_at(h, h->off_schurm, h->t_schurm.per_lv[l].begin),
+                                         st));
+    // otherwise per Schur group, its near and far tiles (adjacent, different target levels) as one launch
+    for (int32_t g = h->schur_merged[l] ? h->schur_gptr[l + 1] : h->schur_gptr[l]; g < h->schur_gptr[l + 1]; ++g) {
       const int64_t b0 = h->schur_near[g].begin, b1 = h->schur_far[g].end;
       PSI_CUDA(h, psi::launch_adj_tiles(AdjKern::Syr2k, h->schur_gvar[g], a, tasks_at(h, h->off_schur, b0), b1 - b0, st));
     }

@@ -11,9 +11,9 @@
 #include <algorithm>
 
 #include "block_inverse.cuh"
-#include "bounded_wait.cuh"
 #include "internal.h"
 #include "kernels.h"
+#include "merged_update.cuh"
 #include "selinv_steps.cuh"
 #include "tile_gemm.cuh"
 
@@ -779,93 +779,17 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
   });
 }
 
-// The Schur updates of a whole level in one launch: the tiles of all its groups,
-// 16 x 8, in group order.  Targets of different groups overlap, so a tile's
-// read-modify-write waits until the groups before its own have finished (same
-// order per target as a launch per group, so the same bits); the products do not
-// wait.  CTAs take their tile by a ticket: the holder of a tile only waits on
-// tiles with lower tickets, which running CTAs hold, and those of the lowest
-// group wait on nothing, so the waits end whatever else is resident; each is
-// bounded in time all the same (bounded_wait.cuh).
-// Warp w computes the k range [w kq, (w + 1) kq) of the tile from fragments loaded
-// straight to registers; the four partial sums are added in warp order.
-// Bound: latency (loads, at most 16 MMAs a warp, the group order).
+// The Schur updates of a whole small level in one launch (merged_update.cuh),
+// operands and targets as in k_schur.
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_schur_merged(FArgs f, const Task* __restrict__ tasks, MergedArgs mq) {
-  constexpr int P = Sc<T>::P, RF = kMergedRows / 8, LDP = kMergedRows + 1;
-  __shared__ double part[4][P][8][LDP];
-  __shared__ int sh_ticket;
-  if (threadIdx.x == 0) sh_ticket = atomicAdd(mq.ticket, 1);  // zeroed long before the previous kernel
-  __syncthreads();
-  const int ticket = sh_ticket, copies = gridDim.y, copy = ticket % copies;
-  const Task tk = tasks[ticket / copies];
-  const int side = copy % f.sides, b = copy / f.sides;
-  const int grp = tk.c >> kMergedShift, cend = tk.c & ((1 << kMergedShift) - 1);
-  const SnMeta m = f.meta[tk.sn];
-  const int s = m.s, r = m.r, ld = s + r;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, q = lane & 3;
-  // this thread's entry of the tile and its target
-  const int ei = tk.m0 + t % kMergedRows, ec = tk.n0 + t / kMergedRows;
-  const bool live = ei < r && ec < cend && ec + side <= ei;
-  T* dst = nullptr;
-  if (live) {
-    const ColDesc cd = f.desc[m.desc + ec];
-    dst = (T*)f.L[side] + b * f.sz.panel + cd.col + f.relidx[cd.rel + ei];
-  }
-  const int need = grp > 0 ? mq.gcnt[grp - 1] : 0;
-  after_previous();
-  const int64_t po = b * f.sz.panel + m.panel + s;
-  const T* B = (const T*)f.L[f.sides - 1 - side] + po;
-  const T* W = (const T*)f.W[side] + po;
-  double acc[RF][P][2] = {};
-  const int kq = (s + 15) / 16 * 4, k0 = warp * kq, k1 = min(s, k0 + kq);  // at most 32
-  if (k0 < k1) {
-    T a[RF][kFB / 4], bf[kFB / 4];
-#pragma unroll
-    for (int u = 0; u < kFB / 4; ++u) {
-      const int k = k0 + 4 * u + q;
-      const bool on = k < k1;
-      bf[u] = on && tk.n0 + g < cend ? B[tk.n0 + g + (int64_t)k * ld] : Sc<T>::zero();
-#pragma unroll
-      for (int h = 0; h < RF; ++h) {
-        const int row = tk.m0 + 8 * h + g;
-        a[h][u] = on && row < r ? W[row + (int64_t)k * ld] : Sc<T>::zero();
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < RF; ++h) {
-      if (tk.m0 + 8 * h >= r) continue;
-#pragma unroll
-      for (int u = 0; u < kFB / 4; ++u)
-        if (k0 + 4 * u < k1) frag_mma<T, 1>(acc[h], a[h] + u, bf + u);
-    }
-  }
-#pragma unroll
-  for (int h = 0; h < RF; ++h)
-#pragma unroll
-    for (int p = 0; p < P; ++p)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) part[warp][p][2 * q + e][8 * h + g] = acc[h][p][e];
-  __syncthreads();
-  double v[P];
-#pragma unroll
-  for (int p = 0; p < P; ++p) {
-    v[p] = part[0][p][t / kMergedRows][t % kMergedRows];
-#pragma unroll
-    for (int w = 1; w < 4; ++w) v[p] += part[w][p][t / kMergedRows][t % kMergedRows];
-  }
-  if (grp > 0 && !cta_wait(mq.done + (int64_t)(grp - 1) * copies + copy, need, mq.spin_ns,
-                           f.status + kFactorTimeoutWord, 20))
-    return;
-  if (live) {
-    T x = ld_cg(dst);
-    if constexpr (P == 1)
-      x -= v[0];
-    else
-      x -= T{v[0], v[1]};
-    *dst = x;
-  }
-  cta_signal(mq.done + (int64_t)grp * copies + copy);
+  merged_update<T, 1>(
+      tasks, mq, f.meta, f.desc, f.relidx, f.sides, f.status + kFactorTimeoutWord,
+      [&](const SnMeta& m, int b, int side, int) {
+        const int64_t po = b * f.sz.panel + m.panel + m.s;
+        return UpdatePair<T>{(const T*)f.W[side] + po, (const T*)f.L[f.sides - 1 - side] + po, m.s + m.r};
+      },
+      [&](int b, int side) { return (T*)f.L[side] + b * f.sz.panel; }, [](T x, T v, bool) { return x - v; });
 }
 
 // Normalisation, diagonal part: M_K = L_KK^{-T} D_K^{-1} L_KK^{-1} = V^T (D_K^{-1} V)

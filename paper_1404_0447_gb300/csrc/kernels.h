@@ -125,9 +125,9 @@ struct FArgs {
   int sides;
 };
 enum class FKern { Panel, Update, VInv, Schur };
-// Status word set when a wait of a merged Schur launch ran out.
-constexpr int kFactorTimeoutWord = 5;
-// One merged Schur launch (k_schur_merged): the level's ticket, and for the
+// Status words set when a wait of a merged launch ran out.
+constexpr int kFactorTimeoutWord = 5, kAdjointTimeoutWord = 6;
+// One merged launch (merged_update.cuh): the level's ticket, and for the
 // level's first group on the tiles per group and the finished tiles per (group,
 // copy), copy = side and batch member.
 struct MergedArgs {
@@ -272,6 +272,7 @@ enum class AdjKern { Ybar, Lhbar, LbarOff, T1, Q, Vpart, Rpart, Syr2k, Dr1, Dr3,
 enum class AdjSn { Seed, Ev, Zbar, Dr2, Df1, Df5, SumParts };
 cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* tasks, int64_t n, cudaStream_t st,
                              bool dep = true);
+cudaError_t launch_adj_merged(const AdjArgs& a, const MergedArgs& q, const Task* t, cudaStream_t st);
 // wmax: the widest supernode of the launch (64 at most where every supernode takes part).
 cudaError_t launch_adj_per_sn(AdjSn k, const AdjArgs& a, const int32_t* sns, int nsn, int wmax, cudaStream_t st,
                               bool dep = true);

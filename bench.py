@@ -422,7 +422,7 @@ def run_ours(args):
         fms.append(e0.elapsed_time(e1))
     h.sync_status(stream=stream)
     f_med = statistics.median(fms)
-    factor_block = {"bound": "tensor", "kernel": "pselinv_factor: k_factor_diag, k_trsm, k_copyback, k_schur "
+    factor_block = {"bound": "tensor", "kernel": "pselinv_factor: k_fdiag, k_fpanel, k_fupdate, k_schur "
                                                 "(FP64 mma.sync m8n8k4) per level, Schur updates in groups "
                                                 "with disjoint targets (no atomics)",
                     "flops": fl_factor, "ms_stats": stats(fms), "achieved": fl_factor / (f_med * 1e-3) / 1e12,

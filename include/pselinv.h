@@ -80,7 +80,9 @@ extern "C" {
 
 /* selected-inversion schedules (Algorithm 3 and Section 3.3) */
 #define PSELINV_PLAIN 0 /* one supernode per launch, reverse postorder */
-#define PSELINV_LEVEL 1 /* one grouped launch per kernel per level of Algorithm 2 */
+#define PSELINV_LEVEL 1 /* one grouped launch per kernel per level of Algorithm 2; from the second
+                           call on replayed from a graph (not while the caller captures `stream` or
+                           times kernels) */
 #define PSELINV_GRAPH 2 /* the LEVEL sequence captured once into a CUDA graph and replayed */
 #define PSELINV_PERSISTENT 3 /* one persistent launch for the whole sweep running every level's work
                                 from one task list with bounded dependency waits and no barrier
@@ -236,12 +238,15 @@ int pselinv_analyze_batch(int32_t k, const int64_t* h_n, const int64_t* const* h
 /*
  * Numeric factorisation A = L D L^T on the device (supernodal, level by
  * level from the leaves; no pivoting, Section 4); it produces the input of
- * the selected inversion.  Per level: the diagonal blocks, the panel solves,
- * then the Schur updates of the ancestors in groups of supernodes whose
- * update targets are disjoint (fixed order, no atomics): L and D, and so X,
- * are bitwise reproducible from run to run.  The handle's X panels serve as
- * scratch (the panel solve's L_{C,K} D_K): a selected inverse computed before
- * is gone.
+ * the selected inversion.  Per level: the panels, 32 columns at a time, then
+ * the Schur updates of the ancestors in groups of supernodes whose update
+ * targets are disjoint (fixed order, no atomics on values): L and D, and so X,
+ * are bitwise reproducible from run to run.  On small levels one launch runs
+ * all groups and orders them by bounded waits (opts.spin_limit_ns).  The
+ * handle's X panels serve as scratch (L_KK D_K below its diagonal 32 x 32
+ * blocks and L_{C,K} D_K): a selected inverse computed before is gone.  From
+ * the second call on the launches are replayed from a graph, unless `stream`
+ * is being captured by the caller.
  *
  * d_values   device, batch x nnz_a values of A's lower CSC in the user's
  *            order (dtype of the handle)
@@ -250,7 +255,8 @@ int pselinv_analyze_batch(int32_t k, const int64_t* h_n, const int64_t* const* h
  * order) and reported by the next pselinv_sync_status or pselinv_logdet as
  * ERR_ZERO_PIVOT / ERR_NONFINITE (message via pselinv_last_error), which
  * also returns the handle to the unfactored state; a selinv enqueued before
- * that check computes with the bad factor.  Errors returned directly:
+ * that check computes with the bad factor.  A wait that ran out is reported
+ * the same way as ERR_TIMEOUT.  Errors returned directly:
  * ERR_ARG, ERR_STATE, ERR_OOM, ERR_CUDA.
  */
 int pselinv_factor(pselinv_handle* h, const void* d_values, void* stream);
@@ -355,9 +361,10 @@ int pselinv_get_panels(pselinv_handle* h, int32_t which, void* out, void* stream
  * work on h: PSELINV_ERR_ZERO_PIVOT / PSELINV_ERR_NONFINITE if the last
  * factorisation met a bad pivot (first column, internal order; reported
  * until the next factorisation, the handle is back to "not factored"),
- * PSELINV_ERR_TIMEOUT if a bounded wait of the PERSISTENT schedule ran out
- * (that call's results are invalid; the flag is cleared and the handle stays
- * usable), PSELINV_ERR_RANGE if a selinv with opts.fp64_emulation met an X
+ * PSELINV_ERR_TIMEOUT if a bounded wait of the factorisation ran out (until
+ * the next factorisation, the handle is back to "not factored"), or one of the
+ * PERSISTENT schedule or of the adjoint (that call's results are invalid; the
+ * flag is cleared and the handle stays usable), PSELINV_ERR_RANGE if a selinv with opts.fp64_emulation met an X
  * that is not positive definite (same treatment).  Returns PSELINV_OK
  * otherwise.
  */
@@ -461,7 +468,7 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream);
  *            function whose output is the X panels
  * d_gradA  device, batch x nnz_a
  * Requires a prior pselinv_selinv on the same factor (uses X, L, D;
- * recomputes Lhat and (L_KK)^{-1}).  Reverse sweep leaves -> root of the
+ * recomputes Lhat from the factor).  Reverse sweep leaves -> root of the
  * recurrence of Algorithm 1 (steps 3, 2, 1 in that order per supernode,
  * scattering into the ancestors' adjoints through the relative indices, in
  * the factorisation's groups of supernodes with disjoint targets: no
@@ -477,12 +484,13 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
  * Kernel timing of the selected inversion (measurement support, no paper
  * counterpart beyond Section 4.2's per-phase timings).  enable != 0 makes
  * every later pselinv_selinv in PLAIN or LEVEL mode record CUDA events on
- * its stream around each kernel class; pselinv_get_timing waits for them
+ * its stream around each kernel class (launched one by one, not replayed from
+ * a graph); pselinv_get_timing waits for them
  * and returns in h_ms[PSELINV_NTIMERS] the summed milliseconds since the
  * previous pselinv_get_timing (or enable), in h_launches[PSELINV_NTIMERS]
  * the kernel launches per class, and resets both.  GRAPH mode does not
  * record.  Classes:
- *   0 normalisation (diagonal inverses, Lhat)   1 step 2 (X_{C,K})
+ *   0 normalisation (M_K, Lhat)                 1 step 2 (X_{C,K})
  *   2 step 3 partial products                    3 step 3 finish (symmetrise)
  */
 #define PSELINV_NTIMERS 4
@@ -501,7 +509,7 @@ int pselinv_get_timing(pselinv_handle* h, double* h_ms, int64_t* h_launches);
  * h_best[0] = split_k_rows, h_best[1] = small_cutoff, h_best[2] =
  * level_tiles, h_best[3] = the fastest mode (h_best holds 4 entries) and
  * that mode's time in *h_best_ms.
- * Overwrites the X panels; drops a captured GRAPH schedule.  Synchronises.
+ * Overwrites the X panels; drops captured graphs.  Synchronises.
  */
 int pselinv_autotune(pselinv_handle* h, int32_t* h_best, double* h_best_ms, void* stream);
 

@@ -315,24 +315,15 @@ __global__ void k_adj_seed(AdjArgs a) {
     }
 }
 
-// Step-3 chunk partials of a supernode summed in chunk order into chunk 0
-// (VPART before the reverse diagonal step, RPART before the factor one);
-// blockIdx.z selects one of gridDim.z CTAs sharing the s x s entries.
+// Entry e of a supernode's step-3 chunk partials (VPART, RPART) summed in chunk
+// order.  The elementwise kernels sum while they read; a pass of its own cost 6 us
+// a level and sweep.
 template <class T>
-__global__ void k_adj_sum_parts(AdjArgs a, const int32_t* __restrict__ sns) {
-  const int k = sns[blockIdx.x], b = blockIdx.y;
-  const Sizes sz = a.k.sz;
-  const SnMeta m = a.k.meta[k];
-  after_previous();
-  if (m.nchunk < 2) return;
-  const int s = m.s;
-  T* part = (T*)a.k.part + b * sz.part + m.part;
-  const int64_t ss = (int64_t)s * s;
-  for (int64_t e = threadIdx.x + (int64_t)blockIdx.z * blockDim.x; e < ss; e += (int64_t)gridDim.z * blockDim.x) {
-    T acc = part[e];
-    for (int c = 1; c < m.nchunk; ++c) acc += part[c * ss + e];
-    part[e] = acc;
-  }
+__device__ __forceinline__ T chunk_sum(const T* part, int nchunk, int64_t ss, int64_t e) {
+  T acc = nchunk > 0 ? part[e] : Sc<T>::zero();
+#pragma unroll 4
+  for (int c = 1; c < nchunk; ++c) acc += part[c * ss + e];
+  return acc;
 }
 
 // Zb = (Xb_KK + Xb_KK^T) / 2 for the supernodes of a level.
@@ -386,7 +377,7 @@ __global__ void k_adj_dr2(AdjArgs a, const int32_t* __restrict__ sns) {
   for (int e = threadIdx.x + zc * blockDim.x; e < s * s; e += blockDim.x * nz) {
     const int t = e % s;
     T vb = 2.0 * W[e] / d[t];
-    if (m.nchunk > 0) vb += part[e];  // chunk partials already summed into chunk 0
+    if (m.nchunk > 0) vb += chunk_sum(part, m.nchunk, (int64_t)s * s, e);
     Z[e] = vb;
   }
 }
@@ -409,7 +400,7 @@ __global__ void k_adj_df1(AdjArgs a, const int32_t* __restrict__ sns) {
   const T* Lb = (const T*)a.Lb + b * sz.panel + m.panel;
   T* W = (T*)a.W1 + b * sz.linv + m.linv;
   const T zero = Sc<T>::zero();
-  auto R = [&](int i, int j) { return m.nchunk > 0 ? part[i + j * s] : zero; };
+  auto R = [&](int i, int j) { return chunk_sum(part, m.nchunk, (int64_t)s * s, i + j * s); };
   auto Lkk = [&](int i, int j) { return i == j ? Sc<T>::one() : (i > j ? Lp[i + (int64_t)j * ld] : zero); };
   // one warp per column t, lanes along the r rows, then along j; entries e of W in
   // blocks of blockDim.x
@@ -531,8 +522,7 @@ static cudaError_t adj_sn_t(AdjSn k, const AdjArgs& a, const int32_t* sns, int n
     case AdjSn::Zbar: return launch_dep(k_adj_zbar<T>, grid, 256, 0, st, dep, a, sns);
     case AdjSn::Dr2: return launch_dep(k_adj_dr2<T>, grid, 256, 0, st, dep, a, sns);
     case AdjSn::Df1: return launch_dep(k_adj_df1<T>, grid, 256, 0, st, dep, a, sns);
-    case AdjSn::Df5: return launch_dep(k_adj_df5<T>, grid, 256, 0, st, dep, a, sns);
-    default: return launch_dep(k_adj_sum_parts<T>, grid, 256, 0, st, dep, a, sns);
+    default: return launch_dep(k_adj_df5<T>, grid, 256, 0, st, dep, a, sns);
   }
 }
 

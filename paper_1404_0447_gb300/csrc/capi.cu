@@ -1297,9 +1297,8 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     PSI_CUDA(h, cudaStreamWaitEvent(lo, ev[l], 0));
     PSI_CUDA(h, tiles(AdjKern::LbarOff, h->t_rect, h->off_rect, l, lo, false));  // after the wait
     PSI_CUDA(h, tiles(AdjKern::Vpart, h->t_gemm2, h->off_gemm2, l, lo, false));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, wmax[l], lo, false));
     // diagonal step: the s x s products as tiles over all supernodes of the level
-    PSI_CUDA(h, tiles(AdjKern::Dr1, h->t_sq, h->off_sq, l, lo));
+    PSI_CUDA(h, tiles(AdjKern::Dr1, h->t_sq, h->off_sq, l, lo, false));
     PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Dr2, a, sns, nsl, wmax[l], lo));
     PSI_CUDA(h, tiles(AdjKern::Dr3, h->t_sq, h->off_sq, l, lo));
     PSI_CUDA(h, tiles(AdjKern::Dr4, h->t_sq, h->off_sq, l, lo));
@@ -1317,7 +1316,6 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     PSI_CUDA(h, tiles(AdjKern::T1, h->t_gemm1, h->off_gemm1, l, st));
     PSI_CUDA(h, tiles(AdjKern::Q, h->t_rect, h->off_rect, l, st));
     PSI_CUDA(h, tiles(AdjKern::Rpart, h->t_gemm2, h->off_gemm2, l, st));
-    PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::SumParts, a, sns, nsl, wmax[l], st));
     PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Df1, a, sns, nsl, wmax[l], st));
     PSI_CUDA(h, tiles(AdjKern::Df2, h->t_sq, h->off_sq, l, st));
     PSI_CUDA(h, tiles(AdjKern::Df3, h->t_sq, h->off_sq, l, st));

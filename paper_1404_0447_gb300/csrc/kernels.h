@@ -269,7 +269,7 @@ struct AdjArgs {
   void* Hb;       // r x s per supernode: Lhat-bar
 };
 enum class AdjKern { Ybar, Lhbar, LbarOff, T1, Q, Vpart, Rpart, Syr2k, Dr1, Dr3, Dr4, Df2, Df3, Df4 };
-enum class AdjSn { Seed, Ev, Zbar, Dr2, Df1, Df5, SumParts };
+enum class AdjSn { Seed, Ev, Zbar, Dr2, Df1, Df5 };
 cudaError_t launch_adj_tiles(AdjKern k, int var, const AdjArgs& a, const Task* tasks, int64_t n, cudaStream_t st,
                              bool dep = true);
 cudaError_t launch_adj_merged(const AdjArgs& a, const MergedArgs& q, const Task* t, cudaStream_t st);

@@ -105,7 +105,8 @@ typedef struct {
                              A = L D U' (pselinv_factor_unsym; Algorithm 1 with step 4); complex
                              non-symmetric handles cap w_max at 112 (shared-memory budget of the
                              diagonal-block factorisation) */
-  int64_t spin_limit_ns;  /* limit for bounded device waits; <= 0 = 1e9 */
+  int64_t spin_limit_ns;  /* limit for bounded device waits; <= 0 = 1e9 (waits inside a factorisation or
+                             an adjoint: at least 1e9) */
   int32_t level_tiles;    /* a level whose step-2 (step-3) tiles number fewer than this gets its slices
                              (row chunks) of C shrunk until it has about this many; 0 = 128 per SM (19456) */
   int32_t min_slice_rows; /* smallest step-2 slice that shrinking makes; 0 = 128 (step-3 chunks: a quarter) */
@@ -242,7 +243,7 @@ int pselinv_analyze_batch(int32_t k, const int64_t* h_n, const int64_t* const* h
  * the Schur updates of the ancestors in groups of supernodes whose update
  * targets are disjoint (fixed order, no atomics on values): L and D, and so X,
  * are bitwise reproducible from run to run.  On small levels one launch runs
- * all groups and orders them by bounded waits (opts.spin_limit_ns).  The
+ * all groups and orders them by bounded waits (opts.spin_limit_ns, at least 1 s).  The
  * handle's X panels serve as scratch (L_KK D_K below its diagonal 32 x 32
  * blocks and L_{C,K} D_K): a selected inverse computed before is gone.  From
  * the second call on the launches are replayed from a graph, unless `stream`

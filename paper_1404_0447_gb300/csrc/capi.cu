@@ -233,7 +233,9 @@ psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
   q.gcnt = (const int32_t*)h->d_gcnt + g0;
   q.done = (int*)h->d_mctr + h->nlevels + (int64_t)g0 * h->opts.batch * (h->opts.unsym ? 2 : 1);
   q.ntile = (int)(r.end - r.begin);
-  q.spin_ns = h->opts.spin_limit_ns > 0 ? h->opts.spin_limit_ns : 1000000000LL;
+  // at least a second, also where the persistent schedule's limit is shorter: a wait
+  // lasts as long as the tiles before it, whatever limit the caller chose for a sweep
+  q.spin_ns = std::max<long long>(h->opts.spin_limit_ns, 1000000000LL);
   return q;
 }
 

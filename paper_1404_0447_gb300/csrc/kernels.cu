@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
 // A_ij -= sum_k W_ik L_jk over the block's 32 columns k, rows i >= j of the
 // whole panel (i > j on the U side), each entry by one thread; one warp per
 // 8 x 8 fragment of a 16 x 8 tile, operands straight to registers (see k_fpanel).
+// Bound: latency near the root, 8 us a step (staged 64 x 8 tiles 8.5).
 constexpr int kFUpdateThreads = 4 * kFUpdateRows;
 template <class T>
 __global__ void __launch_bounds__(kFUpdateThreads) k_fupdate(FArgs f, const Task* __restrict__ tasks) {
@@ -338,7 +339,9 @@ __global__ void __launch_bounds__(kFUpdateThreads) k_fupdate(FArgs f, const Task
 
 // (L_KK)^{-1} off its 32 x 32 diagonal blocks, all supernodes wider than 32 of the
 // task list at once (pivot-free: after the last level): one strip of 8 columns
-// (task n0) per CTA; blockIdx.z = side.
+// (task n0) per CTA; blockIdx.z = side.  Bound: the chain of a strip's blocks, 54 us
+// for all supernodes of a 33 x 29 x 27 grid (inside the level loop, with the block on
+// one SM, (L_KK)^{-1} was most of the 345 us of a 128-wide block).
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_vinv(FArgs f, const Task* __restrict__ tasks) {
   __shared__ VsSmem<T> sm;
@@ -780,7 +783,11 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
 }
 
 // The Schur updates of a whole small level in one launch (merged_update.cuh),
-// operands and targets as in k_schur.
+// operands and targets as in k_schur.  A launch per group and part cost 3 to 5 us
+// however few tiles it held (31 x 31 grid, 103 launches: 590 -> 537 us).  Larger
+// levels keep a launch per group: ordered the same way on their 64 x 8 tiles they
+// gave 0.2 to 0.4% on wide supernodes and lost 2 to 3% on narrow ones, whose short
+// tiles feel the ticket and hold their slots while the group before ends.
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_schur_merged(FArgs f, const Task* __restrict__ tasks, MergedArgs mq) {
   merged_update<T, 1>(

@@ -727,7 +727,7 @@ int ensure_factor_streams(pselinv_handle* h) {
     PSI_CUDA(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     h->fev.push_back(e);
   }
-  if (h->far_after_near.empty()) {
+  if (h->far_after_near[0].empty()) {
     // Per level l: does far(l) wait for near(l), so that level l - 1's panels
     // start beside it?  The pivot chain of a diagonal block and the panel tiles
     // run several times slower beside resident Schur tiles (one FP64 pipe per
@@ -735,7 +735,11 @@ int ensure_factor_streams(pselinv_handle* h) {
     // when far(l) is short against the next level's panels (model: FP64 work at
     // 1 TFLOP/s; 30 us per 32 columns of the widest supernode).
     const int32_t nl = h->nlevels;
-    std::vector<double> t_far(nl, 0.0), t_next(nl, 0.0);
+    // The pivoted panels take longer: 345 us (w / 128)^3 + 30 us for the diagonal
+    // block (one CTA), no blocks of columns (pivoted 40^3 34.6 -> 33.0 ms, 24^3 and
+    // 80^3 the same within 0.2%).
+    std::vector<double> t_far(nl, 0.0), t_next[2];
+    for (auto& t : t_next) t.assign(nl, 0.0);
     for (int32_t l = 0; l < nl; ++l) {
       double far = 0.0, solve = 0.0;
       int wmax = 0;
@@ -746,10 +750,14 @@ int ensure_factor_streams(pselinv_handle* h) {
         wmax = std::max(wmax, m.s);
       }
       t_far[l] = far / 1e12;
-      t_next[l] = 30e-6 * ((wmax + psi::kFactorBlock - 1) / psi::kFactorBlock) + solve / 1e12;
+      const double w = wmax / 128.0;
+      t_next[0][l] = 30e-6 * ((wmax + psi::kFactorBlock - 1) / psi::kFactorBlock) + solve / 1e12;
+      t_next[1][l] = 345e-6 * w * w * w + 30e-6 + solve / 1e12;
     }
-    h->far_after_near.assign(nl, 0);
-    for (int32_t l = 1; l < nl; ++l) h->far_after_near[l] = t_far[l] < 4.0 * t_next[l - 1];
+    for (int bk = 0; bk < 2; ++bk) {
+      h->far_after_near[bk].assign(nl, 0);
+      for (int32_t l = 1; l < nl; ++l) h->far_after_near[bk][l] = t_far[l] < 4.0 * t_next[bk][l - 1];
+    }
   }
   return PSELINV_OK;
 }
@@ -854,7 +862,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
       const psi::Range r = h->t_schurm.per_lv[l];
       const psi::MergedArgs q = merged_args(h, l);
       PSI_CUDA(h, psi::launch_schur_merged(dt, f, q, tasks_at(h, h->off_schurm, r.begin), hi, hidep));
-    } else if (h->far_after_near[l]) {
+    } else if (h->far_after_near[bk][l]) {
       if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       PSI_CUDA(h, schur(h->schur_near, g0, g1, hi, hidep));
       PSI_CUDA(h, cudaEventRecord(ev[3 + 2 * nl + l], hi));

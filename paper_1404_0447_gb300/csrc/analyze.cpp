@@ -543,9 +543,9 @@ int build_schedule(pselinv_handle* h) {
         h->trvar[k] = (int8_t)(ttf < target ? 0 : pick_variant(h->meta[k].s, cplx, o.small_cutoff));
         // fewer 64 x 8 tiles than ~8 per SM: fine tiles, where k is longer than one of their
         // warps takes (level with |C| <= 32: step 2 4.2 us on 64 x 8 tiles, 7.6 on fine ones)
-        if (t2n * o.batch < kFineTiles && rmax > 32 && !o.fp64_emulation) h->s2var[k] = kVarFine;
-        if (t3n * o.batch < kFineTiles && rmax > 32 && !o.fp64_emulation) h->s3var[k] = kVarFine;
-        if (ttn * o.batch < kFineTiles) h->trvar[k] = kVarFine;
+        if (t2n < kFineTiles && rmax > 32 && !o.fp64_emulation) h->s2var[k] = kVarFine;
+        if (t3n < kFineTiles && rmax > 32 && !o.fp64_emulation) h->s3var[k] = kVarFine;
+        if (ttn < kFineTiles) h->trvar[k] = kVarFine;
       }
     }
   }
@@ -608,7 +608,7 @@ int build_schedule(pselinv_handle* h) {
   {
     int64_t nt8 = 0;
     for (int32_t k = 0; k < nsn; ++k) nt8 += (h->meta[k].r + kTileM - 1) / kTileM * ((h->meta[k].s + 7) / 8);
-    const int var = nt8 * o.batch < kFineTiles ? kVarFine : 0;
+    const int var = nt8 < kFineTiles ? kVarFine : 0;
     build(h->t_lhat, true, [&](int32_t) { return var; }, rect);
   }
   // the adjoint's r x s and s x s tile lists: 64 x 8 tiles on levels whose
@@ -628,8 +628,8 @@ int build_schedule(pselinv_handle* h) {
       }
       for (int32_t t = h->level_ptr[l]; t < h->level_ptr[l + 1]; ++t) {
         const int32_t k = h->level_sn[t];
-        rvar[k] = (int8_t)(nr8 * o.batch < kFineTiles ? kVarFine : nr < target ? 0 : by_width(k));
-        qvar[k] = (int8_t)(nq8 * o.batch < kFineTiles ? kVarFine : nq < target ? 0 : by_width(k));
+        rvar[k] = (int8_t)(nr8 < kFineTiles ? kVarFine : nr < target ? 0 : by_width(k));
+        qvar[k] = (int8_t)(nq8 < kFineTiles ? kVarFine : nq < target ? 0 : by_width(k));
       }
     }
   }
@@ -809,7 +809,7 @@ int build_schedule(pselinv_handle* h) {
     TaskList& tm = h->t_schurm;
     tm.tasks.clear();
     tm.per_lv.assign(nl, Range{});
-    const int64_t copies = (int64_t)o.batch * (o.unsym ? 2 : 1);
+    const int64_t copies = o.unsym ? 2 : 1;
     for (int32_t l = 0; l < nl; ++l) {
       const int32_t g0 = h->schur_gptr[l], g1 = h->schur_gptr[l + 1];
       const int64_t begin = (int64_t)tm.tasks.size();

@@ -814,7 +814,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
   };
   auto merged = [&](int32_t l) {
     const psi::Range r = h->t_schurm.per_lv[l];
-    return h->schur_merged[l] && (!bk || (r.end - r.begin) * h->opts.batch <= psi::kMergedTilesPivoted);
+    return h->schur_merged[l] && (!bk || r.end - r.begin <= psi::kMergedTilesPivoted);
   };
   bool hidep = false, lodep = false;  // hi and lo start with a wait on an event
   for (int32_t l = nl - 1; l >= 0; --l) {

@@ -88,16 +88,17 @@ __host__ __device__
 #endif
 constexpr int fpanel_rows(int w) { return w <= 8 ? 64 : w <= 16 ? 32 : 16; }
 // Merged Schur launches: rows of a tile, bits of Task.c that hold the column end,
-// and the most tiles (all batch members and sides) of a level taken by one.
+// and the most tiles (all sides) of a level taken by one, counted per batch member as
+// kFineTiles.
 constexpr int kMergedRows = 16;
 constexpr int kMergedShift = 20;
 // Both parts of a larger level as one launch no longer overlap its far part with the
 // next level's panels, so the line lies lower where the panels take longer: complex
 // ones, and pivoted ones, whose diagonal block is one long CTA (measured at 8, 32
 // and 128 tiles per SM: 24^3 log det step 6,373, 6,189, 6,086 us; 200 x 147 grid
-// 1,589, 1,507, 1,506; 4 complex poles 57.06, 57.11, 57.69 ms; indefinite 8,443,
+// 1,589, 1,507, 1,506; 4 complex poles, counted together, 57.06, 57.11, 57.69 ms; indefinite 8,443,
 // 8,556, 8,997 us; 56^3 547.4, 547.4, 548.1 ms).
-constexpr int64_t kMergedTiles = 64 * 152, kMergedTilesComplex = 32 * 152, kMergedTilesPivoted = 8 * 152;
+constexpr int64_t kMergedTiles = 64 * 152, kMergedTilesComplex = 8 * 152, kMergedTilesPivoted = 8 * 152;
 constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
 // Variants of the tile GEMMs: 64 x (8 << var) for var 0 .. 3, and the fine 16 x 8 tile.
@@ -105,7 +106,8 @@ constexpr int kNumVar = 5;
 constexpr int kVarFine = 4;
 constexpr int var_rows(int var) { return var == kVarFine ? 16 : kTileM; }
 constexpr int var_cols(int var) { return var == kVarFine ? 8 : 8 << var; }
-// A launch with fewer 64 x 8 tiles than this (all batch members) takes fine ones
+// A launch with fewer 64 x 8 tiles than this takes fine ones, counted per batch member
+// (a fine tile sums k in another order: a member's bits must not depend on the batch)
 // (20^3 adjoint step 10.75 -> 9.89 ms, 16 grids of 12^3 2,053 -> 1,994 us; above it a
 // 64 x 8 tile's reuse of the gathered operand wins).
 constexpr int64_t kFineTiles = 8 * 152;

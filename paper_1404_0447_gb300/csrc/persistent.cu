@@ -49,18 +49,24 @@ __global__ void __launch_bounds__(TG_THREADS, Sc<T>::P == 1 ? 8 : 5) k_persisten
   static_assert(sizeof(TileSmem<T, kFine>) <= sizeof(TileSmem<T, 8>), "one buffer for both tiles");
   __shared__ __align__(16) unsigned char smraw[sizeof(TileSmem<T, 8>)];
   __shared__ long long s_item;
+  __shared__ int s_abort;
   const int batch = a.sz.batch;
   const long long total = ntask * batch;
   int* status = a.status;
   for (;;) {
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(p.head, 1);
+    // one thread reads the abort flag for the CTA: threads that read it for themselves
+    // while another CTA raises it would part ways before the barriers of a task
+    if (threadIdx.x == 0) {
+      s_item = (long long)atomicAdd(p.head, 1);
+      s_abort = *(volatile int*)(status + 2);
+    }
     __syncthreads();
     const long long item = s_item;
+    const bool aborted = s_abort != 0;
     __syncthreads();
     if (item >= total) break;
     const PTask pt = list[item / batch];
     const int b = (int)(item % batch);
-    const bool aborted = *(volatile int*)(status + 2) != 0;
     if (aborted) continue;  // drain the list
     const int64_t cb = (int64_t)b * p.nsn;
     switch (pt.kind) {

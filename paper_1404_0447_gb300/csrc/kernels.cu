@@ -1253,7 +1253,7 @@ cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Tas
 cudaError_t launch_schur_merged(int dtype, const FArgs& f, const MergedArgs& q, const Task* t, cudaStream_t st,
                                 bool dep) {
   if (q.ntile <= 0) return cudaSuccess;
-  const dim3 grid(q.ntile, f.sz.batch * f.sides);
+  const dim3 grid(q.ntile, f.sz.batch, f.sides);  // the product of the last two can exceed the limit of one
   if (dtype == PSELINV_C128) return launch_dep(k_schur_merged<Cplx>, grid, TG_THREADS, 0, st, dep, f, t, q);
   return launch_dep(k_schur_merged<double>, grid, TG_THREADS, 0, st, dep, f, t, q);
 }

@@ -40,7 +40,7 @@ __device__ __forceinline__ void merged_update(const Task* __restrict__ tasks, co
   __shared__ int sh_ticket;
   if (threadIdx.x == 0) sh_ticket = atomicAdd(mq.ticket, 1);  // zeroed long before the previous kernel
   __syncthreads();
-  const int ticket = sh_ticket, copies = gridDim.y, copy = ticket % copies;
+  const int ticket = sh_ticket, copies = gridDim.y * gridDim.z, copy = ticket % copies;
   const Task tk = tasks[ticket / copies];
   const int side = copy % sides, b = copy / sides;
   const int grp = tk.c >> kMergedShift, cend = tk.c & ((1 << kMergedShift) - 1);

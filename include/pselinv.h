@@ -375,7 +375,10 @@ int pselinv_sync_status(pselinv_handle* h, void* stream);
  * Debug switches (failure-detection tests; no paper counterpart).  Bit 1
  * (value 2): the next PERSISTENT pselinv_selinv arms one dependency wait
  * that is never satisfied, so it must end by the spin limit with
- * PSELINV_ERR_TIMEOUT from pselinv_sync_status instead of hanging.
+ * PSELINV_ERR_TIMEOUT from pselinv_sync_status instead of hanging.  Bit 2
+ * (value 4): the same for the waits that order the groups of a level in the
+ * next factorisation or pselinv_selinv_adjoint (matrices with a level of two
+ * groups or more; the limit is at least 1 s).
  */
 int pselinv_set_debug(pselinv_handle* h, int32_t flags);
 

@@ -239,6 +239,22 @@ psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
   return q;
 }
 
+// Debug switch 4 (pselinv_set_debug): around one factorisation or adjoint the groups'
+// tile counts, which only the waits of the merged launches read, are out of reach, so
+// that the first wait runs out; the counts are put back on the stream after it.
+int arm_merged_waits(pselinv_handle* h, cudaStream_t st) {
+  if (h->debug_flags & 4)
+    PSI_CUDA(h, cudaMemsetAsync(h->d_gcnt, 0x7f, sizeof(int32_t) * h->schur_gcnt.size(), st));
+  return PSELINV_OK;
+}
+int disarm_merged_waits(pselinv_handle* h, cudaStream_t st) {
+  if (!(h->debug_flags & 4)) return PSELINV_OK;
+  h->debug_flags &= ~4;
+  PSI_CUDA(h, cudaMemcpyAsync(h->d_gcnt, h->schur_gcnt.data(), sizeof(int32_t) * h->schur_gcnt.size(),
+                              cudaMemcpyHostToDevice, st));
+  return PSELINV_OK;
+}
+
 // Upload the tuning-dependent part (metadata, task lists, partial buffers);
 // called again by the autotuner after build_schedule.
 int upload_schedule(pselinv_handle* h) {
@@ -916,9 +932,11 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
                                            sz, st));
   int rc;
   if ((rc = ensure_factor_streams(h))) return rc;
+  if ((rc = arm_merged_waits(h, st))) return rc;
   rc = replay_or_enqueue(h, &h->fgraph_exec[bk], &h->factor_ran[bk], st,
                          [&](cudaStream_t cs) { return enqueue_factor(h, cs, bk); });
   if (rc) return rc;
+  if ((rc = disarm_merged_waits(h, st))) return rc;
   // no host synchronisation: the first bad pivot stays in status words 0-1
   // until the next factorisation and is reported by pselinv_sync_status (and
   // by pselinv_logdet, which synchronises anyway)
@@ -1380,9 +1398,11 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   PSI_CUDA(h, cudaMemsetAsync(h->d_db, 0, B * h->n * es, st));
   PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, std::min(h->max_width, 64), st));
   a.G = nullptr;  // read by the seed only
+  if ((rc = arm_merged_waits(h, st))) return rc;
   rc = replay_or_enqueue(h, &h->agraph_exec, &h->adjoint_ran, st,
                          [&](cudaStream_t cs) { return enqueue_adjoint(h, a, cs); });
   if (rc) return rc;
+  if ((rc = disarm_merged_waits(h, st))) return rc;
   PSI_CUDA(h, psi::launch_gather_values(h->opts.dtype, h->d_xb, (const int64_t*)h->d_valmap, nullptr, h->nnz_a,
                                         d_gradA, sizes(h), st));
   return PSELINV_OK;

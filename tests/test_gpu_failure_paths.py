@@ -52,3 +52,67 @@ def test_persistent_timeouts_with_many_tasks_in_flight(P, batch):
         h.selinv(P.PERSISTENT)
         h.sync_status()
         assert torch.equal(h.panels(0), good)
+
+
+def merged_handle(P, kind, batch=2):
+    """A handle whose small levels hold several groups each, and a function that factors it."""
+    import torch
+    p = synth.convdiff_problem(dims=(7, 6, 5)) if kind == "unsym" else synth.grid3d(7)
+    h = P.SelInv(p.n, p.colptr, p.rowind, dtype=P.C128 if kind == "complex" else P.F64, unsym=int(kind == "unsym"),
+                 batch=batch)
+    assert np.diff(h.symbolic()["group_ptr"]).max() > 1
+    dev = lambda v: torch.tensor(np.tile(v, batch), dtype=h.torch_dtype, device="cuda")  # noqa: E731
+    lo = dev(p.values)
+    if kind == "unsym":
+        up = dev(p.values_up)
+        return h, lambda: h.factor_unsym(lo, up)
+    return h, lambda: (h.factor_bk if kind == "pivoted" else h.factor)(lo)
+
+
+def raises(P, code, f, *a):
+    with pytest.raises(P.PselinvError) as e:
+        f(*a)
+    assert e.value.code == code
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("report", ["sync_status", "logdet"])
+@pytest.mark.parametrize("kind", ["real", "complex", "unsym", "pivoted"])
+def test_factorisation_wait_runs_out(P, kind, report):
+    """Launched (first call) and replayed: ERR_TIMEOUT, the handle back to "not
+    factored", and the next factorisation right."""
+    import torch
+    h, factor = merged_handle(P, kind)
+    good = None
+    for _ in range(2):
+        h.set_debug(4)
+        factor()
+        raises(P, -7, getattr(h, report))
+        raises(P, -8, h.selinv, P.LEVEL)
+        factor()
+        h.selinv(P.LEVEL)
+        h.sync_status()
+        if good is None:
+            h2, factor2 = merged_handle(P, kind)
+            factor2()
+            h2.selinv(P.LEVEL)
+            good = h2.panels(0)
+        assert torch.equal(h.panels(0), good)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["real", "complex"])
+def test_adjoint_wait_runs_out(P, kind):
+    import torch
+    h, factor = merged_handle(P, kind)
+    factor()
+    h.selinv(P.LEVEL)
+    G = h.panels(0).clone()
+    good = h.adjoint(G).clone()
+    h.sync_status()
+    for _ in range(2):
+        h.set_debug(4)
+        h.adjoint(G)
+        raises(P, -7, h.sync_status)
+        assert torch.equal(h.adjoint(G), good)  # X and the factor are untouched
+        h.sync_status()

@@ -364,7 +364,8 @@ int pselinv_get_panels(pselinv_handle* h, int32_t which, void* out, void* stream
  * until the next factorisation, the handle is back to "not factored"),
  * PSELINV_ERR_TIMEOUT if a bounded wait of the factorisation ran out (until
  * the next factorisation, the handle is back to "not factored"), or one of the
- * PERSISTENT schedule or of the adjoint (that call's results are invalid; the
+ * PERSISTENT schedule or of an adjoint since the last pselinv_sync_status, also
+ * one before a later factorisation (that call's results are invalid; the
  * flag is cleared and the handle stays usable), PSELINV_ERR_RANGE if a selinv with opts.fp64_emulation met an X
  * that is not positive definite (same treatment).  Returns PSELINV_OK
  * otherwise.

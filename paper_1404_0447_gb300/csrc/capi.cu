@@ -923,7 +923,9 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   PSI_CUDA(h, cudaMemsetAsync(h->d_L, 0, elem_size(h) * B * h->panel_total, st));
   if (unsym) PSI_CUDA(h, cudaMemsetAsync(h->d_U, 0, elem_size(h) * B * h->panel_total, st));
   PSI_CUDA(h, cudaMemsetAsync(h->d_status, 0x7f, 2 * sizeof(int), st));  // pivot key: unset
-  PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, sizeof(int) * (kStatusWords - 2), st));
+  // not the adjoint's word: an adjoint is reported whatever followed it
+  static_assert(psi::kAdjointTimeoutWord == psi::kFactorTimeoutWord + 1, "cleared up to the factorisation's word");
+  PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + 2, 0, sizeof(int) * (psi::kAdjointTimeoutWord - 2), st));
   if (unsym)
     PSI_CUDA(h, psi::launch_scatter_values_lu(h->opts.dtype, d_lower, d_upper, (const int64_t*)h->d_valmap,
                                               (const uint8_t*)h->d_flipmap, h->nnz_a, h->d_L, h->d_U, sz, st));

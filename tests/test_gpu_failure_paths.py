@@ -116,3 +116,20 @@ def test_adjoint_wait_runs_out(P, kind):
         raises(P, -7, h.sync_status)
         assert torch.equal(h.adjoint(G), good)  # X and the factor are untouched
         h.sync_status()
+
+
+@pytest.mark.gpu
+def test_adjoint_timeout_outlives_the_next_factorisation(P):
+    import torch
+    h, factor = merged_handle(P, "real")
+    factor()
+    h.selinv(P.LEVEL)
+    G = h.panels(0).clone()
+    good = h.adjoint(G).clone()
+    h.set_debug(4)
+    h.adjoint(G)
+    factor()
+    h.selinv(P.LEVEL)
+    raises(P, -7, h.sync_status)
+    h.sync_status()  # reported once
+    assert torch.equal(h.adjoint(G), good)

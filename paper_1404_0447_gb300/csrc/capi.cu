@@ -219,10 +219,12 @@ int ensure_device(pselinv_handle* h) {
   return PSELINV_OK;
 }
 
-// A ticket per level, a count per (Schur group, copy): batch members and sides.
+// A ticket per level, the abort flag of the sequence's launches, a count per (Schur
+// group, copy): batch members and sides.  One memset at the start of a
+// factorisation or an adjoint clears them all.
 int64_t merged_counter_bytes(const pselinv_handle* h) {
   return (int64_t)sizeof(int) *
-         (h->nlevels + (int64_t)h->schur_gcnt.size() * h->opts.batch * (h->opts.unsym ? 2 : 1));
+         (h->nlevels + 1 + (int64_t)h->schur_gcnt.size() * h->opts.batch * (h->opts.unsym ? 2 : 1));
 }
 
 psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
@@ -230,8 +232,9 @@ psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
   const psi::Range r = h->t_schurm.per_lv[l];
   psi::MergedArgs q;
   q.ticket = (int*)h->d_mctr + l;
+  q.abort = (int*)h->d_mctr + h->nlevels;
   q.gcnt = (const int32_t*)h->d_gcnt + g0;
-  q.done = (int*)h->d_mctr + h->nlevels + (int64_t)g0 * h->opts.batch * (h->opts.unsym ? 2 : 1);
+  q.done = (int*)h->d_mctr + h->nlevels + 1 + (int64_t)g0 * h->opts.batch * (h->opts.unsym ? 2 : 1);
   q.ntile = (int)(r.end - r.begin);
   // at least a second, also where the persistent schedule's limit is shorter: a wait
   // lasts as long as the tiles before it, whatever limit the caller chose for a sweep

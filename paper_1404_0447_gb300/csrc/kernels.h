@@ -125,13 +125,15 @@ struct FArgs {
   int sides;
 };
 enum class FKern { Panel, Update, VInv, Schur };
-// Status words set when a wait of a merged launch ran out.
+// Status words set when a wait of a merged launch ran out: the factorisation's until
+// the next factorisation, the adjoint's until pselinv_sync_status has reported it.
 constexpr int kFactorTimeoutWord = 5, kAdjointTimeoutWord = 6;
 // One merged launch (merged_update.cuh): the level's ticket, and for the
 // level's first group on the tiles per group and the finished tiles per (group,
 // copy), copy = side and batch member.
 struct MergedArgs {
   int* ticket;
+  int* abort;        // of the factorisation's or adjoint's launches: set when a wait ran out
   const int32_t* gcnt;
   int* done;
   int ntile;         // tiles of one copy

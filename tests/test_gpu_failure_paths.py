@@ -133,3 +133,17 @@ def test_adjoint_timeout_outlives_the_next_factorisation(P):
     raises(P, -7, h.sync_status)
     h.sync_status()  # reported once
     assert torch.equal(h.adjoint(G), good)
+
+
+@pytest.mark.gpu
+def test_adjoint_after_an_unreported_timeout_is_right(P):
+    import torch
+    h, factor = merged_handle(P, "real")
+    factor()
+    h.selinv(P.LEVEL)
+    G = h.panels(0).clone()
+    good = h.adjoint(G).clone()
+    h.set_debug(4)
+    h.adjoint(G)
+    assert torch.equal(h.adjoint(G), good)
+    raises(P, -7, h.sync_status)

@@ -449,7 +449,10 @@ def _autograd():
 
         @staticmethod
         def backward(ctx, g):
-            return ctx.handle.adjoint(g.contiguous(), G_PANEL), None, None
+            grad = ctx.handle.adjoint(g.contiguous(), G_PANEL)
+            if not torch.cuda.is_current_stream_capturing():
+                ctx.handle.sync_status()  # a bounded wait of the adjoint that ran out raises here
+            return grad, None, None
 
     return LogDet, SelectedInverse
 

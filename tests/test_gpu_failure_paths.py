@@ -147,3 +147,20 @@ def test_adjoint_after_an_unreported_timeout_is_right(P):
     h.adjoint(G)
     assert torch.equal(h.adjoint(G), good)
     raises(P, -7, h.sync_status)
+
+
+@pytest.mark.gpu
+def test_backward_raises_when_a_wait_of_the_adjoint_ran_out(P):
+    import torch
+    p = synth.grid3d(7)
+    h = P.SelInv(p.n, p.colptr, p.rowind)
+    v = torch.tensor(p.values, device="cuda")[None].requires_grad_()
+    P.selected_inverse(v, h).square().sum().backward()
+    good = v.grad.clone()
+    v.grad = None
+    X = P.selected_inverse(v, h)
+    h.set_debug(4)
+    raises(P, -7, X.square().sum().backward)
+    v.grad = None
+    P.selected_inverse(v, h).square().sum().backward()
+    assert torch.equal(v.grad, good)

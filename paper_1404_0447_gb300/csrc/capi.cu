@@ -966,6 +966,14 @@ int factor_timeout(pselinv_handle* h, const int* status) {
   h->factored = h->inverted = false;
   return set_err(h, PSELINV_ERR_TIMEOUT, "a bounded device wait of the factorisation ran out; the factor is invalid");
 }
+// Report of the last factorisation from the status words (host copy).  A wait that
+// ran out leaves updates out, so a bad pivot beside it may be a consequence.
+int factor_error(pselinv_handle* h, const int* status) {
+  if (const int rc = factor_timeout(h, status)) return rc;
+  unsigned long long key;
+  std::memcpy(&key, status, sizeof(key));
+  return pivot_error(h, key);
+}
 }  // namespace
 
 extern "C" {
@@ -1119,13 +1127,7 @@ int pselinv_sync_status(pselinv_handle* h, void* stream) {
   int status[kStatusWords];
   PSI_CUDA(h, cudaMemcpyAsync(status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, st));
   PSI_CUDA(h, cudaStreamSynchronize(st));
-  {
-    unsigned long long key;
-    std::memcpy(&key, status, sizeof(key));
-    const int rc = pivot_error(h, key);
-    if (rc) return rc;
-  }
-  if (const int rc = factor_timeout(h, status)) return rc;
+  if (const int rc = factor_error(h, status)) return rc;
   if (status[psi::kAdjointTimeoutWord]) {
     PSI_CUDA(h, cudaMemsetAsync((int*)h->d_status + psi::kAdjointTimeoutWord, 0, sizeof(int), st));
     PSI_CUDA(h, cudaStreamSynchronize(st));
@@ -1272,10 +1274,7 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream) {
   int status[kStatusWords];
   PSI_CUDA(h, cudaMemcpyAsync(status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, st));
   PSI_CUDA(h, cudaStreamSynchronize(st));
-  unsigned long long key;
-  std::memcpy(&key, status, sizeof(key));
-  if (const int rc = pivot_error(h, key)) return rc;
-  return factor_timeout(h, status);
+  return factor_error(h, status);
 }
 
 }  // extern "C"

@@ -164,3 +164,19 @@ def test_backward_raises_when_a_wait_of_the_adjoint_ran_out(P):
     v.grad = None
     P.selected_inverse(v, h).square().sum().backward()
     assert torch.equal(v.grad, good)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("report", ["sync_status", "logdet"])
+def test_timeout_is_reported_before_a_pivot_it_spoilt(P, report):
+    """Two leaves of pivot 1 each take 1 off the root's 1: without the update that
+    waits, the root's pivot is 0 instead of -1."""
+    import torch
+    h = P.SelInv(3, np.array([0, 2, 4, 5]), np.array([0, 2, 1, 2, 2]), relax=P.RELAX_NONE)
+    assert np.diff(h.symbolic()["group_ptr"]).max() == 2
+    vals = torch.ones(5, dtype=torch.float64, device="cuda")
+    h.set_debug(4)
+    h.factor(vals)
+    raises(P, -7, getattr(h, report))
+    h.factor(vals)
+    assert h.logdet().tolist() == [[0.0, 1.0]]

@@ -30,6 +30,21 @@ __device__ void report_pivot(int* status, int col, bool zero) {
             ((unsigned long long)(unsigned)col << 2) | (zero ? 1ull : 2ull));
 }
 
+// Whether u / d may be taken as u (1 / d) (one division a column, a product of 60
+// cycles instead of a division of 574 per entry): 1 / d is a normal number.
+// Elsewhere (|d| < 2^-1021 or >= 2^1022) the product would lose bits or overflow where
+// the quotient is an ordinary number, and the kernels divide, outside the code that
+// ordinary pivots run: a test and a division in the pivot loop of k_fdiag cost 0.8 to
+// 1.3% of a 24^3 log det step and a 24^3 non-symmetric pass, this form 0 and 0.5%.
+// Complex: division squares |d|, which leaves its own range first.
+__device__ __forceinline__ bool by_reciprocal(double d) {
+  return ((unsigned)__double2hiint(d) >> 20 & 0x7ffu) - 2u < 2043u;
+}
+__device__ __forceinline__ bool by_reciprocal(Cplx) { return true; }
+// A zero in the place of the reciprocal (a normal number has no zero high word).
+__device__ __forceinline__ bool no_reciprocal(double rd) { return __double2hiint(rd) == 0; }
+__device__ __forceinline__ bool no_reciprocal(Cplx) { return false; }
+
 // --------------------------------------------------------------------------
 // value scatter / selected-entry gather (HBM-bound, index driven)
 // --------------------------------------------------------------------------
@@ -150,13 +165,13 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
 #pragma unroll
     for (int e = 0; e < SIDES; ++e) c[e] = i < w ? ((T*)f.L[e] + po)[i] : Sc<T>::zero();  // column 0
     T dl = c[0];  // lane j: d_j, once column j is final
-    for (int j = 0; j + 1 < w; ++j) {
-      const T rd = Sc<T>::one() / shfl(c[0], j);
+    auto column = [&](int j, T dj, bool prod) {
+      const T rd = Sc<T>::one() / dj;
       const int o = (j & 1) * kFB;
       T l[SIDES], u[SIDES];
 #pragma unroll
       for (int e = 0; e < SIDES; ++e) {
-        l[e] = c[e] * rd;
+        l[e] = prod ? c[e] * rd : c[e] / dj;
         sh[e * SD + o + i] = l[e];  // rows above j are not read
         sh[e * SD + 2 * kFB + o + i] = c[e];
         u[e] = shfl(c[e], j + 1);
@@ -169,6 +184,16 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
         if (i > j && i < w) ((T*)f.L[e] + po)[i + (int64_t)j * ld] = l[e];
       }
       if (i == j + 1) dl = c[0];
+    };
+    int j = 0;
+    for (; j + 1 < w; ++j) {
+      const T dj = shfl(c[0], j);
+      if (__any_sync(0xffffffffu, !by_reciprocal(dj))) break;  // a vote: no divergent code in the chain
+      column(j, dj, true);
+    }
+    for (; j + 1 < w; ++j) {  // from the first pivot out of range on
+      const T dj = shfl(c[0], j);
+      column(j, dj, by_reciprocal(dj));
     }
     // off the chain: a test of d_j inside the loop would hold this warp for the
     // FP64 compares of every column
@@ -263,7 +288,7 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
   T* A = (T*)f.L[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   T* Wp = (T*)f.W[side] + b * f.sz.panel + m.panel + (int64_t)c0 * ld;
   const T* Vi = (const T*)f.Linv[f.sides - 1 - side] + b * f.sz.linv + m.linv + c0 + (int64_t)c0 * s;
-  T a[RF][kFB / 4], bf[kFB / 4], rd[2];
+  T a[RF][kFB / 4], bf[kFB / 4], dc[2], rd[2];
 #pragma unroll
   for (int u = 0; u < kFB / 4; ++u) {
     const int k = 4 * u + q, n = 8 * j + g;
@@ -278,7 +303,8 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const int col = 8 * j + 2 * q + e;
-    rd[e] = Sc<T>::one() / (col < w ? ((const T*)f.D + b * f.sz.n + m.f + c0)[col] : Sc<T>::one());
+    dc[e] = col < w ? ((const T*)f.D + b * f.sz.n + m.f + c0)[col] : Sc<T>::one();
+    rd[e] = Sc<T>::one() / dc[e];
   }
   double acc[RF][Sc<T>::P][2] = {};
 #pragma unroll
@@ -298,6 +324,14 @@ __global__ void __launch_bounds__(kFB * 4) k_fpanel(FArgs f, const Task* __restr
       const T v = frag_value<T>(acc[h], e);
       Wp[row + (int64_t)col * ld] = v;
       A[row + (int64_t)col * ld] = v * rd[e];
+    }
+  if (by_reciprocal(dc[0]) && by_reciprocal(dc[1])) return;
+#pragma unroll
+  for (int h = 0; h < RF; ++h)  // behind the stores of every ordinary pivot
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int row = m0 + 8 * h + g, col = 8 * j + 2 * q + e;
+      if (row < ld && col < w && !by_reciprocal(dc[e])) A[row + (int64_t)col * ld] = frag_value<T>(acc[h], e) / dc[e];
     }
 }
 
@@ -427,7 +461,7 @@ __global__ void __launch_bounds__(512) k_factor_diag_bk(const SnMeta* __restrict
   int* perm = reinterpret_cast<int*>(l2 + s);
   __shared__ int sh_kp, sh_kstep, sh_bad, sh_row;  // sh_row: column of the row search still to do, or -1
   __shared__ __align__(16) double rraw[Sc<T>::P];
-  T* rpiv = reinterpret_cast<T*>(rraw);  // 1 / pivot of a 1 x 1 step
+  T* rpiv = reinterpret_cast<T*>(rraw);  // 1 / pivot of a 1 x 1 step; 0: divide by the pivot
   __shared__ double sh_colmax;
   T* P = L + b * sz.panel + m.panel;
   const int nt = blockDim.x, t = threadIdx.x;
@@ -465,7 +499,7 @@ __global__ void __launch_bounds__(512) k_factor_diag_bk(const SnMeta* __restrict
       sh_kp = c;
       sh_kstep = 1;
       sh_row = -1;
-      *rpiv = r0;
+      *rpiv = by_reciprocal(acc) ? r0 : Sc<T>::zero();
       if (ak == 0 || ak > kBkInf || ck > kBkInf) {  // NaN or infinite
         sh_bad = 2;
       } else if (ak == 1 && ck <= 1) {
@@ -500,8 +534,9 @@ __global__ void __launch_bounds__(512) k_factor_diag_bk(const SnMeta* __restrict
           const double absakk = bk_abs(Tp[pk(k, k, s)]);
           if (!(absakk * rowmax >= alpha * colmax * colmax)) {
             sh_kp = imax;
-            if (bk_abs(Tp[pk(imax, imax, s)]) >= alpha * rowmax)
-              *rpiv = Sc<T>::one() / Tp[pk(imax, imax, s)];
+            const T d = Tp[pk(imax, imax, s)];
+            if (bk_abs(d) >= alpha * rowmax)
+              *rpiv = by_reciprocal(d) ? Sc<T>::one() / d : Sc<T>::zero();
             else
               sh_kstep = 2;
           }
@@ -539,8 +574,9 @@ __global__ void __launch_bounds__(512) k_factor_diag_bk(const SnMeta* __restrict
     if (kstep == 1) {
       const T rd = *rpiv;
       const int ck = pk(k, k, s) - k;
+      const bool prod = !no_reciprocal(rd);
       for (int i = k + 1 + t; i < s; i += nt) {
-        const T u = Tp[ck + i], l = u * rd;
+        const T u = Tp[ck + i], l = prod ? u * rd : u / Tp[ck + k];
         l1[i] = u;
         l2[i] = l;
         Tp[ck + i] = l;

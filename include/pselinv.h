@@ -479,7 +479,8 @@ int pselinv_logdet(pselinv_handle* h, double* h_out, void* stream);
  * the factorisation's groups of supernodes with disjoint targets: no
  * atomics, bitwise reproducible), then the adjoint of the supernodal LDL^T
  * root -> leaves.  Allocates its work buffers on first use.  Symmetric
- * handles only (ERR_STATE otherwise).
+ * handles only (ERR_STATE otherwise).  Where a bounded wait inside ran out,
+ * d_gradA is NaN throughout and pselinv_sync_status returns ERR_TIMEOUT.
  */
 #define PSELINV_G_SYMMETRIC 0
 #define PSELINV_G_PANEL 1

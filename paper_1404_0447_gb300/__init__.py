@@ -443,16 +443,15 @@ def _autograd():
         def forward(ctx, values, handle, mode):
             handle.factor(values.detach().contiguous())
             handle.selinv(mode)
-            handle.sync_status()  # a bad pivot of the factorisation raises here
+            handle.sync_status()  # a bad pivot, or a wait that ran out here or in an earlier backward pass, raises
             ctx.handle = handle
             return handle.panels(0)
 
         @staticmethod
         def backward(ctx, g):
-            grad = ctx.handle.adjoint(g.contiguous(), G_PANEL)
-            if not torch.cuda.is_current_stream_capturing():
-                ctx.handle.sync_status()  # a bounded wait of the adjoint that ran out raises here
-            return grad, None, None
+            # not synchronised: where a bounded wait ran out the gradient is NaN and the next
+            # forward pass (or sync_status) raises
+            return ctx.handle.adjoint(g.contiguous(), G_PANEL), None, None
 
     return LogDet, SelectedInverse
 

@@ -95,15 +95,17 @@ __global__ void k_gather_values_lu(const T* __restrict__ XL, const T* __restrict
 
 // out[q] = X at the panel position of stored entry q; with a diagonal mask,
 // off-diagonal entries are doubled (gradient with respect to a stored value
-// that stands for both A_ij and A_ji).
+// that stands for both A_ij and A_ji).  NaN throughout where *invalid is set.
 template <class T>
 __global__ void k_gather_values(const T* __restrict__ X, int64_t panel_total, const int64_t* __restrict__ vmap,
-                                const uint8_t* __restrict__ diagmask, int64_t nnz, T* __restrict__ out) {
+                                const uint8_t* __restrict__ diagmask, int64_t nnz, T* __restrict__ out,
+                                const int* __restrict__ invalid) {
   const int b = blockIdx.y;
   const T* Xb = X + (int64_t)b * panel_total;
   T* o = out + (int64_t)b * nnz;
+  const bool bad = invalid && *invalid;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x) {
-    const T v = Xb[vmap[q]];
+    const T v = bad ? Sc<T>::nan() : Xb[vmap[q]];
     o[q] = (diagmask && !diagmask[q]) ? 2.0 * v : v;
   }
 }
@@ -1186,15 +1188,15 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
 
 template <class T>
 static cudaError_t gather_t(const void* X, const int64_t* vmap, const uint8_t* mask, int64_t nnz, void* out,
-                            const Sizes& sz, cudaStream_t st) {
+                            const Sizes& sz, cudaStream_t st, const int* invalid) {
   k_gather_values<T><<<dim3(blocks_for(nnz, 256), sz.batch), 256, 0, st>>>((const T*)X, sz.panel, vmap, mask, nnz,
-                                                                          (T*)out);
+                                                                          (T*)out, invalid);
   return cudaGetLastError();
 }
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
-                                 void* out, const Sizes& sz, cudaStream_t st) {
-  return dtype == PSELINV_C128 ? gather_t<Cplx>(X, vmap, diagmask, nnz, out, sz, st)
-                               : gather_t<double>(X, vmap, diagmask, nnz, out, sz, st);
+                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid) {
+  return dtype == PSELINV_C128 ? gather_t<Cplx>(X, vmap, diagmask, nnz, out, sz, st, invalid)
+                               : gather_t<double>(X, vmap, diagmask, nnz, out, sz, st, invalid);
 }
 
 // ---- tile-kernel launch for one task range of one variant ----

@@ -160,9 +160,10 @@ cudaError_t launch_scatter_values_lu(int dtype, const void* lower, const void* u
 cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, const int64_t* vmap,
                                     const uint8_t* flip, int64_t nnz, int upper, void* out, const Sizes& sz,
                                     cudaStream_t st);
-// diagmask == nullptr: plain gather; else off-diagonal entries doubled.
+// diagmask == nullptr: plain gather; else off-diagonal entries doubled.  invalid: a
+// device flag; where it is set the output is NaN.
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
-                                 void* out, const Sizes& sz, cudaStream_t st);
+                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid = nullptr);
 // Tile kernels (Trsm, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
 cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st,

@@ -46,6 +46,7 @@ struct Sc<double> {
   static constexpr int P = 1;  // real planes
   __device__ __forceinline__ static double zero() { return 0.0; }
   __device__ __forceinline__ static double one() { return 1.0; }
+  __device__ __forceinline__ static double nan() { return __longlong_as_double(0x7ff8000000000000ll); }
   __device__ __forceinline__ static double plane(double v, int) { return v; }
   __device__ __forceinline__ static bool bad(double v) { return !isfinite(v) || v == 0.0; }
   __device__ __forceinline__ static bool is_zero(double v) { return v == 0.0; }
@@ -55,6 +56,7 @@ struct Sc<Cplx> {
   static constexpr int P = 2;
   __device__ __forceinline__ static Cplx zero() { return {0.0, 0.0}; }
   __device__ __forceinline__ static Cplx one() { return {1.0, 0.0}; }
+  __device__ __forceinline__ static Cplx nan() { return {Sc<double>::nan(), Sc<double>::nan()}; }
   __device__ __forceinline__ static double plane(Cplx v, int p) { return p ? v.im : v.re; }
   __device__ __forceinline__ static bool bad(Cplx v) {
     return !isfinite(v.re) || !isfinite(v.im) || (v.re == 0.0 && v.im == 0.0);

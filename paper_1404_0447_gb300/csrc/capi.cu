@@ -77,10 +77,14 @@ void drop_graphs(pselinv_handle* h) {
 
 // Replay *exec on st; captured first, from enqueue(stream), where it is not there
 // yet.  The capture runs on the handle's own stream, thread-local: nothing of
-// the caller's is captured.
+// the caller's is captured.  On an error nothing has been enqueued on st.
 template <class F>
 int replay(pselinv_handle* h, void** exec, cudaStream_t st, F&& enqueue) {
   if (!*exec) {
+    if (h->debug_flags & 8) {  // debug switch: as if the capture had failed
+      h->debug_flags &= ~8;
+      return cuda_err(h, cudaErrorMemoryAllocation, "cudaGraphInstantiate");
+    }
     if (!h->graph_stream) {
       cudaStream_t ns;
       PSI_CUDA(h, cudaStreamCreateWithFlags(&ns, cudaStreamNonBlocking));
@@ -112,7 +116,8 @@ int replay(pselinv_handle* h, void** exec, cudaStream_t st, F&& enqueue) {
 // a graph node by 0.2 us, and the host's ~2 us per launch is gone, against
 // ~1 ms once for capture and instantiation (so a handle used once never pays).
 // A stream that is being captured by the caller takes the launches themselves,
-// as before.
+// as before, and so does a call whose capture or replay fails (no memory for the
+// graph, say): the launches need nothing that the first call did not have.
 template <class F>
 int replay_or_enqueue(pselinv_handle* h, void** exec, bool* ran, cudaStream_t st, F&& enqueue) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -124,7 +129,9 @@ int replay_or_enqueue(pselinv_handle* h, void** exec, bool* ran, cudaStream_t st
     *ran = true;
     return enqueue(st);
   }
-  return replay(h, exec, st, enqueue);
+  if (replay(h, exec, st, enqueue) == PSELINV_OK) return PSELINV_OK;
+  cudaGetLastError();  // reported by the launches if it persists
+  return enqueue(st);
 }
 
 void free_device(pselinv_handle* h) {
@@ -1052,6 +1059,7 @@ int pselinv_selinv(pselinv_handle* h, int32_t mode, void* stream) {
     bool enqueued = false;
     const auto sweep = [&](cudaStream_t cs) {
       enqueued = true;
+      std::memcpy(h->launches, before, sizeof(before));  // counted once, also after a failed capture
       return enqueue_selinv(h, PSELINV_LEVEL, cs, false);
     };
     const int rc = mode == PSELINV_GRAPH

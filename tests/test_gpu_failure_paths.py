@@ -182,3 +182,51 @@ def test_timeout_is_reported_before_a_pivot_it_spoilt(P, report):
     raises(P, -7, getattr(h, report))
     h.factor(vals)
     assert h.logdet().tolist() == [[0.0, 1.0]]
+
+
+@pytest.mark.gpu
+def test_calls_go_on_without_their_graphs(P):
+    """The second call captures its launches: where that fails, it launches them."""
+    import torch
+    h, factor = merged_handle(P, "real")
+    G = None
+    ref = []
+    for it in range(3):
+        h.set_debug(8 if it == 1 else 0)
+        factor()
+        h.set_debug(8 if it == 1 else 0)
+        h.selinv(P.LEVEL)
+        G = h.panels(0).clone() if G is None else G
+        h.set_debug(8 if it == 1 else 0)
+        out = [h.panels(0).clone(), h.panels(1).clone(), h.adjoint(G).clone()]
+        h.sync_status()
+        ref = ref or out
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", ["GRAPH", "PERSISTENT"])
+def test_schedules_that_are_graphs_report_a_failed_capture(P, mode):
+    import torch
+    h, factor = merged_handle(P, "real")
+    factor()
+    h.set_debug(8)
+    raises(P, -5, h.selinv, getattr(P, mode))
+    h.selinv(getattr(P, mode))
+    h.sync_status()
+    X = h.panels(0).clone()
+    h.selinv(P.LEVEL)
+    assert torch.equal(h.panels(0), X)
+
+
+@pytest.mark.gpu
+def test_launches_are_counted_once_after_a_failed_capture(P):
+    h, factor = merged_handle(P, "real")
+    factor()
+    counts = []
+    for flag in (0, 8, 0, 0):
+        h.set_timing(False)  # resets the counts
+        h.set_debug(flag)
+        h.selinv(P.LEVEL)
+        counts.append(h.get_timing()[1].tolist())
+    assert all(c == counts[0] for c in counts)

@@ -205,7 +205,7 @@ int ensure_device(pselinv_handle* h) {
   if ((rc = alloc(h, &h->d_D, B * h->n * es))) return rc;
   if ((rc = alloc(h, &h->d_lhat, B * h->lhat_total * es))) return rc;
   if ((rc = alloc(h, &h->d_linv, B * h->linv_total * es))) return rc;
-  if ((rc = alloc(h, &h->d_status, sizeof(int) * kStatusWords + sizeof(double) * (6 + 2 * psi::kLogdetCtas) * B))) return rc;
+  if ((rc = alloc(h, &h->d_status, sizeof(int) * kStatusWords + sizeof(double) * (6 + 2 * psi::logdet_parts(h->n)) * B))) return rc;
   if (h->opts.unsym) {
     if ((rc = upload(h, &h->d_flipmap, h->flipmap))) return rc;
     if ((rc = alloc(h, &h->d_U, B * h->panel_total * es))) return rc;

@@ -1033,14 +1033,14 @@ __global__ void k_logdet(const T* __restrict__ D, int64_t n, double* __restrict_
   }
   block_sum2(a, c);
   if (threadIdx.x == 0) {
-    double* w = work + 2 * ((int64_t)b * kLogdetCtas + blockIdx.x);
+    double* w = work + 2 * ((int64_t)b * gridDim.x + blockIdx.x);
     w[0] = a;
     w[1] = c;
   }
 }
 __global__ void k_logdet_sum(const double* __restrict__ work, int parts, double* __restrict__ out) {
   const int b = blockIdx.x;
-  const double* w = work + 2 * (int64_t)b * kLogdetCtas;
+  const double* w = work + 2 * (int64_t)b * parts;
   double a = 0.0, c = 0.0;
   for (int p = threadIdx.x; p < parts; p += blockDim.x) {
     a += w[2 * p];
@@ -1329,7 +1329,7 @@ cudaError_t launch_per_sn(Kern k, const KArgs& a, const int32_t* sns, int nsn, c
 
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* work, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype, const void* E) {
-  const int parts = (int)blocks_for(n, 256, kLogdetCtas);
+  const int parts = logdet_parts(n);
   if (dtype == PSELINV_C128)
     k_logdet<Cplx><<<dim3(parts, batch), 256, 0, st>>>((const Cplx*)D, n, work, ptype, (const Cplx*)E);
   else

@@ -183,8 +183,8 @@ cudaError_t launch_schur_merged(int dtype, const FArgs& f, const MergedArgs& q, 
 cudaError_t launch_vdiag(int dtype, const FArgs& f, const int32_t* sns, int nsn, int wmax, cudaStream_t st);
 cudaError_t launch_ftiles(FKern k, int var, int dtype, const FArgs& f, const Task* t, int64_t n, cudaStream_t st,
                           bool dep = true);
-// work: batch x 2 x kLogdetCtas doubles.
-constexpr int kLogdetCtas = 128;
+// CTAs per batch member; work: batch x 2 x logdet_parts(n) doubles.
+constexpr int logdet_parts(int64_t n) { return n <= 256 ? 1 : n >= 128 * 256 ? 128 : (int)((n + 255) / 256); }
 cudaError_t launch_logdet(int dtype, const void* D, int64_t n, double* work, double* out, int batch, cudaStream_t st,
                           const int8_t* ptype = nullptr, const void* E = nullptr);
 cudaError_t launch_pole_sum(int dtype, const void* X, int64_t panel_total, int batch, const void* w, void* out,

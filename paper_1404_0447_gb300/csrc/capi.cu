@@ -48,19 +48,25 @@ psi::Sizes sizes(const pselinv_handle* h) {
   return s;
 }
 
-template <class T>
-int upload(pselinv_handle* h, void** dst, const std::vector<T>& v) {
-  size_t bytes = sizeof(T) * (v.empty() ? 1 : v.size());
-  PSI_CUDA(h, cudaMalloc(dst, bytes));
-  h->device_bytes += (int64_t)bytes;
-  if (!v.empty()) PSI_CUDA(h, cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
-  return PSELINV_OK;
-}
-
 int alloc(pselinv_handle* h, void** dst, int64_t bytes) {
   if (bytes < 16) bytes = 16;
   PSI_CUDA(h, cudaMalloc(dst, (size_t)bytes));
-  h->device_bytes += bytes;
+  h->dev_alloc.emplace_back(*dst, bytes);
+  return PSELINV_OK;
+}
+
+void release(pselinv_handle* h, void** p) {
+  if (!*p) return;
+  cudaFree(*p);
+  auto& a = h->dev_alloc;
+  a.erase(std::find_if(a.begin(), a.end(), [&](const auto& e) { return e.first == *p; }));
+  *p = nullptr;
+}
+
+template <class T>
+int upload(pselinv_handle* h, void** dst, const std::vector<T>& v) {
+  if (const int rc = alloc(h, dst, (int64_t)(sizeof(T) * v.size()))) return rc;
+  if (!v.empty()) PSI_CUDA(h, cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
   return PSELINV_OK;
 }
 
@@ -142,10 +148,7 @@ void free_device(pselinv_handle* h) {
                    &h->d_xb,   &h->d_lb,   &h->d_db,     &h->d_zb,     &h->d_w1,    &h->d_yb,   &h->d_hb,
                    &h->d_plist, &h->d_pn,  &h->d_pctr, &h->d_xs, &h->d_ls, &h->d_sig, &h->d_lexp, &h->d_gexp, &h->d_crow,
                    &h->d_tctr, &h->d_gctr, &h->d_fbsn, &h->d_gcnt, &h->d_mctr};
-  for (void** p : ptrs) {
-    if (*p) cudaFree(*p);
-    *p = nullptr;
-  }
+  for (void** p : ptrs) release(h, p);
   for (void* e : h->ev_pool) cudaEventDestroy((cudaEvent_t)e);
   h->ev_pool.clear();
   h->ev_used = 0;
@@ -163,7 +166,6 @@ void free_device(pselinv_handle* h) {
   if (h->fs_lo) cudaStreamDestroy((cudaStream_t)h->fs_lo);
   h->fs_hi = h->fs_lo = nullptr;
   h->dev_sym = false;
-  h->device_bytes = 0;
 }
 
 int upload_schedule(pselinv_handle* h);
@@ -273,11 +275,7 @@ int upload_schedule(pselinv_handle* h) {
   int rc;
   void** old[] = {&h->d_meta, &h->d_tasks, &h->d_part, &h->d_ypart, &h->d_plist, &h->d_pn, &h->d_pctr,
                    &h->d_yring, &h->d_pring, &h->d_tctr, &h->d_gcnt, &h->d_mctr};
-  for (void** p : old)
-    if (*p) {
-      cudaFree(*p);
-      *p = nullptr;
-    }
+  for (void** p : old) release(h, p);
   drop_graphs(h);
   if ((rc = upload(h, &h->d_meta, h->meta))) return rc;
   std::vector<psi::Task> all;
@@ -1568,26 +1566,8 @@ int pselinv_get_info(const pselinv_handle* h, pselinv_info* info) {
   info->flops_selinv = h->flops_selinv;
   info->flops_gemm1 = h->flops_gemm1;
   info->bytes_selinv = h->bytes_selinv;
-  // device memory held now (the autotuner reallocates the schedule buffers)
-  if (h->dev_sym) {
-    const int64_t B = h->opts.batch, es = (int64_t)elem_size(h), tasks =
-        (int64_t)(h->t_norm.tasks.size() + h->t_lhat.tasks.size() + h->t_gemm1.tasks.size() + h->t_gemm2.tasks.size() +
-                  h->t_trsm.tasks.size() + h->t_schur.tasks.size() + h->t_schurm.tasks.size() + h->t_fpanel.tasks.size() +
-                  h->t_fupdate.tasks.size() + h->t_vinv.tasks.size() + h->t_rect.tasks.size() +
-                  h->t_pgemm1.tasks.size() + h->t_pgemm2.tasks.size() + h->t_sq.tasks.size());
-    int64_t bytes = (int64_t)(sizeof(psi::SnMeta) * h->meta.size() + sizeof(psi::ColDesc) * h->desc.size() +
-                              4 * h->relidx.size() + 8 * h->valmap.size() + h->diagmask.size() +
-                              4 * h->level_sn.size()) +
-                    (int64_t)sizeof(psi::Task) * tasks +
-                    B * es * (2 * h->panel_total + h->n + h->lhat_total + h->linv_total + h->part_max + h->ypart_max);
-    if (h->d_xb) bytes += B * es * (2 * h->panel_total + h->n + 2 * h->linv_total + 2 * h->lhat_total);
-    if (h->opts.unsym) bytes += h->flipmap.size() + B * es * (2 * h->panel_total + h->lhat_total + h->linv_total);
-    if (h->d_yring) bytes += B * es * psi::kRing * (h->ypart_max + h->part_max);
-    bytes += 4 * (2 * (int64_t)h->nsn + h->nlevels + 1);  // level / parent / level offsets
-    info->device_bytes = bytes;
-  } else {
-    info->device_bytes = 0;
-  }
+  info->device_bytes = 0;
+  for (const auto& e : h->dev_alloc) info->device_bytes += e.second;
   return PSELINV_OK;
 }
 

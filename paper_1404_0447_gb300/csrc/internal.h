@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <climits>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/pselinv.h"
@@ -270,7 +271,7 @@ struct pselinv_handle {
   void* d_w1 = nullptr;     // s x s per supernode
   void* d_yb = nullptr;     // r x s per supernode
   void* d_hb = nullptr;     // r x s per supernode
-  int64_t device_bytes = 0;
+  std::vector<std::pair<void*, int64_t>> dev_alloc;  // device allocations held, with their bytes
   void* d_plist = nullptr;  // persistent schedule
   void* d_pn = nullptr;     // pn1 then pn2
   void* d_pctr = nullptr;   // c1, c2, cr, cf counters, per-level finish counts, dequeue head

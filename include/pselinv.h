@@ -380,7 +380,8 @@ int pselinv_sync_status(pselinv_handle* h, void* stream);
  * (value 4): the same for the waits that order the groups of a level in the
  * next factorisation or pselinv_selinv_adjoint (matrices with a level of two
  * groups or more; the limit is at least 1 s).  Bit 3 (value 8): the next
- * capture of a graph fails as if there were no memory for it.
+ * capture of a graph fails as if there were no memory for it.  Bit 4 (value 16):
+ * the second of the next device allocations fails likewise.
  */
 int pselinv_set_debug(pselinv_handle* h, int32_t flags);
 

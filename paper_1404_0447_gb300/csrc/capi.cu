@@ -24,6 +24,7 @@ int set_err(pselinv_handle* h, int code, const std::string& msg) {
 }
 
 int cuda_err(pselinv_handle* h, cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: the check after a later launch must not find it
   return set_err(h, e == cudaErrorMemoryAllocation ? PSELINV_ERR_OOM : PSELINV_ERR_CUDA,
                  std::string(where) + ": " + cudaGetErrorString(e));
 }
@@ -48,7 +49,15 @@ psi::Sizes sizes(const pselinv_handle* h) {
   return s;
 }
 
+// Keeps what is there: after one of several allocations has failed, the call that is
+// tried again makes the missing ones only.
 int alloc(pselinv_handle* h, void** dst, int64_t bytes) {
+  if (*dst) return PSELINV_OK;
+  if (h->debug_flags & 32) {  // debug switch: the second allocation fails
+    h->debug_flags &= ~32;
+    return cuda_err(h, cudaErrorMemoryAllocation, "cudaMalloc");
+  }
+  if (h->debug_flags & 16) h->debug_flags ^= 16 | 32;
   if (bytes < 16) bytes = 16;
   PSI_CUDA(h, cudaMalloc(dst, (size_t)bytes));
   h->dev_alloc.emplace_back(*dst, bytes);
@@ -272,6 +281,9 @@ int disarm_merged_waits(pselinv_handle* h, cudaStream_t st) {
 // Upload the tuning-dependent part (metadata, task lists, partial buffers);
 // called again by the autotuner after build_schedule.
 int upload_schedule(pselinv_handle* h) {
+  // not usable until all of it is there; after a failure the next factorisation uploads it
+  const bool sym = h->dev_sym, factored = h->factored, inverted = h->inverted;
+  h->dev_sym = h->factored = h->inverted = false;
   int rc;
   void** old[] = {&h->d_meta, &h->d_tasks, &h->d_part, &h->d_ypart, &h->d_plist, &h->d_pn, &h->d_pctr,
                    &h->d_yring, &h->d_pring, &h->d_tctr, &h->d_gcnt, &h->d_mctr};
@@ -320,13 +332,15 @@ int upload_schedule(pselinv_handle* h) {
   pn.insert(pn.end(), h->pn2.begin(), h->pn2.end());
   if ((rc = upload(h, &h->d_pn, pn))) return rc;
   if ((rc = alloc(h, &h->d_pctr, (int64_t)sizeof(int) * (4 * B * h->nsn + h->nlevels + 1)))) return rc;
+  h->dev_sym = sym;
+  h->factored = factored;
+  h->inverted = inverted;
   return PSELINV_OK;
 }
 
 // Ring of kRing level slots for the persistent schedule's partial products
 // (allocated before its graph is captured; dropped with the schedule).
 int ensure_ring(pselinv_handle* h) {
-  if (h->d_yring) return PSELINV_OK;
   const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
   int rc;
   if ((rc = alloc(h, &h->d_yring, B * psi::kRing * h->ypart_max * es))) return rc;
@@ -923,7 +937,7 @@ int factor_impl(pselinv_handle* h, const void* d_lower, const void* d_upper, cud
   const int64_t B = h->opts.batch;
   const bool unsym = d_upper != nullptr;
   h->factored = h->inverted = false;
-  if (bk && !h->d_piv) {
+  if (bk) {
     int rc;
     if ((rc = alloc(h, &h->d_piv, B * h->n * (int64_t)sizeof(int32_t)))) return rc;
     if ((rc = alloc(h, &h->d_ptype, B * h->n))) return rc;
@@ -1378,15 +1392,13 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   if (!h->inverted) return set_err(h, PSELINV_ERR_STATE, "selinv_adjoint needs a prior pselinv_selinv");
   const int64_t B = h->opts.batch, es = (int64_t)elem_size(h);
   int rc;
-  if (!h->d_xb) {
-    if ((rc = alloc(h, &h->d_xb, B * h->panel_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_lb, B * h->panel_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_db, B * h->n * es))) return rc;
-    if ((rc = alloc(h, &h->d_zb, B * h->linv_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_w1, B * h->linv_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_yb, B * h->lhat_total * es))) return rc;
-    if ((rc = alloc(h, &h->d_hb, B * h->lhat_total * es))) return rc;
-  }
+  if ((rc = alloc(h, &h->d_xb, B * h->panel_total * es))) return rc;
+  if ((rc = alloc(h, &h->d_lb, B * h->panel_total * es))) return rc;
+  if ((rc = alloc(h, &h->d_db, B * h->n * es))) return rc;
+  if ((rc = alloc(h, &h->d_zb, B * h->linv_total * es))) return rc;
+  if ((rc = alloc(h, &h->d_w1, B * h->linv_total * es))) return rc;
+  if ((rc = alloc(h, &h->d_yb, B * h->lhat_total * es))) return rc;
+  if ((rc = alloc(h, &h->d_hb, B * h->lhat_total * es))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   psi::AdjArgs a;
   a.k = kargs(h);

@@ -79,3 +79,46 @@ def test_device_bytes_count_the_counters_of_a_batch(P):  # noqa: F811
     use()
     said, used = use()
     assert said <= used <= said + (40 << 20)
+
+
+@pytest.mark.parametrize("what", ["factor", "pivoted", "persistent", "adjoint", "autotune"])
+def test_call_that_ran_out_of_memory_can_be_tried_again(P, what):  # noqa: F811
+    """The second of a call's allocations fails (debug switch): ERR_OOM, and the same
+    call made again allocates what is missing and gives the right bits."""
+    import torch
+    p = synth.grid3d(7)
+    vals = torch.tensor(p.values, device="cuda")
+
+    def call(h, fail):
+        out = []
+        steps = {"factor": lambda: h.factor(vals), "pivoted": lambda: h.factor_bk(vals),
+                 "persistent": lambda: h.selinv(P.PERSISTENT), "adjoint": lambda: out.append(h.adjoint(X)),
+                 "autotune": lambda: h.autotune()}
+        if what not in ("factor", "pivoted"):
+            h.factor(vals)
+            h.selinv(P.LEVEL)
+            X = h.panels(0).clone()
+        elif what == "pivoted":
+            h.factor(vals)
+        if fail:
+            h.set_debug(16)
+            with pytest.raises(P.PselinvError) as e:
+                steps[what]()
+            assert e.value.code == -5
+        if what == "autotune":  # a schedule half replaced: refused until the next factorisation
+            if fail:
+                with pytest.raises(P.PselinvError) as e:
+                    h.selinv(P.LEVEL)
+                assert e.value.code == -8
+            h.factor(vals)
+        else:
+            steps[what]()
+        h.selinv(P.LEVEL) if what != "persistent" else None
+        h.sync_status()
+        return [h.panels(0).clone(), h.panels(1).clone()] + out
+
+    new = lambda: P.SelInv(p.n, p.colptr, p.rowind)  # noqa: E731
+    tuned = what == "autotune"
+    for a, b in zip(call(new(), True), call(new(), False)):
+        # autotune: the trial's step-2 slices stay, which sum in another order
+        assert torch.allclose(a, b, rtol=0, atol=1e-13 * float(b.abs().max())) if tuned else torch.equal(a, b)

@@ -703,7 +703,6 @@ int build_schedule(pselinv_handle* h) {
     // thread: the factor is bitwise reproducible.
     TaskList& tl = h->t_schur;
     const int var = by_rows(0);
-    h->schur_var = var;
     tl.tasks.clear();
     tl.per_lv.assign((size_t)nl * kNumVar, Range{});
     tl.per_sn.assign(nsn, Range{});

@@ -209,7 +209,6 @@ struct pselinv_handle {
   std::vector<int8_t> schur_merged;
   psi::TaskList t_schurm;
   std::vector<int32_t> schur_gcnt;
-  int32_t schur_var = 0;  // tile variant of the Schur tiles of the larger groups
   std::vector<int8_t> s2var, s3var, trvar;  // step-2 / step-3 / panel-solve tile variant per supernode
   psi::TaskList t_sq;     // s x s tiles of each supernode's diagonal block (adjoint products)
   psi::TaskList t_pgemm1; // persistent schedule: step-2 tiles, 64 x 8 and fine

@@ -1216,8 +1216,10 @@ static cudaError_t tiles_tb(Kern k, const KArgs& a, const Task* t, int64_t n, cu
       return launch_dep(k_trsm<T, BN>, grid, TG_THREADS, 0, st, dep, a.meta, t, (const T*)a.L, (const T*)a.Linv, a.sz,
                         a.piv, (T*)a.W);
     case Kern::Lhat:
-      return launch_dep(k_lhat<T, BN>, grid, TG_THREADS, 0, st, dep, a.meta, t, (const T*)a.L, (const T*)a.Linv,
-                        (T*)a.Lhat, a.sz);
+      if constexpr (BN == 8 || BN == kFine)  // a list of 64 x 8 or of fine tiles
+        return launch_dep(k_lhat<T, BN>, grid, TG_THREADS, 0, st, dep, a.meta, t, (const T*)a.L, (const T*)a.Linv,
+                          (T*)a.Lhat, a.sz);
+      return cudaErrorInvalidValue;
     case Kern::Gemm1:
       if (a.XU) return launch_dep(k_gemm1<T, BN, true>, grid, TG_THREADS, 0, st, dep, a, t);
       return launch_dep(k_gemm1<T, BN, false>, grid, TG_THREADS, 0, st, dep, a, t);

@@ -348,13 +348,6 @@ __device__ __forceinline__ void tile_mma(TileSmem<T, BN>& sm, int kbeg, int kend
   }
 }
 
-// Every fragment live.
-template <class T, int BN, class MA, class LA, class LB>
-__device__ __forceinline__ void tile_mma(TileSmem<T, BN>& sm, int kbeg, int kend, const MA& a_by_k_at, const LA& la,
-                                         const LB& lb, Acc<T, BN>& acc) {
-  tile_mma<T, BN>(sm, kbeg, kend, a_by_k_at, la, lb, acc, [](int, int) { return true; });
-}
-
 // Fragments with a row below mlim and a column below nlim (tile-local): a
 // rectangular output's ragged edges.
 struct LiveRect {

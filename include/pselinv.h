@@ -103,8 +103,7 @@ typedef struct {
   int32_t debug_checks;   /* nonzero: kernels bounds-check every index and report */
   int32_t unsym;          /* 0: symmetric A = L D L^T.  1: non-symmetric A with a symmetric pattern,
                              A = L D U' (pselinv_factor_unsym; Algorithm 1 with step 4); complex
-                             non-symmetric handles cap w_max at 112 (shared-memory budget of the
-                             diagonal-block factorisation) */
+                             non-symmetric handles cap w_max at 112 */
   int64_t spin_limit_ns;  /* limit for bounded device waits; <= 0 = 1e9 (waits inside a factorisation or
                              an adjoint: at least 1e9) */
   int32_t level_tiles;    /* a level whose step-2 (step-3) tiles number fewer than this gets its slices

@@ -782,8 +782,9 @@ int ensure_factor_streams(pselinv_handle* h) {
     // 1 TFLOP/s; 30 us per 32 columns of the widest supernode).
     const int32_t nl = h->nlevels;
     // The pivoted panels take longer: 345 us (w / 128)^3 + 30 us for the diagonal
-    // block (one CTA), no blocks of columns (pivoted 40^3 34.6 -> 33.0 ms, 24^3 and
-    // 80^3 the same within 0.2%).
+    // block (one CTA; 305 us alone at w = 128) and the inverse's two launches after
+    // it, no blocks of columns (against the pivot-free estimate: pivoted 40^3 34.6 ->
+    // 33.0 ms, 24^3 and 80^3 the same within 0.2%).
     std::vector<double> t_far(nl, 0.0), t_next[2];
     for (auto& t : t_next) t.assign(nl, 0.0);
     for (int32_t l = 0; l < nl; ++l) {

@@ -70,7 +70,11 @@ struct Range {
 };
 
 constexpr int kMaxWidth = 128;   // widest supernode the kernels accept
-constexpr int kMaxWidthLUComplex = 112;  // complex non-symmetric: two packed triangles in shared memory
+// Complex non-symmetric handles: the documented cap of pselinv_opts.unsym.  The bound
+// behind it (two packed triangles in one CTA's shared memory) went with the kernel that
+// had them; the kernels now take 128, and the cap stays so that the supernodes of such
+// handles, and with them X's bits, stay what they are.
+constexpr int kMaxWidthLUComplex = 112;
 constexpr int kChunkRows = 512;  // rows per step-3 partial product (before the per-level boost)
 constexpr int kTargetTiles = 128 * 152;  // tiles a level should offer the GPU (128 per SM: short tails)
 constexpr int kMinSlice2 = 128;   // smallest step-2 slice the per-level boost makes
@@ -95,10 +99,11 @@ constexpr int kMergedRows = 16;
 constexpr int kMergedShift = 20;
 // Both parts of a larger level as one launch no longer overlap its far part with the
 // next level's panels, so the line lies lower where the panels take longer: complex
-// ones, and pivoted ones, whose diagonal block is one long CTA (measured at 8, 32
-// and 128 tiles per SM: 24^3 log det step 6,373, 6,189, 6,086 us; 200 x 147 grid
-// 1,589, 1,507, 1,506; 4 complex poles, counted together, 57.06, 57.11, 57.69 ms; indefinite 8,443,
-// 8,556, 8,997 us; 56^3 547.4, 547.4, 548.1 ms).
+// ones, and pivoted ones, whose diagonal block is one long CTA.  Measured at 8, 32, 64
+// and 128 tiles per SM, real: 24^3 log det step 6,321, 6,090, 5,925, 5,927 us; 200 x 147
+// grid 1,613, 1,508, 1,508, 1,508; 56^3 545.6, 545.7, 545.5, 545.5 ms.  At 8, 32 and 128,
+// 4 complex poles (counted together) 57.06, 57.11, 57.69 ms; pivoted 26 x 25 x 23 grid
+// 8,443, 8,556, 8,997 us.
 constexpr int64_t kMergedTiles = 64 * 152, kMergedTilesComplex = 8 * 152, kMergedTilesPivoted = 8 * 152;
 constexpr int kFUpdateRows = 16; // rows of a k_fupdate task (8 per warp)
 
@@ -231,13 +236,13 @@ struct pselinv_handle {
   void* d_levelsn = nullptr;
   void* d_fbsn = nullptr;   // fb_sn
   void* d_gcnt = nullptr;   // schur_gcnt
-  // merged Schur launches: per level a ticket, per (group, batch member) the finished
-  // tiles; zeroed at the start of a factorisation
+  // merged launches: per level a ticket, an abort flag, per (group, side, batch member)
+  // the finished tiles; zeroed at the start of a factorisation or an adjoint
   void* d_mctr = nullptr;
   void* d_L = nullptr;      // L panels (unit diagonal implied; D on the diagonal slots)
   void* d_X = nullptr;      // X panels
   void* d_D = nullptr;      // pivots, batch x n
-  void* d_lhat = nullptr;   // normalised factor / factor scratch
+  void* d_lhat = nullptr;   // normalised factor Lhat
   void* d_linv = nullptr;   // inverses of the diagonal blocks
   void* d_part = nullptr;   // step-3 partial products (level-local)
   void* d_ypart = nullptr;  // step-2 partial products (level-local)
@@ -253,7 +258,7 @@ struct pselinv_handle {
   // non-symmetric handles
   void* d_U = nullptr;      // U panels (U'_{j,i} at position (i, j))
   void* d_XU = nullptr;     // XU panels (X_{j,i} at position (i, j))
-  void* d_uhat = nullptr;   // Uhat^T / factor scratch of the U side
+  void* d_uhat = nullptr;   // Uhat^T
   void* d_uinv = nullptr;   // (U'_KK^T)^{-1}
   // FP64 emulation of step 2 on the bf16 tensor cores (opts.fp64_emulation)
   void* d_xs = nullptr;     // slices of the scaled X panels (16 bytes per entry)

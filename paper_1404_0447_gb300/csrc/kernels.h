@@ -14,6 +14,9 @@ namespace psi {
 // launched so calls after_previous() in all its threads before anything else in
 // memory, so that a kernel's end implies the end of all before it; the next one
 // may start only after that wait, so at most one kernel per stream waits resident.
+// One exception: merged_update takes its ticket before the wait.  A level's ticket is
+// touched by its own launch alone, and the memset that clears it precedes the chain's
+// first kernel, which starts in the ordinary way and so after the memset.
 __device__ __forceinline__ void after_previous() {
 #ifdef __CUDA_ARCH__
   cudaGridDependencySynchronize();
@@ -51,7 +54,7 @@ cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, unsigned block, size_t s
 // Per-batch-member sizes (elements of the scalar) of every batched array.
 struct Sizes {
   int64_t panel;  // L and X panels
-  int64_t lhat;   // normalised factor / factor scratch
+  int64_t lhat;   // normalised factor Lhat
   int64_t linv;   // diagonal-block inverses
   int64_t n;      // pivots
   int64_t part;   // step-3 partial products

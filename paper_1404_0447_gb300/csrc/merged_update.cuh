@@ -40,7 +40,7 @@ __device__ __forceinline__ void merged_update(const Task* __restrict__ tasks, co
   constexpr int P = Sc<T>::P, RF = kMergedRows / 8, LDP = kMergedRows + 1, KW = 32;
   __shared__ double part[4][P][8][LDP];
   __shared__ int sh_ticket;
-  if (threadIdx.x == 0) sh_ticket = atomicAdd(mq.ticket, 1);  // zeroed long before the previous kernel
+  if (threadIdx.x == 0) sh_ticket = atomicAdd(mq.ticket, 1);  // zeroed before the chain's first kernel
   __syncthreads();
   const int ticket = sh_ticket, copies = gridDim.y * gridDim.z, copy = ticket % copies;
   const Task tk = tasks[ticket / copies];

@@ -190,13 +190,15 @@ __global__ void __launch_bounds__(32 + SIDES * kFdUpdate) k_fdiag(FArgs f, const
     int j = 0;
     for (; j + 1 < w; ++j) {
       const T dj = shfl(c[0], j);
-      if (__any_sync(0xffffffffu, !by_reciprocal(dj))) break;  // a vote: no divergent code in the chain
+      if constexpr (Sc<T>::P == 1)
+        if (__any_sync(0xffffffffu, !by_reciprocal(dj))) break;  // a vote: no divergent code in the chain
       column(j, dj, true);
     }
-    for (; j + 1 < w; ++j) {  // from the first pivot out of range on
-      const T dj = shfl(c[0], j);
-      column(j, dj, by_reciprocal(dj));
-    }
+    if constexpr (Sc<T>::P == 1)
+      for (; j + 1 < w; ++j) {  // from the first pivot out of range on
+        const T dj = shfl(c[0], j);
+        column(j, dj, by_reciprocal(dj));
+      }
     // off the chain: a test of d_j inside the loop would hold this warp for the
     // FP64 compares of every column
     if (i < w) {

@@ -273,7 +273,7 @@ template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_syr2k_merged(AdjArgs a, const Task* __restrict__ tasks, MergedArgs mq) {
   const Sizes& sz = a.k.sz;
   merged_update<T, 2>(
-      tasks, mq, a.k.meta, a.k.desc, a.k.relidx, 1, a.k.status + kAdjointTimeoutWord,
+      tasks, mq, a.k.meta, a.k.desc, a.k.relidx, 1,
       [&](const SnMeta& m, int b, int, int p) {
         const T* Yb = (const T*)a.Yb + b * sz.lhat + m.lhat;
         const T* Lh = (const T*)a.k.Lhat + b * sz.lhat + m.lhat;

@@ -243,22 +243,27 @@ int ensure_device(pselinv_handle* h) {
   return PSELINV_OK;
 }
 
-// A ticket per level, the abort flag of the sequence's launches, a count per (Schur
-// group, copy): batch members and sides.  One memset at the start of a
-// factorisation or an adjoint clears them all.
+// Counters of the merged launches: a ticket per level, the adjoint's abort flag, a
+// count per (Schur group, copy), copy = batch member and side.  One memset at the
+// start of a factorisation or an adjoint clears them all.
 int64_t merged_counter_bytes(const pselinv_handle* h) {
   return (int64_t)sizeof(int) *
          (h->nlevels + 1 + (int64_t)h->schur_gcnt.size() * h->opts.batch * (h->opts.unsym ? 2 : 1));
 }
 
-int* merged_abort(const pselinv_handle* h) { return (int*)h->d_mctr + h->nlevels; }
+// The abort flag of the factorisation is its status word, which the next one clears.
+// The adjoint's status word outlives it, so its flag is another; the gather of the
+// gradient passes it on (a second address in the merged kernel took 17 registers and 2%
+// of a batch's adjoint).
+int* factor_abort(const pselinv_handle* h) { return (int*)h->d_status + psi::kFactorTimeoutWord; }
+int* adjoint_abort(const pselinv_handle* h) { return (int*)h->d_mctr + h->nlevels; }
 
-psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l) {
+psi::MergedArgs merged_args(const pselinv_handle* h, int32_t l, int* abort) {
   const int32_t g0 = h->schur_gptr[l];
   const psi::Range r = h->t_schurm.per_lv[l];
   psi::MergedArgs q;
   q.ticket = (int*)h->d_mctr + l;
-  q.abort = merged_abort(h);
+  q.abort = abort;
   q.gcnt = (const int32_t*)h->d_gcnt + g0;
   q.done = (int*)h->d_mctr + h->nlevels + 1 + (int64_t)g0 * h->opts.batch * (h->opts.unsym ? 2 : 1);
   q.ntile = (int)(r.end - r.begin);
@@ -907,7 +912,7 @@ int enqueue_factor(pselinv_handle* h, cudaStream_t st, bool bk) {
     if (merged(l)) {  // few tiles: near and far in one launch
       if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
       const psi::Range r = h->t_schurm.per_lv[l];
-      const psi::MergedArgs q = merged_args(h, l);
+      const psi::MergedArgs q = merged_args(h, l, factor_abort(h));
       PSI_CUDA(h, psi::launch_schur_merged(dt, f, q, tasks_at(h, h->off_schurm, r.begin), hi, hidep));
     } else if (h->far_after_near[bk][l]) {
       if (l + 1 < nl && !merged(l + 1)) PSI_CUDA(h, wait(hi, ev[1 + nl + l + 1], hidep));
@@ -1348,8 +1353,8 @@ int enqueue_adjoint(pselinv_handle* h, const psi::AdjArgs& a, cudaStream_t st) {
     PSI_CUDA(h, tiles(AdjKern::Lhbar, h->t_gemm1, h->off_gemm1, l, hi));  // step-2 slices of C
     PSI_CUDA(h, cudaEventRecord(ev[l], hi));
     if (h->schur_merged[l])
-      PSI_CUDA(h, psi::launch_adj_merged(a, merged_args(h, l), tasks_at(h, h->off_schurm, h->t_schurm.per_lv[l].begin),
-                                         hi));
+      PSI_CUDA(h, psi::launch_adj_merged(a, merged_args(h, l, adjoint_abort(h)),
+                                         tasks_at(h, h->off_schurm, h->t_schurm.per_lv[l].begin), hi));
     // otherwise per Schur group, its near and far tiles (adjacent, different target levels) as one launch
     for (int32_t g = h->schur_merged[l] ? h->schur_gptr[l + 1] : h->schur_gptr[l]; g < h->schur_gptr[l + 1]; ++g) {
       const int64_t b0 = h->schur_near[g].begin, b1 = h->schur_far[g].end;
@@ -1430,14 +1435,15 @@ int pselinv_selinv_adjoint(pselinv_handle* h, const void* d_G, int32_t g_kind, v
   PSI_CUDA(h, psi::launch_adj_per_sn(AdjSn::Seed, a, nullptr, h->nsn, std::min(h->max_width, 64), st));
   a.G = nullptr;  // read by the seed only
   if ((rc = arm_merged_waits(h, st))) return rc;
-  rc = replay_or_enqueue(h, &h->agraph_exec, &h->adjoint_ran, st, true,
+  rc = replay_or_enqueue(h, &h->agraph_exec, &h->adjoint_ran, st, false,
                          [&](cudaStream_t cs) { return enqueue_adjoint(h, a, cs); });
   if (rc) return rc;
   if ((rc = disarm_merged_waits(h, st))) return rc;
   // a gradient that a wait spoilt is NaN: nothing has read the status word yet, and a
   // read here would cost a host synchronisation (4% of a gradient on a 20^3 grid)
   PSI_CUDA(h, psi::launch_gather_values(h->opts.dtype, h->d_xb, (const int64_t*)h->d_valmap, nullptr, h->nnz_a,
-                                        d_gradA, sizes(h), st, merged_abort(h)));
+                                        d_gradA, sizes(h), st, adjoint_abort(h),
+                                        (int*)h->d_status + psi::kAdjointTimeoutWord));
   return PSELINV_OK;
 }
 

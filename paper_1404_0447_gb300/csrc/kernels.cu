@@ -95,15 +95,17 @@ __global__ void k_gather_values_lu(const T* __restrict__ XL, const T* __restrict
 
 // out[q] = X at the panel position of stored entry q; with a diagonal mask,
 // off-diagonal entries are doubled (gradient with respect to a stored value
-// that stands for both A_ij and A_ji).  NaN throughout where *invalid is set.
+// that stands for both A_ij and A_ji).  NaN throughout where *invalid is set, which
+// *report then says.
 template <class T>
 __global__ void k_gather_values(const T* __restrict__ X, int64_t panel_total, const int64_t* __restrict__ vmap,
                                 const uint8_t* __restrict__ diagmask, int64_t nnz, T* __restrict__ out,
-                                const int* __restrict__ invalid) {
+                                const int* __restrict__ invalid, int* report) {
   const int b = blockIdx.y;
   const T* Xb = X + (int64_t)b * panel_total;
   T* o = out + (int64_t)b * nnz;
   const bool bad = invalid && *invalid;
+  if (bad && threadIdx.x == 0) *report = 1;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x) {
     const T v = bad ? Sc<T>::nan() : Xb[vmap[q]];
     o[q] = (diagmask && !diagmask[q]) ? 2.0 * v : v;
@@ -831,7 +833,7 @@ __global__ void __launch_bounds__(TG_THREADS, (tile_min_ctas<T, BN>())) k_schur(
 template <class T>
 __global__ void __launch_bounds__(TG_THREADS) k_schur_merged(FArgs f, const Task* __restrict__ tasks, MergedArgs mq) {
   merged_update<T, 1>(
-      tasks, mq, f.meta, f.desc, f.relidx, f.sides, f.status + kFactorTimeoutWord,
+      tasks, mq, f.meta, f.desc, f.relidx, f.sides,
       [&](const SnMeta& m, int b, int side, int) {
         const int64_t po = b * f.sz.panel + m.panel + m.s;
         return UpdatePair<T>{(const T*)f.W[side] + po, (const T*)f.L[f.sides - 1 - side] + po, m.s + m.r};
@@ -1190,15 +1192,15 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
 
 template <class T>
 static cudaError_t gather_t(const void* X, const int64_t* vmap, const uint8_t* mask, int64_t nnz, void* out,
-                            const Sizes& sz, cudaStream_t st, const int* invalid) {
+                            const Sizes& sz, cudaStream_t st, const int* invalid, int* report) {
   k_gather_values<T><<<dim3(blocks_for(nnz, 256), sz.batch), 256, 0, st>>>((const T*)X, sz.panel, vmap, mask, nnz,
-                                                                          (T*)out, invalid);
+                                                                          (T*)out, invalid, report);
   return cudaGetLastError();
 }
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
-                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid) {
-  return dtype == PSELINV_C128 ? gather_t<Cplx>(X, vmap, diagmask, nnz, out, sz, st, invalid)
-                               : gather_t<double>(X, vmap, diagmask, nnz, out, sz, st, invalid);
+                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid, int* report) {
+  return dtype == PSELINV_C128 ? gather_t<Cplx>(X, vmap, diagmask, nnz, out, sz, st, invalid, report)
+                               : gather_t<double>(X, vmap, diagmask, nnz, out, sz, st, invalid, report);
 }
 
 // ---- tile-kernel launch for one task range of one variant ----

@@ -136,7 +136,7 @@ constexpr int kFactorTimeoutWord = 5, kAdjointTimeoutWord = 6;
 // copy), copy = side and batch member.
 struct MergedArgs {
   int* ticket;
-  int* abort;        // of the factorisation's or adjoint's launches: set when a wait ran out
+  int* abort;        // set when a wait ran out: the factorisation's status word, or the adjoint's flag
   const int32_t* gcnt;
   int* done;
   int ntile;         // tiles of one copy
@@ -164,9 +164,10 @@ cudaError_t launch_gather_values_lu(int dtype, const void* XL, const void* XU, c
                                     const uint8_t* flip, int64_t nnz, int upper, void* out, const Sizes& sz,
                                     cudaStream_t st);
 // diagmask == nullptr: plain gather; else off-diagonal entries doubled.  invalid: a
-// device flag; where it is set the output is NaN.
+// device flag; where it is set the output is NaN and *report becomes 1.
 cudaError_t launch_gather_values(int dtype, const void* X, const int64_t* vmap, const uint8_t* diagmask, int64_t nnz,
-                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid = nullptr);
+                                 void* out, const Sizes& sz, cudaStream_t st, const int* invalid = nullptr,
+                                 int* report = nullptr);
 // Tile kernels (Trsm, NormM, Lhat, Gemm1, Gemm2) over n tasks of one tile
 // width variant (BN = 8 << var).
 cudaError_t launch_tiles(Kern k, int var, const KArgs& a, const Task* tasks, int64_t n, cudaStream_t st,

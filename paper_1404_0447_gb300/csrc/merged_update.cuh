@@ -30,13 +30,11 @@ struct UpdatePair {
 
 // pairs(m, b, side, p): operands of product p < NP.  target(b, side): the panels
 // updated.  apply(x, v, diag): the new value of a target x given the products' sum.
-// report: the status word set when a wait runs out (mq.abort ends the launches of
-// this sequence only, so that a later one is not held up by it).
 template <class T, int NP, class PAIRS, class TARGET, class APPLY>
 __device__ __forceinline__ void merged_update(const Task* __restrict__ tasks, const MergedArgs& mq,
                                               const SnMeta* __restrict__ meta, const ColDesc* __restrict__ desc,
-                                              const int32_t* __restrict__ relidx, int sides, int* report,
-                                              const PAIRS& pairs, const TARGET& target, const APPLY& apply) {
+                                              const int32_t* __restrict__ relidx, int sides, const PAIRS& pairs,
+                                              const TARGET& target, const APPLY& apply) {
   constexpr int P = Sc<T>::P, RF = kMergedRows / 8, LDP = kMergedRows + 1, KW = 32;
   __shared__ double part[4][P][8][LDP];
   __shared__ int sh_ticket;
@@ -100,10 +98,7 @@ __device__ __forceinline__ void merged_update(const Task* __restrict__ tasks, co
 #pragma unroll
     for (int w = 1; w < 4; ++w) v[p] += part[w][p][t / kMergedRows][t % kMergedRows];
   }
-  if (grp > 0 && !cta_wait(mq.done + (int64_t)(grp - 1) * copies + copy, need, mq.spin_ns, mq.abort, 20)) {
-    if (t == 0) *(volatile int*)report = 1;
-    return;
-  }
+  if (grp > 0 && !cta_wait(mq.done + (int64_t)(grp - 1) * copies + copy, need, mq.spin_ns, mq.abort, 20)) return;
   if (live) {
     if constexpr (P == 1)
       *dst = apply(ld_cg(dst), v[0], ei == ec);

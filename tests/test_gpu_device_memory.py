@@ -33,7 +33,7 @@ def test_logdet_partials_are_sized_by_the_order(P):  # noqa: F811
 
 @pytest.mark.parametrize("what", ["factor", "autotune", "persistent", "pivoted", "adjoint"])
 def test_device_bytes_count_every_allocation(P, what):  # noqa: F811
-    """device_bytes against what the driver says was taken: an allocation takes whole
+    """device_bytes against what CUDA says was taken: an allocation takes whole
     2 MiB blocks at most, and streams, events and graphs take some blocks more."""
     import torch
     p = synth.grid3d(30)
